@@ -4,6 +4,7 @@
 // accepted mini-batch with the additive repair of the community totals and
 // the exact modularity change dQ(B) with its rollback test.
 #include <atomic>
+#include <type_traits>
 #include <cooperative_groups.h>
 
 #include "chunks.cuh"
@@ -79,7 +80,7 @@ __global__ void k_union(const int32_t* list, const int32_t* nlist, int32_t* stam
 // (level-r parents) restricted to neighbours of the same community.
 template <class WT>
 struct SweepArgs {
-  Adj<WT> out, in;
+  Adj<WT> out, in;  // both directions' rows lie in one pool: out.col == in.col, out.w == in.w
   int directed;
   const int32_t* lab;
   const int32_t* par;
@@ -98,17 +99,54 @@ struct SweepArgs {
   DevScalars* stats;
 };
 
-__device__ inline void hash_add(int32_t* K, int64_t* V, uint32_t mask, int32_t key, int64_t w) {
-  uint32_t h = hash32((uint32_t)key) & mask;
-  while (true) {
-    const int32_t prev = atomicCAS(&K[h], -1, key);
-    if (prev == -1 || prev == key) {
-      atomicAdd((unsigned long long*)&V[h], (unsigned long long)w);
-      return;
-    }
-    h = (h + 1) & mask;
+// A node's shared-memory table: keys and the sums of their weights.  Shared
+// memory has no native 64-bit add (it becomes a compare-and-swap loop that
+// lanes with one key run through one after the other), so sums are kept in
+// 32-bit words: one word when the gains fit int64 (then m < 2^30 and no sum
+// of a node's in- and out-weights reaches 2^31), else a low and a high word
+// with the carry passed on.  Both are exact.  Measured per level-0 sweep of a
+// batch of 10^5 on the 2M-vertex power-law graph, 64-bit sums before: 128-
+// thread blocks 873 -> 263 us, warps 781 -> 456 us, 8-lane groups 398 -> 198.
+template <bool WIDE>
+struct Tab {
+  int32_t* K;
+  uint32_t* lo;
+  uint32_t* hi;  // WIDE only
+  __device__ void clear4(uint32_t k) const {  // slots k .. k + 3, k a multiple of 4
+    *(int4*)(K + k) = make_int4(-1, -1, -1, -1);
+    *(uint4*)(lo + k) = make_uint4(0, 0, 0, 0);
+    if (WIDE) *(uint4*)(hi + k) = make_uint4(0, 0, 0, 0);
   }
-}
+  __device__ void add(uint32_t mask, int32_t key, int64_t w) const {
+    // the upper bits of a multiplicative hash (H = mask + 1 slots)
+    uint32_t h = __umulhi((uint32_t)key * 0x9E3779B1u, mask + 1);
+    while (true) {
+      const int32_t prev = atomicCAS(&K[h], -1, key);
+      if (prev == -1 || prev == key) break;
+      h = (h + 1) & mask;
+    }
+    const uint32_t wl = (uint32_t)w;
+    if (!WIDE) {
+      atomicAdd(&lo[h], wl);
+    } else {
+      const uint32_t old = atomicAdd(&lo[h], wl);
+      const uint32_t up = (uint32_t)((uint64_t)w >> 32) + (old + wl < old ? 1u : 0u);
+      if (up) atomicAdd(&hi[h], up);
+    }
+  }
+  __device__ int64_t sum(uint32_t h) const {
+    return WIDE ? (int64_t)(((uint64_t)hi[h] << 32) | lo[h]) : (int64_t)lo[h];
+  }
+};
+
+// slot bytes of a table in the gain type GT (int64: one-word sums)
+template <class GT>
+constexpr bool wide_sums = sizeof(GT) > 8;
+// a staged entry weight: below m, so one word with one-word sums
+template <class GT>
+using StageW = std::conditional_t<wide_sums<GT>, int64_t, uint32_t>;
+template <class GT>
+constexpr int tab_slot = wide_sums<GT> ? 12 : 8;
 
 __device__ inline int64_t hash_get(const int32_t* K, const int64_t* V, uint32_t mask, int32_t key) {
   uint32_t h = hash32((uint32_t)key) & mask;
@@ -117,62 +155,6 @@ __device__ inline int64_t hash_get(const int32_t* K, const int64_t* V, uint32_t 
     if (k == key) return V[h];
     if (k == -1) return 0;
     h = (h + 1) & mask;
-  }
-}
-
-template <class WT, int MODE>
-__device__ inline void accumulate(const SweepArgs<WT>& A, const Adj<WT>& adj, int32_t v, int32_t cv_, int32_t* K,
-                                  int64_t* V, uint32_t mask, int tid, int nthreads) {
-  // ACC entries per thread per step: their loads and label gathers are all in
-  // flight before the first insert
-  constexpr int ACC = 4;
-  const int64_t o = adj.off[v];
-  const int32_t l = adj.len[v];
-  for (int32_t k0 = tid; k0 < l; k0 += ACC * nthreads) {
-    int32_t u[ACC];
-    int64_t w[ACC];
-#pragma unroll
-    for (int j = 0; j < ACC; ++j) {
-      const int32_t k = k0 + j * nthreads;
-      u[j] = k < l ? adj.col[o + k] : -1;
-      w[j] = k < l ? (int64_t)adj.w[o + k] : 0;
-    }
-    int32_t key[ACC];
-#pragma unroll
-    for (int j = 0; j < ACC; ++j) {
-      key[j] = -1;
-      if (u[j] >= 0 && u[j] != v && (MODE == 0 || A.lab[u[j]] == cv_)) key[j] = MODE == 0 ? A.lab[u[j]] : A.par[u[j]];
-    }
-#pragma unroll
-    for (int j = 0; j < ACC; ++j)
-      if (key[j] >= 0) hash_add(K, V, mask, key[j], w[j]);
-  }
-}
-
-// accumulate() for a row whose offset and length the caller already holds.
-template <class WT, int MODE>
-__device__ inline void accumulate_row(const SweepArgs<WT>& A, const int32_t* col, const WT* wt, int64_t o, int32_t l,
-                                      int32_t v, int32_t cv_, int32_t* K, int64_t* V, uint32_t mask, int tid,
-                                      int nthreads) {
-  constexpr int ACC = 4;
-  for (int32_t k0 = tid; k0 < l; k0 += ACC * nthreads) {
-    int32_t u[ACC];
-    int64_t w[ACC];
-#pragma unroll
-    for (int j = 0; j < ACC; ++j) {
-      const int32_t k = k0 + j * nthreads;
-      u[j] = k < l ? col[o + k] : -1;
-      w[j] = k < l ? (int64_t)wt[o + k] : 0;
-    }
-    int32_t key[ACC];
-#pragma unroll
-    for (int j = 0; j < ACC; ++j) {
-      key[j] = -1;
-      if (u[j] >= 0 && u[j] != v && (MODE == 0 || A.lab[u[j]] == cv_)) key[j] = MODE == 0 ? A.lab[u[j]] : A.par[u[j]];
-    }
-#pragma unroll
-    for (int j = 0; j < ACC; ++j)
-      if (key[j] >= 0) hash_add(K, V, mask, key[j], w[j]);
   }
 }
 
@@ -196,6 +178,41 @@ __device__ inline NodeMeta node_meta(const SweepArgs<WT>& A, int32_t v) {
   m.ko = A.kout[v];
   m.ki = A.kin[v];
   return m;
+}
+
+// Adds a node's entries (its out-row, then its in-row) to its table; weights
+// towards its own community (MODE 0; most entries, once communities have
+// formed) are summed in a register instead, as they would all meet in one
+// slot.
+template <class WT, int MODE, bool WIDE, bool DIR>
+__device__ inline void accumulate(const SweepArgs<WT>& A, const NodeMeta& m, const Tab<WIDE>& T, uint32_t mask,
+                                  int tid, int nthreads, std::conditional_t<WIDE, int64_t, uint32_t>& own) {
+  // ACC entries per thread per step: their loads and label gathers are all in
+  // flight before the first insert
+  constexpr int ACC = 4;
+  const int32_t l = DIR ? m.lo + m.li : m.lo;
+  for (int32_t k0 = tid; k0 < l; k0 += ACC * nthreads) {
+    int32_t u[ACC];
+    std::conditional_t<WIDE, int64_t, uint32_t> w[ACC];
+#pragma unroll
+    for (int j = 0; j < ACC; ++j) {
+      const int32_t k = k0 + j * nthreads;
+      const int64_t at = (!DIR || k < m.lo ? m.oo : m.oi - m.lo) + k;
+      u[j] = k < l ? A.out.col[at] : -1;
+      w[j] = k < l ? A.out.w[at] : 0;
+    }
+    int32_t key[ACC];
+#pragma unroll
+    for (int j = 0; j < ACC; ++j) {
+      key[j] = -1;
+      if (u[j] >= 0 && u[j] != m.v && (MODE == 0 || A.lab[u[j]] == m.a)) key[j] = MODE == 0 ? A.lab[u[j]] : A.par[u[j]];
+    }
+#pragma unroll
+    for (int j = 0; j < ACC; ++j) {
+      if (MODE == 0 && key[j] == m.a) own += w[j];
+      else if (key[j] >= 0) T.add(mask, key[j], w[j]);
+    }
+  }
 }
 
 // Exact gain of v into key (see Eq. 2 with a' = a \ {v}).
@@ -267,50 +284,38 @@ __device__ inline BestG<GT> seg_best(BestG<GT> x) {
   return x;
 }
 
-// Evaluates the slots start, start + step, ... < H of a node's table: the
-// exact gain (as gain_of) into every target but `self`, the best kept in b.
-// EV slots per step have their totals gathered before any gain is computed.
-template <int MODE, class GT>
-__device__ inline void eval_slots(const int32_t* K, const int64_t* V, uint32_t H, uint32_t start, uint32_t step,
-                                  int32_t self, int32_t a, int64_t wa, int64_t ko, int64_t ki, const int64_t* Tout,
+// Evaluates a node's table (H slots, a multiple of 4; thread `start` of
+// `step`): the exact gain (gain_of, with what does not depend on the target
+// collected in g0) into every target but `self`, the best kept in b.  Most
+// slots are empty, so the keys are read four at a time; the occupied ones are
+// emptied on the way, which leaves a clean table for the next node.  The terms
+// may wrap in GT where the gain itself fits, hence the unsigned arithmetic.
+template <int MODE, class GT, class CT>
+__device__ inline void eval_slots(const Tab<wide_sums<GT>>& T, uint32_t H, uint32_t start, uint32_t step, int32_t self,
+                                  int32_t a, int64_t wa, int64_t ko, int64_t ki, int directed, const int64_t* Tout,
                                   const int64_t* Tin, int64_t m, int64_t gn, int64_t gd, int64_t mult, BestG<GT>& b,
-                                  int64_t& pairs) {
-  constexpr int EV = 1;
-  const int64_t tia = MODE == 0 ? Tin[a] : 0, toa = MODE == 0 ? Tout[a] : 0;
-  for (uint32_t k0 = start; k0 < H; k0 += EV * step) {
-    int32_t key[EV];
-    int64_t acc[EV], ti[EV], to[EV];
+                                  CT& pairs) {
+  using UT = std::conditional_t<(sizeof(GT) > 8), unsigned __int128, uint64_t>;
+  const UT cw = (UT)(gd * mult) * (UT)m, co = (UT)gn * (UT)ko, ci = (UT)gn * (UT)ki;
+  UT g0 = 0;
+  if (MODE == 0) g0 = co * (UT)(GT)(Tin[a] - ki) + ci * (UT)(GT)(Tout[a] - ko) - cw * (UT)wa;
+  for (uint32_t k0 = 4 * start; k0 < H; k0 += 4 * step) {
+    const int4 kk = *(const int4*)(T.K + k0);
+    const int32_t key[4] = {kk.x, kk.y, kk.z, kk.w};
+    if ((key[0] & key[1] & key[2] & key[3]) == -1) continue;
 #pragma unroll
-    for (int j = 0; j < EV; ++j) {
-      const uint32_t k = k0 + j * step;
-      key[j] = k < H ? K[k] : -1;
-      if (key[j] == self) key[j] = -1;
-      acc[j] = key[j] >= 0 ? V[k] : 0;
-    }
-#pragma unroll
-    for (int j = 0; j < EV; ++j) {
-      ti[j] = key[j] >= 0 ? Tin[key[j]] : 0;
-      to[j] = key[j] >= 0 ? Tout[key[j]] : 0;
-    }
-#pragma unroll
-    for (int j = 0; j < EV; ++j) {
-      if (key[j] < 0) continue;
+    for (int j = 0; j < 4; ++j) {
+      if (key[j] < 0 || (MODE == 1 && key[j] == self)) continue;
       ++pairs;
-      GT g;
-      if (MODE == 0) {
-        const GT dw = (GT)mult * (GT)(acc[j] - wa);
-        const GT dd = (GT)ko * (GT)(ti[j] - tia + ki) + (GT)ki * (GT)(to[j] - toa + ko);
-        g = (GT)gd * (GT)m * dw - (GT)gn * dd;
-      } else {
-        const GT dw = (GT)mult * (GT)acc[j];
-        const GT dd = (GT)ko * (GT)ti[j] + (GT)ki * (GT)to[j];
-        g = (GT)gd * (GT)m * dw - (GT)gn * dd;
-      }
+      const UT ti = (UT)Tin[key[j]];
+      const UT dd = directed ? co * ti + ci * (UT)Tout[key[j]] : (co + ci) * ti;
+      const GT g = (GT)(g0 + cw * (UT)T.sum(k0 + j) - dd);
       if (g > 0) {
         BestG<GT> c{g, key[j], 1};
         if (better(c, b)) b = c;
       }
     }
+    T.clear4(k0);
   }
 }
 
@@ -339,56 +344,67 @@ __device__ inline void emit_cand(const SweepArgs<WT>& A, int32_t v, int32_t src,
 // node).  All groups
 // of a warp advance together, so the warp-wide shuffles of the argmax see
 // every lane; a group without a node in an iteration only takes part in them.
+// Bound by instructions and by the latency of the dependent loads (row
+// bounds, entries, labels, totals).  Occupancy hides the latter best: staging
+// the next node as the block kernel does (64 registers, 4 blocks a SM) took
+// 681 us where this form took 456.  Fewer instructions then brought warps to
+// 206 us and groups to 176 (2M-vertex power-law graph, batch of 10^5): one
+// multiply to hash, the target-independent terms of the gain collected, keys
+// read four at a time, no separate clearing, no argmax without a candidate.
 template <class WT, int MODE, int G, class GT>
-__global__ void __launch_bounds__(TPB, 5) k_sweep_group(SweepArgs<WT> A, const int32_t* list, const int32_t* nlist) {
+__global__ void __launch_bounds__(TPB, wide_sums<GT> ? 4 : 6) k_sweep_group(SweepArgs<WT> A, const int32_t* list,
+                                                                             const int32_t* nlist) {
   constexpr int HG = G == 8 ? HG8 : HG32;
   constexpr int GPW = 32 / G;  // groups per warp
-  __shared__ int32_t hk[TPB / G][HG];
-  __shared__ int64_t hv[TPB / G][HG];
+  constexpr bool WIDE = wide_sums<GT>;
+  __shared__ __align__(16) int32_t hk[TPB / G][HG];
+  __shared__ __align__(16) uint32_t hv[WIDE ? 2 : 1][TPB / G][HG];
   const int lane = threadIdx.x & 31, gl = threadIdx.x & (G - 1);
-  int32_t* K = hk[threadIdx.x / G];
-  int64_t* V = hv[threadIdx.x / G];
+  const Tab<WIDE> T{hk[threadIdx.x / G], hv[0][threadIdx.x / G], WIDE ? hv[WIDE ? 1 : 0][threadIdx.x / G] : nullptr};
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t ngroups = ((int64_t)gridDim.x * blockDim.x) / G;
   const int32_t nl = *nlist;
   const int64_t mult = A.directed ? 1 : 2;
-  int64_t scanned = 0, pairs = 0, nodes = 0;
-  for (int64_t base = warp * GPW; base < nl; base += ngroups) {
-    const int64_t t = base + lane / G;
+  uint32_t entries = 0, pairs = 0, nodes = 0;
+  // the list is read one node ahead, off the chain of dependent loads
+  int64_t t = warp * GPW + lane / G;
+  int32_t v_next = t < nl ? list[t] : 0;
+  for (uint32_t k = 4 * gl; k < HG; k += 4 * G) T.clear4(k);
+  __syncwarp();
+  for (int64_t base = warp * GPW; base < nl; base += ngroups, t += ngroups) {
     const bool act = t < nl;
-    const int32_t v = act ? list[t] : 0;
-    const int32_t deg = act ? A.out.len[v] + (A.directed ? A.in.len[v] : 0) : 0;
+    const int32_t v = v_next;
+    v_next = t + ngroups < nl ? list[t + ngroups] : 0;
+    NodeMeta cur{};
+    if (act) cur = node_meta(A, v);
+    const int32_t deg = cur.lo + cur.li, a = cur.a;
     int H = G;
     while (H < 2 * deg && H < HG) H <<= 1;
-    for (int k = gl; k < H; k += G) {
-      K[k] = -1;
-      V[k] = 0;
-    }
-    __syncwarp();
     BestG<GT> b{0, 0, 0};
-    int32_t a = 0;
-    if (act) {
-      a = A.lab[v];
-      accumulate<WT, MODE>(A, A.out, v, a, K, V, H - 1, gl, G);
-      if (A.directed) accumulate<WT, MODE>(A, A.in, v, a, K, V, H - 1, gl, G);
-      if (gl == 0) {
-        scanned += deg;
-        ++nodes;
-      }
+    StageW<GT> wa = 0;
+    if (A.directed) accumulate<WT, MODE, WIDE, true>(A, cur, T, H - 1, gl, G, wa);
+    else accumulate<WT, MODE, WIDE, false>(A, cur, T, H - 1, gl, G, wa);
+    if (act && gl == 0) {
+      entries += deg;
+      ++nodes;
     }
     __syncwarp();
-    if (act) {
-      const int64_t wa = MODE == 0 ? hash_get(K, V, H - 1, a) : 0;
-      const int64_t ko = A.kout[v], ki = A.kin[v];
-      eval_slots<MODE, GT>(K, V, (uint32_t)H, (uint32_t)gl, (uint32_t)G, MODE == 0 ? a : v, a, wa, ko, ki, A.Tout,
-                           A.Tin, A.m, A.gn, A.gd, mult, b, pairs);
+    if (MODE == 0) {
+#pragma unroll
+      for (int d = G / 2; d > 0; d >>= 1) wa += __shfl_xor_sync(0xffffffffu, wa, d, G);
     }
-    b = seg_best<GT, G>(b);
-    if (act && gl == 0 && b.have) emit_cand(A, v, MODE == 0 ? a : v, b);
+    if (act)
+      eval_slots<MODE, GT>(T, (uint32_t)H, (uint32_t)gl, (uint32_t)G, MODE == 0 ? a : v, a, (int64_t)wa, cur.ko, cur.ki, A.directed,
+                           A.Tout, A.Tin, A.m, A.gn, A.gd, mult, b, pairs);
+    // most nodes stay where they are: no argmax without a positive gain
+    if (__any_sync(0xffffffffu, b.have)) {
+      b = seg_best<GT, G>(b);
+      if (act && gl == 0 && b.have) emit_cand(A, v, MODE == 0 ? a : v, b);
+    }
     __syncwarp();
   }
-  const int64_t bytes = warp_sum_i64(sweep_bytes<WT, MODE>(A.directed, scanned, nodes, pairs));
-  scanned = warp_sum_i64(scanned);
+  const int64_t bytes = warp_sum_i64(sweep_bytes<WT, MODE>(A.directed, entries, nodes, pairs));
+  const int64_t scanned = warp_sum_i64(entries);
   if (lane == 0 && (scanned | bytes)) {
     atomic_add_i64(A.scanned, scanned);
     atomic_add_i64(&A.stats->sw_entries[G == 32 ? 1 : 0], scanned);
@@ -401,19 +417,22 @@ __global__ void __launch_bounds__(TPB, 5) k_sweep_group(SweepArgs<WT> A, const i
 // Entries of a node's rows staged in registers: entry k of the node is its
 // out-row entry k (k < lo) or its in-row entry k - lo; thread tid holds the
 // entries tid + j * NT.  First the neighbour ids and weights ...
-template <class WT, int NT, int ACC>
-__device__ inline void stage_rows(const SweepArgs<WT>& A, const NodeMeta& m, int32_t (&u)[ACC], int64_t (&w)[ACC]) {
+template <class WT, int NT, int ACC, class SW>
+__device__ inline void stage_rows(const SweepArgs<WT>& A, const NodeMeta& m, int32_t (&u)[ACC], SW (&w)[ACC]) {
+  if (A.directed) {
 #pragma unroll
-  for (int j = 0; j < ACC; ++j) {
-    const int32_t k = (int32_t)threadIdx.x + j * NT;
-    u[j] = -1;
-    w[j] = 0;
-    if (k < m.lo) {
-      u[j] = A.out.col[m.oo + k];
-      w[j] = (int64_t)A.out.w[m.oo + k];
-    } else if (k < m.lo + m.li) {
-      u[j] = A.in.col[m.oi + (k - m.lo)];
-      w[j] = (int64_t)A.in.w[m.oi + (k - m.lo)];
+    for (int j = 0; j < ACC; ++j) {
+      const int32_t k = (int32_t)threadIdx.x + j * NT;
+      const int64_t at = (k < m.lo ? m.oo : m.oi - m.lo) + k;
+      u[j] = k < m.lo + m.li ? A.out.col[at] : -1;
+      w[j] = k < m.lo + m.li ? (SW)A.out.w[at] : 0;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < ACC; ++j) {
+      const int32_t k = (int32_t)threadIdx.x + j * NT;
+      u[j] = k < m.lo ? A.out.col[m.oo + k] : -1;
+      w[j] = k < m.lo ? (SW)A.out.w[m.oo + k] : 0;
     }
   }
 }
@@ -442,70 +461,81 @@ __device__ inline void stage_keys(const SweepArgs<WT>& A, int32_t v, int32_t a, 
 // that has its offsets, lengths and strengths loaded one node further ahead,
 // so a node's fill only inserts into shared memory.  Entries beyond the
 // staged HMAX/2 (not produced by the default bins) are inserted directly.
+// With the evaluation emptying the table, two barriers a node instead of
+// four: 263 -> 215 us for the rows of 97..1024 entries of a 10^5 batch on the
+// 2M-vertex power-law graph, 249 -> 214 us for 10^4 on the R-MAT of 2^20.
 template <class WT, int MODE, int NT, int HMAX, class GT>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, const int32_t* list,
                                                                const int32_t* nlist) {
   extern __shared__ unsigned char smem[];
+  constexpr bool WIDE = wide_sums<GT>;
   __shared__ BestG<GT> wb[NT / 32];
+  __shared__ int64_t wown[NT / 32];
   constexpr int ACC = HMAX / (2 * NT);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const Tab<WIDE> T{(int32_t*)smem, (uint32_t*)smem + HMAX, WIDE ? (uint32_t*)smem + 2 * HMAX : nullptr};
   const int32_t nl = *nlist;
   const int64_t mult = A.directed ? 1 : 2;
   int64_t ent_all = 0, nodes = 0, pairs_all = 0;
   NodeMeta cur{}, nxt{};
   int32_t ek[ACC];
-  int64_t ew[ACC];
+  StageW<GT> ew[ACC];
   if (blockIdx.x < nl) {
     cur = node_meta(A, list[blockIdx.x]);
-    stage_rows<WT, NT, ACC>(A, cur, ek, ew);
+    stage_rows<WT, NT>(A, cur, ek, ew);
     stage_keys<WT, MODE, ACC>(A, cur.v, cur.a, ek);
   }
   if (blockIdx.x + gridDim.x < nl) nxt = node_meta(A, list[blockIdx.x + gridDim.x]);
+  if (blockIdx.x < nl)
+    for (uint32_t k = 4 * threadIdx.x; k < HMAX; k += 4 * NT) T.clear4(k);
+  __syncthreads();
   for (int64_t t = blockIdx.x; t < nl; t += gridDim.x) {
     const int32_t v = cur.v;
-    int64_t* V = (int64_t*)smem;
-    int32_t* K = (int32_t*)(smem + sizeof(int64_t) * HMAX);
     const int64_t d = (int64_t)cur.lo + cur.li;
     uint32_t H = 256;
     while (H < 2 * d && H < HMAX) H <<= 1;
-    for (uint32_t k = threadIdx.x; k < H; k += NT) {
-      K[k] = -1;
-      V[k] = 0;
-    }
-    __syncthreads();
     const int32_t a = cur.a;
+    StageW<GT> own = 0;
 #pragma unroll
-    for (int j = 0; j < ACC; ++j)
-      if (ek[j] >= 0) hash_add(K, V, H - 1, ek[j], ew[j]);
+    for (int j = 0; j < ACC; ++j) {
+      if (MODE == 0 && ek[j] == a) own += ew[j];
+      else if (ek[j] >= 0) T.add(H - 1, ek[j], ew[j]);
+    }
     if (d > ACC * NT) {  // entries beyond the staged ones
       for (int64_t k = ACC * NT + threadIdx.x; k < d; k += NT) {
-        int32_t x;
-        int64_t wx;
-        if (k < cur.lo) {
-          x = A.out.col[cur.oo + k];
-          wx = (int64_t)A.out.w[cur.oo + k];
-        } else {
-          x = A.in.col[cur.oi + (k - cur.lo)];
-          wx = (int64_t)A.in.w[cur.oi + (k - cur.lo)];
-        }
-        int32_t kx[1] = {x};
+        const int64_t at = (k < cur.lo ? cur.oo : cur.oi - cur.lo) + k;
+        const int64_t wx = (int64_t)A.out.w[at];
+        int32_t kx[1] = {A.out.col[at]};
         stage_keys<WT, MODE, 1>(A, v, a, kx);
-        if (kx[0] >= 0) hash_add(K, V, H - 1, kx[0], wx);
+        if (MODE == 0 && kx[0] == a) own += (StageW<GT>)wx;
+        else if (kx[0] >= 0) T.add(H - 1, kx[0], wx);
       }
+    }
+    if (MODE == 0) {
+      if constexpr (WIDE) own = warp_sum_i64(own);
+      else own = __reduce_add_sync(0xffffffffu, own);
+      if (lane == 0) wown[wid] = own;
     }
     __syncthreads();
     const bool has_next = t + gridDim.x < nl;
-    if (has_next) stage_rows<WT, NT, ACC>(A, nxt, ek, ew);  // in flight during the evaluation
-    const int64_t wa = MODE == 0 ? hash_get(K, V, H - 1, a) : 0;
+    if (has_next) stage_rows<WT, NT>(A, nxt, ek, ew);  // in flight during the evaluation
+    int64_t wa = 0;
+    if (MODE == 0) {
+#pragma unroll
+      for (int w = 0; w < NT / 32; ++w) wa += wown[w];
+    }
     const int64_t ko = cur.ko, ki = cur.ki;
     BestG<GT> b{0, 0, 0};
     int64_t pairs = 0;
-    eval_slots<MODE, GT>(K, V, H, threadIdx.x, NT, MODE == 0 ? a : v, a, wa, ko, ki, A.Tout, A.Tin, A.m, A.gn, A.gd,
+    eval_slots<MODE, GT>(T, H, threadIdx.x, NT, MODE == 0 ? a : v, a, wa, ko, ki, A.directed, A.Tout, A.Tin, A.m, A.gn, A.gd,
                          mult, b, pairs);
     if (has_next) stage_keys<WT, MODE, ACC>(A, nxt.v, nxt.a, ek);  // label gathers overlap the argmax
-    b = seg_best<GT, 32>(b);
+    if (__any_sync(0xffffffffu, b.have)) b = seg_best<GT, 32>(b);
     if (lane == 0) wb[wid] = b;
     pairs_all += pairs;
+    // two barriers a node: this one also separates the evaluation (which
+    // empties the table) from the next node's inserts, and the next node's
+    // barrier separates thread 0's reads of wb from their next writes
     __syncthreads();
     if (threadIdx.x == 0) {
       BestG<GT> r = wb[0];
@@ -515,7 +545,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, 
       ent_all += d;
       ++nodes;
     }
-    __syncthreads();
     cur = nxt;
     if (t + 2 * (int64_t)gridDim.x < nl) nxt = node_meta(A, list[t + 2 * (int64_t)gridDim.x]);
   }
@@ -1307,20 +1336,20 @@ static bool sweep_gain_fits_i64(const ldl_ctx& c) {
 // The bins of nodes with at most 2048 entries, in the gain type GT.
 template <class WT, int MODE, class GT>
 static void sweep_bins(ldl_ctx& c, const SweepArgs<WT>& A, int64_t n_hint, cudaEvent_t* kev) {
-  k_sweep_group<WT, MODE, 8, GT><<<grid_for(n_hint * 8, TPB, 5), TPB, 0, c.s>>>(A, c.binT.p, c.dcnt + K_TINY);
+  k_sweep_group<WT, MODE, 8, GT><<<grid_for(n_hint * 8, TPB, 6), TPB, 0, c.s>>>(A, c.binT.p, c.dcnt + K_TINY);
   CKL("k_sweep_group<8>");
   if (kev) CK(cudaEventRecord(kev[1], c.s));
-  k_sweep_group<WT, MODE, 32, GT><<<grid_for(n_hint * 32, TPB, 5), TPB, 0, c.s>>>(A, c.binS.p, c.dcnt + K_SMALL);
+  k_sweep_group<WT, MODE, 32, GT><<<grid_for(n_hint * 32, TPB, 6), TPB, 0, c.s>>>(A, c.binS.p, c.dcnt + K_SMALL);
   CKL("k_sweep_group<32>");
   if (kev) CK(cudaEventRecord(kev[2], c.s));
   {
-    const size_t sm = (sizeof(int64_t) + sizeof(int32_t)) * 2048;
+    const size_t sm = (size_t)tab_slot<GT> * 2048;
     k_sweep_block<WT, MODE, 128, 2048, GT><<<grid_for(n_hint, 1, 16), 128, sm, c.s>>>(A, c.binM.p, c.dcnt + K_MID);
     CKL("k_sweep_block(mid1)");
   }
   if (kev) CK(cudaEventRecord(kev[3], c.s));
   {
-    const size_t sm = (sizeof(int64_t) + sizeof(int32_t)) * HB;
+    const size_t sm = (size_t)tab_slot<GT> * HB;
     CK(cudaFuncSetAttribute(k_sweep_block<WT, MODE, 256, HB, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)sm));
     k_sweep_block<WT, MODE, 256, HB, GT><<<grid_for(n_hint, 1, 4), 256, sm, c.s>>>(A, c.binM2.p, c.dcnt + K_MID2);
