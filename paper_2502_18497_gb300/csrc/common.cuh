@@ -323,18 +323,12 @@ struct DevScalars {
   int64_t need;     // pool slots needed by relocation
   int64_t need2;    // second accumulator (record counts)
   int64_t scanned;  // adjacency entries scanned
-  int64_t err_key;  // packed (index << 8 | status) of the first failing update
-  int64_t pool_top;
-  int64_t seg_n, seg_stot, seg_wtot;  // CSR update: segments, scratch and rebuild totals
+  int64_t err_key;  // packed (index << 8 | status) of the first update invalid by itself
+  int64_t err_seq;  // the same for an update that its predecessors make invalid
+  int64_t agg_recs;  // aggregate records of the batch
+  int64_t seg_n;     // CSR update: segments
+  int64_t plan_bad;  // last CSR update that met an impossible record
   int64_t sw_entries[KS_GROUPS];  // per sweep kernel group: adjacency entries read since statistics
                                   // were enabled
   int64_t sw_bytes[KS_GROUPS];    // algorithmic bytes of the same sweeps
-  int32_t cnt[16];  // list counters
-  int32_t undecided;
-  int32_t pad;
-};
-
-enum {  // indices into DevScalars::cnt
-  C_LIST0 = 0, C_LIST1, C_LIST2, C_LIST3, C_LIST4, C_LIST5, C_LIST6, C_LIST7,
-  C_CAND, C_REC, C_SEG, C_ACC, C_TC, C_X, C_Y, C_Z
 };

@@ -8,6 +8,8 @@
 // loses entries is rebuilt by a flattened scatter in which every kept entry
 // and every inserted entry computes its own destination, so hub rows spread
 // over the whole GPU instead of one warp.
+#include <algorithm>
+
 #include "csr.cuh"
 #include "prims.cuh"
 
@@ -18,146 +20,230 @@ namespace {
 
 constexpr int TPB = 256;
 
-// binary search of col in a sorted row: returns the lower bound index
-__device__ inline int32_t row_lower_bound(const int32_t* col, int64_t off, int32_t len, int32_t c) {
-  int32_t lo = 0, hi = len;
-  while (lo < hi) {
-    const int32_t mid = (lo + hi) >> 1;
-    if (col[off + mid] < c) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
+// ---- planning an update: records -> rows (segments) -> what each row needs
+// A record list: n records, or mul * *n_dev of them with n an upper bound.
+struct RecN {
+  int64_t n;
+  const int32_t* n_dev;
+  int mul;
+  __device__ int64_t count() const { return n_dev ? min(n, (int64_t)mul * *n_dev) : n; }
+};
 
+// Per-record and per-segment arrays of an update (see CsrScratch).
+struct PlanOut {
+  int32_t *pos, *lb, *segid, *pins, *pdel;
+  int64_t* oldw;
+  int64_t *seg, *segrow;
+  int32_t* newcap;
+  int64_t *soff, *woff, *noff;
+  int64_t* nseg;  // device: number of segments
+  u64* bad;       // device: the last plan number that met an impossible record
+  u64 plan;       // this plan's number
+};
+
+struct Rec {
+  int32_t ins, del, head;
+};
+
+// Matches record i in its (sorted) row and says what it does to it; the
+// endpoints of an entry it removes go to *t (rows below t.rows).
 template <class WT>
-__global__ void k_lookup(const int64_t* off, const int32_t* len, const int32_t* col, const WT* w, const u64* keys,
-                         int64_t nrec, int bshift, int32_t* pos, int32_t* lb, int64_t* oldw) {
+__device__ inline Rec match_record(const int64_t* off, const int32_t* len, const int32_t* col, const WT* w,
+                                   const u64* keys, const int64_t* delta, int64_t i, int bshift, const PlanOut& o,
+                                   const DelTrack& t) {
   const u64 cmask = (((u64)1) << bshift) - 1;
-  GRID_STRIDE(i, nrec) {
-    const int64_t row = (int64_t)(keys[i] >> bshift);
-    const int32_t c = (int32_t)(keys[i] & cmask);
-    const int64_t o = off[row];
-    const int32_t l = len[row];
-    const int32_t p = row_lower_bound(col, o, l, c);
-    const bool found = p < l && col[o + p] == c;
-    pos[i] = found ? p : -1;
-    if (lb) lb[i] = p;
-    oldw[i] = found ? (int64_t)w[o + p] : 0;
-  }
-}
-
-// per record: insert / delete flags and segment heads (row changes)
-__global__ void k_rec_flags(const u64* keys, const int64_t* delta, int64_t nrec, int bshift, const int32_t* pos,
-                            const int64_t* oldw, int32_t* fins, int32_t* fdel, int32_t* fhead, int32_t* err) {
-  GRID_STRIDE(i, nrec) {
-    const bool found = pos[i] >= 0;
-    const int64_t nv = (found ? oldw[i] : 0) + delta[i];
-    if (nv < 0 || (!found && nv == 0)) atomicExch(err, 1);
-    fins[i] = (!found && nv > 0) ? 1 : 0;
-    fdel[i] = (found && nv == 0) ? 1 : 0;
-    fhead[i] = (i == 0 || (keys[i] >> bshift) != (keys[i - 1] >> bshift)) ? 1 : 0;
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    fins[nrec] = 0;
-    fdel[nrec] = 0;
-    fhead[nrec] = 0;
-  }
-}
-
-// endpoints of the entries a record removes (rows below t.rows)
-__global__ void k_track_del(const u64* keys, const int32_t* fdel, int64_t nrec, int bshift, DelTrack t) {
-  const u64 cmask = (((u64)1) << bshift) - 1;
-  GRID_STRIDE(i, nrec) {
-    if (!fdel[i]) continue;
-    const int64_t row = (int64_t)(keys[i] >> bshift);
-    if (row >= t.rows) continue;
-    const int32_t col = (int32_t)(keys[i] & cmask);
+  const u64 key = keys[i];
+  const int64_t row = (int64_t)(key >> bshift);
+  const int32_t c = (int32_t)(key & cmask);
+  const int64_t at = off[row];
+  const int32_t l = len[row];
+  const int64_t d = delta[i];
+  Rec r;
+  r.head = i == 0 || (int64_t)(keys[i - 1] >> bshift) != row;
+  const int32_t p = row_lower_bound(col, at, l, c);
+  const bool found = p < l && col[at + p] == c;
+  const int64_t ow = found ? (int64_t)w[at + p] : 0;
+  const int64_t nv = ow + d;
+  o.pos[i] = found ? p : -1;
+  o.lb[i] = p;
+  o.oldw[i] = ow;
+  if (nv < 0 || (!found && nv == 0)) atomicMax((unsigned long long*)o.bad, (unsigned long long)o.plan);
+  r.ins = !found && nv > 0;
+  r.del = found && nv == 0;
+  if (r.del && t.stamp && row < t.rows) {
     // an arc between two different refined communities cannot disconnect
     // either; a parentless endpoint may have just left its community (an
     // emptied node), so such arcs are kept
-    if (t.par && (row == col || (t.par[row] >= 0 && t.par[col] >= 0 && t.par[row] != t.par[col]))) continue;
-    stamp_add(t.stamp, t.ep, (int32_t)row, t.list, t.cnt);
-    stamp_add(t.stamp, t.ep, col, t.list, t.cnt);
-  }
-}
-
-__global__ void k_seg_info(const u64* keys, int64_t nrec, int bshift, const int32_t* fhead, const int64_t* segid,
-                           int64_t* seg_start, int64_t* seg_row) {
-  GRID_STRIDE(i, nrec) {
-    if (fhead[i]) {
-      seg_start[segid[i]] = i;
-      seg_row[segid[i]] = (int64_t)(keys[i] >> bshift);
+    if (!(t.par && (row == c || (t.par[row] >= 0 && t.par[c] >= 0 && t.par[row] != t.par[c])))) {
+      stamp_add(t.stamp, t.ep, (int32_t)row, t.list, t.cnt);
+      stamp_add(t.stamp, t.ep, c, t.list, t.cnt);
     }
   }
+  return r;
 }
 
-// Per segment: new length, whether the row is rebuilt, relocation size.
-__global__ void k_plan(const int64_t* nsegp, int64_t nrec, const int64_t* seg_start, const int64_t* seg_row,
-                       const int64_t* pins, const int64_t* pdel, const int32_t* len, const int32_t* cap,
-                       int32_t* newcap, int64_t* scratch_len, int64_t* work_len, int64_t* need) {
-  const int64_t nseg = *nsegp;
-  GRID_STRIDE(s, nseg) {
-    const int64_t a = seg_start[s];
-    const int64_t b = s + 1 < nseg ? seg_start[s + 1] : nrec;
-    const int64_t row = seg_row[s];
-    const int64_t ins = pins[b] - pins[a], del = pdel[b] - pdel[a];
-    const int64_t l = len[row];
-    const int64_t nl = l - del + ins;
-    const bool rewrite = ins > 0 || del > 0;
-    int32_t nc = 0;
-    if (nl > cap[row]) {
-      int64_t want = nl + (nl >> 1) + 4;
-      want = (want + 3) & ~(int64_t)3;
-      nc = (int32_t)want;
-      atomic_add_i64(need, want);
-    }
-    newcap[s] = nc;
-    scratch_len[s] = rewrite ? l : 0;
-    work_len[s] = rewrite ? l + ins : 0;
+struct SegNeed {
+  int64_t scratch, work, pool;  // old entries to copy, items of the rebuild, pool slots of a relocation
+};
+
+// Segment s (records [a, b)): its new capacity when the row no longer fits,
+// and what its rebuild needs.
+__device__ inline SegNeed plan_segment(const PlanOut& o, int64_t s, int64_t a, int64_t b, const int32_t* len,
+                                       const int32_t* cap) {
+  const int64_t row = o.segrow[s];
+  const int64_t ins = o.pins[b] - o.pins[a], del = o.pdel[b] - o.pdel[a];
+  const int64_t l = len[row];
+  const int64_t nl = l - del + ins;
+  SegNeed q{0, 0, 0};
+  if (nl > cap[row]) {
+    q.pool = nl + (nl >> 1) + 4;
+    q.pool = (q.pool + 3) & ~(int64_t)3;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    scratch_len[nseg] = 0;
-    work_len[nseg] = 0;
+  o.newcap[s] = (int32_t)q.pool;
+  if (ins > 0 || del > 0) {
+    q.scratch = l;
+    q.work = l + ins;
   }
+  return q;
 }
 
-// weight updates in place; deleted entries get weight 0 (live weights are >= 1)
+__device__ inline void publish_plan(const Pub& pub, const PlanOut& o, int64_t need, int64_t nseg, int64_t stot,
+                                    int64_t wtot, int64_t nrec) {
+  const int64_t v[6] = {need, nseg, stot, wtot, nrec, (int64_t)(*(volatile u64*)o.bad == o.plan)};
+  publish<6>(pub, v);
+}
+
+constexpr int PL_TPB = 512;  // records (segments) per tile: one each per thread, as a match is a chain of loads
+
+// Records: one pass over tiles of PL_TPB, with a look-back for the running
+// counts of inserts, deletes and segments.
 template <class WT>
-__global__ void k_update(const int64_t* off, const u64* keys, const int64_t* delta, int64_t nrec, int bshift,
-                         const int32_t* pos, const int64_t* oldw, WT* w) {
-  GRID_STRIDE(i, nrec) {
-    if (pos[i] < 0) continue;
-    const int64_t row = (int64_t)(keys[i] >> bshift);
-    w[off[row] + pos[i]] = (WT)(oldw[i] + delta[i]);
+__global__ void __launch_bounds__(PL_TPB) k_plan_records(const int64_t* off, const int32_t* len, const int32_t* col,
+                                                         const WT* w, const u64* keys, const int64_t* delta, RecN rn,
+                                                         int bshift, PlanOut o, DelTrack t, LookBack q) {
+  __shared__ int64_t s_tile, s_pre[3];
+  if (threadIdx.x == 0) s_tile = atomicAdd(q.ctr, 1);
+  __syncthreads();
+  const int64_t n = rn.count(), tile = s_tile, i = tile * PL_TPB + threadIdx.x;
+  if (tile * PL_TPB >= n && tile > 0) return;
+  Rec r{0, 0, 0};
+  if (i < n) r = match_record<WT>(off, len, col, w, keys, delta, i, bshift, o, t);
+  u64 tot;
+  const u64 ex = block_scan<PL_TPB>((u64)r.ins | ((u64)r.del << 20) | ((u64)r.head << 40), &tot);
+  if (threadIdx.x < 32) {
+    const int64_t agg[3] = {(int64_t)(tot & 0xfffff), (int64_t)((tot >> 20) & 0xfffff), (int64_t)(tot >> 40)};
+    int64_t pre[3];
+    look_back<3>(q.st, tile, agg, pre, q.ep, q.err);
+    if (threadIdx.x == 0) {
+      for (int k = 0; k < 3; ++k) s_pre[k] = pre[k];
+      if ((tile + 1) * PL_TPB >= n) {
+        o.pins[n] = (int32_t)(pre[0] + agg[0]);
+        o.pdel[n] = (int32_t)(pre[1] + agg[1]);
+        *o.nseg = pre[2] + agg[2];
+      }
+    }
+  }
+  __syncthreads();
+  if (i < n) {
+    o.pins[i] = (int32_t)(s_pre[0] + (int64_t)(ex & 0xfffff));
+    o.pdel[i] = (int32_t)(s_pre[1] + (int64_t)((ex >> 20) & 0xfffff));
+    const int64_t seg = s_pre[2] + (int64_t)(ex >> 40);  // heads before i
+    o.segid[i] = (int32_t)(seg + r.head - 1);
+    if (r.head) {
+      o.seg[seg] = i;
+      o.segrow[seg] = (int64_t)(keys[i] >> bshift);
+    }
+  }
+}
+
+// Segments: scratch, rebuild and pool offsets by one pass; the last tile
+// publishes the totals to the host.
+__global__ void __launch_bounds__(PL_TPB) k_plan_segments(const int32_t* len, const int32_t* cap, RecN rn, PlanOut o,
+                                                          LookBack q, Pub pub) {
+  __shared__ int64_t s_tile, s_pre[3];
+  __shared__ int64_t s_sum[3];
+  if (threadIdx.x == 0) s_tile = atomicAdd(q.ctr, 1);
+  __syncthreads();
+  const int64_t n = rn.count(), nseg = *o.nseg, tile = s_tile, s = tile * PL_TPB + threadIdx.x;
+  if (tile * PL_TPB >= nseg && tile > 0) return;
+  SegNeed d{0, 0, 0};
+  if (s < nseg) d = plan_segment(o, s, o.seg[s], s + 1 < nseg ? o.seg[s + 1] : n, len, cap);
+  u64 ex[3];
+  u64 tot[3];
+  ex[0] = block_scan<PL_TPB>((u64)d.scratch, &tot[0]);
+  ex[1] = block_scan<PL_TPB>((u64)d.work, &tot[1]);
+  ex[2] = block_scan<PL_TPB>((u64)d.pool, &tot[2]);
+  if (threadIdx.x < 32) {
+    const int64_t agg[3] = {(int64_t)tot[0], (int64_t)tot[1], (int64_t)tot[2]};
+    int64_t pre[3];
+    look_back<3>(q.st, tile, agg, pre, q.ep, q.err);
+    if (threadIdx.x == 0)
+      for (int k = 0; k < 3; ++k) {
+        s_pre[k] = pre[k];
+        s_sum[k] = pre[k] + agg[k];
+      }
+  }
+  __syncthreads();
+  if (s < nseg) {
+    o.soff[s] = s_pre[0] + (int64_t)ex[0];
+    o.woff[s] = s_pre[1] + (int64_t)ex[1];
+    o.noff[s] = s_pre[2] + (int64_t)ex[2];
+  }
+  if (threadIdx.x == 0 && (tile + 1) * PL_TPB >= nseg) {
+    o.soff[nseg] = s_sum[0];
+    o.woff[nseg] = s_sum[1];
+    publish_plan(pub, o, s_sum[2], nseg, s_sum[0], s_sum[1], n);
+  }
+}
+
+// Both steps in one block for up to PS_TPB records (one launch).
+constexpr int PS_TPB = 1024;
+template <class WT>
+__global__ void __launch_bounds__(PS_TPB) k_plan_small(const int64_t* off, const int32_t* len, const int32_t* cap,
+                                                       const int32_t* col, const WT* w, const u64* keys,
+                                                       const int64_t* delta, RecN rn, int bshift, PlanOut o,
+                                                       DelTrack t, Pub pub) {
+  const int64_t n = rn.count(), i = threadIdx.x;
+  Rec r{0, 0, 0};
+  if (i < n) r = match_record<WT>(off, len, col, w, keys, delta, i, bshift, o, t);
+  u64 tot;
+  const u64 ex = block_scan<PS_TPB>((u64)r.ins | ((u64)r.del << 20) | ((u64)r.head << 40), &tot);
+  const int64_t nseg = (int64_t)(tot >> 40);
+  if (i < n) {
+    const int64_t seg = (int64_t)(ex >> 40);
+    o.pins[i] = (int32_t)(ex & 0xfffff);
+    o.pdel[i] = (int32_t)((ex >> 20) & 0xfffff);
+    o.segid[i] = (int32_t)(seg + r.head - 1);
+    if (r.head) {
+      o.seg[seg] = i;
+      o.segrow[seg] = (int64_t)(keys[i] >> bshift);
+    }
+  }
+  if (i == 0) {
+    o.pins[n] = (int32_t)(tot & 0xfffff);
+    o.pdel[n] = (int32_t)((tot >> 20) & 0xfffff);
+    *o.nseg = nseg;
+  }
+  __syncthreads();
+  SegNeed d{0, 0, 0};
+  if (i < nseg) d = plan_segment(o, i, o.seg[i], i + 1 < nseg ? o.seg[i + 1] : n, len, cap);
+  u64 ts, tw, tp;
+  const u64 es = block_scan<PS_TPB>((u64)d.scratch, &ts);
+  const u64 ew = block_scan<PS_TPB>((u64)d.work, &tw);
+  const u64 en = block_scan<PS_TPB>((u64)d.pool, &tp);
+  if (i < nseg) {
+    o.soff[i] = (int64_t)es;
+    o.woff[i] = (int64_t)ew;
+    o.noff[i] = (int64_t)en;
+  }
+  if (i == 0) {
+    o.soff[nseg] = (int64_t)ts;
+    o.woff[nseg] = (int64_t)tw;
+    publish_plan(pub, o, (int64_t)tp, nseg, (int64_t)ts, (int64_t)tw, n);
   }
 }
 
 // ---- undo log (batches that may be rolled back)
-// Row entries: row, old offset, length and capacity, and where its old
-// contents went in the content log (-1: not rewritten by this update).
-__global__ void k_log_rows(int64_t nseg, const int64_t* seg_row, const int64_t* off, const int32_t* len,
-                           const int32_t* cap, const int64_t* slen, const int64_t* soff, int64_t c0, int64_t* lrow,
-                           int64_t* loff, int32_t* llen, int32_t* lcap, int64_t* lsrc) {
-  GRID_STRIDE(s, nseg) {
-    const int64_t row = seg_row[s];
-    lrow[s] = row;
-    loff[s] = off[row];
-    llen[s] = len[row];
-    lcap[s] = cap[row];
-    lsrc[s] = slen[s] > 0 ? c0 + soff[s] : -1;
-  }
-}
-
-// Weight entries: pool position of each record's entry (-1: absent) and
-// the weight it holds before the update.
-template <class WT>
-__global__ void k_log_weights(const u64* keys, int64_t nrec, int bshift, const int64_t* off, const int32_t* pos,
-                              const int64_t* oldw, int64_t* lpos, WT* lold) {
-  GRID_STRIDE(i, nrec) {
-    lpos[i] = pos[i] >= 0 ? off[(int64_t)(keys[i] >> bshift)] + pos[i] : -1;
-    lold[i] = (WT)oldw[i];
-  }
-}
-
 // Rollback of one row chunk: offsets, lengths and capacities come back; a
 // rewritten row's old contents go back where they were when they lie in the
 // batch's first pool below its first free slot (anything else was written
@@ -229,81 +315,108 @@ constexpr int SEG_RUN = 256;
   }                   \
   }
 
+// First half of an update: the weights of rows that keep their entries change
+// in place, and the rows to rebuild are copied out as they are (into the undo
+// log while a batch is logged).  With a log also: per row its old offset,
+// length and capacity and where its contents went (-1: not rewritten), per
+// record the pool position of its entry (-1: absent) and its old weight.  The
+// three parts touch different entries, so one launch does them all.
 template <class WT>
-__global__ void k_copy_scratch(const int64_t* off, const int64_t* seg_row, int64_t nseg, const int64_t* soff,
-                               int64_t total, const int32_t* col, const WT* w, int32_t* scol, WT* sw) {
-  FOR_SEG_ITEMS(t, s, soff, nseg, total)
-    const int64_t row = seg_row[s];
-    const int64_t k = t - soff[s];
-    scol[t] = col[off[row] + k];
-    sw[t] = w[off[row] + k];
+struct UndoOut {  // null pointers without a log
+  int64_t *lrow, *loff, *lsrc, *lpos;
+  int32_t *llen, *lcap;
+  WT* lold;
+  int64_t c0;  // first free slot of the content log
+};
+
+template <class WT>
+__global__ void k_apply(int64_t nrec, int64_t nseg, int64_t stotal, const u64* keys, const int64_t* delta, int bshift,
+                        PlanOut o, const int64_t* off, const int32_t* len, const int32_t* cap, const int32_t* col,
+                        WT* w, int32_t* scol, WT* sw, UndoOut<WT> u) {
+  GRID_STRIDE(i, nrec) {
+    const int32_t p = o.pos[i];
+    const int64_t at = p >= 0 ? off[(int64_t)(keys[i] >> bshift)] + p : -1;
+    const int64_t ow = o.oldw[i];
+    if (u.lpos) {
+      u.lpos[i] = at;
+      u.lold[i] = (WT)ow;
+    }
+    const int32_t s = o.segid[i];
+    if (p >= 0 && o.woff[s + 1] == o.woff[s]) w[at] = (WT)(ow + delta[i]);
+  }
+  if (u.lrow) {
+    GRID_STRIDE(s, nseg) {
+      const int64_t row = o.segrow[s];
+      u.lrow[s] = row;
+      u.loff[s] = off[row];
+      u.llen[s] = len[row];
+      u.lcap[s] = cap[row];
+      u.lsrc[s] = o.soff[s + 1] > o.soff[s] ? u.c0 + o.soff[s] : -1;
+    }
+  }
+  FOR_SEG_ITEMS(t, s, o.soff, nseg, stotal)
+    const int64_t at = off[o.segrow[s]] + (t - o.soff[s]);
+    scol[t] = col[at];
+    sw[t] = w[at];
   END_SEG_ITEMS
 }
 
-__global__ void k_relocate(int64_t nseg, const int64_t* seg_row, const int32_t* newcap, int64_t* off, int32_t* cap,
-                           int64_t* pool_top) {
-  GRID_STRIDE(s, nseg) {
-    const int32_t nc = newcap[s];
-    if (nc == 0) continue;
-    const int64_t row = seg_row[s];
-    off[row] = (int64_t)atomicAdd((unsigned long long*)pool_top, (unsigned long long)nc);
-    cap[row] = nc;
-  }
-}
-
-// Rebuild of rows with inserts or deletes: item t is either a kept old entry
-// (from scratch) or an inserted record; each computes its sorted position.
+// Second half, for rows with inserts or deletes.  Item t is either a kept old
+// entry (from the copy; its record, if it has one, changes its weight, and a
+// weight of zero drops it) or an inserted record; each computes its sorted
+// position.  A row that outgrew its capacity moves to base + noff.  The row
+// table is written by the same launch: only relocated rows change their
+// offset, and nobody reads that.
 template <class WT>
-__global__ void k_scatter_rows(int64_t nseg, int64_t nrec, const int64_t* seg_start, const int64_t* seg_row,
-                               const int64_t* woff, const int64_t* soff, int64_t total, const int32_t* scol,
-                               const WT* sw, const u64* keys, const int64_t* delta, const int32_t* lb,
-                               const int32_t* fins, const int64_t* pins, const int64_t* pdel, int bshift,
-                               const int64_t* off, int32_t* col, WT* w) {
+__global__ void k_rebuild(int64_t nrec, int64_t nseg, int64_t total, int64_t base, PlanOut o, const int32_t* scol,
+                          const WT* sw, const u64* keys, const int64_t* delta, int bshift, int64_t* off, int32_t* len,
+                          int32_t* cap, int32_t* col, WT* w) {
   const u64 cmask = (((u64)1) << bshift) - 1;
-  FOR_SEG_ITEMS(t, s, woff, nseg, total)
-    const int64_t a = seg_start[s];
-    const int64_t b = s + 1 < nseg ? seg_start[s + 1] : nrec;
-    const int64_t row = seg_row[s];
-    const int64_t lold = (woff[s + 1] - woff[s]) - (pins[b] - pins[a]);
-    const int64_t k = t - woff[s];
+  GRID_STRIDE(s, nseg) {
+    if (o.woff[s + 1] == o.woff[s]) continue;
+    const int64_t a = o.seg[s], b = s + 1 < nseg ? o.seg[s + 1] : nrec;
+    const int64_t row = o.segrow[s];
+    len[row] += (o.pins[b] - o.pins[a]) - (o.pdel[b] - o.pdel[a]);
+    if (o.newcap[s]) {
+      off[row] = base + o.noff[s];
+      cap[row] = o.newcap[s];
+    }
+  }
+  FOR_SEG_ITEMS(t, s, o.woff, nseg, total)
+    const int64_t a = o.seg[s];
+    const int64_t b = s + 1 < nseg ? o.seg[s + 1] : nrec;
+    const int64_t to = o.newcap[s] ? base + o.noff[s] : off[o.segrow[s]];
+    const int32_t ia = o.pins[a], da = o.pdel[a];
+    const int64_t lold = (o.woff[s + 1] - o.woff[s]) - (o.pins[b] - ia);
+    const int64_t k = t - o.woff[s];
     if (k < lold) {
-      const int64_t i = k;
-      const WT x = sw[soff[s] + i];
-      if (x == 0) continue;  // deleted
-      const int32_t c = scol[soff[s] + i];
+      const int32_t c = scol[o.soff[s] + k];
+      WT x = sw[o.soff[s] + k];
       // records of this segment with a smaller column
       int64_t lo = a, hi = b;
       while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;
         if ((int32_t)(keys[mid] & cmask) < c) lo = mid + 1; else hi = mid;
       }
-      const int64_t dst = i - (pdel[lo] - pdel[a]) + (pins[lo] - pins[a]);
-      col[off[row] + dst] = c;
-      w[off[row] + dst] = x;
+      if (lo < b && (int32_t)(keys[lo] & cmask) == c) {
+        x = (WT)((int64_t)x + delta[lo]);
+        if (x == 0) continue;  // deleted
+      }
+      const int64_t dst = to + k - (o.pdel[lo] - da) + (o.pins[lo] - ia);
+      col[dst] = c;
+      w[dst] = x;
     } else {
       const int64_t q = k - lold;  // q-th insert of the segment
       int64_t lo = a, hi = b - 1;
-      while (lo < hi) {  // first J with pins[J] - pins[a] >= q and fins[J]
+      while (lo < hi) {  // the record J with q inserts before it that is one itself
         const int64_t mid = (lo + hi) >> 1;
-        if (pins[mid + 1] - pins[a] <= q) lo = mid + 1; else hi = mid;
+        if (o.pins[mid + 1] - ia <= q) lo = mid + 1; else hi = mid;
       }
-      const int64_t J = lo;
-      const int64_t dst = (int64_t)lb[J] - (pdel[J] - pdel[a]) + q;
-      col[off[row] + dst] = (int32_t)(keys[J] & cmask);
-      w[off[row] + dst] = (WT)delta[J];
-      (void)fins;
+      const int64_t dst = to + (int64_t)o.lb[lo] - (o.pdel[lo] - da) + q;
+      col[dst] = (int32_t)(keys[lo] & cmask);
+      w[dst] = (WT)delta[lo];
     }
   END_SEG_ITEMS
-}
-
-__global__ void k_set_len(int64_t nseg, int64_t nrec, const int64_t* seg_start, const int64_t* seg_row,
-                          const int64_t* pins, const int64_t* pdel, int32_t* len) {
-  GRID_STRIDE(s, nseg) {
-    const int64_t a = seg_start[s];
-    const int64_t b = s + 1 < nseg ? seg_start[s + 1] : nrec;
-    const int64_t row = seg_row[s];
-    len[row] = (int32_t)(len[row] - (pdel[b] - pdel[a]) + (pins[b] - pins[a]));
-  }
 }
 
 // compaction: every live entry is one item (rows located through the scan of
@@ -385,18 +498,6 @@ void csr_build(SlackCSR<WT>& g, int64_t n, const u64* keys, const int64_t* vals,
   }
 }
 
-template <class WT>
-void csr_lookup(const SlackCSR<WT>& g, const u64* keys, int64_t nrec, int bshift, int32_t* pos, int64_t* oldw,
-                CsrScratch& S, Prims& P, cudaStream_t s, int32_t* d_nseg) {
-  (void)P;
-  (void)S;
-  (void)d_nseg;
-  if (nrec <= 0) return;
-  k_lookup<WT><<<grid_for(nrec, TPB), TPB, 0, s>>>(g.off.p, g.len.p, g.col.p, g.w.p, keys, nrec, bshift, pos, nullptr,
-                                                   oldw);
-  CKL("k_lookup");
-}
-
 // Copy every row into a fresh pool of `cap_total + extra` slots.
 template <class WT>
 static void compact_pool(SlackCSR<WT>& g, int64_t extra, CsrScratch& S, Prims& P, cudaStream_t s) {
@@ -439,64 +540,57 @@ static void compact_pool(SlackCSR<WT>& g, int64_t extra, CsrScratch& S, Prims& P
 }
 
 template <class WT>
-void csr_apply(SlackCSR<WT>& g, const u64* keys, const int64_t* delta, int64_t nrec, int bshift, CsrScratch& S,
-               Prims& P, cudaStream_t s, DevScalars* d_sc, const DelTrack* trk) {
-  if (nrec <= 0) return;
-  S.pos.reserve(nrec + 1, s);
-  S.lb.reserve(nrec + 1, s);
-  S.oldw.reserve(nrec + 1, s);
-  S.fins.reserve(nrec + 1, s);
-  S.fdel.reserve(nrec + 1, s);
-  S.fhead.reserve(nrec + 1, s);
-  S.pins.reserve(nrec + 1, s);
-  S.pdel.reserve(nrec + 1, s);
-  S.segid.reserve(nrec + 1, s);
-  const int gr = grid_for(nrec, TPB);
-  k_lookup<WT><<<gr, TPB, 0, s>>>(g.off.p, g.len.p, g.col.p, g.w.p, keys, nrec, bshift, S.pos.p, S.lb.p, S.oldw.p);
-  CKL("k_lookup");
-  CK(cudaMemsetAsync(&d_sc->cnt[C_Z], 0, sizeof(int32_t), s));
-  k_rec_flags<<<gr, TPB, 0, s>>>(keys, delta, nrec, bshift, S.pos.p, S.oldw.p, S.fins.p, S.fdel.p, S.fhead.p,
-                                 &d_sc->cnt[C_Z]);
-  CKL("k_rec_flags");
-  if (trk) {
-    k_track_del<<<gr, TPB, 0, s>>>(keys, S.fdel.p, nrec, bshift, *trk);
-    CKL("k_track_del");
+int64_t csr_apply(SlackCSR<WT>& g, const u64* keys, const int64_t* delta, int64_t n_max, const int32_t* n_dev, int mul,
+                  int bshift, CsrScratch& S, Prims& P, cudaStream_t s, DevScalars* d_sc, const DelTrack* trk) {
+  if (n_max <= 0) return 0;
+  S.pos.reserve(n_max + 1, s);
+  S.lb.reserve(n_max + 1, s);
+  S.oldw.reserve(n_max + 1, s);
+  S.pins.reserve(n_max + 1, s);
+  S.pdel.reserve(n_max + 1, s);
+  S.segid.reserve(n_max + 1, s);
+  // the segment count stays on the device: one segment per record bounds it
+  S.seg.reserve(n_max + 1, s);
+  S.segrow.reserve(n_max + 1, s);
+  S.newcap.reserve(n_max + 1, s);
+  S.soff.reserve(n_max + 2, s);
+  S.woff.reserve(n_max + 2, s);
+  S.noff.reserve(n_max + 2, s);
+  const RecN rn{n_max, n_dev, mul};
+  const PlanOut o{S.pos.p,  S.lb.p,     S.segid.p,  S.pins.p, S.pdel.p, S.oldw.p,     S.seg.p,
+                  S.segrow.p, S.newcap.p, S.soff.p, S.woff.p, S.noff.p, &d_sc->seg_n, (u64*)&d_sc->plan_bad,
+                  ++S.plans};
+  const DelTrack t = trk ? *trk : DelTrack{};
+  // Up to one record per thread of a block, one launch plans the update: 6.2 us
+  // for a few records and 7.5 for some hundred, where the two tiled launches
+  // take 8.9 and 9.9 and the gap between them.  Beyond, one block would match
+  // several records per thread one after the other.
+  const Pub pub = P.pub_begin(P.rd_owner);
+  if (n_max <= PS_TPB) {
+    k_plan_small<WT><<<1, PS_TPB, 0, s>>>(g.off.p, g.len.p, g.cap.p, g.col.p, g.w.p, keys, delta, rn, bshift, o, t,
+                                          pub);
+    CKL("k_plan_small");
+  } else {
+    const int tiles = div_up(n_max, PL_TPB);
+    const LookBack q1 = look_back_begin(P, 3 * (int64_t)tiles, s);
+    k_plan_records<WT><<<tiles, PL_TPB, 0, s>>>(g.off.p, g.len.p, g.col.p, g.w.p, keys, delta, rn, bshift, o, t, q1);
+    CKL("k_plan_records");
+    const LookBack q2 = look_back_begin(P, 3 * (int64_t)tiles, s);
+    k_plan_segments<<<tiles, PL_TPB, 0, s>>>(g.len.p, g.cap.p, rn, o, q2, pub);
+    CKL("k_plan_segments");
   }
-  scan_exclusive_i32_to(S.fins.p, S.pins.p, nrec + 1, nullptr, nrec + 1, nullptr, P, s);
-  scan_exclusive_i32_to(S.fdel.p, S.pdel.p, nrec + 1, nullptr, nrec + 1, nullptr, P, s);
-  // the segment count stays on the device: segment arrays are sized for one
-  // segment per record, and the plan and its scans read the count there
-  scan_exclusive_i32_to(S.fhead.p, S.segid.p, nrec, nullptr, nrec, &d_sc->seg_n, P, s);
-  S.seg.reserve(nrec + 1, s);
-  S.segrow.reserve(nrec + 1, s);
-  S.newcap.reserve(nrec + 1, s);
-  S.slen.reserve(nrec + 2, s);
-  S.wlen.reserve(nrec + 2, s);
-  S.soff.reserve(nrec + 2, s);
-  S.woff.reserve(nrec + 2, s);
-  k_seg_info<<<gr, TPB, 0, s>>>(keys, nrec, bshift, S.fhead.p, S.segid.p, S.seg.p, S.segrow.p);
-  CKL("k_seg_info");
-  CK(cudaMemsetAsync(&d_sc->need, 0, sizeof(int64_t), s));
-  k_plan<<<gr, TPB, 0, s>>>(&d_sc->seg_n, nrec, S.seg.p, S.segrow.p, S.pins.p, S.pdel.p, g.len.p, g.cap.p,
-                            S.newcap.p, S.slen.p, S.wlen.p, &d_sc->need);
-  CKL("k_plan");
-  scan_exclusive_to(S.slen.p, S.soff.p, 1, &d_sc->seg_n, nrec + 1, &d_sc->seg_stot, P, s);
-  scan_exclusive_to(S.wlen.p, S.woff.p, 1, &d_sc->seg_n, nrec + 1, &d_sc->seg_wtot, P, s);
-  static_assert(offsetof(DevScalars, seg_stot) == offsetof(DevScalars, seg_n) + 8 &&
-                    offsetof(DevScalars, seg_wtot) == offsetof(DevScalars, seg_n) + 16,
-                "adjacent totals");
-  int64_t tot[4] = {0, 0, 0, 0};  // need, nseg, scratch total, rebuild total
-  int32_t bad = 0;
-  const HostRead rr[3] = {{&d_sc->need, &tot[0], sizeof(int64_t)}, {&d_sc->seg_n, &tot[1], 3 * sizeof(int64_t)},
-                          {&d_sc->cnt[C_Z], &bad, sizeof(int32_t)}};
-  P.read(rr, 3, s);
-  if (bad) ldl_throw(LDL_E_INVALID, "internal: adjacency update would make a weight negative");
-  const int64_t need = tot[0], nseg = tot[1], stotal = tot[2], wtotal = tot[3];
-  const int gs = grid_for(nseg, TPB);
+  int64_t tot[6];
+  P.pub_wait(P.rd_owner, tot, 6);
+  const int64_t need = tot[0], nseg = tot[1], stotal = tot[2], wtotal = tot[3], nrec = tot[4];
+  if (tot[5]) ldl_throw(LDL_E_INVALID, "internal: adjacency update would make a weight negative");
+  if (nrec <= 0) return 0;
   if (g.pool_top + need > g.col.cap) compact_pool<WT>(g, need, S, P, s);
   DBuf<WT>& sw = S.template sw_of<WT>();
+  UndoOut<WT> u{};
+  int32_t* scol = nullptr;
+  WT* swp = nullptr;
   if (g.logging) {
-    // everything a rollback needs, reserved and written before any change
+    // everything a rollback needs, reserved before any change
     g.lrow.reserve(g.rtop + nseg + 1, s, true);
     g.loff.reserve(g.rtop + nseg + 1, s, true);
     g.lsrc.reserve(g.rtop + nseg + 1, s, true);
@@ -506,55 +600,32 @@ void csr_apply(SlackCSR<WT>& g, const u64* keys, const int64_t* delta, int64_t n
     g.lold.reserve(g.wtop + nrec + 1, s, true);
     g.lcol.reserve(g.ctop + stotal + 1, s, true);
     g.lw.reserve(g.ctop + stotal + 1, s, true);
-    if (nseg > 0) {
-      k_log_rows<<<gs, TPB, 0, s>>>(nseg, S.segrow.p, g.off.p, g.len.p, g.cap.p, S.slen.p, S.soff.p, g.ctop,
-                                    g.lrow.p + g.rtop, g.loff.p + g.rtop, g.llen.p + g.rtop, g.lcap.p + g.rtop,
-                                    g.lsrc.p + g.rtop);
-      CKL("k_log_rows");
-    }
-    k_log_weights<WT><<<gr, TPB, 0, s>>>(keys, nrec, bshift, g.off.p, S.pos.p, S.oldw.p, g.lpos.p + g.wtop,
-                                         g.lold.p + g.wtop);
-    CKL("k_log_weights");
+    u = {g.lrow.p + g.rtop, g.loff.p + g.rtop, g.lsrc.p + g.rtop, g.lpos.p + g.wtop,
+         g.llen.p + g.rtop, g.lcap.p + g.rtop, g.lold.p + g.wtop, g.ctop};
+    scol = g.lcol.p + g.ctop;
+    swp = g.lw.p + g.ctop;
+  } else {
+    S.scol.reserve(stotal + 1, s);
+    sw.reserve(stotal + 1, s);
+    scol = S.scol.p;
+    swp = sw.p;
+  }
+  k_apply<WT><<<grid_for(std::max(nrec, (stotal + 7) / 8), TPB), TPB, 0, s>>>(
+      nrec, nseg, stotal, keys, delta, bshift, o, g.off.p, g.len.p, g.cap.p, g.col.p, g.w.p, scol, swp, u);
+  CKL("k_apply");
+  if (g.logging) {
     g.events.push_back({false, g.rtop, nseg, g.wtop, nrec, 0, g.col.p});
     g.rtop += nseg;
     g.wtop += nrec;
+    g.ctop += stotal;
   }
-  k_update<WT><<<gr, TPB, 0, s>>>(g.off.p, keys, delta, nrec, bshift, S.pos.p, S.oldw.p, g.w.p);
-  CKL("k_update");
   if (wtotal > 0) {
-    // the rows to rebuild, as they are before the rewrite (weights already
-    // updated): while a batch is logged they go straight into the undo log,
-    // which the rebuild then reads
-    int32_t* scol = nullptr;
-    WT* swp = nullptr;
-    if (g.logging) {
-      scol = g.lcol.p + g.ctop;
-      swp = g.lw.p + g.ctop;
-      g.ctop += stotal;
-    } else {
-      S.scol.reserve(stotal + 1, s);
-      sw.reserve(stotal + 1, s);
-      scol = S.scol.p;
-      swp = sw.p;
-    }
-    if (stotal > 0) {
-      k_copy_scratch<WT><<<grid_for((stotal + 7) / 8, TPB), TPB, 0, s>>>(g.off.p, S.segrow.p, nseg, S.soff.p, stotal,
-                                                                         g.col.p, g.w.p, scol, swp);
-      CKL("k_copy_scratch");
-    }
-    if (need > 0) {
-      CK(cudaMemcpyAsync(&d_sc->pool_top, &g.pool_top, sizeof(int64_t), cudaMemcpyHostToDevice, s));
-      k_relocate<<<gs, TPB, 0, s>>>(nseg, S.segrow.p, S.newcap.p, g.off.p, g.cap.p, &d_sc->pool_top);
-      CKL("k_relocate");
-      g.pool_top += need;
-    }
-    k_scatter_rows<WT><<<grid_for((wtotal + 7) / 8, TPB), TPB, 0, s>>>(nseg, nrec, S.seg.p, S.segrow.p, S.woff.p, S.soff.p,
-                                                             wtotal, scol, swp, keys, delta, S.lb.p, S.fins.p,
-                                                             S.pins.p, S.pdel.p, bshift, g.off.p, g.col.p, g.w.p);
-    CKL("k_scatter_rows");
-    k_set_len<<<gs, TPB, 0, s>>>(nseg, nrec, S.seg.p, S.segrow.p, S.pins.p, S.pdel.p, g.len.p);
-    CKL("k_set_len");
+    k_rebuild<WT><<<grid_for(std::max(nseg, (wtotal + 7) / 8), TPB), TPB, 0, s>>>(
+        nrec, nseg, wtotal, g.pool_top, o, scol, swp, keys, delta, bshift, g.off.p, g.len.p, g.cap.p, g.col.p, g.w.p);
+    CKL("k_rebuild");
+    g.pool_top += need;
   }
+  return nrec;
 }
 
 template <class WT>
@@ -638,11 +709,7 @@ template void csr_build<int32_t>(SlackCSR<int32_t>&, int64_t, const u64*, const 
                                  CsrScratch&, Prims&, cudaStream_t);
 template void csr_build<int64_t>(SlackCSR<int64_t>&, int64_t, const u64*, const int64_t*, int64_t, int, int,
                                  CsrScratch&, Prims&, cudaStream_t);
-template void csr_lookup<int32_t>(const SlackCSR<int32_t>&, const u64*, int64_t, int, int32_t*, int64_t*,
-                                  CsrScratch&, Prims&, cudaStream_t, int32_t*);
-template void csr_lookup<int64_t>(const SlackCSR<int64_t>&, const u64*, int64_t, int, int32_t*, int64_t*,
-                                  CsrScratch&, Prims&, cudaStream_t, int32_t*);
-template void csr_apply<int32_t>(SlackCSR<int32_t>&, const u64*, const int64_t*, int64_t, int, CsrScratch&, Prims&,
-                                 cudaStream_t, DevScalars*, const DelTrack*);
-template void csr_apply<int64_t>(SlackCSR<int64_t>&, const u64*, const int64_t*, int64_t, int, CsrScratch&, Prims&,
-                                 cudaStream_t, DevScalars*, const DelTrack*);
+template int64_t csr_apply<int32_t>(SlackCSR<int32_t>&, const u64*, const int64_t*, int64_t, const int32_t*, int, int,
+                                    CsrScratch&, Prims&, cudaStream_t, DevScalars*, const DelTrack*);
+template int64_t csr_apply<int64_t>(SlackCSR<int64_t>&, const u64*, const int64_t*, int64_t, const int32_t*, int, int,
+                                    CsrScratch&, Prims&, cudaStream_t, DevScalars*, const DelTrack*);

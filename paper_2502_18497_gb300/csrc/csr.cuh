@@ -4,16 +4,16 @@
 #include "prims.cuh"
 
 struct CsrScratch {
-  DBuf<int64_t> seg, segrow, oldw, rs, tmp64, pins, pdel, segid, slen, wlen, soff, woff;
-  DBuf<int32_t> pos, lb, newcap, fins, fdel, fhead, scol, sw32;
+  DBuf<int64_t> seg, segrow, oldw, rs, tmp64, soff, woff, noff;
+  DBuf<int32_t> pos, lb, newcap, pins, pdel, segid, scol, sw32;
   DBuf<int64_t> sw64;
+  u64 plans = 0;  // updates planned so far
   template <class WT>
   DBuf<WT>& sw_of();
   void release() {
-    DBuf<int64_t>* a[] = {&seg, &segrow, &oldw, &rs, &tmp64, &pins, &pdel, &segid, &slen, &wlen, &soff, &woff,
-                          &sw64};
+    DBuf<int64_t>* a[] = {&seg, &segrow, &oldw, &rs, &tmp64, &soff, &woff, &noff, &sw64};
     for (auto* b : a) b->release();
-    DBuf<int32_t>* c[] = {&pos, &lb, &newcap, &fins, &fdel, &fhead, &scol, &sw32};
+    DBuf<int32_t>* c[] = {&pos, &lb, &newcap, &pins, &pdel, &segid, &scol, &sw32};
     for (auto* b : c) b->release();
   }
 };
@@ -28,11 +28,15 @@ template <class WT>
 void csr_build(SlackCSR<WT>& g, int64_t n, const u64* keys, const int64_t* vals, int64_t nrec, int bshift,
                int slack_pct, CsrScratch& S, Prims& P, cudaStream_t s);
 
-// For each sorted unique record key: pos[i] = entry index in its row (or -1)
-// and oldw[i] = current weight (or 0).  d_nseg is a device counter.
-template <class WT>
-void csr_lookup(const SlackCSR<WT>& g, const u64* keys, int64_t nrec, int bshift, int32_t* pos, int64_t* oldw,
-                CsrScratch& S, Prims& P, cudaStream_t s, int32_t* d_nseg);
+// Binary search of col in a sorted row: the lower bound index.
+__device__ inline int32_t row_lower_bound(const int32_t* col, int64_t off, int32_t len, int32_t c) {
+  int32_t lo = 0, hi = len;
+  while (lo < hi) {
+    const int32_t mid = (lo + hi) >> 1;
+    if (col[off + mid] < c) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
 
 // Where csr_apply records the endpoints (row and column) of the entries it
 // removes, for records whose row is below `rows`: a dedup stamp with its
@@ -57,8 +61,10 @@ template <class WT>
 cudaError_t csr_txn_rollback(SlackCSR<WT>& g, cudaStream_t s);
 
 // Add delta to each record's entry: absent entries are inserted, entries that
-// reach zero are removed (their endpoints go to *trk when given).
-// Synchronises once (pool growth decision).
+// reach zero are removed (their endpoints go to *trk when given).  n_max
+// records, or mul * *n_dev of them (device count, n_max an upper bound).
+// Waits for the host once (pool growth decision) and returns the number of
+// records.
 template <class WT>
-void csr_apply(SlackCSR<WT>& g, const u64* keys, const int64_t* delta, int64_t nrec, int bshift, CsrScratch& S,
-               Prims& P, cudaStream_t s, DevScalars* d_sc, const DelTrack* trk = nullptr);
+int64_t csr_apply(SlackCSR<WT>& g, const u64* keys, const int64_t* delta, int64_t n_max, const int32_t* n_dev, int mul,
+                  int bshift, CsrScratch& S, Prims& P, cudaStream_t s, DevScalars* d_sc, const DelTrack* trk = nullptr);

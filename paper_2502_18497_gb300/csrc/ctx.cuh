@@ -43,11 +43,14 @@ struct LevelState {
 
 // Device counters (indices into ldl_ctx::dcnt).
 enum {
-  K_U = 0, K_S, K_USTAR, K_MV, K_M0, K_D, K_C, K_R, K_R2, K_X, K_T, K_E, K_E2, K_CH, K_CAND, K_B,
-  K_UNDEC, K_SMALL, K_MID, K_LARGE, K_REC, K_CREC, K_NREC, K_ERR, K_TMP, K_TMP2, K_CHG, K_MID2, K_TINY, K_CLU,
+  K_U = 0, K_S, K_USTAR, K_MV, K_M0, K_D, K_C, K_R, K_R2, K_X, K_T, K_CH, K_CAND, K_B,
+  K_UNDEC, K_SMALL, K_MID, K_LARGE, K_REC, K_CREC, K_ERR, K_TMP, K_TMP2, K_CHG, K_MID2, K_TINY, K_CLU,
   K_G,
   K_HUBG,      // hubs of the current hub group
   K_A0 = 32,   // K_A0 + r: |A^r|
+  K_NR = 40,   // summed records of the last sort_reduce
+  K_NU,        // distinct edges of the batch
+  K_FL,        // summed records of a flush
   K_BRK0 = 48, // K_BRK0 + r: endpoints of deleted level-r arcs
   K_PEND0 = 56, // K_PEND0 + r: pending weight records of level r
   K_COUNT = 64
@@ -75,7 +78,7 @@ struct ldl_ctx {
 
   // dedup stamps (one int32 per node id) and lists
   DBuf<int32_t> stS, stU, stMv, stB, stM0, stD, stC, stR, stX, stT, stE, stCh, stL;
-  DBuf<int32_t> lU, lS, lUstar, lMv, lM0, lD, lC, lR, lR2, lX, lT, lE, lE2, lCh, lChg, lTmp, lG;
+  DBuf<int32_t> lU, lS, lUstar, lMv, lM0, lD, lC, lR, lR2, lX, lT, lE2, lCh, lChg, lTmp, lG;
   DBuf<int32_t> comp;  // connected-component labels of the refinement's re-check
   DBuf<int32_t> nbr;   // per leaving node: its neighbours in its old refined community
   DBuf<int32_t> ckf;   // per refined community: stamp when its connectivity must be computed
@@ -97,9 +100,7 @@ struct ldl_ctx {
   // records
   DBuf<u64> rk, rv, tk, tv, rk2, rv2;
   DBuf<int64_t> rsum, rsum2;
-  DBuf<int32_t> ndx;
-  DBuf<int64_t> ndko, ndki;
-  DBuf<u64> crk, crv, fk, trk, trv;
+  DBuf<u64> crk, crv, trk, trv;
   DBuf<u64> flk;      // a pending list's summed records (keys) ...
   DBuf<int64_t> flv;  // ... and their weight changes
   DBuf<int64_t> chunk_pre;
@@ -179,6 +180,11 @@ inline int64_t* Kin_of(ldl_ctx& c) { return c.directed ? c.Kin.p : c.Kout.p; }
 // this point: a one-block kernel writes them into the pinned page and then the
 // sequence number, which the host polls (a stream error ends the wait).
 void host_read(ldl_ctx& c, const HostRead* r, int n);
+// The same for values that a kernel publishes itself (scan.cuh): the page and
+// the sequence number for it, then the wait for its n payload words.  One
+// read at a time: nothing else is read between the two.
+Pub pub_begin(ldl_ctx& c);
+void pub_wait(ldl_ctx& c, int64_t* out, int n);
 int32_t rd_cnt(ldl_ctx& c, int idx);
 void zero_cnt(ldl_ctx& c, int idx);
 // One launch that clears several counters (bit i of mask: dcnt[i]) and up to

@@ -18,7 +18,23 @@ __device__ inline void set_err(unsigned long long* err, int64_t idx, int code) {
   atomicMin(err, ((unsigned long long)idx << 8) | (unsigned long long)code);
 }
 
-__global__ void k_validate(const ldl_update* u, int64_t cnt, int64_t n, unsigned long long* err) {
+// Start of a batch: every counter, and the scalars that ingest adds to.
+__global__ void k_batch_begin(int32_t* dcnt, DevScalars* sc) {
+  const int t = threadIdx.x;
+  if (t < K_COUNT) dcnt[t] = 0;
+  if (t == 0) {
+    sc->scanned = 0;
+    sc->dm = 0;
+    sc->agg_recs = 0;
+    sc->err_key = -1;
+    sc->err_seq = -1;
+  }
+}
+
+// Checks each update by itself and makes its edge key (an update that fails
+// gets key 0: the batch is rejected before anything uses it).
+__global__ void k_upd_keys(const ldl_update* u, int64_t cnt, int64_t n, int bits, int directed, u64* keys, u64* vals,
+                           unsigned long long* err) {
   GRID_STRIDE(i, cnt) {
     const ldl_update x = u[i];
     int code = 0;
@@ -26,13 +42,11 @@ __global__ void k_validate(const ldl_update* u, int64_t cnt, int64_t n, unsigned
     else if (x.op != LDL_INSERT && x.op != LDL_DELETE && x.op != LDL_REWEIGHT) code = LDL_E_INVALID;
     else if (x.op == LDL_INSERT && x.w < 1) code = LDL_E_INVALID;
     else if (x.op == LDL_REWEIGHT && x.w < 0) code = LDL_E_NEG_WEIGHT;
-    if (code) set_err(err, i, code);
-  }
-}
-
-__global__ void k_upd_keys(const ldl_update* u, int64_t cnt, int bits, int directed, u64* keys, u64* vals) {
-  GRID_STRIDE(i, cnt) {
-    int64_t a = u[i].src, b = u[i].dst;
+    int64_t a = x.src, b = x.dst;
+    if (code) {
+      set_err(err, i, code);
+      a = b = 0;
+    }
     if (!directed && a > b) {
       int64_t t = a; a = b; b = t;
     }
@@ -41,23 +55,49 @@ __global__ void k_upd_keys(const ldl_update* u, int64_t cnt, int bits, int direc
   }
 }
 
-__global__ void k_unique_starts(const u64* keys, int64_t n, const int32_t* flag, const int64_t* pos, u64* ukeys,
-                                int64_t* ustart) {
-  GRID_STRIDE(i, n) {
-    if (flag[i]) {
-      ukeys[pos[i]] = keys[i];
-      ustart[pos[i]] = i;
+// The distinct keys of a sorted list and where each starts, in one pass with
+// look-back (their number in *nu).
+constexpr int UQ_TPB = 512;
+__global__ void __launch_bounds__(UQ_TPB) k_unique(const u64* keys, int64_t n, u64* ukeys, int64_t* ustart,
+                                                   int32_t* nu, LookBack q) {
+  __shared__ int64_t s_tile, s_pre;
+  if (threadIdx.x == 0) s_tile = atomicAdd(q.ctr, 1);
+  __syncthreads();
+  const int64_t tile = s_tile, i = tile * UQ_TPB + threadIdx.x;
+  const u64 k = i < n ? keys[i] : 0;
+  const bool head = i < n && (i == 0 || keys[i - 1] != k);
+  u64 tot;
+  const u64 ex = block_scan<UQ_TPB>(head ? 1 : 0, &tot);
+  if (threadIdx.x < 32) {
+    const int64_t agg[1] = {(int64_t)tot};
+    int64_t pre[1];
+    look_back<1>(q.st, tile, agg, pre, q.ep, q.err);
+    if (threadIdx.x == 0) {
+      s_pre = pre[0];
+      if ((tile + 1) * UQ_TPB >= n) *nu = (int32_t)(pre[0] + agg[0]);
     }
+  }
+  __syncthreads();
+  if (head) {
+    ukeys[s_pre + (int64_t)ex] = k;
+    ustart[s_pre + (int64_t)ex] = i;
   }
 }
 
-// Per edge key: apply its updates in array order to the current weight.
-__global__ void k_seq(const ldl_update* u, int64_t cnt, const u64* vals, const int64_t* ustart, int64_t nu,
-                      const u64* ukeys, const int64_t* oldw, int bits, int directed, int64_t* delta,
-                      unsigned long long* err, int64_t* dm) {
+// Per distinct edge: its current weight, its updates in array order on top,
+// and the arcs whose weight changes (an undirected edge's mirror too).
+__global__ void k_seq(const ldl_update* u, int64_t cnt, const u64* vals, const int64_t* ustart, const int32_t* nup,
+                      const u64* ukeys, const int64_t* off, const int32_t* len, const int32_t* col, const int32_t* wt,
+                      int bits, int directed, unsigned long long* err, int64_t* dm, u64* ok, u64* ov, int32_t* na) {
+  const int64_t nu = *nup;
   GRID_STRIDE(k, nu) {
     const int64_t s = ustart[k], e = (k + 1 < nu) ? ustart[k + 1] : cnt;
-    const int64_t w0 = oldw[k];
+    const u64 key = ukeys[k];
+    const u64 a = key >> bits, b = key & ((((u64)1) << bits) - 1);
+    const int64_t o = off[a];
+    const int32_t l = len[a];
+    const int32_t at = row_lower_bound(col, o, l, (int32_t)b);
+    const int64_t w0 = at < l && col[o + at] == (int32_t)b ? wt[o + at] : 0;
     int64_t cur = w0;
     for (int64_t t = s; t < e; ++t) {
       const int64_t idx = (int64_t)vals[t];
@@ -80,29 +120,15 @@ __global__ void k_seq(const ldl_update* u, int64_t cnt, const u64* vals, const i
       }
     }
     const int64_t d = cur - w0;
-    delta[k] = d;
-    if (d) {
-      const u64 key = ukeys[k];
-      const int64_t a = (int64_t)(key >> bits), b = (int64_t)(key & ((((u64)1) << bits) - 1));
-      atomic_add_i64(dm, (directed || a == b) ? d : 2 * d);
-    }
-  }
-}
-
-__global__ void k_emit_arcs(const u64* ukeys, const int64_t* delta, int64_t nu, int bits, int directed, u64* ok,
-                            u64* ov, int32_t* cnt) {
-  GRID_STRIDE(k, nu) {
-    const int64_t d = delta[k];
     if (!d) continue;
-    const u64 key = ukeys[k];
-    const u64 a = key >> bits, b = key & ((((u64)1) << bits) - 1);
-    int32_t p = atomicAdd(cnt, 1);
+    const bool two = !directed && a != b;
+    atomic_add_i64(dm, two ? 2 * d : d);
+    const int32_t p = atomicAdd(na, two ? 2 : 1);
     ok[p] = key;
     ov[p] = (u64)d;
-    if (!directed && a != b) {
-      p = atomicAdd(cnt, 1);
-      ok[p] = (b << bits) | a;
-      ov[p] = (u64)d;
+    if (two) {
+      ok[p + 1] = (b << bits) | a;
+      ov[p + 1] = (u64)d;
     }
   }
 }
@@ -199,8 +225,9 @@ __device__ inline void warp_append_rec(bool want, u64 key, int64_t v, u64* pk, u
   }
 }
 
-__global__ void k_chain_records(const u64* keys, const int64_t* vals, int64_t n, int bits, int q0, int top, int self,
+__global__ void k_chain_records(const u64* keys, const int64_t* vals, int64_t n, const int32_t* n_dev, int bits, int q0, int top, int self,
                                 int add_k, int directed, Chain ch, int32_t* pcnt) {
+  if (n_dev) n = min(n, (int64_t)*n_dev);
   const u64 mask = (((u64)1) << bits) - 1;
   const int lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -576,23 +603,18 @@ __global__ void k_singletons(const int32_t* l, const int32_t* n, const int32_t* 
 }
 
 // ---------------------------------------------------------------- aggregate
+// The nodes of D whose parent changed, and the entries of their rows.
 __global__ void k_changed(const int32_t* lD, const int32_t* nD, const int32_t* par, const int32_t* par_old,
-                          int32_t* stC, int32_t epC, int32_t* lC, int32_t* nC) {
+                          int32_t* stC, int32_t epC, int32_t* lC, int32_t* nC, const int32_t* len_out,
+                          const int32_t* len_in, int64_t* acc_out, int64_t* acc_in) {
   const int32_t n = *nD;
+  int64_t so = 0, si = 0;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t u = lD[k];
-    if (par[u] != par_old[u]) stamp_add(stC, epC, u, lC, nC);
-  }
-}
-
-template <class WT>
-__global__ void k_deg_sum(Adj<WT> out, Adj<WT> in, const int32_t* l, const int32_t* n, int64_t* acc_out,
-                          int64_t* acc_in) {
-  const int32_t m = *n;
-  int64_t so = 0, si = 0;
-  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
-    so += (int64_t)out.len[l[k]];
-    si += (int64_t)in.len[l[k]];
+    if (par[u] != par_old[u] && stamp_add(stC, epC, u, lC, nC)) {
+      so += len_out[u];
+      si += len_in[u];
+    }
   }
   so = warp_sum_i64(so);
   si = warp_sum_i64(si);
@@ -675,83 +697,58 @@ __global__ void k_emit(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* par, 
   }
 }
 
-// Node records (strength moves between parents) and children-list records.
+// Children-list records of the changed nodes; their strengths move from the
+// old parent's ancestors to the new one's, up to level `top` (the parents'
+// own strengths moved with the members; a supernode's are its members' sums).
 __global__ void k_emit_nodes(const int32_t* lC, const int32_t* nC, const int32_t* par, const int32_t* par_old,
-                             const int64_t* kout, const int64_t* kin, int bits, int32_t* ndx, int64_t* ndko,
-                             int64_t* ndki, int32_t* nnd, u64* ck, u64* cv, int32_t* ncr) {
+                             const int64_t* kout, const int64_t* kin, int bits, int q0, int top, int directed,
+                             Chain ch, u64* ck, u64* cv, int32_t* ncr) {
   const int32_t n = *nC;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t u = lC[k];
     const int32_t po = par_old[u], pn = par[u];
-    if (ndx) {
-      if (po >= 0) {
-        const int32_t p = atomicAdd(nnd, 1);
-        ndx[p] = po;
-        ndko[p] = -kout[u];
-        ndki[p] = -kin[u];
-      }
-      const int32_t p = atomicAdd(nnd, 1);
-      ndx[p] = pn;
-      ndko[p] = kout[u];
-      ndki[p] = kin[u];
-    }
-    if (po >= 0) {
-      const int32_t p = atomicAdd(ncr, 1);
-      ck[p] = ((u64)po << bits) | (u64)u;
-      cv[p] = (u64)(int64_t)-1;
-    }
-    const int32_t p = atomicAdd(ncr, 1);
+    const int32_t p = atomicAdd(ncr, po >= 0 ? 2 : 1);
     ck[p] = ((u64)pn << bits) | (u64)u;
     cv[p] = (u64)(int64_t)1;
-  }
-}
-
-// Strength moves (node, out delta, in delta) of level-q0 nodes carried to
-// every ancestor level up to `top` (the strengths of a supernode are the sums
-// of its members').
-__global__ void k_chain_nodes(const int32_t* ndx, const int64_t* ndko, const int64_t* ndki, const int32_t* n,
-                              int q0, int top, int directed, Chain ch) {
-  const int32_t m = *n;
-  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
-    int32_t x = ndx[k];
-    const int64_t ko = ndko[k], ki = ndki[k];
-    for (int q = q0; q < top; ++q) {
-      x = ch.par[q][x];
-      if (x < 0) break;
-      atomic_add_i64(&ch.kout[q + 1][x], ko);
-      if (directed) atomic_add_i64(&ch.kin[q + 1][x], ki);
+    if (po >= 0) {
+      ck[p + 1] = ((u64)po << bits) | (u64)u;
+      cv[p + 1] = (u64)(int64_t)-1;
     }
-  }
-}
-
-__global__ void k_exist_cands(const int32_t* lC, const int32_t* nC, const int32_t* par, const int32_t* par_old,
-                              int32_t* stE, int32_t epE, int32_t* lE, int32_t* nE) {
-  const int32_t n = *nC;
-  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    const int32_t u = lC[k];
-    if (par_old[u] >= 0) stamp_add(stE, epE, par_old[u], lE, nE);
-    stamp_add(stE, epE, par[u], lE, nE);
+    const int64_t ko = kout[u], ki = kin[u];
+    for (int side = 0; side < 2; ++side) {
+      int32_t x = side ? pn : po;
+      for (int q = q0; q < top && x >= 0; ++q) {
+        x = ch.par[q][x];
+        if (x < 0) break;
+        atomic_add_i64(&ch.kout[q + 1][x], side ? ko : -ko);
+        if (directed) atomic_add_i64(&ch.kin[q + 1][x], side ? ki : -ki);
+      }
+    }
   }
 }
 
 // Existence after a level-q0 aggregate step, for the candidate level-q0 nodes
-// (old and new parents of the changed nodes): a node with members appears
-// (it has no parent yet); a node left without members dies and leaves its
-// parent, and a parent that thereby loses its last member dies in turn, up
-// the chain to level top.  The walk that takes a parent's member count to
-// zero carries on with that parent, so each death is handled once, and the
-// counts above q0 only fall meanwhile.  (An emptied node stays listed among
-// its parent's children; readers of the lists check the parent.)
+// (old and new parents of the changed nodes, each handled by the thread that
+// claims it): a node with members appears (it has no parent yet); a node left
+// without members dies and leaves its parent, and a parent that thereby loses
+// its last member dies in turn, up the chain to level top.  The walk that
+// takes a parent's member count to zero carries on with that parent, so each
+// death is handled once, and the counts above q0 only fall meanwhile.  (An
+// emptied node stays listed among its parent's children; readers of the
+// lists check the parent.)
 struct ExistChain {
   int32_t* cnt[8];
   uint8_t* alive[8];
   int32_t* par[8];
 };
 
-__global__ void k_exist_chain(const int32_t* lE, const int32_t* nE, int q0, int top, ExistChain ch, int32_t* err) {
-  const int32_t n = *nE;
-  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    int32_t x = lE[k];
+__global__ void k_exist_chain(const int32_t* lC, const int32_t* nC, const int32_t* par, const int32_t* par_old,
+                              int32_t* stE, int32_t epE, int q0, int top, ExistChain ch, int32_t* err) {
+  const int32_t n = *nC;
+  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < 2 * n; k += gridDim.x * blockDim.x) {
+    const int32_t u = lC[k >> 1];
+    int32_t x = (k & 1) ? par_old[u] : par[u];
+    if (x < 0 || !stamp_claim(stE, epE, x)) continue;
     int q = q0;
     const int32_t c = ch.cnt[q][x];
     if (!ch.alive[q][x]) {
@@ -775,35 +772,35 @@ __global__ void k_exist_chain(const int32_t* lE, const int32_t* nE, int q0, int 
   }
 }
 
-__global__ void k_relabel(const int32_t* l, const int32_t* n, const int32_t* par, const int32_t* lab,
-                          int32_t* lab_up) {
-  const int32_t m = *n;
-  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
-    const int32_t u = l[k];
-    lab_up[par[u]] = lab[u];
-  }
-}
-
-__global__ void k_nf_records(const u64* keys, int64_t n, int bits, const uint8_t* alive, int32_t* stA, int32_t epA,
-                             int32_t* lA, int32_t* nA) {
+// Level r + 1 after level r's aggregate step: the images of the frontier and
+// dissolved nodes take their labels, and NextFrontier is marked: the images of
+// U* and D (D's old parents too) and the endpoints of the level's nr weight
+// records, as far as they exist.  (Stamps make the three lists one set, so one
+// launch goes through them all; without stA only the labels are written.)
+__global__ void k_next_level(const int32_t* lU, const int32_t* nU, const int32_t* lD, const int32_t* nD,
+                             const int32_t* par, const int32_t* par_old, const int32_t* lab, int32_t* lab_up,
+                             const u64* keys, const int32_t* nr, int64_t nr_max, int bits, const uint8_t* alive,
+                             int32_t* stA, int32_t epA, int32_t* lA, int32_t* nA, int64_t* agg_recs) {
+  const int64_t mu = *nU, md = *nD;
+  const int64_t mr = keys ? min((int64_t)*nr, nr_max) : 0;
   const u64 mask = (((u64)1) << bits) - 1;
-  GRID_STRIDE(t, n) {
-    const int32_t x = (int32_t)(keys[t] >> bits), y = (int32_t)(keys[t] & mask);
-    if (alive[x]) stamp_add(stA, epA, x, lA, nA);
-    if (alive[y]) stamp_add(stA, epA, y, lA, nA);
-  }
-}
-
-__global__ void k_nf_nodes(const int32_t* l, const int32_t* n, const int32_t* par, const int32_t* par_old,
-                           const uint8_t* alive, int32_t* stA, int32_t epA, int32_t* lA, int32_t* nA) {
-  const int32_t m = *n;
-  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
-    const int32_t u = l[k];
-    const int32_t p = par[u];
-    if (p >= 0 && alive[p]) stamp_add(stA, epA, p, lA, nA);
-    if (par_old) {
-      const int32_t q = par_old[u];
-      if (q >= 0 && alive[q]) stamp_add(stA, epA, q, lA, nA);
+  if (blockIdx.x == 0 && threadIdx.x == 0 && mr) atomic_add_i64(agg_recs, mr);
+  GRID_STRIDE(t, mu + md + mr) {
+    if (t < mu + md) {
+      const int32_t u = t < mu ? lU[t] : lD[t - mu];
+      const int32_t p = par[u];
+      lab_up[p] = lab[u];
+      if (!stA) continue;
+      if (p >= 0 && alive[p]) stamp_add(stA, epA, p, lA, nA);
+      if (t >= mu) {
+        const int32_t q = par_old[u];
+        if (q >= 0 && alive[q]) stamp_add(stA, epA, q, lA, nA);
+      }
+    } else if (stA) {
+      const u64 key = keys[t - mu - md];
+      const int32_t x = (int32_t)(key >> bits), y = (int32_t)(key & mask);
+      if (alive[x]) stamp_add(stA, epA, x, lA, nA);
+      if (alive[y]) stamp_add(stA, epA, y, lA, nA);
     }
   }
 }
@@ -944,8 +941,16 @@ static void reset_err(ldl_ctx& c) {
 
 static unsigned long long* err_ptr(ldl_ctx& c) { return (unsigned long long*)&c.d_sc->err_key; }
 
+static void throw_at(int64_t key, const char* what) {
+  char buf[160];
+  snprintf(buf, sizeof buf, "%s: status %d at update %lld", what, (int)(key & 255), (long long)(key >> 8));
+  ldl_throw((ldl_status)(key & 255), buf);
+}
+
 int64_t ingest(ldl_ctx& c, const ldl_update* upd, int64_t count, int on_device, int64_t* dm) {
   *dm = 0;
+  k_batch_begin<<<1, K_COUNT, 0, c.s>>>(c.dcnt, c.d_sc);
+  CKL("k_batch_begin");
   if (count <= 0) return 0;
   const ldl_update* du = upd;
   if (!on_device) {
@@ -953,51 +958,38 @@ int64_t ingest(ldl_ctx& c, const ldl_update* upd, int64_t count, int on_device, 
     CK(cudaMemcpyAsync(c.upd.p, upd, sizeof(ldl_update) * (size_t)count, cudaMemcpyHostToDevice, c.s));
     du = c.upd.p;
   }
-  reset_err(c);
-  const int g = grid_for(count, TPB);
-  k_validate<<<g, TPB, 0, c.s>>>(du, count, c.n, err_ptr(c));
-  CKL("k_validate");
-  throw_err(c, err_ptr(c), "invalid update");
-  c.rk.reserve(2 * count + 2, c.s);
-  c.rv.reserve(2 * count + 2, c.s);
-  k_upd_keys<<<g, TPB, 0, c.s>>>(du, count, c.bits, c.directed, c.rk.p, c.rv.p);
-  CKL("k_upd_keys");
-  sort_pairs(c.rk, c.rv, c.tk, c.tv, count, 2 * c.bits, c.P, c.s);
-  // unique keys and their first positions
-  c.P.flag.reserve(count + 1, c.s);
-  c.P.pos.reserve(count + 1, c.s);
+  // (rk, rv) may change places with (tk, tv) in the sort, and takes the arcs
+  // of both directions at the end
+  const int64_t arcs = c.directed ? count : 2 * count;
+  for (DBuf<u64>* b : {&c.rk, &c.rv, &c.tk, &c.tv, &c.trk, &c.trv}) b->reserve(2 * count + 2, c.s);
   c.rk2.reserve(count + 1, c.s);
   c.rsum.reserve(count + 1, c.s);
-  c.rsum2.reserve(count + 1, c.s);
-  heads_launch(c.rk.p, count, c.P.flag.p, c.s);
-  const int64_t nu = scan_exclusive_i32(c.P.flag.p, c.P.pos.p, count, c.P, c.s, true);
-  k_unique_starts<<<g, TPB, 0, c.s>>>(c.rk.p, count, c.P.flag.p, c.P.pos.p, c.rk2.p, c.rsum.p);
-  CKL("k_unique_starts");
-  c.CS.pos.reserve(nu + 1, c.s);
-  c.CS.oldw.reserve(nu + 1, c.s);
-  csr_lookup<int32_t>(c.lv[0].out0, c.rk2.p, nu, c.bits, c.CS.pos.p, c.CS.oldw.p, c.CS, c.P, c.s,
-                      &c.d_sc->cnt[C_SEG]);
-  CK(cudaMemsetAsync(&c.d_sc->dm, 0, sizeof(int64_t), c.s));
-  k_seq<<<grid_for(nu, TPB), TPB, 0, c.s>>>(du, count, c.rv.p, c.rsum.p, nu, c.rk2.p, c.CS.oldw.p, c.bits,
-                                            c.directed, c.rsum2.p, err_ptr(c), &c.d_sc->dm);
+  unsigned long long* err = (unsigned long long*)&c.d_sc->err_key;
+  unsigned long long* err_seq = (unsigned long long*)&c.d_sc->err_seq;
+  const int g = grid_for(count, TPB);
+  k_upd_keys<<<g, TPB, 0, c.s>>>(du, count, c.n, c.bits, c.directed, c.rk.p, c.rv.p, err);
+  CKL("k_upd_keys");
+  sort_pairs(c.rk, c.rv, c.tk, c.tv, count, 2 * c.bits, c.P, c.s);
+  const int tiles = div_up(count, UQ_TPB);
+  const LookBack q = look_back_begin(c.P, tiles, c.s);
+  k_unique<<<tiles, UQ_TPB, 0, c.s>>>(c.rk.p, count, c.rk2.p, c.rsum.p, c.dcnt + K_NU, q);
+  CKL("k_unique");
+  const auto& g0 = c.lv[0].out0;
+  k_seq<<<g, TPB, 0, c.s>>>(du, count, c.rv.p, c.rsum.p, c.dcnt + K_NU, c.rk2.p, g0.off.p, g0.len.p, g0.col.p, g0.w.p,
+                            c.bits, c.directed, err_seq, &c.d_sc->dm, c.trk.p, c.trv.p, c.dcnt + K_REC);
   CKL("k_seq");
-  throw_err(c, err_ptr(c), "invalid update sequence");
-  {
-    const HostRead r{&c.d_sc->dm, dm, sizeof(int64_t)};
-    host_read(c, &r, 1);
-  }
+  // the changed arcs in order (each once, no change zero), on directed graphs
+  // followed by their in-direction records
+  sort_reduce(c.trk, c.trv, c.tk, c.tv, arcs, c.dcnt + K_REC, c.bits, c.directed, c.n, c.rk.p, (int64_t*)c.rv.p,
+              c.dcnt + K_NR, c.P, c.s);
+  int64_t e1 = -1, e2 = -1;
+  int32_t na = 0;
+  const HostRead rr[4] = {{err, &e1, sizeof(int64_t)}, {err_seq, &e2, sizeof(int64_t)},
+                          {&c.d_sc->dm, dm, sizeof(int64_t)}, {c.dcnt + K_NR, &na, sizeof(int32_t)}};
+  host_read(c, rr, 4);
+  if (e1 != -1) throw_at(e1, "invalid update");
+  if (e2 != -1) throw_at(e2, "invalid update sequence");
   if (c.m + *dm >= ((int64_t)1 << 50) || c.m + *dm < 0) ldl_throw(LDL_E_OVERFLOW, "total weight m would reach 2^50");
-  zero_cnt(c, K_REC);
-  // up to two arcs per distinct key (an undirected edge and its mirror); the
-  // sort above may have swapped rk / rv with its scratch, so their capacity
-  // is only known to cover `count`
-  c.rk.reserve(2 * nu + 2, c.s);
-  c.rv.reserve(2 * nu + 2, c.s);
-  k_emit_arcs<<<grid_for(nu, TPB), TPB, 0, c.s>>>(c.rk2.p, c.rsum2.p, nu, c.bits, c.directed, c.rk.p, c.rv.p,
-                                                  c.dcnt + K_REC);
-  CKL("k_emit_arcs");
-  const int64_t na = rd_cnt(c, K_REC);
-  sort_pairs(c.rk, c.rv, c.tk, c.tv, na, 2 * c.bits, c.P, c.s);
   return na;
 }
 
@@ -1019,29 +1011,23 @@ static void combine_in_out(ldl_ctx& c, const u64* keys, const u64* vals, int64_t
   CK(cudaMemcpyAsync(c.rv2.p + nr, c.trv.p, sizeof(u64) * (size_t)nr, cudaMemcpyDeviceToDevice, c.s));
 }
 
-// apply sorted unique records to a level's adjacency (both directions); the
-// endpoints of arcs that disappear are recorded for the level's next
-// refinement
-static void apply_level(ldl_ctx& c, int r, const u64* keys, const int64_t* vals, int64_t nr) {
-  if (nr <= 0) return;
+// Applies sorted unique records (directed: followed by their in-direction
+// copies) to a level's adjacency; the endpoints of arcs that disappear are
+// recorded for the level's next refinement.  nr records, or *n_dev of them
+// with nr an upper bound; returns their number.
+static int64_t apply_records(ldl_ctx& c, int r, const u64* keys, const int64_t* vals, int64_t nr,
+                             const int32_t* n_dev) {
   LevelState& Lr = c.lv[r];
   // a deleted arc can only disconnect the refined community holding both of
   // its endpoints (refined communities are connected); until the level's next
   // split its parents change only where a node empties and leaves its parent
   const DelTrack trk{Lr.stK.p, Lr.brk_ep, Lr.lK.p, c.dcnt + K_BRK0 + r, c.n, r < c.T ? Lr.par.p : nullptr};
-  const u64* k = keys;
-  const u64* v = (const u64*)vals;
-  int64_t m = nr;
-  if (c.directed) {
-    combine_in_out(c, keys, (const u64*)vals, nr);
-    k = c.rk2.p;
-    v = c.rv2.p;
-    m = 2 * nr;
-  }
-  if (r == 0)
-    csr_apply<int32_t>(c.lv[0].out0, k, (const int64_t*)v, m, c.bits, c.CS, c.P, c.s, c.d_sc, &trk);
-  else
-    csr_apply<int64_t>(c.lv[r].out, k, (const int64_t*)v, m, c.bits, c.CS, c.P, c.s, c.d_sc, &trk);
+  const int mul = c.directed ? 2 : 1;
+  const int64_t m = r == 0 ? csr_apply<int32_t>(c.lv[0].out0, keys, vals, mul * nr, n_dev, mul, c.bits, c.CS, c.P, c.s,
+                                                c.d_sc, &trk)
+                           : csr_apply<int64_t>(c.lv[r].out, keys, vals, mul * nr, n_dev, mul, c.bits, c.CS, c.P, c.s,
+                                                c.d_sc, &trk);
+  return m / mul;
 }
 
 static Chain chain_of(ldl_ctx& c, const int32_t* epA) {
@@ -1062,9 +1048,9 @@ static Chain chain_of(ldl_ctx& c, const int32_t* epA) {
 
 // Records of level q0 onto the pending lists of level q0 (with `self`) and
 // of every level above: each list is grown (keeping its contents) to hold n
-// more.
-static void chain_records(ldl_ctx& c, const u64* keys, const int64_t* vals, int64_t n, int q0, bool self,
-                          bool add_k) {
+// more (n_dev: their device count, n bounds it).
+static void chain_records(ldl_ctx& c, const u64* keys, const int64_t* vals, int64_t n, const int32_t* n_dev, int q0,
+                          bool self, bool add_k) {
   if (n <= 0 || (!self && q0 >= c.T)) return;
   if (n > INT32_MAX / 2) ldl_throw(LDL_E_OVERFLOW, "too many weight records in one step for the 32-bit counters");
   for (int q = self ? q0 : q0 + 1; q <= c.T; ++q) {
@@ -1075,14 +1061,13 @@ static void chain_records(ldl_ctx& c, const u64* keys, const int64_t* vals, int6
     L.pv.reserve(L.pend_ub + n + 1, c.s, true);
     L.pend_ub += n;
   }
-  k_chain_records<<<grid_for(n, TPB), TPB, 0, c.s>>>(keys, vals, n, c.bits, q0, c.T, self ? 1 : 0, add_k ? 1 : 0,
+  k_chain_records<<<grid_for(n, TPB), TPB, 0, c.s>>>(keys, vals, n, n_dev, c.bits, q0, c.T, self ? 1 : 0, add_k ? 1 : 0,
                                                      c.directed, chain_of(c, nullptr), c.dcnt + K_PEND0);
   CKL("k_chain_records");
 }
 
-void pending_reset(ldl_ctx& c) {
+void pending_reset(ldl_ctx& c) {  // the device counters are cleared by ingest
   for (auto& L : c.lv) L.pend_ub = 0;
-  CK(cudaMemsetAsync(c.dcnt + K_PEND0, 0, sizeof(int32_t) * 8, c.s));
 }
 
 // Level q's pending records, sorted by (row, col) and summed per arc (zero
@@ -1095,20 +1080,19 @@ void flush_level(ldl_ctx& c, int q, int64_t known) {
   L.pend_ub = 0;
   zero_cnt(c, K_PEND0 + q);
   if (n <= 0) return;
-  sort_pairs(L.pk, L.pv, c.tk, c.tv, n, 2 * c.bits, c.P, c.s);
   // own output buffers: a flush may run while the caller's records sit in rk / rv
-  c.flk.reserve(n + 1, c.s);
-  c.flv.reserve(n + 1, c.s);
-  const int64_t nr = reduce_by_key(L.pk.p, L.pv.p, n, c.flk.p, c.flv.p, c.P, c.s);
+  c.flk.reserve((c.directed ? 2 : 1) * n + 1, c.s);
+  c.flv.reserve((c.directed ? 2 : 1) * n + 1, c.s);
+  int32_t* nr = c.dcnt + K_FL;
+  sort_reduce(L.pk, L.pv, c.tk, c.tv, n, nullptr, c.bits, c.directed, c.n, c.flk.p, c.flv.p, nr, c.P, c.s);
   c.res.pending_records += n;
-  c.res.pending_applied += nr;
-  apply_level(c, q, c.flk.p, c.flv.p, nr);
+  c.res.pending_applied += apply_records(c, q, c.flk.p, c.flv.p, n, nr);
 }
 
 void repair_batch(ldl_ctx& c, int64_t na, const int32_t* epA, int32_t epT, int64_t dm) {
   if (na <= 0) return;
   // Algorithm 1, applying the batch: it changes level 0
-  apply_level(c, 0, c.rk.p, (const int64_t*)c.rv.p, na);
+  apply_records(c, 0, c.rk.p, (const int64_t*)c.rv.p, na, nullptr);
   // statistic repair: m, degrees, community totals (exactly, with sum_C K_out K_in)
   LevelState& L0 = c.lv[0];
   {
@@ -1146,7 +1130,7 @@ void repair_batch(ldl_ctx& c, int64_t na, const int32_t* epA, int32_t epT, int64
   CKL("k_chain_frontier");
   // the aggregate chain: W_q(anc(i), anc(j)) += delta and the strengths of
   // every level above 0; the weights are applied when each level is next read
-  chain_records(c, c.rk.p, (const int64_t*)c.rv.p, na, 0, false, true);
+  chain_records(c, c.rk.p, (const int64_t*)c.rv.p, na, nullptr, 0, false, true);
 }
 
 void pushdown(ldl_ctx& c, int r, int32_t epCh, int64_t moved_ub) {
@@ -1303,21 +1287,11 @@ int32_t split(ldl_ctx& c, int r, int32_t epD, int32_t epX) {
   return renamed ? rd_cnt(c, K_D) : nleft;
 }
 
-// Row entries of the changed nodes (list lC, count on the device, at most
-// n_hint) into need (out-rows) and need2 (in-rows).
+// deg: out-row and in-row entries of the changed nodes (k_changed); returns
+// the bound on the records (their count is at dcnt[K_REC])
 template <class WT>
-static void deg_sum(ldl_ctx& c, Adj<WT> out, Adj<WT> in, int64_t n_hint) {
-  static_assert(offsetof(DevScalars, need2) == offsetof(DevScalars, need) + 8, "adjacent accumulators");
-  CK(cudaMemsetAsync(&c.d_sc->need, 0, 2 * sizeof(int64_t), c.s));
-  k_deg_sum<WT><<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(out, in, c.lC.p, c.dcnt + K_C, &c.d_sc->need,
-                                                        &c.d_sc->need2);
-  CKL("k_deg_sum");
-}
-
-// deg: out-row and in-row entries of the changed nodes (deg_sum)
-template <class WT>
-static void emit_records(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t nC, int32_t epC, bool build,
-                         const int64_t (&deg)[2]) {
+static int64_t emit_records(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t nC, int32_t epC, bool build,
+                            const int64_t (&deg)[2]) {
   // at most a subtract and an add record per visited entry; in the static
   // build no node had a parent (no subtract records) and every node is
   // changed (no in-row records), so one record per out-row entry
@@ -1325,13 +1299,19 @@ static void emit_records(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t nC,
   if (cap > INT32_MAX) ldl_throw(LDL_E_OVERFLOW, "aggregate records beyond the 32-bit record counter");
   c.rk2.reserve(cap, c.s);
   c.rv2.reserve(cap, c.s);
-  zero_cnt(c, K_REC);
   ChunkMap m = chunk_map(c, c.lC.p, c.dcnt + K_C, nC, out.len, in.len);
   k_emit<WT><<<grid_for((int64_t)nC * 64, TPB, 16), TPB, 0, c.s>>>(out, in, m, c.lv[r].par.p, c.par_old.p,
                                                                           c.stC.p, epC, c.bits, c.rk2.p, c.rv2.p,
                                                                           c.dcnt + K_REC, cap, c.dcnt + K_ERR);
   CKL("k_emit");
+  return cap;
 }
+
+// Above this many records a step reads their exact number before it sorts them
+// and queues them on the levels above: up to four times as many are reserved
+// as come, which costs memory where the buffers are large and nothing but the
+// read (about 8 us) to avoid.
+constexpr int64_t AGG_EXACT = 1 << 20;
 
 void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bool build, int32_t nD) {
   (void)epD;
@@ -1339,101 +1319,97 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
   LevelState& N = c.lv[r + 1];
   // changed nodes
   sub_begin(c);
-  zero_cnt(c, K_C);
-  k_changed<<<grid_for(nD, TPB), TPB, 0, c.s>>>(c.lD.p, c.dcnt + K_D, L.par.p, c.par_old.p, c.stC.p, epC, c.lC.p,
-                                                c.dcnt + K_C);
-  CKL("k_changed");
-  // the changed nodes' row entries (lC is a subset of lD, so nD bounds the
-  // launch); one read returns them with |C| and |U*| (for the relabelling)
-  if (r == 0) deg_sum<int32_t>(c, adj_out0(c), adj_in0(c), nD);
-  else deg_sum<int64_t>(c, adj_out(c, r), adj_in(c, r), nD);
-  int32_t nC = 0, nUs = 0;
-  int64_t deg[2] = {0, 0};
+  static_assert(offsetof(DevScalars, need2) == offsetof(DevScalars, need) + 8, "adjacent accumulators");
   {
-    const HostRead rr[3] = {{c.dcnt + K_C, &nC, sizeof(int32_t)}, {c.dcnt + K_USTAR, &nUs, sizeof(int32_t)},
-                            {&c.d_sc->need, deg, 2 * sizeof(int64_t)}};
-    host_read(c, rr, 3);
+    ZeroSpans z;
+    z.mask = cnt_bit(K_C) | cnt_bit(K_REC) | cnt_bit(K_CREC);
+    z.p[0] = &c.d_sc->need;
+    z.nw[0] = 2;
+    zero_many(c, z);
   }
-  int64_t nr = 0;
+  int32_t nC = 0;
+  int64_t deg[2] = {0, 0};
+  if (nD > 0) {
+    const int32_t* lo = r == 0 ? adj_out0(c).len : adj_out(c, r).len;
+    const int32_t* li = r == 0 ? adj_in0(c).len : adj_in(c, r).len;
+    k_changed<<<grid_for(nD, TPB), TPB, 0, c.s>>>(c.lD.p, c.dcnt + K_D, L.par.p, c.par_old.p, c.stC.p, epC, c.lC.p,
+                                                  c.dcnt + K_C, lo, li, &c.d_sc->need, &c.d_sc->need2);
+    CKL("k_changed");
+    const HostRead rr[2] = {{c.dcnt + K_C, &nC, sizeof(int32_t)}, {&c.d_sc->need, deg, 2 * sizeof(int64_t)}};
+    host_read(c, rr, 2);
+  }
+  int64_t nr = 0;  // bound on the level r+1 records (their number is at dcnt[K_NR])
   if (nC > 0) {
-    if (r == 0) emit_records<int32_t>(c, r, adj_out0(c), adj_in0(c), nC, epC, build, deg);
-    else emit_records<int64_t>(c, r, adj_out(c, r), adj_in(c, r), nC, epC, build, deg);
-    // node and children records (they need only the parents), so that one
-    // read returns both record counts
-    c.ndx.reserve(2 * (int64_t)nC + 2, c.s);
-    c.ndko.reserve(2 * (int64_t)nC + 2, c.s);
-    c.ndki.reserve(2 * (int64_t)nC + 2, c.s);
+    int64_t nrec = r == 0 ? emit_records<int32_t>(c, r, adj_out0(c), adj_in0(c), nC, epC, build, deg)
+                          : emit_records<int64_t>(c, r, adj_out(c, r), adj_in(c, r), nC, epC, build, deg);
     c.crk.reserve(2 * (int64_t)nC + 2, c.s);
     c.crv.reserve(2 * (int64_t)nC + 2, c.s);
-    {
-      ZeroSpans z;
-      z.mask = cnt_bit(K_NREC) | cnt_bit(K_CREC);
-      zero_many(c, z);
-    }
     k_emit_nodes<<<grid_for(nC, TPB), TPB, 0, c.s>>>(c.lC.p, c.dcnt + K_C, L.par.p, c.par_old.p, L.kout.p,
-                                                     kin_of(c, r), c.bits, c.ndx.p, c.ndko.p, c.ndki.p,
-                                                     c.dcnt + K_NREC, c.crk.p, c.crv.p, c.dcnt + K_CREC);
+                                                     kin_of(c, r), c.bits, r + 1, build ? r + 1 : c.T, c.directed,
+                                                     chain_of(c, nullptr), c.crk.p, c.crv.p, c.dcnt + K_CREC);
     CKL("k_emit_nodes");
-    int32_t nrec32 = 0, ncr32 = 0;
-    {
-      const HostRead rr[2] = {{c.dcnt + K_REC, &nrec32, sizeof(int32_t)}, {c.dcnt + K_CREC, &ncr32, sizeof(int32_t)}};
-      host_read(c, rr, 2);
-    }
-    const int64_t nrec = nrec32, ncr = ncr32;
-    if (nrec > c.rk2.cap) ldl_throw(LDL_E_INVALID, "internal: aggregate records exceed their bound");
     sub_end(c, SU_AGG_EMIT);
     sub_begin(c);
-    sort_pairs(c.rk2, c.rv2, c.tk, c.tv, nrec, 2 * c.bits, c.P, c.s);
-    c.rk.reserve(nrec + 1, c.s);
-    c.rv.reserve(nrec + 1, c.s);
-    c.rsum.reserve(nrec + 1, c.s);
-    nr = reduce_by_key(c.rk2.p, c.rv2.p, nrec, c.rk.p, c.rsum.p, c.P, c.s);
-    CK(cudaMemcpyAsync(c.rv.p, c.rsum.p, sizeof(int64_t) * (size_t)nr, cudaMemcpyDeviceToDevice, c.s));
-    c.res.agg_records += nr;
-    sub_end(c, SU_AGG_SORT);
-    sub_begin(c);
-    sort_pairs(c.crk, c.crv, c.tk, c.tv, ncr, 2 * c.bits, c.P, c.s);
-    // keep the level r+1 record keys for NextFrontier
-    c.fk.reserve(nr + 1, c.s);
-    if (nr) CK(cudaMemcpyAsync(c.fk.p, c.rk.p, sizeof(u64) * (size_t)nr, cudaMemcpyDeviceToDevice, c.s));
     if (build) {
       // level r+1 starts empty: build its adjacency and the children lists
+      int32_t nrec32 = 0, ncr32 = 0;
+      {
+        const HostRead rr[2] = {{c.dcnt + K_REC, &nrec32, sizeof(int32_t)},
+                                {c.dcnt + K_CREC, &ncr32, sizeof(int32_t)}};
+        host_read(c, rr, 2);
+      }
+      const int64_t cnt = nrec32, ncr = ncr32;
+      if (cnt > nrec) ldl_throw(LDL_E_INVALID, "internal: aggregate records exceed their bound");
+      sort_pairs(c.rk2, c.rv2, c.tk, c.tv, cnt, 2 * c.bits, c.P, c.s);
+      c.rk.reserve(cnt + 1, c.s);
+      c.rsum.reserve(cnt + 1, c.s);
+      nr = reduce_by_key(c.rk2.p, c.rv2.p, cnt, c.rk.p, c.rsum.p, c.P, c.s);
+      c.res.agg_records += nr;
+      sub_end(c, SU_AGG_SORT);
+      sub_begin(c);
+      sort_pairs(c.crk, c.crv, c.tk, c.tv, ncr, 2 * c.bits, c.P, c.s);
       if (c.directed) {
-        combine_in_out(c, c.rk.p, c.rv.p, nr);
+        combine_in_out(c, c.rk.p, (const u64*)c.rsum.p, nr);
         csr_build<int64_t>(N.out, 2 * c.n, c.rk2.p, (const int64_t*)c.rv2.p, 2 * nr, c.bits, 25, c.CS, c.P, c.s);
       } else {
         csr_build<int64_t>(N.out, c.n, c.rk.p, c.rsum.p, nr, c.bits, 25, c.CS, c.P, c.s);
       }
       csr_build<int32_t>(L.children, c.n, c.crk.p, (const int64_t*)c.crv.p, ncr, c.bits, 25, c.CS, c.P, c.s);
     } else {
+      const int32_t* cnt_dev = c.dcnt + K_REC;
+      if (nrec > AGG_EXACT) {
+        const int64_t cnt = rd_cnt(c, K_REC);
+        if (cnt > nrec) ldl_throw(LDL_E_INVALID, "internal: aggregate records exceed their bound");
+        nrec = cnt;
+        cnt_dev = nullptr;
+      }
+      c.rk.reserve(nrec + 1, c.s);
+      c.rsum.reserve(nrec + 1, c.s);
+      if (nrec > 0)
+        sort_reduce(c.rk2, c.rv2, c.tk, c.tv, nrec, cnt_dev, c.bits, false, 0, c.rk.p, c.rsum.p, c.dcnt + K_NR, c.P,
+                    c.s);
+      nr = nrec;
+      if (nrec > AGG_EXACT) nr = rd_cnt(c, K_NR);
+      sub_end(c, SU_AGG_SORT);
+      sub_begin(c);
       // the level r+1 records join its pending list and, mapped through the
-      // current parents, the lists of the levels above; the strength moves
-      // reach every ancestor level at once
-      chain_records(c, c.rk.p, (const int64_t*)c.rv.p, nr, r + 1, true, false);
-      csr_apply<int32_t>(L.children, c.crk.p, (const int64_t*)c.crv.p, ncr, c.bits, c.CS, c.P, c.s, c.d_sc);
+      // current parents, the lists of the levels above
+      chain_records(c, c.rk.p, c.rsum.p, nr, c.dcnt + K_NR, r + 1, true, false);
+      sort_pairs(c.crk, c.crv, c.tk, c.tv, 2 * (int64_t)nC, 2 * c.bits, c.P, c.s, 0, c.dcnt + K_CREC);
+      csr_apply<int32_t>(L.children, c.crk.p, (const int64_t*)c.crv.p, 2 * (int64_t)nC, c.dcnt + K_CREC, 1, c.bits,
+                         c.CS, c.P, c.s, c.d_sc);
     }
     sub_end(c, SU_AGG_APPLY);
     sub_begin(c);
-    if (!build && r + 1 < c.T) {
-      k_chain_nodes<<<grid_for(2 * (int64_t)nC, TPB), TPB, 0, c.s>>>(c.ndx.p, c.ndko.p, c.ndki.p, c.dcnt + K_NREC,
-                                                                      r + 1, c.T, c.directed, chain_of(c, nullptr));
-      CKL("k_chain_nodes");
-    }
-    sub_end(c, SU_AGG_UP);
-    sub_begin(c);
     // existence: appear at r+1, emptied nodes cascade upwards
-    int32_t epE = c.next_epoch();
-    zero_cnt(c, K_E);
-    k_exist_cands<<<grid_for(nC, TPB), TPB, 0, c.s>>>(c.lC.p, c.dcnt + K_C, L.par.p, c.par_old.p, c.stE.p, epE,
-                                                      c.lE.p, c.dcnt + K_E);
-    CKL("k_exist_cands");
     ExistChain ech{};
     for (int q = 0; q <= c.T && q < 8; ++q) {
       ech.cnt[q] = c.lv[q].cnt.p;
       ech.alive[q] = c.lv[q].alive.p;
       ech.par[q] = c.lv[q].par.p;
     }
-    k_exist_chain<<<grid_for(2 * (int64_t)nC, TPB), TPB, 0, c.s>>>(c.lE.p, c.dcnt + K_E, r + 1, c.T, ech,
+    k_exist_chain<<<grid_for(2 * (int64_t)nC, TPB), TPB, 0, c.s>>>(c.lC.p, c.dcnt + K_C, L.par.p, c.par_old.p,
+                                                                    c.stE.p, c.next_epoch(), r + 1, c.T, ech,
                                                                     c.dcnt + K_ERR);
     CKL("k_exist_chain");
     // the error flag K_ERR is read once at the end of the batch (or of the static build)
@@ -1441,33 +1417,13 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
     sub_end(c, SU_AGG_EMIT);
     sub_begin(c);
   }
-  // relabel the level-(r+1) images of frontier and dissolved nodes
-  if (nUs > 0) {
-    k_relabel<<<grid_for(nUs, TPB), TPB, 0, c.s>>>(c.lUstar.p, c.dcnt + K_USTAR, L.par.p, L.lab.p, N.lab.p);
-    CKL("k_relabel");
-  }
-  if (nD > 0) {
-    k_relabel<<<grid_for(nD, TPB), TPB, 0, c.s>>>(c.lD.p, c.dcnt + K_D, L.par.p, L.lab.p, N.lab.p);
-    CKL("k_relabel");
-  }
-  // NextFrontier for level r+1
-  if (epA_next) {
-    if (nr > 0) {
-      k_nf_records<<<grid_for(nr, TPB), TPB, 0, c.s>>>(c.fk.p, nr, c.bits, N.alive.p, N.stA.p,
-                                                       epA_next, N.lA.p, c.dcnt + K_A0 + r + 1);
-      CKL("k_nf_records");
-    }
-    if (nD > 0) {
-      k_nf_nodes<<<grid_for(nD, TPB), TPB, 0, c.s>>>(c.lD.p, c.dcnt + K_D, L.par.p, c.par_old.p, N.alive.p, N.stA.p,
-                                                     epA_next, N.lA.p, c.dcnt + K_A0 + r + 1);
-      CKL("k_nf_nodes");
-    }
-    if (nUs > 0) {
-      k_nf_nodes<<<grid_for(nUs, TPB), TPB, 0, c.s>>>(c.lUstar.p, c.dcnt + K_USTAR, L.par.p, nullptr, N.alive.p,
-                                                      N.stA.p, epA_next, N.lA.p, c.dcnt + K_A0 + r + 1);
-      CKL("k_nf_nodes");
-    }
-  }
+  // |U*| stays on the device: the grid is bounded by two blocks per SM
+  const bool recs = nC > 0 && epA_next;
+  k_next_level<<<device_sms() * 2, TPB, 0, c.s>>>(c.lUstar.p, c.dcnt + K_USTAR, c.lD.p, c.dcnt + K_D, L.par.p,
+                                                  c.par_old.p, L.lab.p, N.lab.p, recs ? c.rk.p : nullptr,
+                                                  c.dcnt + K_NR, nr, c.bits, N.alive.p, epA_next ? N.stA.p : nullptr,
+                                                  epA_next, N.lA.p, c.dcnt + K_A0 + r + 1, &c.d_sc->agg_recs);
+  CKL("k_next_level");
   sub_end(c, SU_AGG_EXIST);
 }
 

@@ -110,6 +110,33 @@ __global__ void k_zero(int32_t* dcnt, ZeroSpans z) {
 }
 }  // namespace
 
+// Polls the mapped sequence word until the read `seq` has arrived.  Every so
+// often it asks the stream: an error ends the wait with that error; an idle
+// stream whose write is still not seen falls back to a full synchronisation
+// before failing.
+static void wait_page(ldl_ctx& c, int64_t seq) {
+  for (uint64_t spins = 1; c.h_pub[0] != seq; ++spins) {
+    if ((spins & 4095) == 0) {
+      const cudaError_t e = cudaStreamQuery(c.s);
+      if (e == cudaErrorNotReady) continue;
+      CK(e);
+      CK(cudaStreamSynchronize(c.s));
+      if (c.h_pub[0] != seq) ldl_throw(LDL_E_CUDA, "internal: a published value never reached the host");
+    }
+  }
+  std::atomic_thread_fence(std::memory_order_acquire);
+}
+
+Pub pub_begin(ldl_ctx& c) {
+  ++c.syncs;
+  return Pub{c.d_pub, ++c.pub_seq};
+}
+
+void pub_wait(ldl_ctx& c, int64_t* out, int n) {
+  wait_page(c, c.pub_seq);
+  for (int i = 0; i < n; ++i) out[i] = c.h_pub[1 + i];
+}
+
 void host_read(ldl_ctx& c, const HostRead* r, int n) {
   ++c.syncs;
   PubReq q{};
@@ -126,19 +153,7 @@ void host_read(ldl_ctx& c, const HostRead* r, int n) {
   const int64_t seq = ++c.pub_seq;
   k_publish<<<1, 64, 0, c.s>>>(q, (unsigned char*)(c.d_pub + 1), c.d_pub, seq);
   CKL("k_publish");
-  // Poll the mapped sequence word.  Every so often ask the stream: an error
-  // ends the wait with that error; an idle stream whose write is still not
-  // seen falls back to a full synchronisation before failing.
-  for (uint64_t spins = 1; c.h_pub[0] != seq; ++spins) {
-    if ((spins & 4095) == 0) {
-      const cudaError_t e = cudaStreamQuery(c.s);
-      if (e == cudaErrorNotReady) continue;
-      CK(e);
-      CK(cudaStreamSynchronize(c.s));
-      if (c.h_pub[0] != seq) ldl_throw(LDL_E_CUDA, "internal: a published value never reached the host");
-    }
-  }
-  std::atomic_thread_fence(std::memory_order_acquire);
+  wait_page(c, seq);
   const unsigned char* pay = (const unsigned char*)(c.h_pub + 1);
   for (int i = 0; i < n; ++i) memcpy(r[i].dst, pay + q.off[i], (size_t)r[i].bytes);
 }
@@ -210,7 +225,7 @@ void alloc_globals(ldl_ctx& c) {
     CK(cudaMemsetAsync(b->p, 0, sizeof(int32_t) * (size_t)n, c.s));
   }
   DBuf<int32_t>* ls[] = {&c.lU, &c.lS, &c.lUstar, &c.lMv, &c.lM0, &c.lD, &c.lC, &c.lR, &c.lR2, &c.lX, &c.lT,
-                         &c.lE, &c.lE2, &c.lCh, &c.lChg, &c.lTmp, &c.lG, &c.comp, &c.nbr, &c.cv, &c.csrc, &c.cdst, &c.cst, &c.bv,
+                         &c.lE2, &c.lCh, &c.lChg, &c.lTmp, &c.lG, &c.comp, &c.nbr, &c.cv, &c.csrc, &c.cdst, &c.cst, &c.bv,
                          &c.bsrc, &c.bdst, &c.oldlab, &c.par_old, &c.lab_before, &c.binT, &c.binS, &c.binM, &c.binM2, &c.binC, &c.binL};
   for (auto* b : ls) b->exact(n);
   c.best.exact(n);
@@ -230,23 +245,25 @@ void alloc_globals(ldl_ctx& c) {
   CK(cudaMemsetAsync(c.dcnt, 0, sizeof(int32_t) * K_COUNT, c.s));
   c.P.rd = [](void* owner, const HostRead* r, int n) { host_read(*(ldl_ctx*)owner, r, n); };
   c.P.rd_owner = &c;
+  c.P.pub_begin = [](void* owner) { return pub_begin(*(ldl_ctx*)owner); };
+  c.P.pub_wait = [](void* owner, int64_t* out, int n) { pub_wait(*(ldl_ctx*)owner, out, n); };
 }
 
 void free_all(ldl_ctx& c) {
   if (c.s) cudaStreamSynchronize(c.s);
   for (auto& L : c.lv) L.release();
   DBuf<int64_t>* b64[] = {&c.Kout, &c.Kin, &c.e, &c.cghi, &c.snapKo, &c.snapKi, &c.snapE, &c.binLoff, &c.binLsz,
-                          &c.gvals, &c.rsum, &c.rsum2, &c.ndko, &c.ndki,
+                          &c.gvals, &c.rsum, &c.rsum2, 
                           &c.chunk_pre, &c.hub_ecnt, &c.hub_epre, &c.pb_hi};
   for (auto* b : b64) b->release();
   DBuf<int32_t>* b32[] = {&c.stS, &c.stU, &c.stMv, &c.stB, &c.stM0, &c.stD, &c.stC, &c.stR, &c.stX, &c.stT,
                           &c.stE, &c.stCh, &c.stL, &c.lG, &c.comp, &c.nbr, &c.ckf, &c.lU, &c.lS, &c.lUstar, &c.lMv, &c.lM0, &c.lD, &c.lC, &c.lR,
-                          &c.lR2, &c.lX, &c.lT, &c.lE, &c.lE2, &c.lCh, &c.lChg, &c.lTmp, &c.cv, &c.csrc,
+                          &c.lR2, &c.lX, &c.lT, &c.lE2, &c.lCh, &c.lChg, &c.lTmp, &c.cv, &c.csrc,
                           &c.cdst, &c.cst, &c.bv, &c.bsrc, &c.bdst, &c.best, &c.role, &c.oldlab, &c.par_old,
-                          &c.lab_before, &c.binT, &c.binS, &c.binM, &c.binM2, &c.binC, &c.binL, &c.gkeys, &c.ndx,
+                          &c.lab_before, &c.binT, &c.binS, &c.binM, &c.binM2, &c.binC, &c.binL, &c.gkeys, 
                           &c.glist, &c.hcnt};
   for (auto* b : b32) b->release();
-  DBuf<u64>* bu[] = {&c.rk, &c.rv, &c.tk, &c.tv, &c.rk2, &c.rv2, &c.crk, &c.crv, &c.fk, &c.trk, &c.trv, &c.flk};
+  DBuf<u64>* bu[] = {&c.rk, &c.rv, &c.tk, &c.tv, &c.rk2, &c.rv2, &c.crk, &c.crv, &c.trk, &c.trv, &c.flk};
   for (auto* b : bu) b->release();
   c.flv.release();
   c.cglo.release();
@@ -418,7 +435,7 @@ static void static_build(ldl_ctx& c) {
 // they are freed here and grow again to what batches use.
 static void release_build_scratch(ldl_ctx& c) {
   CK(cudaStreamSynchronize(c.s));
-  DBuf<u64>* bu[] = {&c.rk, &c.rv, &c.tk, &c.tv, &c.rk2, &c.rv2, &c.crk, &c.crv, &c.fk, &c.trk, &c.trv};
+  DBuf<u64>* bu[] = {&c.rk, &c.rv, &c.tk, &c.tv, &c.rk2, &c.rv2, &c.crk, &c.crv, &c.trk, &c.trv};
   for (auto* b : bu) b->release();
   c.rsum.release();
   c.rsum2.release();
@@ -431,9 +448,7 @@ static void release_build_scratch(ldl_ctx& c) {
   c.pb_c.release();
   c.CS.release();
   c.P.hist.release();
-  c.P.pos.release();
   c.P.usum.release();
-  c.P.flag.release();
 }
 
 // ---------------------------------------------------------------- transactions
@@ -520,15 +535,12 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
   memset(&c.res, 0, sizeof(c.res));
   c.syncs = 0;
   pending_reset(c);
-  CK(cudaMemsetAsync(&c.d_sc->scanned, 0, sizeof(int64_t), c.s));
   const int T = c.T;
   int64_t dm = 0;
   stage_begin(c);
   const int64_t na = ingest(c, upd, count, on_device, &dm);
   stage_end(c, ST_INGEST);
   const int32_t epCh = c.next_epoch();
-  zero_cnt(c, K_CH);
-  zero_cnt(c, K_ERR);
   if (na == 0) {
     c.res.n_changed = 0;
     return;
@@ -536,10 +548,8 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
   if (!c.prm.no_rollback) txn_begin(c);
   std::vector<int32_t> epA(T + 2, 0);
   for (int r = 0; r <= T; ++r) {
-    epA[r] = c.next_epoch();
-    zero_cnt(c, K_A0 + r);
+    epA[r] = c.next_epoch();  // the lists' counters were cleared at the start of ingest
     c.lv[r].brk_ep = c.next_epoch();
-    zero_cnt(c, K_BRK0 + r);
   }
   stage_begin(c);
   const int32_t epT = c.next_epoch();
@@ -627,11 +637,12 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
   int32_t nchg = 0, err = 0, scan_bad = 0;
   int32_t* scan_flag = scan_error_flag(c.P);
   {
-    const HostRead rr[4] = {{c.dcnt + K_CHG, &nchg, sizeof(int32_t)},
+    const HostRead rr[5] = {{c.dcnt + K_CHG, &nchg, sizeof(int32_t)},
                             {c.dcnt + K_ERR, &err, sizeof(int32_t)},
                             {&c.d_sc->scanned, &c.res.edges_scanned, sizeof(int64_t)},
+                            {&c.d_sc->agg_recs, &c.res.agg_records, sizeof(int64_t)},
                             {scan_flag, &scan_bad, sizeof(int32_t)}};
-    host_read(c, rr, scan_flag ? 4 : 3);
+    host_read(c, rr, scan_flag ? 5 : 4);
   }
   c.res.n_changed = nchg;
   c.res.host_syncs = c.syncs;

@@ -65,8 +65,7 @@ struct ChunkCountIn {
 
 // whole input in one tile: scan and total in one launch
 template <class In>
-__global__ void k_scan_one(In in, int64_t* out, int64_t n, const int64_t* n_dev, int64_t* total) {
-  if (n_dev) n += *n_dev;
+__global__ void k_scan_one(In in, int64_t* out, int64_t n, int64_t* total) {
   const int64_t base = (int64_t)threadIdx.x * SC_ITEMS;
   int64_t loc[SC_ITEMS];
   int64_t s = 0;
@@ -95,14 +94,11 @@ __global__ void k_scan_one(In in, int64_t* out, int64_t n, const int64_t* n_dev,
 // *err and carries on (the host turns the flag into LDL_E_TIMEOUT).
 constexpr int LB_ITEMS = 8;
 constexpr int LB_TILE = SC_THREADS * LB_ITEMS;
-constexpr uint32_t LB_SPINS = 1u << 20;
 
 template <class In>
-__global__ void __launch_bounds__(SC_THREADS) k_scan_lb(In in, int64_t* out, int64_t n, const int64_t* n_dev,
-                                                        u64* st, int32_t* ctr, uint32_t ep, int64_t* total,
-                                                        int32_t* err) {
+__global__ void __launch_bounds__(SC_THREADS) k_scan_lb(In in, int64_t* out, int64_t n, u64* st, int32_t* ctr,
+                                                        uint32_t ep, int64_t* total, int32_t* err) {
   __shared__ int64_t s_tile, s_pre;
-  if (n_dev) n += *n_dev;  // launched for an upper bound; tiles past n leave at once
   if (threadIdx.x == 0) s_tile = atomicAdd(ctr, 1);
   __syncthreads();
   const int64_t tile = s_tile;
@@ -170,11 +166,24 @@ __global__ void __launch_bounds__(SC_THREADS) k_scan_lb(In in, int64_t* out, int
 constexpr int RS_THREADS = 256;
 constexpr int RS_ITEMS = 8;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
+// A sort's extras: the device count of its pairs (else the host's n), and,
+// with tbits > 0, the read transposes each key ((row, col) -> (col + row_off,
+// row) with tbits per half) and the result goes behind the n input pairs.
+struct RsExt {
+  const int32_t* n_dev;
+  int tbits;
+  int64_t row_off;
+  int64_t* zero;  // n words cleared on the way (null: none)
+};
+__device__ inline u64 transposed(u64 key, int bits, int64_t row_off) {
+  return (((key & ((((u64)1) << bits) - 1)) + (u64)row_off) << bits) | (key >> bits);
+}
 static_assert(RS_THREADS == 256 && SC_THREADS == 256, "one thread per digit");
 
 // Digit histogram of tile b (RS_TILE keys from b * RS_TILE) into column b
 // of ghist (digit-major: ghist[d * nb + b]).
-__device__ inline void rs_hist_tile(const u64* keys, int64_t n, int shift, int64_t nb, int64_t* ghist, int64_t b) {
+__device__ inline void rs_hist_tile(const u64* keys, int64_t n, int shift, int64_t nb, int64_t* ghist, int64_t b,
+                                    int tbits = 0, int64_t row_off = 0) {
   __shared__ uint32_t h[256];
   for (int i = threadIdx.x; i < 256; i += RS_THREADS) h[i] = 0;
   const int lane = threadIdx.x & 31;
@@ -182,7 +191,9 @@ __device__ inline void rs_hist_tile(const u64* keys, int64_t n, int shift, int64
   int d[RS_ITEMS];
   for (int k = 0; k < RS_ITEMS; ++k) {  // all loads in flight before any shuffle
     const int64_t i = base + (int64_t)k * RS_THREADS + threadIdx.x;
-    d[k] = i < n ? (int)((keys[i] >> shift) & 255) : 256;
+    u64 x = i < n ? keys[i] : 0;
+    if (tbits) x = transposed(x, tbits, row_off);
+    d[k] = i < n ? (int)((x >> shift) & 255) : 256;
   }
   __syncthreads();
   for (int k = 0; k < RS_ITEMS; ++k) {
@@ -195,8 +206,13 @@ __device__ inline void rs_hist_tile(const u64* keys, int64_t n, int shift, int64
   __syncthreads();  // h is reset by the block's next tile
 }
 
-__global__ void k_rs_hist(const u64* keys, int64_t n, int shift, int64_t nb, int64_t* ghist) {
-  rs_hist_tile(keys, n, shift, nb, ghist, blockIdx.x);
+__global__ void k_rs_hist(const u64* keys, int64_t n, int shift, int64_t nb, int64_t* ghist, RsExt x, int first,
+                          int in_off) {
+  if (x.n_dev) n = min(n, (int64_t)*x.n_dev);
+  if (x.zero && first)
+    for (int64_t i = (int64_t)blockIdx.x * RS_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * RS_THREADS)
+      x.zero[i] = 0;
+  rs_hist_tile(in_off ? keys + n : keys, n, shift, nb, ghist, blockIdx.x, first ? x.tbits : 0, x.row_off);
 }
 
 // One block per digit: exclusive scan of the digit's tile counts in place
@@ -236,7 +252,8 @@ __global__ void __launch_bounds__(SC_THREADS) k_rs_dscan(int64_t* ghist, int64_t
 // tile b) is the exclusive prefix of the digit totals dtot at d plus the
 // per-digit scanned tile count goff[d * nb + b].
 __device__ inline void rs_scatter_tile(const u64* keys, const u64* vals, u64* okeys, u64* ovals, int64_t n, int shift,
-                                       int64_t nb, const int64_t* goff, const int64_t* dtot, int64_t b) {
+                                       int64_t nb, const int64_t* goff, const int64_t* dtot, int64_t b, int tbits = 0,
+                                       int64_t row_off = 0) {
   constexpr int NW = RS_THREADS / WARP;
   __shared__ int32_t whist[NW][256];  // per-warp digit counts, then per-warp exclusive bases
   __shared__ int32_t tstart[256];     // tile-local start of each digit
@@ -245,7 +262,7 @@ __device__ inline void rs_scatter_tile(const u64* keys, const u64* vals, u64* ok
   __shared__ u64 sv[RS_TILE];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int64_t base = b * RS_TILE;
-  const int tile_n = (int)min((int64_t)RS_TILE, n - base);
+  const int tile_n = (int)max((int64_t)0, min((int64_t)RS_TILE, n - base));
   for (int d = lane; d < 256; d += 32) whist[wid][d] = 0;
   {
     int64_t total;
@@ -259,6 +276,7 @@ __device__ inline void rs_scatter_tile(const u64* keys, const u64* vals, u64* ok
     const bool valid = li < tile_n;
     key[k] = valid ? keys[base + li] : 0;
     val[k] = valid ? vals[base + li] : 0;
+    if (tbits) key[k] = transposed(key[k], tbits, row_off);
   }
   for (int k = 0; k < RS_ITEMS; ++k) {
     const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
@@ -307,28 +325,50 @@ __device__ inline void rs_scatter_tile(const u64* keys, const u64* vals, u64* ok
 
 __global__ void __launch_bounds__(RS_THREADS, 4) k_rs_scatter(const u64* keys, const u64* vals, u64* okeys,
                                                               u64* ovals, int64_t n, int shift, int64_t nb,
-                                                              const int64_t* goff, const int64_t* dtot) {
-  rs_scatter_tile(keys, vals, okeys, ovals, n, shift, nb, goff, dtot, blockIdx.x);
+                                                              const int64_t* goff, const int64_t* dtot, RsExt x,
+                                                              int first, int in_off, int out_off) {
+  if (x.n_dev) n = min(n, (int64_t)*x.n_dev);
+  rs_scatter_tile(in_off ? keys + n : keys, in_off ? vals + n : vals, out_off ? okeys + n : okeys,
+                  out_off ? ovals + n : ovals, n, shift, nb, goff, dtot, blockIdx.x, first ? x.tbits : 0, x.row_off);
 }
 
 // The whole multi-tile sort in one cooperative launch (all nb tiles'
 // blocks co-resident): per 8-bit pass the tile histograms, the per-digit
 // scans over tiles and the scatter, separated by grid barriers, ping-ponging
-// between (keys, vals) and (tk, tv).  Replaces three launches per pass.
+// between (keys, vals) and (tk, tv).  Replaces three launches per pass.  A
+// transposing sort ping-pongs between the place behind its input and (tk,
+// tv) such that the last pass ends there.
 __global__ void __launch_bounds__(RS_THREADS, 4) k_rs_coop(u64* keys, u64* vals, u64* tk, u64* tv, int64_t n,
-                                                           int lo_bit, int bits, int64_t nb, int64_t* ghist,
-                                                           int64_t* dtot) {
+                                                           int lo_bit, int bits, int64_t* ghist, int64_t* dtot,
+                                                           RsExt x) {
   cg::grid_group grid = cg::this_grid();
+  if (x.n_dev) n = min(n, (int64_t)*x.n_dev);
+  const int64_t nb = (n + RS_TILE - 1) / RS_TILE;
+  if (x.zero)
+    for (int64_t i = (int64_t)blockIdx.x * RS_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * RS_THREADS)
+      x.zero[i] = 0;
   u64 *ik = keys, *iv = vals, *ok = tk, *ov = tv;
+  u64 *nk = keys, *nv = vals;  // written by the pass after the first
+  if (x.tbits) {
+    nk = keys + n;
+    nv = vals + n;
+    if (((bits - lo_bit + 7) / 8) & 1) {
+      ok = nk; ov = nv;
+      nk = tk; nv = tv;
+    }
+  }
   for (int shift = lo_bit; shift < bits; shift += 8) {
-    for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) rs_hist_tile(ik, n, shift, nb, ghist, b);
+    const int tb = shift == lo_bit ? x.tbits : 0;
+    for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) rs_hist_tile(ik, n, shift, nb, ghist, b, tb, x.row_off);
     grid.sync();
     for (int d = blockIdx.x; d < 256; d += gridDim.x) rs_dscan_digit(ghist, nb, dtot, d);
     grid.sync();
-    for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) rs_scatter_tile(ik, iv, ok, ov, n, shift, nb, ghist, dtot, b);
+    for (int64_t b = blockIdx.x; b < nb; b += gridDim.x)
+      rs_scatter_tile(ik, iv, ok, ov, n, shift, nb, ghist, dtot, b, tb, x.row_off);
     grid.sync();
-    u64* t = ik; ik = ok; ok = t;
-    t = iv; iv = ov; ov = t;
+    ik = ok; iv = ov;
+    u64* t = ok; ok = nk; nk = t;
+    t = ov; ov = nv; nv = t;
   }
 }
 
@@ -337,12 +377,92 @@ __global__ void __launch_bounds__(RS_THREADS, 4) k_rs_coop(u64* keys, u64* vals,
 // contiguous sub-tile (rounds of 32, stable), the block turns the per-warp
 // digit counts into positions, the pairs are placed in shared memory in
 // digit order and read back in the same warp-contiguous layout.
-__global__ void __launch_bounds__(RS_THREADS) k_rs_small(u64* keys, u64* vals, int n, int lo_bit, int bits) {
+struct RsSmall {
+  int32_t whist[RS_THREADS / WARP][256];
+  int32_t tstart[256];
+  u64 sk[RS_TILE];
+  u64 sv[RS_TILE];
+};
+
+__device__ inline void rs_small_passes(RsSmall& m, u64 (&key)[RS_ITEMS], u64 (&val)[RS_ITEMS], int n, int lo_bit,
+                                       int bits) {
   constexpr int NW = RS_THREADS / WARP;
-  __shared__ int32_t whist[NW][256];
-  __shared__ int32_t tstart[256];
-  __shared__ u64 sk[RS_TILE];
-  __shared__ u64 sv[RS_TILE];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  for (int shift = lo_bit; shift < bits; shift += 8) {
+    for (int d = lane; d < 256; d += 32) m.whist[wid][d] = 0;
+    __syncwarp();
+    int rk[RS_ITEMS];
+    for (int k = 0; k < RS_ITEMS; ++k) {
+      const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
+      const int d = li < n ? (int)((key[k] >> shift) & 255) : 256;
+      const unsigned peers = __match_any_sync(0xffffffffu, d);
+      const int before = d < 256 ? m.whist[wid][d] : 0;
+      rk[k] = before + __popc(peers & ((1u << lane) - 1u));
+      __syncwarp();
+      if (d < 256 && lane == __ffs(peers) - 1) m.whist[wid][d] = before + __popc(peers);
+      __syncwarp();
+    }
+    __syncthreads();
+    int cnt = 0;
+    for (int w = 0; w < NW; ++w) {  // thread = digit (RS_THREADS == 256)
+      const int c = m.whist[w][tid];
+      m.whist[w][tid] = cnt;
+      cnt += c;
+    }
+    int64_t total;
+    m.tstart[tid] = (int32_t)block_excl_scan_i64(cnt, &total);
+    __syncthreads();
+    for (int k = 0; k < RS_ITEMS; ++k) {
+      const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
+      if (li < n) {
+        const int d = (int)((key[k] >> shift) & 255);
+        const int p = m.tstart[d] + m.whist[wid][d] + rk[k];
+        m.sk[p] = key[k];
+        m.sv[p] = val[k];
+      }
+    }
+    __syncthreads();
+    for (int k = 0; k < RS_ITEMS; ++k) {
+      const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
+      if (li < n) {
+        key[k] = m.sk[li];
+        val[k] = m.sv[li];
+      }
+    }
+    __syncthreads();  // whist, tstart and the staging buffers are rewritten next pass
+  }
+}
+
+__global__ void __launch_bounds__(RS_THREADS) k_rs_small(u64* keys, u64* vals, int n, const int32_t* n_dev, int lo_bit,
+                                                         int bits) {
+  __shared__ RsSmall m;
+  if (n_dev) n = min(n, *n_dev);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  u64 key[RS_ITEMS], val[RS_ITEMS];
+  for (int k = 0; k < RS_ITEMS; ++k) {
+    const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
+    key[k] = li < n ? keys[li] : 0;
+    val[k] = li < n ? vals[li] : 0;
+  }
+  rs_small_passes(m, key, val, n, lo_bit, bits);
+  for (int k = 0; k < RS_ITEMS; ++k) {
+    const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
+    if (li < n) {
+      keys[li] = key[k];
+      vals[li] = val[k];
+    }
+  }
+}
+
+// Sort by the low 2 * bits key bits, sum per key with zero sums dropped, and
+// with `both` the same records transposed behind them, in (row, col) order
+// (rows from row_off): sort_reduce() for n <= RS_TILE in one launch.
+__global__ void __launch_bounds__(RS_THREADS) k_rs_small_reduce(const u64* keys, const u64* vals, int n,
+                                                                const int32_t* n_dev, int bits, int both,
+                                                                int64_t row_off, u64* okeys, int64_t* ovals,
+                                                                int32_t* nr) {
+  __shared__ RsSmall m;
+  if (n_dev) n = min(n, *n_dev);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   u64 key[RS_ITEMS], val[RS_ITEMS];
   for (int k = 0; k < RS_ITEMS; ++k) {
@@ -350,54 +470,81 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_small(u64* keys, u64* vals, i
     key[k] = li < n ? keys[li] : 0;
     val[k] = li < n ? vals[li] : 0;
   }
-  for (int shift = lo_bit; shift < bits; shift += 8) {
-    for (int d = lane; d < 256; d += 32) whist[wid][d] = 0;
-    __syncwarp();
-    int rk[RS_ITEMS];
-    for (int k = 0; k < RS_ITEMS; ++k) {
-      const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
-      const int d = li < n ? (int)((key[k] >> shift) & 255) : 256;
-      const unsigned peers = __match_any_sync(0xffffffffu, d);
-      const int before = d < 256 ? whist[wid][d] : 0;
-      rk[k] = before + __popc(peers & ((1u << lane) - 1u));
-      __syncwarp();
-      if (d < 256 && lane == __ffs(peers) - 1) whist[wid][d] = before + __popc(peers);
-      __syncwarp();
-    }
-    __syncthreads();
-    int cnt = 0;
-    for (int w = 0; w < NW; ++w) {  // thread = digit (RS_THREADS == 256)
-      const int c = whist[w][tid];
-      whist[w][tid] = cnt;
-      cnt += c;
-    }
-    int64_t total;
-    tstart[tid] = (int32_t)block_excl_scan_i64(cnt, &total);
-    __syncthreads();
-    for (int k = 0; k < RS_ITEMS; ++k) {
-      const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
-      if (li < n) {
-        const int d = (int)((key[k] >> shift) & 255);
-        const int p = tstart[d] + whist[wid][d] + rk[k];
-        sk[p] = key[k];
-        sv[p] = val[k];
-      }
-    }
-    __syncthreads();
-    for (int k = 0; k < RS_ITEMS; ++k) {
-      const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
-      if (li < n) {
-        key[k] = sk[li];
-        val[k] = sv[li];
-      }
-    }
-    __syncthreads();  // whist, tstart and the staging buffers are rewritten next pass
+  rs_small_passes(m, key, val, n, 0, 2 * bits);
+  // sorted pairs into shared memory, RS_ITEMS consecutive ones per thread
+  for (int k = 0; k < RS_ITEMS; ++k) {
+    const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
+    m.sk[li] = key[k];
+    m.sv[li] = val[k];
   }
+  __syncthreads();
+  const int i0 = tid * RS_ITEMS;
+  int heads = 0;
+  int64_t sum = 0;
+  for (int k = 0; k < RS_ITEMS; ++k) {
+    const int i = i0 + k;
+    key[k] = m.sk[i];
+    heads += i < n && (i == 0 || key[k] != m.sk[i - 1]);
+    sum += i < n ? (int64_t)m.sv[i] : 0;
+  }
+  // segment numbers, and running sums whose differences at the segments' ends
+  // are the segment sums (both modulo 2^64)
+  int64_t nseg64, all;
+  int seg = (int)block_excl_scan_i64(heads, &nseg64);
+  int64_t run = block_excl_scan_i64(sum, &all);
+  const int nseg = (int)nseg64;
+  u64 hk[RS_ITEMS];
+  int64_t hr[RS_ITEMS];
+  int hs = 0;
+  for (int k = 0; k < RS_ITEMS; ++k) {
+    const int i = i0 + k;
+    if (i < n && (i == 0 || key[k] != m.sk[i - 1])) {
+      hk[hs] = key[k];
+      hr[hs] = run;
+      ++hs;
+    }
+    run += i < n ? (int64_t)m.sv[i] : 0;
+  }
+  __syncthreads();
+  for (int k = 0; k < hs; ++k) {
+    m.sk[seg + k] = hk[k];
+    m.sv[seg + k] = (u64)hr[k];
+  }
+  __syncthreads();
+  int live = 0;
+  for (int k = 0; k < RS_ITEMS; ++k) {
+    const int s = i0 + k;
+    hk[k] = s < nseg ? m.sk[s] : 0;
+    hr[k] = s < nseg ? (s + 1 < nseg ? (int64_t)m.sv[s + 1] : all) - (int64_t)m.sv[s] : 0;
+    live += hr[k] != 0;
+  }
+  int64_t nlive;
+  int p = (int)block_excl_scan_i64(live, &nlive);  // its barriers also end the reads above
+  for (int k = 0; k < RS_ITEMS; ++k)
+    if (hr[k] != 0) {
+      okeys[p] = hk[k];
+      ovals[p] = hr[k];
+      m.sk[p] = transposed(hk[k], bits, row_off);
+      m.sv[p] = (u64)hr[k];
+      ++p;
+    }
+  if (tid == 0) *nr = (int32_t)nlive;
+  if (!both) return;
+  __syncthreads();
+  n = (int)nlive;
+  for (int k = 0; k < RS_ITEMS; ++k) {
+    const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
+    key[k] = li < n ? m.sk[li] : 0;
+    val[k] = li < n ? m.sv[li] : 0;
+  }
+  __syncthreads();
+  // the records are in (row, col) order: a stable sort on the new row alone
+  rs_small_passes(m, key, val, n, bits, 2 * bits + 1);
   for (int k = 0; k < RS_ITEMS; ++k) {
     const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
     if (li < n) {
-      keys[li] = key[k];
-      vals[li] = val[k];
+      okeys[n + li] = key[k];
+      ovals[n + li] = (int64_t)val[k];
     }
   }
 }
@@ -420,7 +567,7 @@ constexpr int CS_NW = CS_THREADS / WARP;
 constexpr int CS_MAX = CS_CL * CS_TILE;
 
 __global__ void __cluster_dims__(CS_CL, 1, 1) __launch_bounds__(CS_THREADS, 1)
-    k_rs_cluster(u64* keys, u64* vals, int n, int lo_bit, int bits) {
+    k_rs_cluster(u64* keys, u64* vals, int n, int lo_bit, int bits, RsExt x) {
   extern __shared__ u64 cs_smem[];
   u64* sk = cs_smem;
   u64* sv = cs_smem + CS_TILE;
@@ -432,12 +579,19 @@ __global__ void __cluster_dims__(CS_CL, 1, 1) __launch_bounds__(CS_THREADS, 1)
   const int c = (int)cl.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int base = c * CS_TILE;
+  if (x.n_dev) n = min(n, *x.n_dev);
   const int tile_n = max(0, min(CS_TILE, n - base));
   u64 key[CS_ITEMS], val[CS_ITEMS];
   for (int k = 0; k < CS_ITEMS; ++k) {
     const int li = wid * (CS_ITEMS * 32) + k * 32 + lane;
     key[k] = li < tile_n ? keys[base + li] : 0;
     val[k] = li < tile_n ? vals[base + li] : 0;
+    if (x.tbits) key[k] = transposed(key[k], x.tbits, x.row_off);
+    if (x.zero && li < tile_n) x.zero[base + li] = 0;
+  }
+  if (x.tbits) {  // the result goes behind the input
+    keys += n;
+    vals += n;
   }
   for (int shift = lo_bit; shift < bits; shift += 8) {
     for (int d = lane; d < 256; d += 32) whist[wid][d] = 0;
@@ -522,18 +676,14 @@ __global__ void __cluster_dims__(CS_CL, 1, 1) __launch_bounds__(CS_THREADS, 1)
 }
 
 // ---------------------------------------------------------------- reduce by key
-__global__ void k_heads(const u64* keys, int64_t n, int32_t* flag) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    flag[i] = (i == 0 || keys[i] != keys[i - 1]) ? 1 : 0;
-}
-
 // Segment sums of sorted keys: each thread takes RBK_RUN consecutive pairs.
 // A segment that starts and ends inside the run is stored; a segment that
 // crosses a run boundary is added atomically at its head (usum is zeroed
 // first).  The head of a run's leading partial segment is found by a binary
 // search for the first equal key.
 constexpr int RBK_RUN = 8;
-__global__ void k_segsum(const u64* keys, const u64* vals, int64_t n, int64_t* usum) {
+__global__ void k_segsum(const u64* keys, const u64* vals, int64_t n, const int32_t* n_dev, int64_t* usum) {
+  if (n_dev) n = min(n, (int64_t)*n_dev);
   const int64_t nt = (n + RBK_RUN - 1) / RBK_RUN;
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nt; r += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i0 = r * RBK_RUN, i1 = min(i0 + RBK_RUN, n);
@@ -563,19 +713,58 @@ __global__ void k_segsum(const u64* keys, const u64* vals, int64_t n, int64_t* u
   }
 }
 
-// flag = segment head with a nonzero sum
-__global__ void k_nonzero_heads(const u64* keys, const int64_t* usum, int64_t n, int32_t* flag) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    flag[i] = (i == 0 || keys[i] != keys[i - 1]) && usum[i] != 0;
-}
-
-__global__ void k_compact_pairs(const u64* ukeys, const int64_t* usum, int64_t nu, const int32_t* flag,
-                                const int64_t* pos, u64* okeys, int64_t* ovals) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nu; i += (int64_t)gridDim.x * blockDim.x)
-    if (flag[i]) {
-      okeys[pos[i]] = ukeys[i];
-      ovals[pos[i]] = usum[i];
+// Compacts the segment heads with nonzero sums (keys, sums) in one pass with
+// look-back; the last tile writes their number.
+__global__ void __launch_bounds__(SC_THREADS) k_reduce_out(const u64* keys, const int64_t* usum, int64_t n,
+                                                           const int32_t* n_dev, u64* okeys, int64_t* ovals,
+                                                           int32_t* nr, int64_t* nr64, LookBack q) {
+  __shared__ int64_t s_tile, s_pre;
+  if (n_dev) n = min(n, (int64_t)*n_dev);
+  if (threadIdx.x == 0) s_tile = atomicAdd(q.ctr, 1);
+  __syncthreads();
+  const int64_t tile = s_tile;
+  if (tile * LB_TILE >= n && tile > 0) return;
+  // warp-contiguous rounds, so that a warp's loads are whole lines
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t base = tile * LB_TILE + wid * (LB_ITEMS * 32);
+  u64 key[LB_ITEMS];
+  int64_t sum[LB_ITEMS];
+  unsigned live = 0, mask[LB_ITEMS];
+  int cnt = 0;
+  for (int k = 0; k < LB_ITEMS; ++k) {
+    const int64_t i = base + k * 32 + lane;
+    key[k] = i < n ? keys[i] : 0;
+    sum[k] = i < n && (i == 0 || key[k] != keys[i - 1]) ? usum[i] : 0;
+    mask[k] = __ballot_sync(0xffffffffu, sum[k] != 0);
+    live |= (sum[k] != 0 ? 1u : 0u) << k;
+    cnt += __popc(mask[k]);
+  }
+  // exclusive offset of the warp: only lane 0 contributes its count
+  u64 tot;
+  u64 ex = block_scan<SC_THREADS>(lane == 0 ? (u64)cnt : 0, &tot);
+  ex = __shfl_sync(0xffffffffu, ex, 0);
+  if (threadIdx.x < 32) {
+    const int64_t agg[1] = {(int64_t)tot};
+    int64_t pre[1];
+    look_back<1>(q.st, tile, agg, pre, q.ep, q.err);
+    if (threadIdx.x == 0) {
+      s_pre = pre[0];
+      if ((tile + 1) * LB_TILE >= n) {
+        if (nr) *nr = (int32_t)(pre[0] + agg[0]);
+        if (nr64) *nr64 = pre[0] + agg[0];
+      }
     }
+  }
+  __syncthreads();
+  int64_t p = s_pre + (int64_t)ex;
+  for (int k = 0; k < LB_ITEMS; ++k) {
+    if ((live >> k) & 1u) {
+      const int64_t at = p + __popc(mask[k] & ((1u << lane) - 1u));
+      okeys[at] = key[k];
+      ovals[at] = sum[k];
+    }
+    p += __popc(mask[k]);
+  }
 }
 
 }  // namespace
@@ -605,19 +794,22 @@ static uint32_t lb_begin(Prims& P, int64_t n, cudaStream_t s) {
   return P.lb_ep;
 }
 
-// n items, or (n_dev != nullptr) *n_dev + n items with n_max an upper bound;
-// the total goes to total_dev (device) when given.
+LookBack look_back_begin(Prims& P, int64_t words, cudaStream_t s) {
+  const uint32_t ep = lb_begin(P, words * LB_TILE, s);
+  return LookBack{P.lb_st.p, P.lb_ctl.p + ep, ep, P.lb_ctl.p + 256};
+}
+
+// n items; the total goes to total_dev (device) when given.
 template <class In>
-static void scan_launch(In in, int64_t* out, int64_t n, const int64_t* n_dev, int64_t n_max, int64_t* total_dev,
-                        Prims& P, cudaStream_t s) {
-  if (n_max <= SC_TILE) {
-    k_scan_one<In><<<1, SC_THREADS, 0, s>>>(in, out, n, n_dev, total_dev);
+static void scan_launch(In in, int64_t* out, int64_t n, int64_t* total_dev, Prims& P, cudaStream_t s) {
+  if (n <= SC_TILE) {
+    k_scan_one<In><<<1, SC_THREADS, 0, s>>>(in, out, n, total_dev);
     CKL("k_scan_one");
   } else {
-    const uint32_t ep = lb_begin(P, n_max, s);
-    const int64_t tiles = (n_max + LB_TILE - 1) / LB_TILE;
-    k_scan_lb<In><<<(unsigned)tiles, SC_THREADS, 0, s>>>(in, out, n, n_dev, P.lb_st.p, P.lb_ctl.p + ep, ep,
-                                                         total_dev, P.lb_ctl.p + 256);
+    const uint32_t ep = lb_begin(P, n, s);
+    const int64_t tiles = (n + LB_TILE - 1) / LB_TILE;
+    k_scan_lb<In><<<(unsigned)tiles, SC_THREADS, 0, s>>>(in, out, n, P.lb_st.p, P.lb_ctl.p + ep, ep, total_dev,
+                                                         P.lb_ctl.p + 256);
     CKL("k_scan_lb");
   }
 }
@@ -626,7 +818,7 @@ template <class T>
 static int64_t scan_t(const T* in, int64_t* out, int64_t n, Prims& P, cudaStream_t s, bool want_total) {
   if (n <= 0) return 0;
   P.bsum.reserve(2, s);
-  scan_launch(ArrayIn<T>{in}, out, n, nullptr, n, P.bsum.p + 1, P, s);
+  scan_launch(ArrayIn<T>{in}, out, n, P.bsum.p + 1, P, s);
   if (!want_total) return -1;
   int64_t tot = 0;
   const HostRead r{P.bsum.p + 1, &tot, sizeof(int64_t)};
@@ -642,21 +834,9 @@ int64_t scan_exclusive_i32(const int32_t* in, int64_t* out, int64_t n, Prims& P,
   return scan_t<int32_t>(in, out, n, P, s, want_total);
 }
 
-void scan_exclusive_to(const int64_t* in, int64_t* out, int64_t n, const int64_t* n_dev, int64_t n_max,
-                       int64_t* total_dev, Prims& P, cudaStream_t s) {
-  if (n_max <= 0) return;
-  scan_launch(ArrayIn<int64_t>{in}, out, n, n_dev, n_max, total_dev, P, s);
-}
-
-void scan_exclusive_i32_to(const int32_t* in, int64_t* out, int64_t n, const int64_t* n_dev, int64_t n_max,
-                           int64_t* total_dev, Prims& P, cudaStream_t s) {
-  if (n_max <= 0) return;
-  scan_launch(ArrayIn<int32_t>{in}, out, n, n_dev, n_max, total_dev, P, s);
-}
-
 void scan_chunk_counts(const int32_t* list, const int32_t* nlist, int64_t n_hint, const int32_t* la,
                        const int32_t* lb, int32_t chunk, int64_t* out, Prims& P, cudaStream_t s) {
-  scan_launch(ChunkCountIn{list, nlist, n_hint, la, lb, chunk}, out, n_hint + 1, nullptr, n_hint + 1, nullptr, P, s);
+  scan_launch(ChunkCountIn{list, nlist, n_hint, la, lb, chunk}, out, n_hint + 1, nullptr, P, s);
 }
 
 int32_t* scan_error_flag(Prims& P) { return P.lb_ctl.cap ? P.lb_ctl.p + 256 : nullptr; }
@@ -675,8 +855,8 @@ bool scan_wait_gives_up(cudaStream_t s) {
     const uint32_t ep = lb_begin(P, n, s);
     const int32_t one = 1;
     CK(cudaMemcpyAsync(P.lb_ctl.p + ep, &one, sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    k_scan_lb<ArrayIn<int64_t>><<<1, SC_THREADS, 0, s>>>(ArrayIn<int64_t>{in}, out, n, nullptr, P.lb_st.p, P.lb_ctl.p + ep, ep, out + n,
-                                                P.lb_ctl.p + 256);
+    k_scan_lb<ArrayIn<int64_t>><<<1, SC_THREADS, 0, s>>>(ArrayIn<int64_t>{in}, out, n, P.lb_st.p, P.lb_ctl.p + ep, ep,
+                                                          out + n, P.lb_ctl.p + 256);
     CKL("k_scan_lb");
     CK(cudaMemcpyAsync(&bad, P.lb_ctl.p + 256, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
@@ -692,14 +872,11 @@ bool scan_wait_gives_up(cudaStream_t s) {
   return bad != 0;
 }
 
-void radix_sort_pairs(u64*& keys, u64*& vals, u64*& tk, u64*& tv, int64_t n, int bits, Prims& P, cudaStream_t s,
-                      int lo_bit) {
-  if (n <= 1 || bits <= lo_bit) return;
-  if (n <= RS_TILE) {
-    k_rs_small<<<1, RS_THREADS, 0, s>>>(keys, vals, (int)n, lo_bit, bits);
-    CKL("k_rs_small");
-    return;
-  }
+// Launches the sort of n pairs (an upper bound with x.n_dev).  A plain sort's
+// result is in (keys, vals) afterwards, which may have been swapped with (tk,
+// tv); a transposing one's lies behind its input.
+static void sort_launch(u64*& keys, u64*& vals, u64*& tk, u64*& tv, int64_t n, int bits, Prims& P, cudaStream_t s,
+                        int lo_bit, const RsExt& x) {
   if (n <= CS_MAX) {  // one cluster, the pairs kept on chip
     const int smem = 2 * CS_TILE * (int)sizeof(u64);
     static thread_local int cs_attr_dev = -1;
@@ -709,7 +886,7 @@ void radix_sort_pairs(u64*& keys, u64*& vals, u64*& tk, u64*& tv, int64_t n, int
       CK(cudaFuncSetAttribute(k_rs_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
       cs_attr_dev = dev;
     }
-    k_rs_cluster<<<CS_CL, CS_THREADS, smem, s>>>(keys, vals, (int)n, lo_bit, bits);
+    k_rs_cluster<<<CS_CL, CS_THREADS, smem, s>>>(keys, vals, (int)n, lo_bit, bits, x);
     CKL("k_rs_cluster");
     return;
   }
@@ -722,51 +899,108 @@ void radix_sort_pairs(u64*& keys, u64*& vals, u64*& tk, u64*& tv, int64_t n, int
   const int64_t coop_max = (int64_t)coop_per_sm * device_sms();
   if (nb <= coop_max && nb <= 1024) {
     const int grid = (int)std::max<int64_t>(nb, std::min<int64_t>(256, coop_max));
-    int64_t n_ = n, nb_ = nb;
+    int64_t n_ = n;
     int lo_ = lo_bit, bits_ = bits;
     int64_t *gh = P.hist.p, *dt = P.bsum.p;
-    void* args[] = {&keys, &vals, &tk, &tv, &n_, &lo_, &bits_, &nb_, &gh, &dt};
+    RsExt x_ = x;
+    void* args[] = {&keys, &vals, &tk, &tv, &n_, &lo_, &bits_, &gh, &dt, &x_};
     CK(cudaLaunchCooperativeKernel((const void*)k_rs_coop, dim3(grid), dim3(RS_THREADS), args, 0, s));
     CKL("k_rs_coop");
-    for (int shift = lo_bit; shift < bits; shift += 8) {  // where the result ended up
-      u64* t = keys; keys = tk; tk = t;
-      t = vals; vals = tv; tv = t;
-    }
+    if (!x.tbits)
+      for (int shift = lo_bit; shift < bits; shift += 8) {  // where the result ended up
+        u64* t = keys; keys = tk; tk = t;
+        t = vals; vals = tv; tv = t;
+      }
     return;
   }
+  // three launches per pass; (place, behind its n pairs?) as in k_rs_coop
+  struct Place {
+    u64 *k, *v;
+    int off;
+  };
+  Place in{keys, vals, 0}, out{tk, tv, 0}, nxt{keys, vals, 0};
+  if (x.tbits) {
+    nxt.off = 1;
+    if (((bits - lo_bit + 7) / 8) & 1) std::swap(out, nxt);
+  }
   for (int shift = lo_bit; shift < bits; shift += 8) {
-    k_rs_hist<<<(unsigned)nb, RS_THREADS, 0, s>>>(keys, n, shift, nb, P.hist.p);
+    const int first = shift == lo_bit;
+    k_rs_hist<<<(unsigned)nb, RS_THREADS, 0, s>>>(in.k, n, shift, nb, P.hist.p, x, first, in.off);
     CKL("k_rs_hist");
     k_rs_dscan<<<256, SC_THREADS, 0, s>>>(P.hist.p, nb, P.bsum.p);
     CKL("k_rs_dscan");
-    k_rs_scatter<<<(unsigned)nb, RS_THREADS, 0, s>>>(keys, vals, tk, tv, n, shift, nb, P.hist.p, P.bsum.p);
+    k_rs_scatter<<<(unsigned)nb, RS_THREADS, 0, s>>>(in.k, in.v, out.k, out.v, n, shift, nb, P.hist.p, P.bsum.p, x,
+                                                     first, in.off, out.off);
     CKL("k_rs_scatter");
-    u64* t = keys; keys = tk; tk = t;
-    t = vals; vals = tv; tv = t;
+    in = out;
+    std::swap(out, nxt);
+    if (!x.tbits) {
+      u64* t = keys; keys = tk; tk = t;
+      t = vals; vals = tv; tv = t;
+    }
   }
 }
 
-void heads_launch(const u64* keys, int64_t n, int32_t* flag, cudaStream_t s) {
-  if (n <= 0) return;
-  k_heads<<<grid_for(n, 256), 256, 0, s>>>(keys, n, flag);
-  CKL("k_heads");
+void radix_sort_pairs(u64*& keys, u64*& vals, u64*& tk, u64*& tv, int64_t n, int bits, Prims& P, cudaStream_t s,
+                      int lo_bit, const int32_t* n_dev) {
+  if (n <= 1 || bits <= lo_bit) return;
+  if (n <= RS_TILE) {
+    k_rs_small<<<1, RS_THREADS, 0, s>>>(keys, vals, (int)n, n_dev, lo_bit, bits);
+    CKL("k_rs_small");
+    return;
+  }
+  sort_launch(keys, vals, tk, tv, n, bits, P, s, lo_bit, RsExt{n_dev, 0, 0, nullptr});
+}
+
+void sort_reduce(DBuf<u64>& k, DBuf<u64>& v, DBuf<u64>& tk, DBuf<u64>& tv, int64_t n, const int32_t* n_dev, int bits,
+                 bool both, int64_t row_off, u64* okeys, int64_t* ovals, int32_t* nr, Prims& P, cudaStream_t s) {
+  if (n <= RS_TILE) {
+    // one block sorts, sums and transposes: 7.6 us for a few records and 11.4
+    // for some hundred, where the launches of the larger sizes take 16.4 and
+    // 23.5 and the gaps between them
+    k_rs_small_reduce<<<1, RS_THREADS, 0, s>>>(k.p, v.p, (int)n, n_dev, bits, both ? 1 : 0, row_off, okeys, ovals, nr);
+    CKL("k_rs_small_reduce");
+    return;
+  }
+  tk.reserve(n, s);
+  tv.reserve(n, s);
+  P.usum.reserve(n + 1, s);
+  u64 *kp = k.p, *vp = v.p, *tkp = tk.p, *tvp = tv.p;
+  // a segment crossing a run boundary is summed atomically into a slot the sort zeroes
+  sort_launch(kp, vp, tkp, tvp, n, 2 * bits, P, s, 0, RsExt{n_dev, 0, 0, P.usum.p});
+  if (kp != k.p) {
+    swap_buf(k, tk);
+    swap_buf(v, tv);
+  }
+  k_segsum<<<grid_for((n + RBK_RUN - 1) / RBK_RUN, 256), 256, 0, s>>>(k.p, v.p, n, n_dev, P.usum.p);
+  CKL("k_segsum");
+  const int tiles = div_up(n, LB_TILE);
+  const LookBack q = look_back_begin(P, tiles, s);
+  k_reduce_out<<<tiles, SC_THREADS, 0, s>>>(k.p, P.usum.p, n, n_dev, okeys, ovals, nr, nullptr, q);
+  CKL("k_reduce_out");
+  if (both) {
+    // in (row, col) order already: a stable sort on the new row alone
+    u64 *ok = okeys, *ov = (u64*)ovals, *t1 = tk.p, *t2 = tv.p;
+    sort_launch(ok, ov, t1, t2, n, 2 * bits + 1, P, s, bits, RsExt{nr, bits, row_off, nullptr});
+  }
 }
 
 int64_t reduce_by_key(const u64* keys, const u64* vals, int64_t n, u64* okeys, int64_t* ovals, Prims& P,
                       cudaStream_t s) {
   if (n <= 0) return 0;
-  P.flag.reserve(n + 1, s);
-  P.pos.reserve(n + 1, s);
   P.usum.reserve(n + 1, s);
   // a segment crossing a run boundary is summed atomically into a zeroed slot
   CK(cudaMemsetAsync(P.usum.p, 0, sizeof(int64_t) * (size_t)n, s));
-  k_segsum<<<grid_for((n + RBK_RUN - 1) / RBK_RUN, 256), 256, 0, s>>>(keys, vals, n, P.usum.p);
+  k_segsum<<<grid_for((n + RBK_RUN - 1) / RBK_RUN, 256), 256, 0, s>>>(keys, vals, n, nullptr, P.usum.p);
   CKL("k_segsum");
-  const int g = grid_for(n, 256);
-  k_nonzero_heads<<<g, 256, 0, s>>>(keys, P.usum.p, n, P.flag.p);
-  CKL("k_nonzero_heads");
-  const int64_t nz = scan_exclusive_i32(P.flag.p, P.pos.p, n, P, s, true);
-  k_compact_pairs<<<g, 256, 0, s>>>(keys, P.usum.p, n, P.flag.p, P.pos.p, okeys, ovals);
-  CKL("k_compact_pairs");
+  const int tiles = div_up(n, LB_TILE);
+  const LookBack q = look_back_begin(P, tiles, s);
+  P.bsum.reserve(2, s);
+  k_reduce_out<<<tiles, SC_THREADS, 0, s>>>(keys, P.usum.p, n, nullptr, okeys, ovals, nullptr, P.bsum.p, q);
+  CKL("k_reduce_out");
+  int64_t nz = 0;
+  const HostRead r{P.bsum.p, &nz, sizeof(int64_t)};
+  P.read(&r, 1, s);
   return nz;
 }
+

@@ -1,0 +1,110 @@
+// Device-side building blocks of single-pass scans: block scans of small
+// packed counts and the decoupled look-back over tiles for several sums at
+// once, and the write of a kernel's result into the host's mapped page.
+#pragma once
+#include "common.cuh"
+
+// Exclusive scan of one value per thread over a block of NT threads; several
+// counts may be packed into the word as long as none overflows its field.
+template <int NT>
+__device__ inline u64 block_scan(u64 v, u64* total) {
+  __shared__ u64 wsum[NT / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  u64 x = v;
+  for (int d = 1; d < 32; d <<= 1) {
+    const u64 y = __shfl_up_sync(0xffffffffu, x, d);
+    if (lane >= d) x += y;
+  }
+  if (lane == 31) wsum[wid] = x;
+  __syncthreads();
+  if (wid == 0) {
+    u64 s = lane < NT / 32 ? wsum[lane] : 0;
+    for (int d = 1; d < 32; d <<= 1) {
+      const u64 y = __shfl_up_sync(0xffffffffu, s, d);
+      if (lane >= d) s += y;
+    }
+    if (lane < NT / 32) wsum[lane] = s;
+  }
+  __syncthreads();
+  const u64 before = wid ? wsum[wid - 1] : 0;
+  *total = wsum[NT / 32 - 1];
+  __syncthreads();
+  return before + x - v;
+}
+
+// Decoupled look-back over tiles for NC sums at once (see k_scan_lb for the
+// scheme and why the waits end): tile t's words are st[t * NC ..], each
+// (value << 10 | epoch << 2 | status) with status 1 = the tile's own sum and
+// 2 = the inclusive prefix; a tile whose words differ in status is being
+// rewritten and read again.  Run by warp 0 with the tile's sums in every lane;
+// returns the exclusive prefixes in every lane.  Past LB_SPINS polls it sets
+// *err and carries on.
+constexpr uint32_t LB_SPINS = 1u << 20;
+
+template <int NC>
+__device__ inline void look_back(u64* st, int64_t tile, const int64_t (&agg)[NC], int64_t (&pre)[NC], uint32_t ep,
+                                 int32_t* err) {
+  const int lane = threadIdx.x & 31;
+  const u64 tag = (u64)(ep & 255u) << 2;
+#pragma unroll
+  for (int k = 0; k < NC; ++k) pre[k] = 0;
+  if (tile > 0) {
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+      if (lane == k) atomicExch((unsigned long long*)&st[tile * NC + k], ((u64)agg[k] << 10) | tag | 1u);
+    uint32_t spins = 0;
+    for (int64_t j0 = tile - 1;;) {
+      const int64_t j = j0 - lane;
+      u64 x[NC];
+      u64 all = 3, any = 0;
+      bool fresh = true;
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        x[k] = j >= 0 ? *(volatile const u64*)&st[j * NC + k] : 0;
+        fresh = fresh && ((x[k] >> 2) & 255u) == (ep & 255u);
+        all &= x[k];
+        any |= x[k] & 3u;
+      }
+      const bool ready = j < 0 || (fresh && all != 0 && any == all);
+      const unsigned rmask = __ballot_sync(0xffffffffu, ready);
+      const unsigned pmask = __ballot_sync(0xffffffffu, j >= 0 && ready && any == 2u);
+      const int nr = rmask == 0xffffffffu ? 32 : __ffs(~rmask) - 1;  // nearest tile not ready
+      const int fp = pmask ? __ffs(pmask) - 1 : 32;                  // nearest inclusive prefix
+      if (fp < nr || nr == 32) {
+        const int upto = fp < 32 ? fp : 31;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+          int64_t v = j >= 0 && lane <= upto ? (int64_t)(x[k] >> 10) : 0;
+          for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+          pre[k] += v;
+        }
+        if (fp < 32 || j0 < 32) break;  // a prefix, or every tile before this one, was summed
+        j0 -= 32;
+        continue;
+      }
+      if (++spins > LB_SPINS) {
+        if (lane == 0) atomicExch(err, 1);
+        break;
+      }
+      __nanosleep(32);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < NC; ++k)
+    if (lane == k) atomicExch((unsigned long long*)&st[tile * NC + k], ((u64)(pre[k] + agg[k]) << 10) | tag | 2u);
+}
+
+// A kernel's result for the host: 64-bit words into the mapped page, then the
+// read's sequence number (written by one thread).
+struct Pub {
+  int64_t* page;  // word 0: sequence number, then the payload
+  int64_t seq;
+};
+
+template <int N>
+__device__ inline void publish(const Pub& p, const int64_t (&v)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) p.page[1 + i] = v[i];
+  __threadfence_system();  // the payload is visible to the host before the sequence number
+  *(volatile int64_t*)p.page = p.seq;
+}

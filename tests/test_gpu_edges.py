@@ -86,3 +86,51 @@ def test_sweep_bins(ldl, directed, weight):
         d.apply(b)
         msgs = compare_states(o, d, f"batch {t}")
         assert not msgs, "\n".join(msgs[:8])
+
+
+def _dense_batch(g, size, seed):
+    """`size` updates of distinct arcs (edges) of a graph on few vertices: half
+    inserts anywhere, a few deletes and reweights of arcs that exist."""
+    rng = np.random.default_rng(seed)
+    src, col, _ = g.arcs()
+    keep = (src < col) if not g.directed else (src != col)
+    have = src[keep] * g.n + col[keep]
+    old = rng.permutation(have)[: min(size // 4, len(have))]
+    new = np.unique(rng.integers(0, g.n, 3 * size) * g.n + rng.integers(0, g.n, 3 * size))
+    if not g.directed:
+        new = new[new // g.n < new % g.n]
+    new = rng.permutation(np.setdiff1d(new[new // g.n != new % g.n], old))[: size - len(old)]
+    key = np.concatenate([new, old])
+    op = np.zeros(len(key), np.int64)
+    op[len(new):] = 1 + np.arange(len(old)) % 2
+    w = np.where(op == 1, 0, rng.integers(1, 5, len(key)))
+    return rng.permutation(np.stack([key // g.n, key % g.n, op, w], 1)).astype(np.int32)
+
+
+# update counts at and beside the tiles and size classes of the batch's sorts,
+# scans and adjacency updates (512, 1024, 2048, 49152 pairs, then one launch
+# per sorting phase from 1.2M)
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("size", [1, 2, 256, 511, 512, 513, 1023, 1024, 1025, 2047, 2048, 2049, 24576, 24577, 49152,
+                                  49153, 1_300_000])
+def test_batch_sizes(ldl, directed, size):
+    n = 3000 if size > 100_000 else 1500
+    rng = np.random.default_rng(size)
+    v = np.arange(n)
+    src = np.repeat(v, 6)
+    dst = np.where(rng.random(6 * n) < 0.8, src // 30 * 30 + rng.integers(0, 30, 6 * n), rng.integers(0, n, 6 * n))
+    dst = np.minimum(dst, n - 1)
+    keep = src != dst if directed else src < dst
+    key = np.unique(src[keep] * n + dst[keep])
+    g = csr_from_arcs(n, key // n, key % n, rng.integers(1, 5, len(key)), directed)
+    o, d = Oracle(g), ldl.LDL.from_graph(g)
+    b = _dense_batch(g, size, size + 1)
+    assert len(b) == size
+    undo = b.copy()[: size // 2]
+    undo = undo[undo[:, 2] == 0]  # the second batch deletes some of what the first brought
+    undo[:, 2:] = (1, 0)
+    for t, x in enumerate((b, undo) if len(undo) else (b,)):
+        assert o.apply(x) == 0
+        d.apply(x)
+        msgs = compare_states(o, d, f"batch {t}")
+        assert not msgs, "\n".join(msgs[:8])
