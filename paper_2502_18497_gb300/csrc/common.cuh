@@ -315,13 +315,10 @@ constexpr int KS_EVENTS = 10;
 __host__ __device__ constexpr int ks_interval_group(int j) { return j < 5 ? j : j == 5 ? -1 : j == 7 ? 5 : 6; }
 
 struct DevScalars {
-  I128 dq;          // numerator change of the current mini-batch
-  I128 dp;          // change of sum_C K_out K_in
-  I128 p_old, p_new;
-  int64_t de;       // change of sum_C e_C
+  int64_t home[10];  // accumulators when the counter arena is used up (CommitAcc, RepairAcc, ...)
+  int64_t home2[10];
   int64_t dm;       // change of m (batch)
-  int64_t need;     // pool slots needed by relocation
-  int64_t need2;    // second accumulator (record counts)
+  int64_t sums[2];  // home of ldl_ctx::sums
   int64_t scanned;  // adjacency entries scanned
   int64_t err_key;  // packed (index << 8 | status) of the first update invalid by itself
   int64_t err_seq;  // the same for an update that its predecessors make invalid

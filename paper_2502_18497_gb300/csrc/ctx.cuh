@@ -28,7 +28,7 @@ struct LevelState {
   DBuf<int32_t> stK, lK;         // endpoints of arcs deleted since the level was last refined
   int32_t brk_ep = 0;            // epoch of stK
   // weight records of this level not yet applied to its adjacency (levels >= 1
-  // of a batch update: unsorted, unreduced; count in dcnt[K_PEND0 + r])
+  // of a batch update: unsorted, unreduced; count in cp[K_PEND0 + r])
   DBuf<u64> pk, pv;
   int64_t pend_ub = 0;           // host bound on the pending count
   bool allocated = false;
@@ -41,7 +41,7 @@ struct LevelState {
   }
 };
 
-// Device counters (indices into ldl_ctx::dcnt).
+// Device counters (indices into ldl_ctx::cp).
 enum {
   K_U = 0, K_S, K_USTAR, K_MV, K_M0, K_D, K_C, K_R, K_R2, K_X, K_T, K_CH, K_CAND, K_B,
   K_UNDEC, K_SMALL, K_MID, K_LARGE, K_REC, K_CREC, K_ERR, K_TMP, K_TMP2, K_CHG, K_MID2, K_TINY, K_CLU,
@@ -53,7 +53,21 @@ enum {
   K_FL,        // summed records of a flush
   K_BRK0 = 48, // K_BRK0 + r: endpoints of deleted level-r arcs
   K_PEND0 = 56, // K_PEND0 + r: pending weight records of level r
+  K_TICKET = 47,  // blocks through (pub_tail)
   K_COUNT = 64
+};
+constexpr int ARENA_WORDS = 8192;
+
+// Exact changes of a mini-batch: the Eq. 1 numerator, sum_C K_out K_in, sum_C e_C.
+struct CommitAcc {
+  I128 dq, dp;
+  int64_t de;
+};
+// The batch's statistic repair: sum over the touched communities of K_out K_in
+// before and after, and the change of sum_C e_C.
+struct RepairAcc {
+  I128 p_old, p_new;
+  int64_t de;
 };
 
 struct ldl_ctx {
@@ -73,7 +87,19 @@ struct ldl_ctx {
   i128 Psum = 0;               // sum_C K_out K_in
 
   DevScalars* d_sc = nullptr;
+  // Device counters.  cp[k] is where counter k lives now: clearing a counter
+  // takes the next word of an arena that one launch clears at the start of a
+  // batch (a memset per counter cost 4.5 us each, 75 times a batch on the
+  // R-MAT of 2^20), or, with the arena used up, its home word in dcnt.
   int32_t* dcnt = nullptr;
+  int32_t* cp[64] = {nullptr};
+  int32_t* arena = nullptr;
+  int32_t arena_top = 0;
+  CommitAcc* acc = nullptr;    // of the last mini-batch
+  RepairAcc* racc = nullptr;   // of the batch's statistic repair
+  int64_t* sums = nullptr;     // two accumulators of the last sweep or aggregate step
+  // whether the last sweep of (level, mode) had hub rows (scheduling only)
+  uint8_t hubs_seen[8][2] = {{0}};
   int32_t epoch = 0;
 
   // dedup stamps (one int32 per node id) and lists
@@ -104,7 +130,7 @@ struct ldl_ctx {
   DBuf<u64> flk;      // a pending list's summed records (keys) ...
   DBuf<int64_t> flv;  // ... and their weight changes
   DBuf<int64_t> chunk_pre;
-  DBuf<int64_t> hub_ecnt, hub_epre, pb_hi;
+  DBuf<int64_t> hub_epre, pb_hi;
   DBuf<uint64_t> pb_lo;
   DBuf<int32_t> pb_c;
   DBuf<ldl_update> upd;
@@ -175,7 +201,6 @@ inline Adj<int64_t> adj_in(ldl_ctx& c, int r) {
 inline int64_t* kin_of(ldl_ctx& c, int r) { return c.directed ? c.lv[r].kin.p : c.lv[r].kout.p; }
 inline int64_t* Kin_of(ldl_ctx& c) { return c.directed ? c.Kin.p : c.Kout.p; }
 
-// host reads of device counters (synchronise)
 // Copies device values to the host once the context's stream has reached
 // this point: a one-block kernel writes them into the pinned page and then the
 // sequence number, which the host polls (a stream error ends the wait).
@@ -187,16 +212,12 @@ Pub pub_begin(ldl_ctx& c);
 void pub_wait(ldl_ctx& c, int64_t* out, int n);
 int32_t rd_cnt(ldl_ctx& c, int idx);
 void zero_cnt(ldl_ctx& c, int idx);
-// One launch that clears several counters (bit i of mask: dcnt[i]) and up to
-// ZERO_SPANS spans of 64-bit device words (p[i], nw[i] <= K_COUNT words).
-constexpr int ZERO_SPANS = 3;
-struct ZeroSpans {
-  uint64_t mask = 0;
-  int64_t* p[ZERO_SPANS] = {nullptr, nullptr, nullptr};
-  int32_t nw[ZERO_SPANS] = {0, 0, 0};
-};
-inline uint64_t cnt_bit(int idx) { return 1ull << idx; }
-void zero_many(ldl_ctx& c, const ZeroSpans& z);
+// `words` zeroed words, 16-byte aligned: from the arena, else `home` cleared.
+void* fresh(ldl_ctx& c, int words, void* home);
+// A read that a kernel's last block performs (scan.cuh): begin before the
+// launch, wait after it, with the same list.
+Tail tail_begin(ldl_ctx& c, const HostRead* r, int n);
+void tail_wait(ldl_ctx& c, const HostRead* r, int n);
 void set_cnt(ldl_ctx& c, int idx, int32_t v);
 
 // stage timing

@@ -19,9 +19,10 @@ __device__ inline void set_err(unsigned long long* err, int64_t idx, int code) {
 }
 
 // Start of a batch: every counter, and the scalars that ingest adds to.
-__global__ void k_batch_begin(int32_t* dcnt, DevScalars* sc) {
+__global__ void k_batch_begin(int32_t* dcnt, int32_t* arena, DevScalars* sc) {
   const int t = threadIdx.x;
   if (t < K_COUNT) dcnt[t] = 0;
+  for (int i = t; i < ARENA_WORDS / 4; i += blockDim.x) ((int4*)arena)[i] = make_int4(0, 0, 0, 0);
   if (t == 0) {
     sc->scanned = 0;
     sc->dm = 0;
@@ -144,13 +145,19 @@ __global__ void k_transpose(const u64* k, const u64* v, int64_t n, int bits, u64
 }
 
 // ---------------------------------------------------------------- repair
+// The communities that the changed arcs touch, and the sum of their K_out *
+// K_in as it is (the totals change in k_stat_arcs).
 __global__ void k_dirty(const u64* keys, int64_t na, int bits, const int32_t* lab, int32_t* stT, int32_t epT,
-                        int32_t* lT, int32_t* nT) {
+                        int32_t* lT, int32_t* nT, const int64_t* Kout, const int64_t* Kin, I128* acc) {
   const u64 mask = (((u64)1) << bits) - 1;
+  i128 s = 0;
   GRID_STRIDE(i, na) {
-    stamp_add(stT, epT, lab[keys[i] >> bits], lT, nT);
-    stamp_add(stT, epT, lab[keys[i] & mask], lT, nT);
+    const int32_t a = lab[keys[i] >> bits], b = lab[keys[i] & mask];
+    if (stamp_add(stT, epT, a, lT, nT)) s += (i128)Kout[a] * Kin[a];
+    if (stamp_add(stT, epT, b, lT, nT)) s += (i128)Kout[b] * Kin[b];
   }
+  s = warp_sum_i128(s);
+  if ((threadIdx.x & 31) == 0) atomic_add_i128(acc, s);
 }
 
 // sum over listed communities of K_out * K_in into an int128 accumulator
@@ -199,6 +206,8 @@ struct Chain {
   int32_t* stA[8];        // frontier A^q: stamp, epoch, list
   int32_t epA[8];
   int32_t* lA[8];
+  int32_t* nA[8];         // its length
+  int32_t* np[8];         // pending records of level q
 };
 
 // Weight records (keys, vals) of level q0 carried up the hierarchy: with
@@ -226,7 +235,7 @@ __device__ inline void warp_append_rec(bool want, u64 key, int64_t v, u64* pk, u
 }
 
 __global__ void k_chain_records(const u64* keys, const int64_t* vals, int64_t n, const int32_t* n_dev, int bits, int q0, int top, int self,
-                                int add_k, int directed, Chain ch, int32_t* pcnt) {
+                                int add_k, int directed, Chain ch) {
   if (n_dev) n = min(n, (int64_t)*n_dev);
   const u64 mask = (((u64)1) << bits) - 1;
   const int lane = threadIdx.x & 31;
@@ -242,7 +251,7 @@ __global__ void k_chain_records(const u64* keys, const int64_t* vals, int64_t n,
       d = vals[t];
     }
     int32_t x = (int32_t)(key >> bits), y = (int32_t)(key & mask);
-    if (self) warp_append_rec(on, key, d, ch.pk[q0], ch.pv[q0], &pcnt[q0]);
+    if (self) warp_append_rec(on, key, d, ch.pk[q0], ch.pv[q0], ch.np[q0]);
     for (int q = q0; q < top; ++q) {
       if (on) {
         x = ch.par[q][x];
@@ -254,7 +263,7 @@ __global__ void k_chain_records(const u64* keys, const int64_t* vals, int64_t n,
         atomic_add_i64(&ch.kout[q + 1][x], d);
         if (directed) atomic_add_i64(&ch.kin[q + 1][y], d);
       }
-      warp_append_rec(on, ((u64)x << bits) | (u64)(uint32_t)y, d, ch.pk[q + 1], ch.pv[q + 1], &pcnt[q + 1]);
+      warp_append_rec(on, ((u64)x << bits) | (u64)(uint32_t)y, d, ch.pk[q + 1], ch.pv[q + 1], ch.np[q + 1]);
     }
   }
 }
@@ -262,13 +271,13 @@ __global__ void k_chain_records(const u64* keys, const int64_t* vals, int64_t n,
 // InitFrontier above level 0: A^{q+1} = pi_q(A^q) for every q < top, by
 // walking each node of A^0 up its parent chain.  A walk stops at a node that
 // is already marked: the walk that marked it goes on above it.
-__global__ void k_chain_frontier(const int32_t* l0, const int32_t* n0, int top, Chain ch, int32_t* nA) {
+__global__ void k_chain_frontier(const int32_t* l0, const int32_t* n0, int top, Chain ch) {
   const int32_t m = *n0;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
     int32_t x = l0[k];
     for (int q = 0; q < top; ++q) {
       x = ch.par[q][x];
-      if (x < 0 || !stamp_add(ch.stA[q + 1], ch.epA[q + 1], x, ch.lA[q + 1], &nA[q + 1])) break;
+      if (x < 0 || !stamp_add(ch.stA[q + 1], ch.epA[q + 1], x, ch.lA[q + 1], ch.nA[q + 1])) break;
     }
   }
 }
@@ -277,13 +286,14 @@ __global__ void k_chain_frontier(const int32_t* l0, const int32_t* n0, int top, 
 // Children of each listed level-(q+1) node take its label at level q.
 __global__ void k_push(ChunkMap m, const int32_t* lab_up, Adj<int32_t> ch_adj, const int32_t* par, int32_t* lab,
                        int32_t* olist, int32_t* nout, int32_t* stCh, int32_t epCh, int32_t* lCh, int32_t* nCh,
-                       int32_t* lab_before) {
+                       int32_t* lab_before, Tail tail) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = m.pre[m.n_hint];
+  __shared__ ChunkPre sh;
+  const int64_t total = chunk_begin(m, sh);
   for (int64_t c = warp; c < total; c += nw) {
-    const Chunk ch = chunk_of(m, c);
+    const Chunk ch = chunk_of(m, sh, c);
     if (ch.row < 0) continue;
     const int32_t L = lab_up[ch.v];
     const int64_t o = ch_adj.off[ch.v];
@@ -303,6 +313,7 @@ __global__ void k_push(ChunkMap m, const int32_t* lab_up, Adj<int32_t> ch_adj, c
       if (olist) warp_append(valid, u, olist, nout);
     }
   }
+  pub_tail(tail);
 }
 
 // ---------------------------------------------------------------- dissolve
@@ -365,7 +376,7 @@ __global__ void k_leave(const int32_t* lU, const int32_t* nU, const uint8_t* ali
                         const int32_t* labN, int32_t* par, int32_t* par_old, const int64_t* kout, const int64_t* kin,
                         int64_t* kout1, int64_t* kin1, int32_t* cnt1, int directed, int32_t* stL, int32_t epL,
                         int32_t* stD, int32_t epD, int32_t* lD, int32_t* nD, int32_t* stX, int32_t epX, int32_t* lX,
-                        int32_t* nX, int32_t* nbr) {
+                        int32_t* nX, int32_t* nbr, Tail tail) {
   const int32_t n = *nU;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t u = lU[k];
@@ -387,6 +398,7 @@ __global__ void k_leave(const int32_t* lU, const int32_t* nU, const uint8_t* ali
     atomicAdd(&cnt1[u], 1);
     stamp_add(stD, epD, u, lD, nD);
   }
+  pub_tail(tail);
 }
 
 // A refined community that lost nodes stays connected when every node that
@@ -401,9 +413,10 @@ __global__ void k_leave_degree(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = m.pre[m.n_hint];
+  __shared__ ChunkPre sh;
+  const int64_t total = chunk_begin(m, sh);
   for (int64_t c = warp; c < total; c += nw) {
-    const Chunk ch = chunk_of(m, c);
+    const Chunk ch = chunk_of(m, sh, c);
     if (ch.row < 0) continue;
     const int32_t v = ch.v;
     const int32_t X = par_old[v];
@@ -423,13 +436,14 @@ __global__ void k_leave_degree(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_
 // is in doubt (flagged, or their seed node left); each starts as its own
 // component.
 __global__ void k_members(Adj<int32_t> ch_adj, ChunkMap m, const int32_t* par, const int32_t* stL, int32_t epL,
-                          const int32_t* ckf, int32_t epF, int32_t* comp, int32_t* lG, int32_t* nG) {
+                          const int32_t* ckf, int32_t epF, int32_t* comp, int32_t* lG, int32_t* nG, Tail tail) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = m.pre[m.n_hint];
+  __shared__ ChunkPre sh;
+  const int64_t total = chunk_begin(m, sh);
   for (int64_t c = warp; c < total; c += nw) {
-    const Chunk ch = chunk_of(m, c);
+    const Chunk ch = chunk_of(m, sh, c);
     if (ch.row < 0) continue;
     const int32_t X = ch.v;
     if (ckf[X] != epF && stL[X] != epL) continue;
@@ -446,6 +460,7 @@ __global__ void k_members(Adj<int32_t> ch_adj, ChunkMap m, const int32_t* par, c
       warp_append(want, u, lG, nG);
     }
   }
+  pub_tail(tail);
 }
 
 // Root of x's tree.  Parent links only point to smaller ids of the same
@@ -525,9 +540,10 @@ __global__ void k_uf(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* par, co
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = m.pre[m.n_hint];
+  __shared__ ChunkPre sh;
+  const int64_t total = chunk_begin(m, sh);
   for (int64_t c = warp; c < total; c += nw) {
-    const Chunk ch = chunk_of(m, c);
+    const Chunk ch = chunk_of(m, sh, c);
     if (ch.row < 0) continue;
     const int32_t u = ch.v;
     const int32_t X = par[u];
@@ -565,7 +581,7 @@ __global__ void k_uf_final(const int32_t* lG, const int32_t* nG, int32_t* comp) 
 __global__ void k_rename(const int32_t* lG, const int32_t* nG, const int32_t* comp, const uint8_t* alive,
                          const int32_t* stL, int32_t epL, int32_t* par, int32_t* par_old, const int64_t* kout,
                          const int64_t* kin, int64_t* kout1, int64_t* kin1, int32_t* cnt1, int directed,
-                         int32_t* stD, int32_t epD, int32_t* lD, int32_t* nD) {
+                         int32_t* stD, int32_t epD, int32_t* lD, int32_t* nD, Tail tail) {
   const int32_t n = *nG;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t u = lG[k];
@@ -583,6 +599,7 @@ __global__ void k_rename(const int32_t* lG, const int32_t* nG, const int32_t* co
     atomicAdd(&cnt1[root], 1);
     stamp_add(stD, epD, u, lD, nD);
   }
+  pub_tail(tail);
 }
 
 // the listed nodes that are singleton refined communities
@@ -606,7 +623,7 @@ __global__ void k_singletons(const int32_t* l, const int32_t* n, const int32_t* 
 // The nodes of D whose parent changed, and the entries of their rows.
 __global__ void k_changed(const int32_t* lD, const int32_t* nD, const int32_t* par, const int32_t* par_old,
                           int32_t* stC, int32_t epC, int32_t* lC, int32_t* nC, const int32_t* len_out,
-                          const int32_t* len_in, int64_t* acc_out, int64_t* acc_in) {
+                          const int32_t* len_in, int64_t* acc_out, int64_t* acc_in, Tail tail) {
   const int32_t n = *nD;
   int64_t so = 0, si = 0;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -620,6 +637,7 @@ __global__ void k_changed(const int32_t* lD, const int32_t* nD, const int32_t* p
   si = warp_sum_i64(si);
   if ((threadIdx.x & 31) == 0 && so) atomic_add_i64(acc_out, so);
   if ((threadIdx.x & 31) == 0 && si) atomic_add_i64(acc_in, si);
+  pub_tail(tail);
 }
 
 // Subtract-add records of Eq. 3 for every arc incident to a changed node,
@@ -632,9 +650,10 @@ __global__ void k_emit(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* par, 
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = m.pre[m.n_hint];
+  __shared__ ChunkPre sh;
+  const int64_t total = chunk_begin(m, sh);
   for (int64_t c = warp; c < total; c += nw) {
-    const Chunk ch = chunk_of(m, c);
+    const Chunk ch = chunk_of(m, sh, c);
     if (ch.row < 0) continue;
     const int32_t u = ch.v;
     const int32_t po = par_old[u], pn = par[u];
@@ -902,12 +921,13 @@ __global__ void k_esum(const int64_t* e, const int64_t* Kout, const int64_t* Kin
 }
 
 __global__ void k_changed_final(const int32_t* lCh, const int32_t* nCh, const int32_t* lab,
-                                const int32_t* lab_before, int32_t* out, int32_t* nout) {
+                                const int32_t* lab_before, int32_t* out, int32_t* nout, Tail tail) {
   const int32_t n = *nCh;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t u = lCh[k];
     if (lab[u] != lab_before[u]) out[atomicAdd(nout, 1)] = u;
   }
+  pub_tail(tail);
 }
 
 __global__ void k_gather(const int32_t* ids, int32_t k, const int32_t* lab, int32_t* out) {
@@ -949,7 +969,9 @@ static void throw_at(int64_t key, const char* what) {
 
 int64_t ingest(ldl_ctx& c, const ldl_update* upd, int64_t count, int on_device, int64_t* dm) {
   *dm = 0;
-  k_batch_begin<<<1, K_COUNT, 0, c.s>>>(c.dcnt, c.d_sc);
+  c.arena_top = 0;
+  for (int k = 0; k < K_COUNT; ++k) c.cp[k] = c.dcnt + k;
+  k_batch_begin<<<1, 1024, 0, c.s>>>(c.dcnt, c.arena, c.d_sc);
   CKL("k_batch_begin");
   if (count <= 0) return 0;
   const ldl_update* du = upd;
@@ -972,20 +994,20 @@ int64_t ingest(ldl_ctx& c, const ldl_update* upd, int64_t count, int on_device, 
   sort_pairs(c.rk, c.rv, c.tk, c.tv, count, 2 * c.bits, c.P, c.s);
   const int tiles = div_up(count, UQ_TPB);
   const LookBack q = look_back_begin(c.P, tiles, c.s);
-  k_unique<<<tiles, UQ_TPB, 0, c.s>>>(c.rk.p, count, c.rk2.p, c.rsum.p, c.dcnt + K_NU, q);
+  k_unique<<<tiles, UQ_TPB, 0, c.s>>>(c.rk.p, count, c.rk2.p, c.rsum.p, c.cp[K_NU], q);
   CKL("k_unique");
   const auto& g0 = c.lv[0].out0;
-  k_seq<<<g, TPB, 0, c.s>>>(du, count, c.rv.p, c.rsum.p, c.dcnt + K_NU, c.rk2.p, g0.off.p, g0.len.p, g0.col.p, g0.w.p,
-                            c.bits, c.directed, err_seq, &c.d_sc->dm, c.trk.p, c.trv.p, c.dcnt + K_REC);
+  k_seq<<<g, TPB, 0, c.s>>>(du, count, c.rv.p, c.rsum.p, c.cp[K_NU], c.rk2.p, g0.off.p, g0.len.p, g0.col.p, g0.w.p,
+                            c.bits, c.directed, err_seq, &c.d_sc->dm, c.trk.p, c.trv.p, c.cp[K_REC]);
   CKL("k_seq");
   // the changed arcs in order (each once, no change zero), on directed graphs
   // followed by their in-direction records
-  sort_reduce(c.trk, c.trv, c.tk, c.tv, arcs, c.dcnt + K_REC, c.bits, c.directed, c.n, c.rk.p, (int64_t*)c.rv.p,
-              c.dcnt + K_NR, c.P, c.s);
+  sort_reduce(c.trk, c.trv, c.tk, c.tv, arcs, c.cp[K_REC], c.bits, c.directed, c.n, c.rk.p, (int64_t*)c.rv.p,
+              c.cp[K_NR], c.P, c.s);
   int64_t e1 = -1, e2 = -1;
   int32_t na = 0;
   const HostRead rr[4] = {{err, &e1, sizeof(int64_t)}, {err_seq, &e2, sizeof(int64_t)},
-                          {&c.d_sc->dm, dm, sizeof(int64_t)}, {c.dcnt + K_NR, &na, sizeof(int32_t)}};
+                          {&c.d_sc->dm, dm, sizeof(int64_t)}, {c.cp[K_NR], &na, sizeof(int32_t)}};
   host_read(c, rr, 4);
   if (e1 != -1) throw_at(e1, "invalid update");
   if (e2 != -1) throw_at(e2, "invalid update sequence");
@@ -1021,7 +1043,7 @@ static int64_t apply_records(ldl_ctx& c, int r, const u64* keys, const int64_t* 
   // a deleted arc can only disconnect the refined community holding both of
   // its endpoints (refined communities are connected); until the level's next
   // split its parents change only where a node empties and leaves its parent
-  const DelTrack trk{Lr.stK.p, Lr.brk_ep, Lr.lK.p, c.dcnt + K_BRK0 + r, c.n, r < c.T ? Lr.par.p : nullptr};
+  const DelTrack trk{Lr.stK.p, Lr.brk_ep, Lr.lK.p, c.cp[K_BRK0 + r], c.n, r < c.T ? Lr.par.p : nullptr};
   const int mul = c.directed ? 2 : 1;
   const int64_t m = r == 0 ? csr_apply<int32_t>(c.lv[0].out0, keys, vals, mul * nr, n_dev, mul, c.bits, c.CS, c.P, c.s,
                                                 c.d_sc, &trk)
@@ -1042,6 +1064,8 @@ static Chain chain_of(ldl_ctx& c, const int32_t* epA) {
     ch.stA[q] = L.stA.p;
     ch.lA[q] = L.lA.p;
     ch.epA[q] = epA ? epA[q] : 0;
+    ch.nA[q] = c.cp[K_A0 + q];
+    ch.np[q] = c.cp[K_PEND0 + q];
   }
   return ch;
 }
@@ -1062,7 +1086,7 @@ static void chain_records(ldl_ctx& c, const u64* keys, const int64_t* vals, int6
     L.pend_ub += n;
   }
   k_chain_records<<<grid_for(n, TPB), TPB, 0, c.s>>>(keys, vals, n, n_dev, c.bits, q0, c.T, self ? 1 : 0, add_k ? 1 : 0,
-                                                     c.directed, chain_of(c, nullptr), c.dcnt + K_PEND0);
+                                                     c.directed, chain_of(c, nullptr));
   CKL("k_chain_records");
 }
 
@@ -1083,50 +1107,38 @@ void flush_level(ldl_ctx& c, int q, int64_t known) {
   // own output buffers: a flush may run while the caller's records sit in rk / rv
   c.flk.reserve((c.directed ? 2 : 1) * n + 1, c.s);
   c.flv.reserve((c.directed ? 2 : 1) * n + 1, c.s);
-  int32_t* nr = c.dcnt + K_FL;
+  int32_t* nr = c.cp[K_FL];
   sort_reduce(L.pk, L.pv, c.tk, c.tv, n, nullptr, c.bits, c.directed, c.n, c.flk.p, c.flv.p, nr, c.P, c.s);
   c.res.pending_records += n;
   c.res.pending_applied += apply_records(c, q, c.flk.p, c.flv.p, n, nr);
 }
 
-void repair_batch(ldl_ctx& c, int64_t na, const int32_t* epA, int32_t epT, int64_t dm) {
+void repair_done(ldl_ctx& c, const RepairAcc& a, int64_t dm) {
+  c.m += dm;
+  c.E += a.de;
+  c.Psum += i128_of(a.p_new.hi, a.p_new.lo) - i128_of(a.p_old.hi, a.p_old.lo);
+}
+
+void repair_batch(ldl_ctx& c, int64_t na, const int32_t* epA, int32_t epT) {
   if (na <= 0) return;
   // Algorithm 1, applying the batch: it changes level 0
   apply_records(c, 0, c.rk.p, (const int64_t*)c.rv.p, na, nullptr);
-  // statistic repair: m, degrees, community totals (exactly, with sum_C K_out K_in)
+  // statistic repair: degrees, community totals (exactly, with sum_C K_out K_in)
   LevelState& L0 = c.lv[0];
-  {
-    static_assert(offsetof(DevScalars, p_new) == offsetof(DevScalars, p_old) + sizeof(I128), "adjacent scalars");
-    ZeroSpans z;
-    z.mask = cnt_bit(K_T);
-    z.p[0] = (int64_t*)&c.d_sc->p_old;
-    z.nw[0] = (int32_t)(2 * sizeof(I128) / sizeof(int64_t));
-    z.p[1] = &c.d_sc->de;
-    z.nw[1] = 1;
-    zero_many(c, z);
-  }
-  k_dirty<<<grid_for(na, TPB), TPB, 0, c.s>>>(c.rk.p, na, c.bits, L0.lab.p, c.stT.p, epT, c.lT.p, c.dcnt + K_T);
+  zero_cnt(c, K_T);
+  c.racc = (RepairAcc*)fresh(c, sizeof(RepairAcc) / 4, c.d_sc->home2);
+  k_dirty<<<grid_for(na, TPB), TPB, 0, c.s>>>(c.rk.p, na, c.bits, L0.lab.p, c.stT.p, epT, c.lT.p, c.cp[K_T], c.Kout.p,
+                                              Kin_of(c), &c.racc->p_old);
   CKL("k_dirty");
-  k_psum<<<grid_for(2 * na, TPB), TPB, 0, c.s>>>(c.lT.p, c.dcnt + K_T, c.Kout.p, Kin_of(c), &c.d_sc->p_old);
-  CKL("k_psum");
   k_stat_arcs<<<grid_for(na, TPB), TPB, 0, c.s>>>(c.rk.p, (const int64_t*)c.rv.p, na, c.bits, c.directed, L0.lab.p,
-                                                  L0.kout.p, kin_of(c, 0), c.Kout.p, Kin_of(c), c.e.p, &c.d_sc->de,
-                                                  L0.stA.p, epA[0], L0.lA.p, c.dcnt + K_A0);
+                                                  L0.kout.p, kin_of(c, 0), c.Kout.p, Kin_of(c), c.e.p, &c.racc->de,
+                                                  L0.stA.p, epA[0], L0.lA.p, c.cp[K_A0]);
   CKL("k_stat_arcs");
-  k_psum<<<grid_for(2 * na, TPB), TPB, 0, c.s>>>(c.lT.p, c.dcnt + K_T, c.Kout.p, Kin_of(c), &c.d_sc->p_new);
+  k_psum<<<grid_for(2 * na, TPB), TPB, 0, c.s>>>(c.lT.p, c.cp[K_T], c.Kout.p, Kin_of(c), &c.racc->p_new);
   CKL("k_psum");
-  I128 p_old, p_new;
-  int64_t de = 0;
-  const HostRead rr[3] = {{&c.d_sc->p_old, &p_old, sizeof(I128)}, {&c.d_sc->p_new, &p_new, sizeof(I128)},
-                          {&c.d_sc->de, &de, sizeof(int64_t)}};
-  host_read(c, rr, 3);
-  c.m += dm;
-  c.E += de;
-  c.Psum += i128_of(p_new.hi, p_new.lo) - i128_of(p_old.hi, p_old.lo);
   if (c.T == 0) return;
   // InitFrontier: A^{q+1} = pi_q(A^q) along the chain
-  k_chain_frontier<<<grid_for(2 * na, TPB), TPB, 0, c.s>>>(L0.lA.p, c.dcnt + K_A0, c.T, chain_of(c, epA),
-                                                           c.dcnt + K_A0);
+  k_chain_frontier<<<grid_for(2 * na, TPB), TPB, 0, c.s>>>(L0.lA.p, c.cp[K_A0], c.T, chain_of(c, epA));
   CKL("k_chain_frontier");
   // the aggregate chain: W_q(anc(i), anc(j)) += delta and the strengths of
   // every level above 0; the weights are applied when each level is next read
@@ -1147,15 +1159,18 @@ void pushdown(ldl_ctx& c, int r, int32_t epCh, int64_t moved_ub) {
     Adj<int32_t> ch{L.children.off.p, L.children.len.p, L.children.col.p, L.children.w.p};
     int32_t* dst = q > 0 ? bufs[flip] : nullptr;
     zero_cnt(c, idxs[flip]);
-    ChunkMap m = chunk_map(c, src, c.dcnt + idx, n, L.children.len.p, nullptr);
-    k_push<<<grid_for((int64_t)n * 64, TPB, 16), TPB, 0, c.s>>>(
-        m, c.lv[q + 1].lab.p, ch, L.par.p, L.lab.p, dst, c.dcnt + idxs[flip], q == 0 ? c.stCh.p : nullptr, epCh,
-        c.lCh.p, c.dcnt + K_CH, c.lab_before.p);
+    ChunkMap m = chunk_map(c, src, c.cp[idx], n, L.children.len.p, nullptr);
+    int32_t nn = 0;
+    const HostRead rr{c.cp[idxs[flip]], &nn, sizeof(int32_t)};
+    k_push<<<chunk_grid(n), TPB, 0, c.s>>>(
+        m, c.lv[q + 1].lab.p, ch, L.par.p, L.lab.p, dst, c.cp[idxs[flip]], q == 0 ? c.stCh.p : nullptr, epCh,
+        c.lCh.p, c.cp[K_CH], c.lab_before.p, q > 0 ? tail_begin(c, &rr, 1) : Tail{});
     CKL("k_push");
     if (q > 0) {
+      tail_wait(c, &rr, 1);
       src = bufs[flip];
       idx = idxs[flip];
-      n = rd_cnt(c, idx);
+      n = nn;
       flip ^= 1;
     }
   }
@@ -1167,13 +1182,13 @@ int32_t dissolve_all(ldl_ctx& c, int r, int32_t epD) {
   LevelState& L = c.lv[r];
   LevelState& N = c.lv[r + 1];
   zero_cnt(c, K_D);
-  k_alive_list<<<grid_for(c.n, TPB), TPB, 0, c.s>>>(r ? L.alive.p : nullptr, c.n, c.lD.p, c.dcnt + K_D);
+  k_alive_list<<<grid_for(c.n, TPB), TPB, 0, c.s>>>(r ? L.alive.p : nullptr, c.n, c.lD.p, c.cp[K_D]);
   CKL("k_alive_list");
-  k_stamp_list<<<grid_for(c.n, TPB), TPB, 0, c.s>>>(c.lD.p, c.dcnt + K_D, c.stD.p, epD);
+  k_stamp_list<<<grid_for(c.n, TPB), TPB, 0, c.s>>>(c.lD.p, c.cp[K_D], c.stD.p, epD);
   CKL("k_stamp_list");
   const int32_t nd = rd_cnt(c, K_D);
   if (nd > 0) {
-    k_dissolve<<<grid_for(nd, TPB), TPB, 0, c.s>>>(c.lD.p, c.dcnt + K_D, L.par.p, c.par_old.p, L.kout.p,
+    k_dissolve<<<grid_for(nd, TPB), TPB, 0, c.s>>>(c.lD.p, c.cp[K_D], L.par.p, c.par_old.p, L.kout.p,
                                                    kin_of(c, r), N.kout.p, kin_of(c, r + 1), N.cnt.p, c.directed);
     CKL("k_dissolve");
   }
@@ -1183,8 +1198,8 @@ int32_t dissolve_all(ldl_ctx& c, int r, int32_t epD) {
 void singletons_of(ldl_ctx& c, int r, const int32_t* list, int idx_n, int64_t n_hint, int32_t* out, int idx_out) {
   zero_cnt(c, idx_out);
   if (n_hint > 0) {
-    k_singletons<<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(list, c.dcnt + idx_n, c.lv[r].par.p, c.lv[r + 1].cnt.p, out,
-                                                         c.dcnt + idx_out);
+    k_singletons<<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(list, c.cp[idx_n], c.lv[r].par.p, c.lv[r + 1].cnt.p, out,
+                                                         c.cp[idx_out]);
     CKL("k_singletons");
   }
 }
@@ -1198,8 +1213,8 @@ void reset_par(ldl_ctx& c, int r, int32_t nD) {
 
 template <class WT>
 static void leave_degree(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t nD, int32_t epL, int32_t epF) {
-  ChunkMap m = chunk_map(c, c.lD.p, c.dcnt + K_D, nD, out.len, c.directed ? in.len : nullptr);
-  k_leave_degree<WT><<<grid_for((int64_t)nD * 64, TPB, 16), TPB, 0, c.s>>>(out, in, m, c.lv[r].par.p, c.par_old.p,
+  ChunkMap m = chunk_map(c, c.lD.p, c.cp[K_D], nD, out.len, c.directed ? in.len : nullptr);
+  k_leave_degree<WT><<<chunk_grid(nD), TPB, 0, c.s>>>(out, in, m, c.lv[r].par.p, c.par_old.p,
                                                                            c.stL.p, epL, c.nbr.p, c.ckf.p, epF);
   CKL("k_leave_degree");
 }
@@ -1207,11 +1222,11 @@ static void leave_degree(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t nD,
 template <class WT>
 static void union_find(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t nG, int32_t epL) {
   LevelState& L = c.lv[r];
-  k_uf_sample<WT><<<grid_for((int64_t)nG * 32, TPB, 16), TPB, 0, c.s>>>(out, in, c.directed, c.lG.p, c.dcnt + K_G,
+  k_uf_sample<WT><<<grid_for((int64_t)nG * 32, TPB, 16), TPB, 0, c.s>>>(out, in, c.directed, c.lG.p, c.cp[K_G],
                                                                        L.par.p, c.stL.p, epL, c.comp.p);
   CKL("k_uf_sample");
-  ChunkMap m = chunk_map(c, c.lG.p, c.dcnt + K_G, nG, out.len, c.directed ? in.len : nullptr);
-  k_uf<WT><<<grid_for((int64_t)nG * 64, TPB, 16), TPB, 0, c.s>>>(out, in, m, L.par.p, L.alive.p, c.stL.p, epL,
+  ChunkMap m = chunk_map(c, c.lG.p, c.cp[K_G], nG, out.len, c.directed ? in.len : nullptr);
+  k_uf<WT><<<chunk_grid(nG), TPB, 0, c.s>>>(out, in, m, L.par.p, L.alive.p, c.stL.p, epL,
                                                                   c.comp.p);
   CKL("k_uf");
 }
@@ -1232,59 +1247,58 @@ static void union_find(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t nG, i
 int32_t split(ldl_ctx& c, int r, int32_t epD, int32_t epX) {
   LevelState& L = c.lv[r];
   LevelState& N = c.lv[r + 1];
-  {
-    ZeroSpans z;
-    z.mask = cnt_bit(K_D) | cnt_bit(K_X);
-    zero_many(c, z);
-  }
+  zero_cnt(c, K_D);
+  zero_cnt(c, K_X);
   const int32_t epF = c.next_epoch();  // communities whose connectivity is in doubt
   // The level's deleted-arc endpoints and U* stay on the device: both kernels
   // stride over their lists' counts with a grid bounded by the node count.
   const int gs = grid_for(c.n, TPB, 4);
-  k_brk_check<<<gs, TPB, 0, c.s>>>(L.lK.p, c.dcnt + K_BRK0 + r, L.alive.p, L.par.p, c.stX.p, epX, c.lX.p,
-                                   c.dcnt + K_X, c.ckf.p, epF);
+  k_brk_check<<<gs, TPB, 0, c.s>>>(L.lK.p, c.cp[K_BRK0 + r], L.alive.p, L.par.p, c.stX.p, epX, c.lX.p,
+                                   c.cp[K_X], c.ckf.p, epF);
   CKL("k_brk_check");
   const int32_t epL = c.next_epoch();
-  k_leave<<<gs, TPB, 0, c.s>>>(c.lUstar.p, c.dcnt + K_USTAR, L.alive.p, L.lab.p, N.lab.p, L.par.p, c.par_old.p,
+  int32_t cnt2[2] = {0, 0};
+  const HostRead rd[2] = {{c.cp[K_D], &cnt2[0], sizeof(int32_t)}, {c.cp[K_X], &cnt2[1], sizeof(int32_t)}};
+  k_leave<<<gs, TPB, 0, c.s>>>(c.lUstar.p, c.cp[K_USTAR], L.alive.p, L.lab.p, N.lab.p, L.par.p, c.par_old.p,
                                L.kout.p, kin_of(c, r), N.kout.p, kin_of(c, r + 1), N.cnt.p, c.directed, c.stL.p, epL,
-                               c.stD.p, epD, c.lD.p, c.dcnt + K_D, c.stX.p, epX, c.lX.p, c.dcnt + K_X, c.nbr.p);
+                               c.stD.p, epD, c.lD.p, c.cp[K_D], c.stX.p, epX, c.lX.p, c.cp[K_X], c.nbr.p,
+                               tail_begin(c, rd, 2));
   CKL("k_leave");
-  int32_t cnt2[2] = {0, 0};  // K_D, then K_X (adjacent counters)
-  {
-    const HostRead rr[2] = {{c.dcnt + K_D, &cnt2[0], sizeof(int32_t)}, {c.dcnt + K_X, &cnt2[1], sizeof(int32_t)}};
-    host_read(c, rr, 2);
-  }
+  tail_wait(c, rd, 2);
   const int32_t nleft = cnt2[0], nx = cnt2[1];
-  bool renamed = false;  // k_rename appends to lD; otherwise |D| = nleft
+  int32_t nD = nleft;  // k_rename appends to lD
   if (nx > 0) {
     if (nleft > 0) {
       if (r == 0) leave_degree<int32_t>(c, r, adj_out0(c), adj_in0(c), nleft, epL, epF);
       else leave_degree<int64_t>(c, r, adj_out(c, r), adj_in(c, r), nleft, epL, epF);
     }
     zero_cnt(c, K_G);
+    int32_t nG = 0;
+    const HostRead rg{c.cp[K_G], &nG, sizeof(int32_t)};
     Adj<int32_t> ch{L.children.off.p, L.children.len.p, L.children.col.p, L.children.w.p};
-    ChunkMap m = chunk_map(c, c.lX.p, c.dcnt + K_X, nx, L.children.len.p, nullptr);
-    k_members<<<grid_for((int64_t)nx * 64, TPB, 16), TPB, 0, c.s>>>(ch, m, L.par.p, c.stL.p, epL, c.ckf.p, epF,
-                                                                   c.comp.p, c.lG.p, c.dcnt + K_G);
+    ChunkMap m = chunk_map(c, c.lX.p, c.cp[K_X], nx, L.children.len.p, nullptr);
+    k_members<<<chunk_grid(nx), TPB, 0, c.s>>>(ch, m, L.par.p, c.stL.p, epL, c.ckf.p, epF,
+                                                                   c.comp.p, c.lG.p, c.cp[K_G], tail_begin(c, &rg, 1));
     CKL("k_members");
-    const int32_t nG = rd_cnt(c, K_G);
+    tail_wait(c, &rg, 1);
     c.res.split_members += nG;
-    renamed = nG > 0;
     if (nG > 0) {
       if (r == 0) union_find<int32_t>(c, r, adj_out0(c), adj_in0(c), nG, epL);
       else union_find<int64_t>(c, r, adj_out(c, r), adj_in(c, r), nG, epL);
-      k_uf_final<<<grid_for(nG, TPB), TPB, 0, c.s>>>(c.lG.p, c.dcnt + K_G, c.comp.p);
+      k_uf_final<<<grid_for(nG, TPB), TPB, 0, c.s>>>(c.lG.p, c.cp[K_G], c.comp.p);
       CKL("k_uf_final");
-      k_rename<<<grid_for(nG, TPB), TPB, 0, c.s>>>(c.lG.p, c.dcnt + K_G, c.comp.p, L.alive.p, c.stL.p, epL, L.par.p,
+      const HostRead rn{c.cp[K_D], &nD, sizeof(int32_t)};
+      k_rename<<<grid_for(nG, TPB), TPB, 0, c.s>>>(c.lG.p, c.cp[K_G], c.comp.p, L.alive.p, c.stL.p, epL, L.par.p,
                                                    c.par_old.p, L.kout.p, kin_of(c, r), N.kout.p, kin_of(c, r + 1),
-                                                   N.cnt.p, c.directed, c.stD.p, epD, c.lD.p, c.dcnt + K_D);
+                                                   N.cnt.p, c.directed, c.stD.p, epD, c.lD.p, c.cp[K_D], tail_begin(c, &rn, 1));
       CKL("k_rename");
+      tail_wait(c, &rn, 1);
     }
   }
   // the deletions of this level are consumed
   L.brk_ep = c.next_epoch();
   zero_cnt(c, K_BRK0 + r);
-  return renamed ? rd_cnt(c, K_D) : nleft;
+  return nD;
 }
 
 // deg: out-row and in-row entries of the changed nodes (k_changed); returns
@@ -1299,10 +1313,10 @@ static int64_t emit_records(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t 
   if (cap > INT32_MAX) ldl_throw(LDL_E_OVERFLOW, "aggregate records beyond the 32-bit record counter");
   c.rk2.reserve(cap, c.s);
   c.rv2.reserve(cap, c.s);
-  ChunkMap m = chunk_map(c, c.lC.p, c.dcnt + K_C, nC, out.len, in.len);
-  k_emit<WT><<<grid_for((int64_t)nC * 64, TPB, 16), TPB, 0, c.s>>>(out, in, m, c.lv[r].par.p, c.par_old.p,
+  ChunkMap m = chunk_map(c, c.lC.p, c.cp[K_C], nC, out.len, in.len);
+  k_emit<WT><<<chunk_grid(nC), TPB, 0, c.s>>>(out, in, m, c.lv[r].par.p, c.par_old.p,
                                                                           c.stC.p, epC, c.bits, c.rk2.p, c.rv2.p,
-                                                                          c.dcnt + K_REC, cap, c.dcnt + K_ERR);
+                                                                          c.cp[K_REC], cap, c.cp[K_ERR]);
   CKL("k_emit");
   return cap;
 }
@@ -1319,24 +1333,18 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
   LevelState& N = c.lv[r + 1];
   // changed nodes
   sub_begin(c);
-  static_assert(offsetof(DevScalars, need2) == offsetof(DevScalars, need) + 8, "adjacent accumulators");
-  {
-    ZeroSpans z;
-    z.mask = cnt_bit(K_C) | cnt_bit(K_REC) | cnt_bit(K_CREC);
-    z.p[0] = &c.d_sc->need;
-    z.nw[0] = 2;
-    zero_many(c, z);
-  }
+  for (int k : {K_C, K_REC, K_CREC}) zero_cnt(c, k);
+  c.sums = (int64_t*)fresh(c, 4, c.d_sc->sums);
   int32_t nC = 0;
   int64_t deg[2] = {0, 0};
   if (nD > 0) {
     const int32_t* lo = r == 0 ? adj_out0(c).len : adj_out(c, r).len;
     const int32_t* li = r == 0 ? adj_in0(c).len : adj_in(c, r).len;
-    k_changed<<<grid_for(nD, TPB), TPB, 0, c.s>>>(c.lD.p, c.dcnt + K_D, L.par.p, c.par_old.p, c.stC.p, epC, c.lC.p,
-                                                  c.dcnt + K_C, lo, li, &c.d_sc->need, &c.d_sc->need2);
+    const HostRead rr[2] = {{c.cp[K_C], &nC, sizeof(int32_t)}, {c.sums, deg, 2 * sizeof(int64_t)}};
+    k_changed<<<grid_for(nD, TPB), TPB, 0, c.s>>>(c.lD.p, c.cp[K_D], L.par.p, c.par_old.p, c.stC.p, epC, c.lC.p,
+                                                  c.cp[K_C], lo, li, c.sums, c.sums + 1, tail_begin(c, rr, 2));
     CKL("k_changed");
-    const HostRead rr[2] = {{c.dcnt + K_C, &nC, sizeof(int32_t)}, {&c.d_sc->need, deg, 2 * sizeof(int64_t)}};
-    host_read(c, rr, 2);
+    tail_wait(c, rr, 2);
   }
   int64_t nr = 0;  // bound on the level r+1 records (their number is at dcnt[K_NR])
   if (nC > 0) {
@@ -1344,9 +1352,9 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
                           : emit_records<int64_t>(c, r, adj_out(c, r), adj_in(c, r), nC, epC, build, deg);
     c.crk.reserve(2 * (int64_t)nC + 2, c.s);
     c.crv.reserve(2 * (int64_t)nC + 2, c.s);
-    k_emit_nodes<<<grid_for(nC, TPB), TPB, 0, c.s>>>(c.lC.p, c.dcnt + K_C, L.par.p, c.par_old.p, L.kout.p,
+    k_emit_nodes<<<grid_for(nC, TPB), TPB, 0, c.s>>>(c.lC.p, c.cp[K_C], L.par.p, c.par_old.p, L.kout.p,
                                                      kin_of(c, r), c.bits, r + 1, build ? r + 1 : c.T, c.directed,
-                                                     chain_of(c, nullptr), c.crk.p, c.crv.p, c.dcnt + K_CREC);
+                                                     chain_of(c, nullptr), c.crk.p, c.crv.p, c.cp[K_CREC]);
     CKL("k_emit_nodes");
     sub_end(c, SU_AGG_EMIT);
     sub_begin(c);
@@ -1354,8 +1362,8 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
       // level r+1 starts empty: build its adjacency and the children lists
       int32_t nrec32 = 0, ncr32 = 0;
       {
-        const HostRead rr[2] = {{c.dcnt + K_REC, &nrec32, sizeof(int32_t)},
-                                {c.dcnt + K_CREC, &ncr32, sizeof(int32_t)}};
+        const HostRead rr[2] = {{c.cp[K_REC], &nrec32, sizeof(int32_t)},
+                                {c.cp[K_CREC], &ncr32, sizeof(int32_t)}};
         host_read(c, rr, 2);
       }
       const int64_t cnt = nrec32, ncr = ncr32;
@@ -1376,7 +1384,7 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
       }
       csr_build<int32_t>(L.children, c.n, c.crk.p, (const int64_t*)c.crv.p, ncr, c.bits, 25, c.CS, c.P, c.s);
     } else {
-      const int32_t* cnt_dev = c.dcnt + K_REC;
+      const int32_t* cnt_dev = c.cp[K_REC];
       if (nrec > AGG_EXACT) {
         const int64_t cnt = rd_cnt(c, K_REC);
         if (cnt > nrec) ldl_throw(LDL_E_INVALID, "internal: aggregate records exceed their bound");
@@ -1386,7 +1394,7 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
       c.rk.reserve(nrec + 1, c.s);
       c.rsum.reserve(nrec + 1, c.s);
       if (nrec > 0)
-        sort_reduce(c.rk2, c.rv2, c.tk, c.tv, nrec, cnt_dev, c.bits, false, 0, c.rk.p, c.rsum.p, c.dcnt + K_NR, c.P,
+        sort_reduce(c.rk2, c.rv2, c.tk, c.tv, nrec, cnt_dev, c.bits, false, 0, c.rk.p, c.rsum.p, c.cp[K_NR], c.P,
                     c.s);
       nr = nrec;
       if (nrec > AGG_EXACT) nr = rd_cnt(c, K_NR);
@@ -1394,9 +1402,9 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
       sub_begin(c);
       // the level r+1 records join its pending list and, mapped through the
       // current parents, the lists of the levels above
-      chain_records(c, c.rk.p, c.rsum.p, nr, c.dcnt + K_NR, r + 1, true, false);
-      sort_pairs(c.crk, c.crv, c.tk, c.tv, 2 * (int64_t)nC, 2 * c.bits, c.P, c.s, 0, c.dcnt + K_CREC);
-      csr_apply<int32_t>(L.children, c.crk.p, (const int64_t*)c.crv.p, 2 * (int64_t)nC, c.dcnt + K_CREC, 1, c.bits,
+      chain_records(c, c.rk.p, c.rsum.p, nr, c.cp[K_NR], r + 1, true, false);
+      sort_pairs(c.crk, c.crv, c.tk, c.tv, 2 * (int64_t)nC, 2 * c.bits, c.P, c.s, 0, c.cp[K_CREC]);
+      csr_apply<int32_t>(L.children, c.crk.p, (const int64_t*)c.crv.p, 2 * (int64_t)nC, c.cp[K_CREC], 1, c.bits,
                          c.CS, c.P, c.s, c.d_sc);
     }
     sub_end(c, SU_AGG_APPLY);
@@ -1408,9 +1416,9 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
       ech.alive[q] = c.lv[q].alive.p;
       ech.par[q] = c.lv[q].par.p;
     }
-    k_exist_chain<<<grid_for(2 * (int64_t)nC, TPB), TPB, 0, c.s>>>(c.lC.p, c.dcnt + K_C, L.par.p, c.par_old.p,
+    k_exist_chain<<<grid_for(2 * (int64_t)nC, TPB), TPB, 0, c.s>>>(c.lC.p, c.cp[K_C], L.par.p, c.par_old.p,
                                                                     c.stE.p, c.next_epoch(), r + 1, c.T, ech,
-                                                                    c.dcnt + K_ERR);
+                                                                    c.cp[K_ERR]);
     CKL("k_exist_chain");
     // the error flag K_ERR is read once at the end of the batch (or of the static build)
   } else {
@@ -1419,10 +1427,10 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
   }
   // |U*| stays on the device: the grid is bounded by two blocks per SM
   const bool recs = nC > 0 && epA_next;
-  k_next_level<<<device_sms() * 2, TPB, 0, c.s>>>(c.lUstar.p, c.dcnt + K_USTAR, c.lD.p, c.dcnt + K_D, L.par.p,
+  k_next_level<<<device_sms() * 2, TPB, 0, c.s>>>(c.lUstar.p, c.cp[K_USTAR], c.lD.p, c.cp[K_D], L.par.p,
                                                   c.par_old.p, L.lab.p, N.lab.p, recs ? c.rk.p : nullptr,
-                                                  c.dcnt + K_NR, nr, c.bits, N.alive.p, epA_next ? N.stA.p : nullptr,
-                                                  epA_next, N.lA.p, c.dcnt + K_A0 + r + 1, &c.d_sc->agg_recs);
+                                                  c.cp[K_NR], nr, c.bits, N.alive.p, epA_next ? N.stA.p : nullptr,
+                                                  epA_next, N.lA.p, c.cp[K_A0 + r + 1], &c.d_sc->agg_recs);
   CKL("k_next_level");
   sub_end(c, SU_AGG_EXIST);
 }
@@ -1456,17 +1464,17 @@ void level_free(ldl_ctx& c, int r) { c.lv[r].release(); }
 
 int32_t alive_list(ldl_ctx& c, int r, int32_t* list, int idx) {
   zero_cnt(c, idx);
-  k_alive_list<<<grid_for(c.n, TPB), TPB, 0, c.s>>>(r ? c.lv[r].alive.p : nullptr, c.n, list, c.dcnt + idx);
+  k_alive_list<<<grid_for(c.n, TPB), TPB, 0, c.s>>>(r ? c.lv[r].alive.p : nullptr, c.n, list, c.cp[idx]);
   CKL("k_alive_list");
   return rd_cnt(c, idx);
 }
 
-void changed_labels_launch(ldl_ctx& c) {
+void changed_labels(ldl_ctx& c, const HostRead* rr, int n) {
   // strides over the candidates' device count with a grid bounded by the node count
-  zero_cnt(c, K_CHG);
-  k_changed_final<<<grid_for(c.n, TPB, 4), TPB, 0, c.s>>>(c.lCh.p, c.dcnt + K_CH, c.lv[0].lab.p, c.lab_before.p,
-                                                          c.lChg.p, c.dcnt + K_CHG);
+  k_changed_final<<<grid_for(c.n, TPB, 2), TPB, 0, c.s>>>(c.lCh.p, c.cp[K_CH], c.lv[0].lab.p, c.lab_before.p, c.lChg.p,
+                                                          c.cp[K_CHG], tail_begin(c, rr, n));
   CKL("k_changed_final");
+  tail_wait(c, rr, n);
 }
 
 void upload_graph(ldl_ctx& c, int64_t nnz, const int64_t* row_ptr, const int32_t* col, const int32_t* w) {
@@ -1539,15 +1547,17 @@ void upload_graph(ldl_ctx& c, int64_t nnz, const int64_t* row_ptr, const int32_t
   CK(cudaMemsetAsync(L0.alive.p, 1, (size_t)n, c.s));
   CK(cudaMemcpyAsync(c.Kout.p, L0.kout.p, sizeof(int64_t) * (size_t)n, cudaMemcpyDeviceToDevice, c.s));
   if (c.directed) CK(cudaMemcpyAsync(c.Kin.p, L0.kin.p, sizeof(int64_t) * (size_t)n, cudaMemcpyDeviceToDevice, c.s));
-  CK(cudaMemsetAsync(&c.d_sc->de, 0, sizeof(int64_t), c.s));
-  CK(cudaMemsetAsync(&c.d_sc->p_new, 0, sizeof(I128), c.s));
-  k_esum<<<grid_for(n, TPB), TPB, 0, c.s>>>(c.e.p, c.Kout.p, Kin_of(c), n, &c.d_sc->de, &c.d_sc->p_new);
+  c.racc = (RepairAcc*)c.d_sc->home2;
+  CK(cudaMemsetAsync(c.racc, 0, sizeof(RepairAcc), c.s));
+  k_esum<<<grid_for(n, TPB), TPB, 0, c.s>>>(c.e.p, c.Kout.p, Kin_of(c), n, &c.racc->de, &c.racc->p_new);
   CKL("k_esum");
   DevScalars h;
   CK(cudaMemcpyAsync(&h, c.d_sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, c.s));
   CK(cudaStreamSynchronize(c.s));
   c.m = h.dm;
   if (c.m >= ((int64_t)1 << 50)) ldl_throw(LDL_E_OVERFLOW, "total weight m reaches 2^50");
-  c.E = h.de;
-  c.Psum = i128_of(h.p_new.hi, h.p_new.lo);
+  RepairAcc ra;
+  memcpy(&ra, h.home2, sizeof(ra));
+  c.E = ra.de;
+  c.Psum = i128_of(ra.p_new.hi, ra.p_new.lo);
 }

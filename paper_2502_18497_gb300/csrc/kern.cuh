@@ -19,26 +19,31 @@ constexpr int32_t BIN_MAX[4] = {32, 128, 1024, 2048};
 // ---- sweep.cu
 void expand_set(ldl_ctx& c, int r, const int32_t* list, int idx_n, int32_t* stamp, int32_t ep, int32_t* olist,
                 int idx_out, int64_t n_hint);
-void filter_alive(ldl_ctx& c, int r, const int32_t* list, int idx_n, int32_t* olist, int idx_out, int64_t n_hint);
+// U = U* = the existing nodes of A^r (lists lU and lUstar, stamp stU with
+// epU); returns when the read rr has arrived.
+void frontier(ldl_ctx& c, int r, int32_t epU, const HostRead* rr, int n);
 void union_into(ldl_ctx& c, const int32_t* list, int idx_n, int32_t* stamp, int32_t ep, int32_t* olist, int idx_out,
                 int64_t n_hint);
-// BestMove (mode 0) / BestRef (mode 1) over the listed nodes; the candidates
-// and their count (counter K_CAND) stay on the device.  Returns the list's
-// length (dcnt[idx_n]), read with the sweep's bin counts.
-int32_t sweep(ldl_ctx& c, int r, int mode, const int32_t* list, int idx_n, int64_t n_hint);
-// Decoupling filter over the last sweep's candidates: returns their number
-// and the number accepted (the accepted moves are in bv / bsrc / bdst), and
-// counter `extra` (when >= 0) read in the same host wait.
-struct DecoupleOut {
-  int32_t nc, nb, extra;
+// BestMove (mode 0) / BestRef (mode 1) over the listed nodes, then the
+// decoupling filter over the candidates: the list's length, the number of
+// candidates and the number accepted (in bv / bsrc / bdst).
+struct SweepOut {
+  int32_t nlist, nc, nb;
 };
-DecoupleOut decouple(ldl_ctx& c, int extra = -1);
-// Launches the commit of a mini-batch; commit_read then reads its outcome
-// (with the counter dcnt[extra_idx] in the same read when extra is given).
+SweepOut sweep(ldl_ctx& c, int r, int mode, const int32_t* list, int idx_n, int64_t n_hint);
+// Decoupling filter over the last sweep's candidates; the values of `extra`
+// arrive in the same host wait.
+struct DecoupleOut {
+  int32_t nc, nb, rounds;
+};
+DecoupleOut decouple(ldl_ctx& c, const HostRead* extra = nullptr, int n_extra = 0);
+// Launches the commit of a mini-batch; commit_expand then expands the next
+// frontier U = V + N(V) and reads the outcome and |U|.
 void commit_move(ldl_ctx& c, int r, int32_t nb, int32_t epB, int32_t epT, int32_t epCh);
-CommitOut commit_read(ldl_ctx& c, int extra_idx, int32_t* extra);
+CommitOut commit_expand(ldl_ctx& c, int r, int32_t nb, int32_t ep, int32_t* nU);
 void rollback_move(ldl_ctx& c, int r, int32_t nb, int32_t ntc);
-void mark_moved(ldl_ctx& c, int r, int32_t nb, int32_t epMv, int32_t epM0);
+// moved nodes into lMv (level 0: lM0 too), and the next U (nU nodes) into U*
+void mark_moved(ldl_ctx& c, int r, int32_t nb, int32_t epMv, int32_t epM0, int32_t epU, int32_t nU);
 void commit_ref(ldl_ctx& c, int r, int32_t nb);
 void spexpand(ldl_ctx& c, int r, int32_t nb, int32_t epD, int32_t epR, int32_t* lR, int idx_R);
 
@@ -48,7 +53,9 @@ void spexpand(ldl_ctx& c, int r, int32_t nb, int32_t epD, int32_t epR, int32_t* 
 int64_t ingest(ldl_ctx& c, const ldl_update* upd, int64_t count, int on_device, int64_t* dm);
 // Apply the level-0 arcs to the adjacency and repair every statistic along
 // the parent chain; marks InitFrontier in the A lists (epA per level).
-void repair_batch(ldl_ctx& c, int64_t na, const int32_t* epA, int32_t epT, int64_t dm);
+// The sums that change m, E and P stay on the device (c.racc) until repair_done.
+void repair_batch(ldl_ctx& c, int64_t na, const int32_t* epA, int32_t epT);
+void repair_done(ldl_ctx& c, const RepairAcc& a, int64_t dm);
 void pending_reset(ldl_ctx& c);
 // known: the level's pending record count when the caller has read it, else -1
 void flush_level(ldl_ctx& c, int q, int64_t known = -1);
@@ -57,7 +64,7 @@ void pushdown(ldl_ctx& c, int r, int32_t epCh, int64_t moved_ub);
 int32_t dissolve_all(ldl_ctx& c, int r, int32_t epD);
 int32_t split(ldl_ctx& c, int r, int32_t epD, int32_t epX);
 // the listed level-r nodes that are singleton refined communities -> out
-// (their count stays on the device, at dcnt[idx_out])
+// (their count stays on the device, at cp[idx_out])
 void singletons_of(ldl_ctx& c, int r, const int32_t* list, int idx_n, int64_t n_hint, int32_t* out, int idx_out);
 // nD = |D| (list lD), the nodes whose refined community changed.
 void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bool build, int32_t nD);
@@ -73,6 +80,6 @@ void level_free(ldl_ctx& c, int r);
 int32_t alive_list(ldl_ctx& c, int r, int32_t* list, int idx);
 void reset_par(ldl_ctx& c, int r, int32_t nD);
 // the level-0 nodes whose label differs from the batch's start -> lChg
-// (count at dcnt[K_CHG], read by the caller)
-void changed_labels_launch(ldl_ctx& c);
+// (count at cp[K_CHG], which the caller clears); the read rr ends it
+void changed_labels(ldl_ctx& c, const HostRead* rr, int n);
 void gather_labels(ldl_ctx& c, const int32_t* ids, int32_t k, int32_t* out);

@@ -140,13 +140,6 @@ __global__ void __launch_bounds__(256) k_snapshot(SnapList l, unsigned char* dst
       for (int64_t b = l.bytes[r] & ~(int64_t)15; b < l.bytes[r]; ++b) dst[l.off[r] + b] = l.src[r][b];
 }
 
-// clears the counters named by the mask and up to ZERO_SPANS spans of 64-bit words
-__global__ void k_zero(int32_t* dcnt, ZeroSpans z) {
-  const int t = threadIdx.x;
-  if (t < K_COUNT && ((z.mask >> t) & 1ull)) dcnt[t] = 0;
-  for (int i = 0; i < ZERO_SPANS; ++i)
-    if (z.p[i] && t < z.nw[i]) z.p[i][t] = 0;
-}
 }  // namespace
 
 // Polls the mapped sequence word until the read `seq` has arrived.  Every so
@@ -199,22 +192,61 @@ void host_read(ldl_ctx& c, const HostRead* r, int n) {
 
 int32_t rd_cnt(ldl_ctx& c, int idx) {
   int32_t v = 0;
-  const HostRead r{c.dcnt + idx, &v, sizeof(int32_t)};
+  const HostRead r{c.cp[idx], &v, sizeof(int32_t)};
   host_read(c, &r, 1);
   return v;
 }
 
-void zero_cnt(ldl_ctx& c, int idx) { CK(cudaMemsetAsync(c.dcnt + idx, 0, sizeof(int32_t), c.s)); }
+void zero_cnt(ldl_ctx& c, int idx) {
+  if (c.arena_top < ARENA_WORDS) {
+    c.cp[idx] = c.arena + c.arena_top++;
+    return;
+  }
+  c.cp[idx] = c.dcnt + idx;
+  CK(cudaMemsetAsync(c.cp[idx], 0, sizeof(int32_t), c.s));
+}
 
-void zero_many(ldl_ctx& c, const ZeroSpans& z) {
-  for (int i = 0; i < ZERO_SPANS; ++i)
-    if (z.nw[i] < 0 || z.nw[i] > K_COUNT) ldl_throw(LDL_E_INVALID, "internal: zero span too long");
-  k_zero<<<1, K_COUNT, 0, c.s>>>(c.dcnt, z);
-  CKL("k_zero");
+void* fresh(ldl_ctx& c, int words, void* home) {
+  const int at = (c.arena_top + 3) & ~3;
+  if (at + words <= ARENA_WORDS) {
+    c.arena_top = at + words;
+    return c.arena + at;
+  }
+  CK(cudaMemsetAsync(home, 0, sizeof(int32_t) * (size_t)words, c.s));
+  return home;
+}
+
+Tail tail_begin(ldl_ctx& c, const HostRead* r, int n) {
+  Tail t{};
+  if (n > TAIL_MAX) ldl_throw(LDL_E_INVALID, "internal: host read of too many values");
+  int32_t off = 0;
+  for (int i = 0; i < n; ++i) {
+    t.src[i] = (const uint32_t*)r[i].src;
+    t.off[i] = off;
+    t.words[i] = r[i].bytes / 4;
+    off += t.words[i];
+  }
+  if (off * 4 > PUB_BYTES) ldl_throw(LDL_E_INVALID, "internal: host read too large");
+  t.n = n;
+  zero_cnt(c, K_TICKET);
+  t.ticket = c.cp[K_TICKET];
+  const Pub p = pub_begin(c);
+  t.page = p.page;
+  t.seq = p.seq;
+  return t;
+}
+
+void tail_wait(ldl_ctx& c, const HostRead* r, int n) {
+  wait_page(c, c.pub_seq);
+  const unsigned char* pay = (const unsigned char*)(c.h_pub + 1);
+  for (int i = 0; i < n; ++i) {
+    memcpy(r[i].dst, pay, (size_t)r[i].bytes);
+    pay += r[i].bytes;
+  }
 }
 
 void set_cnt(ldl_ctx& c, int idx, int32_t v) {
-  k_set_i32<<<1, 1, 0, c.s>>>(c.dcnt + idx, v);
+  k_set_i32<<<1, 1, 0, c.s>>>(c.cp[idx], v);
   CKL("k_set_i32");
 }
 
@@ -282,6 +314,10 @@ void alloc_globals(ldl_ctx& c) {
   CK(cudaMemsetAsync(c.d_sc, 0, sizeof(DevScalars), c.s));
   c.dcnt = (int32_t*)dalloc(sizeof(int32_t) * K_COUNT);
   CK(cudaMemsetAsync(c.dcnt, 0, sizeof(int32_t) * K_COUNT, c.s));
+  c.arena = (int32_t*)dalloc(sizeof(int32_t) * ARENA_WORDS);
+  CK(cudaMemsetAsync(c.arena, 0, sizeof(int32_t) * ARENA_WORDS, c.s));
+  c.arena_top = 0;
+  for (int k = 0; k < K_COUNT; ++k) c.cp[k] = c.dcnt + k;
   c.P.rd = [](void* owner, const HostRead* r, int n) { host_read(*(ldl_ctx*)owner, r, n); };
   c.P.rd_owner = &c;
   c.P.pub_begin = [](void* owner) { return pub_begin(*(ldl_ctx*)owner); };
@@ -293,7 +329,7 @@ void free_all(ldl_ctx& c) {
   for (auto& L : c.lv) L.release();
   DBuf<int64_t>* b64[] = {&c.Kout, &c.Kin, &c.e, &c.cghi, &c.snapKo, &c.snapKi, &c.snapE, &c.binLoff, &c.binLsz,
                           &c.gvals, &c.rsum, &c.rsum2, 
-                          &c.chunk_pre, &c.hub_ecnt, &c.hub_epre, &c.pb_hi};
+                          &c.chunk_pre, &c.hub_epre, &c.pb_hi};
   for (auto* b : b64) b->release();
   DBuf<int32_t>* b32[] = {&c.stS, &c.stU, &c.stMv, &c.stB, &c.stM0, &c.stD, &c.stC, &c.stR, &c.stX, &c.stT,
                           &c.stE, &c.stCh, &c.stL, &c.lG, &c.comp, &c.nbr, &c.ckf, &c.lU, &c.lS, &c.lUstar, &c.lMv, &c.lM0, &c.lD, &c.lC, &c.lR,
@@ -317,6 +353,8 @@ void free_all(ldl_ctx& c) {
   if (c.dcnt) dfree(c.dcnt);
   c.d_sc = nullptr;
   c.dcnt = nullptr;
+  if (c.arena) dfree(c.arena);
+  c.arena = nullptr;
   if (c.h_pub) cudaFreeHost((void*)c.h_pub);
   c.h_pub = nullptr;
   c.d_pub = nullptr;
@@ -351,14 +389,9 @@ static int64_t move_loop(ldl_ctx& c, int r, int rounds, int32_t epU, int32_t epM
     expand_set(c, r, c.lU.p, K_U, c.stS.p, epS, c.lS.p, K_S, nU);
     stage_end(c, ST_EXPAND);
     // |S| stays on the device: the sweep's kernels stride over it (n bounds
-    // their grids) and it comes back with the sweep's bin counts (β test)
-    stage_begin(c);
-    const int32_t nS = sweep(c, r, 0, c.lS.p, K_S, c.n);
-    stage_end(c, ST_BEST);
-    stage_begin(c);
-    const DecoupleOut dd = decouple(c);
-    stage_end(c, ST_DECOUPLE);
-    const int32_t nc = dd.nc, nb = dd.nb;
+    // their grids) and it comes back with the candidates (β test)
+    const SweepOut so = sweep(c, r, 0, c.lS.p, K_S, c.n);
+    const int32_t nS = so.nlist, nc = so.nc, nb = so.nb;
     if (nc == 0) break;
     c.res.rejected += nc - nb;
     if (nb == 0) break;
@@ -370,9 +403,8 @@ static int64_t move_loop(ldl_ctx& c, int r, int rounds, int32_t epU, int32_t epM
     // rolled-back mini-batch ends the loop and its expansion is dropped
     const int32_t epS2 = c.next_epoch();
     zero_cnt(c, K_U);
-    expand_set(c, r, c.bv.p, K_B, c.stS.p, epS2, c.lU.p, K_U, nb);
     int32_t nU2 = 0;
-    const CommitOut co = commit_read(c, K_U, &nU2);
+    const CommitOut co = commit_expand(c, r, nb, epS2, &nU2);
     if (co.dq < 0) {
       rollback_move(c, r, nb, co.ntc);
       c.res.rollbacks++;
@@ -383,11 +415,8 @@ static int64_t move_loop(ldl_ctx& c, int r, int rounds, int32_t epU, int32_t epM
     c.Psum += co.dp;
     c.res.moves += nb;
     committed += nb;
-    mark_moved(c, r, nb, epMv, epM0);
+    mark_moved(c, r, nb, epMv, epM0, epU, nU2);
     stage_end(c, ST_COMMIT);
-    stage_begin(c);
-    union_into(c, c.lU.p, K_U, c.stU.p, epU, c.lUstar.p, K_USTAR, nU2);
-    stage_end(c, ST_EXPAND);
     nU = nU2;
     if (co.dq * (i128)ainv < Q0) break;
     if ((int64_t)nb * binv < (int64_t)nS) break;
@@ -407,15 +436,14 @@ static int64_t refine_loop(ldl_ctx& c, int r, int rounds, int32_t epD, int32_t n
   const int64_t binv = c.prm.beta_inv;
   for (int j = 0; j < rounds; ++j) {
     // R is a subset of D, so nD bounds the sweep's launch; |R| comes back with
-    // the sweep's bin counts (an empty R ends the loop before any filter)
+    // the candidates (an empty R ends the loop and does not count)
     c.res.rounds++;
-    const int32_t nR = sweep(c, r, 1, R, iR, nD);
+    const SweepOut so = sweep(c, r, 1, R, iR, nD);
+    const int32_t nR = so.nlist, nc = so.nc, nb = so.nb;
     if (nR == 0) {
       c.res.rounds--;
       break;
     }
-    const DecoupleOut dd = decouple(c);
-    const int32_t nc = dd.nc, nb = dd.nb;
     if (nc == 0) break;
     c.res.rejected += nc - nb;
     if (nb == 0) break;
@@ -601,33 +629,47 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
   }
   stage_begin(c);
   const int32_t epT = c.next_epoch();
-  repair_batch(c, na, epA.data(), epT, dm);
+  repair_batch(c, na, epA.data(), epT);
+  if (c.prm.N == 0) {  // no pass reads the repair's sums
+    RepairAcc ra{};
+    const HostRead rr{c.racc, &ra, sizeof(ra)};
+    host_read(c, &rr, 1);
+    repair_done(c, ra, dm);
+  }
   stage_end(c, ST_REPAIR);
   const int64_t ainv = c.prm.alpha_inv;
   for (int pass = 0; pass < c.prm.N; ++pass) {
-    const i128 Qpass = qnum(c);
+    i128 Qpass = qnum(c);  // of the first pass: once the repair's sums are back
     const int32_t epM0 = c.next_epoch();
     zero_cnt(c, K_M0);
     int32_t nM0 = -1;  // |level-0 moves of the pass|, final once level 0 is done
     for (int r = 0; r <= T; ++r) {
-      // |A^r| stays on the device: the filter strides over it with a grid of
+      // |A^r| stays on the device: the kernel strides over it with a grid of
       // two blocks per SM, and one read returns |U|, the level's pending
-      // record count for its flush and, from level 1 on, |M0|
+      // record count for its flush and, from level 1 on, |M0| (on the first
+      // visit: the statistic repair's sums)
+      const int32_t epU = c.next_epoch();
       zero_cnt(c, K_U);
-      filter_alive(c, r, c.lv[r].lA.p, K_A0 + r, c.lU.p, K_U, std::min<int64_t>(c.n, (int64_t)device_sms() * 512));
+      zero_cnt(c, K_USTAR);
       int32_t nU = 0, nP = 0, m0 = 0;
-      {
-        const HostRead rr[3] = {{c.dcnt + K_U, &nU, sizeof(int32_t)},
-                                {c.dcnt + K_PEND0 + r, &nP, sizeof(int32_t)},
-                                {c.dcnt + K_M0, &m0, sizeof(int32_t)}};
-        host_read(c, rr, r > 0 ? 3 : 2);
-        if (r > 0) nM0 = m0;
+      RepairAcc ra{};
+      const bool first = pass == 0 && r == 0;
+      HostRead rr[3] = {{c.cp[K_U], &nU, sizeof(int32_t)},
+                        {c.cp[K_PEND0 + r], &nP, sizeof(int32_t)},
+                        {c.cp[K_M0], &m0, sizeof(int32_t)}};
+      if (first) {
+        rr[2].src = c.racc;
+        rr[2].dst = &ra;
+        rr[2].bytes = (int32_t)sizeof(ra);
       }
+      frontier(c, r, epU, rr, 3);
+      if (first) {
+        repair_done(c, ra, dm);
+        Qpass = qnum(c);
+      }
+      if (r > 0) nM0 = m0;
       if (nU == 0) continue;
       if (r < 8) c.res.frontier_nodes[r] += nU;
-      const int32_t epU = c.next_epoch();
-      zero_cnt(c, K_USTAR);
-      union_into(c, c.lU.p, K_U, c.stU.p, epU, c.lUstar.p, K_USTAR, nU);
       const int32_t epMv = c.next_epoch();
       zero_cnt(c, K_MV);
       stage_begin(c);
@@ -655,42 +697,44 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
         stage_end(c, ST_AGG);
       }
     }
-    // frontiers of the next pass: A^0 = Expand_0(level-0 moves), others empty
+    // frontiers of the next pass: A^0 = Expand_0(level-0 moves), others empty.
+    // The expansion holds the moved nodes themselves, so A^0 is empty exactly
+    // when no level-0 node moved.
+    if (pass + 1 == c.prm.N) break;
     if (nM0 < 0) nM0 = rd_cnt(c, K_M0);
+    if (nM0 == 0) break;
+    if ((qnum(c) - Qpass) * (i128)ainv < Qpass) break;
     for (int r = 0; r <= T; ++r) {
       epA[r] = c.next_epoch();
       zero_cnt(c, K_A0 + r);
     }
-    // the expansion holds the moved nodes themselves, so A^0 is empty
-    // exactly when no level-0 node moved
-    if (nM0 == 0) break;
     expand_set(c, 0, c.lM0.p, K_M0, c.lv[0].stA.p, epA[0], c.lv[0].lA.p, K_A0, nM0);
-    if ((qnum(c) - Qpass) * (i128)ainv < Qpass) break;
   }
   stage_begin(c);
   {
-    // the pending counts of every level above 0 in one read (K_PEND0 + r are
-    // adjacent; a flush changes no other level's list)
+    // the pending counts of every level above 0 in one read (a flush changes
+    // no other level's list)
     int32_t np[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (T >= 1) {
-      const HostRead rr{c.dcnt + K_PEND0 + 1, np, (int32_t)(sizeof(int32_t) * (size_t)std::min(T, 7))};
-      host_read(c, &rr, 1);
-    }
-    for (int r = 1; r <= T; ++r) flush_level(c, r, np[r - 1]);
+    HostRead rr[8];
+    int k = 0;
+    for (int r = 1; r <= T; ++r)
+      if (c.lv[r].pend_ub > 0) rr[k++] = {c.cp[K_PEND0 + r], &np[r], sizeof(int32_t)};
+    if (k) host_read(c, rr, k);
+    for (int r = 1; r <= T; ++r) flush_level(c, r, np[r]);
   }
   stage_end(c, ST_AGG);
-  changed_labels_launch(c);
-  // one read: changed labels, the internal error flag, entries scanned and
-  // the look-back scans' error flag
+  // one read: changed labels, the internal error flag, entries scanned, the
+  // aggregate records and the look-back scans' error flag
   int32_t nchg = 0, err = 0, scan_bad = 0;
   int32_t* scan_flag = scan_error_flag(c.P);
   {
-    const HostRead rr[5] = {{c.dcnt + K_CHG, &nchg, sizeof(int32_t)},
-                            {c.dcnt + K_ERR, &err, sizeof(int32_t)},
+    zero_cnt(c, K_CHG);
+    const HostRead rr[5] = {{c.cp[K_CHG], &nchg, sizeof(int32_t)},
+                            {c.cp[K_ERR], &err, sizeof(int32_t)},
                             {&c.d_sc->scanned, &c.res.edges_scanned, sizeof(int64_t)},
                             {&c.d_sc->agg_recs, &c.res.agg_records, sizeof(int64_t)},
                             {scan_flag, &scan_bad, sizeof(int32_t)}};
-    host_read(c, rr, scan_flag ? 5 : 4);
+    changed_labels(c, rr, scan_flag ? 5 : 4);
   }
   c.res.n_changed = nchg;
   c.res.host_syncs = c.syncs;

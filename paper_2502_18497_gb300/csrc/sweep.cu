@@ -29,19 +29,20 @@ std::atomic<int64_t> g_hub_table_slots{HUB_TABLE_SLOTS};
 static_assert(BIN_MAX[0] == HG8 / 2 && BIN_MAX[1] == HG32 / 2 && BIN_MAX[2] == 2048 / 2 &&
                   BIN_MAX[3] == HB / 2 && BIN_MAX[3] == MID_DEG,
               "bin bounds and table sizes");
-constexpr int EVAL_CH = 4096;  // hub table slots evaluated per block
+constexpr int EVAL_CH = 1024;  // hub table slots evaluated per block
 
 // ---------------------------------------------------------------- expand
 // out = U plus every out- and in-neighbour of U (dedup by stamp).
 template <class WT>
 __global__ void k_expand(Adj<WT> out, Adj<WT> in, ChunkMap m, int32_t* stamp, int32_t ep, int32_t* olist,
-                         int32_t* nout) {
+                         int32_t* nout, Tail tail) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = m.pre[m.n_hint];
+  __shared__ ChunkPre sh;
+  const int64_t total = chunk_begin(m, sh);
   for (int64_t c = warp; c < total; c += nw) {
-    const Chunk ch = chunk_of(m, c);
+    const Chunk ch = chunk_of(m, sh, c);
     if (ch.first && lane == 0) stamp_add(stamp, ep, ch.v, olist, nout);
     if (ch.row < 0) continue;
     const Adj<WT>& A = ch.row ? in : out;
@@ -57,15 +58,24 @@ __global__ void k_expand(Adj<WT> out, Adj<WT> in, ChunkMap m, int32_t* stamp, in
       warp_append(want, u, olist, nout);
     }
   }
+  pub_tail(tail);
 }
 
-__global__ void k_filter_alive(const int32_t* list, const int32_t* nlist, const uint8_t* alive, int32_t* olist,
-                               int32_t* nout) {
+// U = U* = the existing nodes of a frontier list (each listed once).
+__global__ void k_frontier(const int32_t* list, const int32_t* nlist, const uint8_t* alive, int32_t* lU, int32_t* nU,
+                           int32_t* stU, int32_t epU, int32_t* lUs, int32_t* nUs, Tail tail) {
   const int32_t nl = *nlist;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nl; t += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t v = list[t];
-    if (!alive || alive[v]) olist[atomicAdd(nout, 1)] = v;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  // warp-uniform trip counts, so that appends aggregate over the warp
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < nl; base += stride) {
+    const int64_t t = base + (threadIdx.x & 31);
+    const int32_t v = t < nl ? list[t] : 0;
+    const bool on = t < nl && (!alive || alive[v]);
+    if (on) stU[v] = epU;
+    warp_append(on, v, lU, nU);
+    warp_append(on, v, lUs, nUs);
   }
+  pub_tail(tail);
 }
 
 __global__ void k_union(const int32_t* list, const int32_t* nlist, int32_t* stamp, int32_t ep, int32_t* olist,
@@ -562,7 +572,7 @@ __global__ void k_bin(Adj<WT> out, Adj<WT> in, int directed, const int32_t* list
                       int32_t* bt, int32_t* nt, int32_t* bs, int32_t* ns, int32_t* bm, int32_t* nm, int32_t* bm2,
                       int32_t* nm2, int32_t* bc, int32_t* nc, int32_t* bl, int32_t* nlarge, int64_t* lsz,
                       int64_t* tabtop, int32_t t0, int32_t t1, int32_t t2, int32_t t3,
-                      int32_t cluster_max) {
+                      int32_t cluster_max, Tail tail) {
   const int32_t nl = *nlist;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   // warp-uniform trip count so that the appends can be warp-aggregated
@@ -590,6 +600,7 @@ __global__ void k_bin(Adj<WT> out, Adj<WT> in, int directed, const int32_t* list
       atomicAdd((unsigned long long*)tabtop, (unsigned long long)sz);
     }
   }
+  pub_tail(tail);
 }
 
 // ---------------------------------------------------------------- cluster bin
@@ -736,29 +747,36 @@ __global__ void k_hub_init(int32_t* K, int64_t* V, int64_t total) {
   }
 }
 
-__global__ void k_eval_counts(const int32_t* hcnt, int32_t nh, int64_t* ecnt) {
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i <= nh; i += gridDim.x * blockDim.x)
-    ecnt[i] = i < nh ? (hcnt[i] + EVAL_CH - 1) / EVAL_CH : 0;
+// Table offsets, evaluation chunks (at most one table slot in two is occupied)
+// and cleared slot counts of nh hubs, by one block.
+__global__ void __launch_bounds__(1024) k_hub_plan(int32_t nh, const int64_t* lsz, int64_t* loff, int64_t* epre,
+                                                   int32_t* hcnt) {
+  int64_t o = 0, e = 0;
+  for (int32_t i0 = 0; i0 < nh; i0 += 1024) {
+    const int32_t i = i0 + threadIdx.x;
+    const int64_t sz = i < nh ? lsz[i] : 0;
+    u64 ot, et;
+    const u64 ox = block_scan<1024>((u64)sz, &ot);
+    const u64 ex = block_scan<1024>((u64)((sz / 2 + EVAL_CH - 1) / EVAL_CH), &et);
+    if (i < nh) {
+      loff[i] = o + (int64_t)ox;
+      epre[i] = e + (int64_t)ex;
+      hcnt[i] = 0;
+    }
+    o += (int64_t)ot;
+    e += (int64_t)et;
+  }
+  if (threadIdx.x == 0) epre[nh] = e;
 }
 
-// listed slots back to empty (after the evaluation)
-__global__ void k_hub_clear(int32_t nh, const int64_t* loff, const int64_t* epre, const int32_t* hcnt,
-                            const int32_t* glist, int32_t* gK, int64_t* gV) {
-  const int64_t total = epre[nh];
-  for (int64_t e = blockIdx.x; e < total; e += gridDim.x) {
-    int64_t lo = 0, hi = nh;
-    while (hi - lo > 1) {
-      const int64_t mid = (lo + hi) >> 1;
-      if (epre[mid] <= e) lo = mid; else hi = mid;
-    }
-    const int64_t s0 = (e - epre[lo]) * EVAL_CH, s1 = min((int64_t)hcnt[lo], s0 + EVAL_CH);
-    const int32_t* L = glist + loff[lo] / 2;
-    for (int64_t j = s0 + threadIdx.x; j < s1; j += blockDim.x) {
-      const int64_t slot = loff[lo] + L[j];
-      gK[slot] = -1;
-      gV[slot] = 0;
-    }
+// The hub of evaluation chunk e.
+__device__ inline int64_t hub_of(const int64_t* epre, int32_t nh, int64_t e) {
+  int64_t lo = 0, hi = nh;
+  while (hi - lo > 1) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (epre[mid] <= e) lo = mid; else hi = mid;
   }
+  return lo;
 }
 
 template <class WT, int MODE>
@@ -767,10 +785,11 @@ __global__ void k_hub_acc(SweepArgs<WT> A, ChunkMap m, const int64_t* loff, cons
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = m.pre[m.n_hint];
+  __shared__ ChunkPre sh;
+  const int64_t total = chunk_begin(m, sh);
   int64_t scanned = 0;
   for (int64_t c = warp; c < total; c += nw) {
-    const Chunk ch = chunk_of(m, c);
+    const Chunk ch = chunk_of(m, sh, c);
     if (ch.row < 0) continue;
     const int32_t v = ch.v;
     const int32_t cv_ = A.lab[v];
@@ -837,18 +856,17 @@ __global__ void __launch_bounds__(TPB) k_hub_eval(SweepArgs<WT> A, const int32_t
   const int64_t mult = A.directed ? 1 : 2;
   const int64_t total = epre[nh];
   for (int64_t e = blockIdx.x; e < total; e += gridDim.x) {
-    int64_t lo = 0, hi = nh;
-    while (hi - lo > 1) {
-      const int64_t mid = (lo + hi) >> 1;
-      if (epre[mid] <= e) lo = mid; else hi = mid;
-    }
-    const int64_t i = lo;
+    const int64_t i = hub_of(epre, nh, e);
     const int32_t v = hubs[i];
     const int32_t* K = gK + loff[i];
     const int64_t* V = gV + loff[i];
     const uint32_t H = (uint32_t)lsz[i];
     const int64_t s0 = (e - epre[i]) * EVAL_CH;
     const int64_t s1 = min((int64_t)hcnt[i], s0 + EVAL_CH);
+    if (s0 >= s1) {  // fewer targets than the table could hold
+      if (threadIdx.x == 0) pb_c[e] = -1;
+      continue;
+    }
     const int32_t* Lst = glist + loff[i] / 2;
     const int32_t a = A.lab[v];
     const int64_t wa = MODE == 0 ? hash_get(K, V, H - 1, a) : 0;
@@ -885,9 +903,11 @@ __global__ void __launch_bounds__(TPB) k_hub_eval(SweepArgs<WT> A, const int32_t
   }
 }
 
+// The best of each hub's chunks, and the listed slots back to empty.
 template <class WT, int MODE>
-__global__ void k_hub_final(SweepArgs<WT> A, const int32_t* hubs, int32_t nh, const int64_t* epre,
-                            const int64_t* pb_hi, const uint64_t* pb_lo, const int32_t* pb_c) {
+__global__ void k_hub_final(SweepArgs<WT> A, const int32_t* hubs, int32_t nh, const int64_t* loff,
+                            const int64_t* epre, const int64_t* pb_hi, const uint64_t* pb_lo, const int32_t* pb_c,
+                            const int32_t* hcnt, const int32_t* glist, int32_t* gK, int64_t* gV) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -903,6 +923,17 @@ __global__ void k_hub_final(SweepArgs<WT> A, const int32_t* hubs, int32_t nh, co
       const int32_t v = hubs[i];
       atomic_add_i64(&A.stats->sw_bytes[6], sweep_bytes<WT, MODE>(A.directed, 0, 1, 0));
       if (b.have) emit_cand(A, v, MODE == 0 ? A.lab[v] : v, b);
+    }
+  }
+  const int64_t total = epre[nh];
+  for (int64_t e = blockIdx.x; e < total; e += gridDim.x) {
+    const int64_t i = hub_of(epre, nh, e);
+    const int64_t s0 = (e - epre[i]) * EVAL_CH, s1 = min((int64_t)hcnt[i], s0 + EVAL_CH);
+    const int32_t* L = glist + loff[i] / 2;
+    for (int64_t j = s0 + threadIdx.x; j < s1; j += blockDim.x) {
+      const int64_t slot = loff[i] + L[j];
+      gK[slot] = -1;
+      gV[slot] = 0;
     }
   }
 }
@@ -1022,7 +1053,7 @@ __global__ void __launch_bounds__(DEC_THREADS) k_dec_block(const int32_t* ncp, c
                                                            const int32_t* dst, const int64_t* ghi,
                                                            const uint64_t* glo, int32_t* role, int32_t* best,
                                                            int32_t* bv, int32_t* bsrc, int32_t* bdst, int32_t* nb,
-                                                           int32_t* stat) {
+                                                           int32_t* stat, Tail tail) {
   extern __shared__ unsigned char dsm[];
   int64_t* sghi = (int64_t*)dsm;
   uint64_t* sglo = (uint64_t*)(dsm + sizeof(int64_t) * DEC_SMALL);
@@ -1030,8 +1061,9 @@ __global__ void __launch_bounds__(DEC_THREADS) k_dec_block(const int32_t* ncp, c
   __shared__ int32_t left;
   const int tid = threadIdx.x;
   const int32_t nc = *ncp;
-  if (nc > DEC_SMALL) {  // left to the multi-block rounds
-    if (tid == 0) *stat = -2;
+  if (nc > DEC_SMALL || nc <= 0) {  // left to the multi-block rounds, or nothing to filter
+    if (tid == 0) *stat = nc > 0 ? -2 : 0;
+    pub_tail(tail);
     return;
   }
   // state per owned candidate: 0 undecided, 1 accepted, 2 rejected, 3 accepted
@@ -1110,37 +1142,47 @@ __global__ void __launch_bounds__(DEC_THREADS) k_dec_block(const int32_t* ncp, c
     }
   }
   if (tid == 0) *stat = ok ? rounds : -1;
+  pub_tail(tail);
 }
 
 // ---------------------------------------------------------------- commit (move)
+// Labels and marks of the accepted moves; a touched community is listed with
+// its totals as they are (they change in k_commit_e).
+__device__ inline void touch(int32_t c, int32_t* stT, int32_t epT, int32_t* lT, int32_t* nT, const int64_t* Kout,
+                             const int64_t* Kin, const int64_t* e, int64_t* sko, int64_t* ski, int64_t* se) {
+  if (!stamp_claim(stT, epT, c)) return;
+  const int32_t k = atomicAdd(nT, 1);
+  lT[k] = c;
+  sko[k] = Kout[c];
+  ski[k] = Kin[c];
+  se[k] = e[c];
+}
+
 __global__ void k_commit_mark(int32_t nb, const int32_t* bv, const int32_t* bsrc, const int32_t* bdst,
                               int32_t* lab, int32_t* oldlab, int32_t* stB, int32_t epB, int32_t* stT, int32_t epT,
                               int32_t* lT, int32_t* nT, int32_t* stCh, int32_t epCh, int32_t* lCh, int32_t* nCh,
-                              int32_t* lab_before, int level0) {
+                              int32_t* lab_before, int level0, const int64_t* Kout, const int64_t* Kin,
+                              const int64_t* e, int64_t* sko, int64_t* ski, int64_t* se) {
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) {
     const int32_t v = bv[i];
     oldlab[v] = bsrc[i];
     stB[v] = epB;
     if (level0 && stamp_add(stCh, epCh, v, lCh, nCh)) lab_before[v] = bsrc[i];
     lab[v] = bdst[i];
-    stamp_add(stT, epT, bsrc[i], lT, nT);
-    stamp_add(stT, epT, bdst[i], lT, nT);
+    touch(bsrc[i], stT, epT, lT, nT, Kout, Kin, e, sko, ski, se);
+    touch(bdst[i], stT, epT, lT, nT, Kout, Kin, e, sko, ski, se);
   }
 }
 
-__global__ void k_snap(const int32_t* lT, const int32_t* nT, const int64_t* Kout, const int64_t* Kin,
-                       const int64_t* e, int64_t* sko, int64_t* ski, int64_t* se) {
-  const int32_t n = *nT;
-  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    const int32_t c = lT[k];
-    sko[k] = Kout[c];
-    ski[k] = Kin[c];
-    se[k] = e[c];
-  }
-}
-
-__global__ void k_commit_K(int32_t nb, const int32_t* bv, const int32_t* bsrc, const int32_t* bdst,
-                           const int64_t* kout, const int64_t* kin, int64_t* Kout, int64_t* Kin, int directed) {
+// Internal-weight repair: every arc with a moved endpoint is counted once
+// (from the moved tail's out-row, or from the moved head's in-row when the
+// tail did not move).  The same launch moves the nodes' strengths between the
+// community totals.
+template <class WT>
+__global__ void k_commit_e(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* bsrc, const int32_t* bdst,
+                           const int32_t* lab, const int32_t* oldlab, const int32_t* stB, int32_t epB, int64_t* e,
+                           int32_t nb, const int32_t* bv, const int64_t* kout, const int64_t* kin, int64_t* Kout,
+                           int64_t* Kin, int directed) {
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) {
     const int32_t v = bv[i];
     atomic_add_i64(&Kout[bsrc[i]], -kout[v]);
@@ -1150,20 +1192,13 @@ __global__ void k_commit_K(int32_t nb, const int32_t* bv, const int32_t* bsrc, c
       atomic_add_i64(&Kin[bdst[i]], kin[v]);
     }
   }
-}
-
-// Internal-weight repair: every arc with a moved endpoint is counted once
-// (from the moved tail's out-row, or from the moved head's in-row when the
-// tail did not move).
-template <class WT>
-__global__ void k_commit_e(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* bsrc, const int32_t* bdst,
-                           const int32_t* lab, const int32_t* oldlab, const int32_t* stB, int32_t epB, int64_t* e) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = m.pre[m.n_hint];
+  __shared__ ChunkPre sh;
+  const int64_t total = chunk_begin(m, sh);
   for (int64_t c = warp; c < total; c += nw) {
-    const Chunk ch = chunk_of(m, c);
+    const Chunk ch = chunk_of(m, sh, c);
     if (ch.row < 0) continue;
     const int32_t a = bsrc[ch.idx], b = bdst[ch.idx];
     int64_t da = 0, db = 0;
@@ -1201,7 +1236,7 @@ __global__ void k_commit_e(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* b
 // dQ(B) = sum over touched communities of gd*m*de_C - gn*d(K_out K_in).
 __global__ void k_commit_dq(const int32_t* lT, const int32_t* nT, const int64_t* Kout, const int64_t* Kin,
                             const int64_t* e, const int64_t* sko, const int64_t* ski, const int64_t* se, int64_t m,
-                            int64_t gn, int64_t gd, DevScalars* sc) {
+                            int64_t gn, int64_t gd, CommitAcc* sc) {
   const int32_t n = *nT;
   i128 dq = 0, dp = 0;
   int64_t de = 0;
@@ -1236,11 +1271,20 @@ __global__ void k_rollback(int32_t nb, const int32_t* bv, const int32_t* bsrc, i
   }
 }
 
+// After a mini-batch that stays: its nodes are moved nodes of the level (and
+// of the pass, on level 0), and the next U joins U*.
 __global__ void k_mark_moved(int32_t nb, const int32_t* bv, int32_t* stMv, int32_t epMv, int32_t* lMv, int32_t* nMv,
-                             int32_t* stM0, int32_t epM0, int32_t* lM0, int32_t* nM0) {
+                             int32_t* stM0, int32_t epM0, int32_t* lM0, int32_t* nM0, int32_t nU, const int32_t* lU,
+                             int32_t* stU, int32_t epU, int32_t* lUs, int32_t* nUs) {
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) {
     stamp_add(stMv, epMv, bv[i], lMv, nMv);
     if (stM0) stamp_add(stM0, epM0, bv[i], lM0, nM0);
+  }
+  const int32_t stride = gridDim.x * blockDim.x;
+  for (int32_t base = blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < nU; base += stride) {
+    const int32_t t = base + (threadIdx.x & 31);
+    const int32_t v = t < nU ? lU[t] : 0;
+    warp_append(t < nU && stamp_claim(stU, epU, v), v, lUs, nUs);
   }
 }
 
@@ -1270,9 +1314,10 @@ __global__ void k_spexpand(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* l
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = m.pre[m.n_hint];
+  __shared__ ChunkPre sh;
+  const int64_t total = chunk_begin(m, sh);
   for (int64_t c = warp; c < total; c += nw) {
-    const Chunk ch = chunk_of(m, c);
+    const Chunk ch = chunk_of(m, sh, c);
     if (ch.row < 0) continue;
     const Adj<WT>& A = ch.row ? in : out;
     const int64_t o = A.off[ch.v];
@@ -1293,33 +1338,39 @@ __global__ void k_spexpand(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* l
 }  // namespace
 
 // ================================================================== host side
-static int chunk_grid(int64_t n_hint) { return grid_for(n_hint * 64, TPB, 16); }
 
-void expand_set(ldl_ctx& c, int r, const int32_t* list, int idx_n, int32_t* stamp, int32_t ep, int32_t* olist,
-                int idx_out, int64_t n_hint) {
-  if (n_hint <= 0) return;
+static void expand_tail(ldl_ctx& c, int r, const int32_t* list, int idx_n, int32_t* stamp, int32_t ep, int32_t* olist,
+                        int idx_out, int64_t n_hint, const Tail& tail) {
   const int g = chunk_grid(n_hint);
   if (r == 0) {
     Adj<int32_t> o = adj_out0(c), i = adj_in0(c);
-    ChunkMap m = chunk_map(c, list, c.dcnt + idx_n, n_hint, o.len, c.directed ? i.len : nullptr);
-    k_expand<int32_t><<<g, TPB, 0, c.s>>>(o, i, m, stamp, ep, olist, c.dcnt + idx_out);
+    ChunkMap m = chunk_map(c, list, c.cp[idx_n], n_hint, o.len, c.directed ? i.len : nullptr);
+    k_expand<int32_t><<<g, TPB, 0, c.s>>>(o, i, m, stamp, ep, olist, c.cp[idx_out], tail);
   } else {
     Adj<int64_t> o = adj_out(c, r), i = adj_in(c, r);
-    ChunkMap m = chunk_map(c, list, c.dcnt + idx_n, n_hint, o.len, c.directed ? i.len : nullptr);
-    k_expand<int64_t><<<g, TPB, 0, c.s>>>(o, i, m, stamp, ep, olist, c.dcnt + idx_out);
+    ChunkMap m = chunk_map(c, list, c.cp[idx_n], n_hint, o.len, c.directed ? i.len : nullptr);
+    k_expand<int64_t><<<g, TPB, 0, c.s>>>(o, i, m, stamp, ep, olist, c.cp[idx_out], tail);
   }
   CKL("k_expand");
 }
 
-void filter_alive(ldl_ctx& c, int r, const int32_t* list, int idx_n, int32_t* olist, int idx_out, int64_t n_hint) {
-  k_filter_alive<<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(list, c.dcnt + idx_n, r ? c.lv[r].alive.p : nullptr, olist,
-                                                         c.dcnt + idx_out);
-  CKL("k_filter_alive");
+void expand_set(ldl_ctx& c, int r, const int32_t* list, int idx_n, int32_t* stamp, int32_t ep, int32_t* olist,
+                int idx_out, int64_t n_hint) {
+  if (n_hint <= 0) return;
+  expand_tail(c, r, list, idx_n, stamp, ep, olist, idx_out, n_hint, Tail{});
+}
+
+void frontier(ldl_ctx& c, int r, int32_t epU, const HostRead* rr, int n) {
+  LevelState& L = c.lv[r];
+  k_frontier<<<grid_for(c.n, TPB, 2), TPB, 0, c.s>>>(L.lA.p, c.cp[K_A0 + r], r ? L.alive.p : nullptr, c.lU.p, c.cp[K_U],
+                                                     c.stU.p, epU, c.lUstar.p, c.cp[K_USTAR], tail_begin(c, rr, n));
+  CKL("k_frontier");
+  tail_wait(c, rr, n);
 }
 
 void union_into(ldl_ctx& c, const int32_t* list, int idx_n, int32_t* stamp, int32_t ep, int32_t* olist, int idx_out,
                 int64_t n_hint) {
-  k_union<<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(list, c.dcnt + idx_n, stamp, ep, olist, c.dcnt + idx_out);
+  k_union<<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(list, c.cp[idx_n], stamp, ep, olist, c.cp[idx_out]);
   CKL("k_union");
 }
 
@@ -1336,15 +1387,15 @@ static bool sweep_gain_fits_i64(const ldl_ctx& c) {
 // The bins of nodes with at most 2048 entries, in the gain type GT.
 template <class WT, int MODE, class GT>
 static void sweep_bins(ldl_ctx& c, const SweepArgs<WT>& A, int64_t n_hint, cudaEvent_t* kev) {
-  k_sweep_group<WT, MODE, 8, GT><<<grid_for(n_hint * 8, TPB, 6), TPB, 0, c.s>>>(A, c.binT.p, c.dcnt + K_TINY);
+  k_sweep_group<WT, MODE, 8, GT><<<grid_for(n_hint * 8, TPB, 6), TPB, 0, c.s>>>(A, c.binT.p, c.cp[K_TINY]);
   CKL("k_sweep_group<8>");
   if (kev) CK(cudaEventRecord(kev[1], c.s));
-  k_sweep_group<WT, MODE, 32, GT><<<grid_for(n_hint * 32, TPB, 6), TPB, 0, c.s>>>(A, c.binS.p, c.dcnt + K_SMALL);
+  k_sweep_group<WT, MODE, 32, GT><<<grid_for(n_hint * 32, TPB, 6), TPB, 0, c.s>>>(A, c.binS.p, c.cp[K_SMALL]);
   CKL("k_sweep_group<32>");
   if (kev) CK(cudaEventRecord(kev[2], c.s));
   {
     const size_t sm = (size_t)tab_slot<GT> * 2048;
-    k_sweep_block<WT, MODE, 128, 2048, GT><<<grid_for(n_hint, 1, 16), 128, sm, c.s>>>(A, c.binM.p, c.dcnt + K_MID);
+    k_sweep_block<WT, MODE, 128, 2048, GT><<<grid_for(n_hint, 1, 16), 128, sm, c.s>>>(A, c.binM.p, c.cp[K_MID]);
     CKL("k_sweep_block(mid1)");
   }
   if (kev) CK(cudaEventRecord(kev[3], c.s));
@@ -1352,7 +1403,7 @@ static void sweep_bins(ldl_ctx& c, const SweepArgs<WT>& A, int64_t n_hint, cudaE
     const size_t sm = (size_t)tab_slot<GT> * HB;
     CK(cudaFuncSetAttribute(k_sweep_block<WT, MODE, 256, HB, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)sm));
-    k_sweep_block<WT, MODE, 256, HB, GT><<<grid_for(n_hint, 1, 4), 256, sm, c.s>>>(A, c.binM2.p, c.dcnt + K_MID2);
+    k_sweep_block<WT, MODE, 256, HB, GT><<<grid_for(n_hint, 1, 4), 256, sm, c.s>>>(A, c.binM2.p, c.cp[K_MID2]);
     CKL("k_sweep_block(mid2)");
   }
 }
@@ -1369,8 +1420,11 @@ static cudaEvent_t* kstats_events(ldl_ctx& c) {
 }
 
 template <class WT, int MODE>
-static int32_t sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_t* list, int idx_n,
-                       int64_t n_hint) {
+static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_t* list, int idx_n,
+                        int64_t n_hint) {
+  if (MODE == 0) stage_begin(c);  // refinement is timed as a whole
+  for (int k : {K_CAND, K_TINY, K_SMALL, K_MID, K_MID2, K_CLU, K_LARGE}) zero_cnt(c, k);
+  c.sums = (int64_t*)fresh(c, 2, c.d_sc->sums);
   LevelState& L = c.lv[r];
   SweepArgs<WT> A;
   A.out = out;
@@ -1395,23 +1449,29 @@ static int32_t sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_t
   A.cdst = c.cdst.p;
   A.cghi = c.cghi.p;
   A.cglo = c.cglo.p;
-  A.ncand = c.dcnt + K_CAND;
+  A.ncand = c.cp[K_CAND];
   A.scanned = &c.d_sc->scanned;
   A.stats = c.d_sc;
-  {
-    ZeroSpans z;
-    z.mask = cnt_bit(K_CAND) | cnt_bit(K_TINY) | cnt_bit(K_SMALL) | cnt_bit(K_MID) | cnt_bit(K_MID2) |
-             cnt_bit(K_CLU) | cnt_bit(K_LARGE);
-    z.p[0] = &c.d_sc->need;
-    z.nw[0] = 1;
-    zero_many(c, z);
-  }
-  k_bin<WT><<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(out, in, c.directed, list, c.dcnt + idx_n, c.binT.p,
-                                                     c.dcnt + K_TINY, c.binS.p, c.dcnt + K_SMALL, c.binM.p,
-                                                     c.dcnt + K_MID, c.binM2.p, c.dcnt + K_MID2, c.binC.p,
-                                                     c.dcnt + K_CLU, c.binL.p, c.dcnt + K_LARGE, c.binLsz.p,
-                                                     &c.d_sc->need, c.bin_deg[0], c.bin_deg[1], c.bin_deg[2],
-                                                     c.bin_deg[3], std::min(c.prm.cluster_max_deg, CLUSTER_DEG));
+  // the bins' sizes, the hub tables' size and the list's length in one read
+  int32_t ct = 0, cs = 0, cm = 0, cm2 = 0, cc = 0, ch = 0, nlist = 0;
+  int64_t tab = 0;
+  const HostRead rb[8] = {{c.cp[K_TINY], &ct, sizeof(int32_t)},  {c.cp[K_SMALL], &cs, sizeof(int32_t)},
+                          {c.cp[K_MID], &cm, sizeof(int32_t)},   {c.cp[K_MID2], &cm2, sizeof(int32_t)},
+                          {c.cp[K_CLU], &cc, sizeof(int32_t)},   {c.cp[K_LARGE], &ch, sizeof(int32_t)},
+                          {c.cp[idx_n], &nlist, sizeof(int32_t)}, {c.sums, &tab, sizeof(int64_t)}};
+  // Hub rows need their tables' size on the host before they are swept.  Where
+  // the last sweep of this level and mode had none, the filter is launched
+  // straight behind the sweeps and one read returns its outcome and the hub
+  // count; should there be hubs after all, they are swept and the filter,
+  // which leaves its scratch as it found it, runs again on all candidates.
+  uint8_t& expect = c.hubs_seen[r][MODE];
+  const bool early = expect || c.kstats;
+  k_bin<WT><<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(out, in, c.directed, list, c.cp[idx_n], c.binT.p, c.cp[K_TINY],
+                                                     c.binS.p, c.cp[K_SMALL], c.binM.p, c.cp[K_MID], c.binM2.p,
+                                                     c.cp[K_MID2], c.binC.p, c.cp[K_CLU], c.binL.p, c.cp[K_LARGE],
+                                                     c.binLsz.p, c.sums, c.bin_deg[0], c.bin_deg[1], c.bin_deg[2],
+                                                     c.bin_deg[3], std::min(c.prm.cluster_max_deg, CLUSTER_DEG),
+                                                     early ? tail_begin(c, rb, 8) : Tail{});
   CKL("k_bin");
   // Every bin but the hubs is swept by a grid-stride kernel that reads its
   // bin's count on the device, so these launch before the counts come back
@@ -1425,21 +1485,16 @@ static int32_t sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_t
     const size_t sm = (sizeof(int64_t) + sizeof(int32_t)) * CL_SLOTS;
     CK(cudaFuncSetAttribute(k_sweep_cluster<WT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     const int ncl = (int)std::min<int64_t>(n_hint, std::max(1, device_sms() * 2 / CL));
-    k_sweep_cluster<WT, MODE><<<ncl * CL, TPB, sm, c.s>>>(A, c.binC.p, c.dcnt + K_CLU);
+    k_sweep_cluster<WT, MODE><<<ncl * CL, TPB, sm, c.s>>>(A, c.binC.p, c.cp[K_CLU]);
     CKL("k_sweep_cluster");
   }
   if (kev) CK(cudaEventRecord(kev[5], c.s));
-  // counters K_SMALL .. K_CLU, the hub tables' size and the list's length in one read
-  int32_t cn[K_CLU - K_SMALL + 1];
-  int64_t tab = 0;
-  int32_t nlist = 0;
-  {
-    const HostRead rr[3] = {{c.dcnt + K_SMALL, cn, (int32_t)sizeof(cn)}, {&c.d_sc->need, &tab, sizeof(int64_t)},
-                            {c.dcnt + idx_n, &nlist, sizeof(int32_t)}};
-    host_read(c, rr, 3);
+  DecoupleOut dd{};
+  if (early) tail_wait(c, rb, 8);
+  else {
+    const HostRead ro[3] = {rb[5], rb[6], rb[7]};
+    dd = decouple(c, ro, 3);
   }
-  const int32_t ct = cn[K_TINY - K_SMALL], cs = cn[0], cm = cn[K_MID - K_SMALL], cm2 = cn[K_MID2 - K_SMALL];
-  const int32_t cc = cn[K_CLU - K_SMALL], ch = cn[K_LARGE - K_SMALL];
   if (kev) CK(cudaEventRecord(kev[6], c.s));  // the wait above is charged to no kernel
   if (ch > 0) {
     // Hub tables hold 2..4 slots per entry.  When all hubs' tables together
@@ -1476,9 +1531,6 @@ static int32_t sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_t
     }
     c.glist.reserve(tab_use / 2 + 1, c.s);
     c.hcnt.reserve(ch + 1, c.s);
-    // table sizes end with a zero so that each group's offset scan has a total
-    CK(cudaMemsetAsync(c.binLsz.p + ch, 0, sizeof(int64_t), c.s));
-    c.hub_ecnt.reserve(ch + 2, c.s);
     c.hub_epre.reserve(ch + 2, c.s);
     const int64_t ech = tab_use / 2 / EVAL_CH + ch + 1;  // bounds the evaluation chunks of any group
     c.pb_hi.reserve(ech, c.s);
@@ -1490,32 +1542,26 @@ static int32_t sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_t
       const int32_t* L = c.binL.p + g0;
       int64_t* Lsz = c.binLsz.p + g0;
       int64_t* Loff = c.binLoff.p + g0;
-      const int32_t* cntp = c.dcnt + K_LARGE;
+      const int32_t* cntp = c.cp[K_LARGE];
       if (gb.size() > 2) {
         set_cnt(c, K_HUBG, nh);
-        cntp = c.dcnt + K_HUBG;
+        cntp = c.cp[K_HUBG];
       }
-      CK(cudaMemsetAsync(c.hcnt.p, 0, sizeof(int32_t) * (size_t)(nh + 1), c.s));
-      // table offsets per hub of the group, in list order
-      scan_exclusive(Lsz, Loff, nh + 1, c.P, c.s, false);
+      // table offsets and evaluation chunks per hub of the group, in list order
+      k_hub_plan<<<1, 1024, 0, c.s>>>(nh, Lsz, Loff, c.hub_epre.p, c.hcnt.p);
+      CKL("k_hub_plan");
       ChunkMap m = chunk_map(c, L, cntp, nh, out.len, c.directed ? in.len : nullptr);
       k_hub_acc<WT, MODE><<<grid_for((int64_t)nh * 2048, TPB, 16), TPB, 0, c.s>>>(
           A, m, Loff, Lsz, c.gkeys.p, c.gvals.p, c.glist.p, c.hcnt.p);
       CKL("k_hub_acc");
       if (kev && gi + 2 == gb.size()) CK(cudaEventRecord(kev[8], c.s));
-      // evaluation chunks per hub from its occupied-slot count (device only)
-      k_eval_counts<<<grid_for(nh + 1, TPB), TPB, 0, c.s>>>(c.hcnt.p, nh, c.hub_ecnt.p);
-      CKL("k_eval_counts");
-      scan_exclusive(c.hub_ecnt.p, c.hub_epre.p, nh + 1, c.P, c.s, false);
       const int ge = grid_for(ech, 1, 8);
       k_hub_eval<WT, MODE><<<ge, TPB, 0, c.s>>>(A, L, nh, Loff, Lsz, c.hub_epre.p, c.gkeys.p, c.gvals.p, c.glist.p,
                                                 c.hcnt.p, c.pb_hi.p, c.pb_lo.p, c.pb_c.p);
       CKL("k_hub_eval");
-      k_hub_final<WT, MODE><<<grid_for((int64_t)nh * 32, TPB), TPB, 0, c.s>>>(A, L, nh, c.hub_epre.p, c.pb_hi.p,
-                                                                             c.pb_lo.p, c.pb_c.p);
+      k_hub_final<WT, MODE><<<std::max(ge, grid_for((int64_t)nh * 32, TPB)), TPB, 0, c.s>>>(
+          A, L, nh, Loff, c.hub_epre.p, c.pb_hi.p, c.pb_lo.p, c.pb_c.p, c.hcnt.p, c.glist.p, c.gkeys.p, c.gvals.p);
       CKL("k_hub_final");
-      k_hub_clear<<<ge, TPB, 0, c.s>>>(nh, Loff, c.hub_epre.p, c.hcnt.p, c.glist.p, c.gkeys.p, c.gvals.p);
-      CKL("k_hub_clear");
     }
   } else if (kev) {
     CK(cudaEventRecord(kev[7], c.s));
@@ -1531,16 +1577,24 @@ static int32_t sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_t
     c.ks_launch[3] += cm2 > 0;
     c.ks_launch[4] += cc > 0;
     c.ks_launch[5] += ch > 0;
-    c.ks_launch[6] += ch > 0 ? 3 : 0;  // evaluation, final reduction, clearing
+    c.ks_launch[6] += ch > 0 ? 2 : 0;  // evaluation, final reduction with the clearing
   }
-  return nlist;
+  if (MODE == 0) stage_end(c, ST_BEST);
+  expect = ch > 0;
+  if (early || ch > 0) {
+    if (MODE == 0) stage_begin(c);
+    dd = decouple(c);
+    if (MODE == 0) stage_end(c, ST_DECOUPLE);
+  }
+  c.res.decouple_rounds += dd.rounds;
+  return {nlist, dd.nc, dd.nb};
 }
 
 extern "C" void ldl_debug_hub_table_slots(int64_t slots) {
   g_hub_table_slots.store(slots > 0 ? slots : HUB_TABLE_SLOTS);
 }
 
-int32_t sweep(ldl_ctx& c, int r, int mode, const int32_t* list, int idx_n, int64_t n_hint) {
+SweepOut sweep(ldl_ctx& c, int r, int mode, const int32_t* list, int idx_n, int64_t n_hint) {
   if (r == 0) {
     if (mode == 0) return sweep_t<int32_t, 0>(c, r, adj_out0(c), adj_in0(c), list, idx_n, n_hint);
     return sweep_t<int32_t, 1>(c, r, adj_out0(c), adj_in0(c), list, idx_n, n_hint);
@@ -1549,29 +1603,25 @@ int32_t sweep(ldl_ctx& c, int r, int mode, const int32_t* list, int idx_n, int64
   return sweep_t<int64_t, 1>(c, r, adj_out(c, r), adj_in(c, r), list, idx_n, n_hint);
 }
 
-DecoupleOut decouple(ldl_ctx& c, int extra) {
+DecoupleOut decouple(ldl_ctx& c, const HostRead* extra, int n_extra) {
   // The single-block filter runs first and reads the candidate count on the
   // device; one read then returns the count, the accepted number and the
   // filter's status (-2: too many candidates for one block).
-  static_assert(K_B == K_CAND + 1 && K_UNDEC == K_CAND + 2, "adjacent counters");
   zero_cnt(c, K_B);
+  int32_t nc = 0, nb = 0, stat = 0;
+  HostRead rr[TAIL_MAX] = {{c.cp[K_CAND], &nc, sizeof(int32_t)}, {c.cp[K_B], &nb, sizeof(int32_t)},
+                           {c.cp[K_UNDEC], &stat, sizeof(int32_t)}};
+  for (int i = 0; i < n_extra; ++i) rr[3 + i] = extra[i];
   CK(cudaFuncSetAttribute(k_dec_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DEC_SMEM));
-  k_dec_block<<<1, DEC_THREADS, DEC_SMEM, c.s>>>(c.dcnt + K_CAND, c.cv.p, c.csrc.p, c.cdst.p, c.cghi.p, c.cglo.p,
-                                                 c.role.p, c.best.p, c.bv.p, c.bsrc.p, c.bdst.p, c.dcnt + K_B,
-                                                 c.dcnt + K_UNDEC);
+  k_dec_block<<<1, DEC_THREADS, DEC_SMEM, c.s>>>(c.cp[K_CAND], c.cv.p, c.csrc.p, c.cdst.p, c.cghi.p, c.cglo.p,
+                                                 c.role.p, c.best.p, c.bv.p, c.bsrc.p, c.bdst.p, c.cp[K_B],
+                                                 c.cp[K_UNDEC], tail_begin(c, rr, 3 + n_extra));
   CKL("k_dec_block");
-  int32_t out[3], ex = 0;
-  {
-    const HostRead rr[2] = {{c.dcnt + K_CAND, out, (int32_t)sizeof(out)},
-                            {c.dcnt + (extra >= 0 ? extra : K_CAND), &ex, sizeof(int32_t)}};
-    host_read(c, rr, extra >= 0 ? 2 : 1);
-  }
-  const int32_t nc = out[0];
-  if (nc <= 0) return {0, 0, ex};
-  if (out[2] != -2) {
-    if (out[2] < 0) ldl_throw(LDL_E_INVALID, "internal: decoupling did not converge");
-    c.res.decouple_rounds += out[2];
-    return {nc, out[1], ex};
+  tail_wait(c, rr, 3 + n_extra);
+  if (nc <= 0) return {0, 0, 0};
+  if (stat != -2) {
+    if (stat < 0) ldl_throw(LDL_E_INVALID, "internal: decoupling did not converge");
+    return {nc, nb, stat};
   }
   // many candidates: one cooperative launch of co-resident blocks runs all rounds
   int per_sm = 0;
@@ -1579,92 +1629,76 @@ DecoupleOut decouple(ldl_ctx& c, int extra) {
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dec_grid, TPB, 0));
   const int g = std::max(1, std::min(grid_for(nc, TPB), sms * per_sm));
   zero_cnt(c, K_B);
-  static_assert(K_TMP2 == K_TMP + 1, "adjacent counters");
   int32_t ncv = nc;
   int32_t* cst = c.cst.p;
   const int32_t *cvp = c.cv.p, *srcp = c.csrc.p, *dstp = c.cdst.p;
   const int64_t* ghi = c.cghi.p;
   const uint64_t* glo = c.cglo.p;
   int32_t *role = c.role.p, *best = c.best.p, *bv = c.bv.p, *bsrc = c.bsrc.p, *bdst = c.bdst.p;
-  int32_t* nbp = c.dcnt + K_B;
-  int32_t* undec = c.dcnt + K_TMP;  // K_TMP, K_TMP2: the two round counters
-  int32_t* stat = c.dcnt + K_UNDEC;
-  void* args[] = {&ncv, &cst, &cvp, &srcp, &dstp, &ghi, &glo, &role, &best, &bv, &bsrc, &bdst, &nbp, &undec, &stat};
+  int32_t* nbp = c.cp[K_B];
+  int32_t* undec = (int32_t*)fresh(c, 2, c.d_sc->home);  // the two round counters
+  int32_t* statp = c.cp[K_UNDEC];
+  void* args[] = {&ncv, &cst, &cvp, &srcp, &dstp, &ghi, &glo, &role, &best, &bv, &bsrc, &bdst, &nbp, &undec, &statp};
   CK(cudaLaunchCooperativeKernel((const void*)k_dec_grid, dim3(g), dim3(TPB), args, 0, c.s));
   CKL("k_dec_grid");
-  int32_t fin[2];  // K_B, K_UNDEC
-  const HostRead rr{c.dcnt + K_B, fin, sizeof(fin)};
-  host_read(c, &rr, 1);
-  if (fin[1] < 0) ldl_throw(LDL_E_INVALID, "internal: decoupling did not converge");
-  c.res.decouple_rounds += fin[1];
-  return {nc, fin[0], ex};
+  const HostRead rf[2] = {{c.cp[K_B], &nb, sizeof(int32_t)}, {c.cp[K_UNDEC], &stat, sizeof(int32_t)}};
+  host_read(c, rf, 2);
+  if (stat < 0) ldl_throw(LDL_E_INVALID, "internal: decoupling did not converge");
+  return {nc, nb, stat};
 }
-
 
 void commit_move(ldl_ctx& c, int r, int32_t nb, int32_t epB, int32_t epT, int32_t epCh) {
   LevelState& L = c.lv[r];
   const int g = grid_for(nb, TPB);
-  {
-    // K_T, and the mini-batch's ΔQ numerator, Δ sum K_out K_in and Δ sum e_C
-    static_assert(offsetof(DevScalars, dp) == offsetof(DevScalars, dq) + sizeof(I128), "adjacent scalars");
-    ZeroSpans z;
-    z.mask = cnt_bit(K_T);
-    z.p[0] = (int64_t*)&c.d_sc->dq;
-    z.nw[0] = (int32_t)(2 * sizeof(I128) / sizeof(int64_t));
-    z.p[1] = &c.d_sc->de;
-    z.nw[1] = 1;
-    zero_many(c, z);
-  }
+  zero_cnt(c, K_T);
+  c.acc = (CommitAcc*)fresh(c, sizeof(CommitAcc) / 4, c.d_sc->home);
   k_commit_mark<<<g, TPB, 0, c.s>>>(nb, c.bv.p, c.bsrc.p, c.bdst.p, L.lab.p, c.oldlab.p, c.stB.p, epB, c.stT.p, epT,
-                                    c.lT.p, c.dcnt + K_T, c.stCh.p, epCh, c.lCh.p, c.dcnt + K_CH, c.lab_before.p,
-                                    r == 0);
+                                    c.lT.p, c.cp[K_T], c.stCh.p, epCh, c.lCh.p, c.cp[K_CH], c.lab_before.p, r == 0,
+                                    c.Kout.p, Kin_of(c), c.e.p, c.snapKo.p, c.snapKi.p, c.snapE.p);
   CKL("k_commit_mark");
-  k_snap<<<grid_for(2 * (int64_t)nb, TPB), TPB, 0, c.s>>>(c.lT.p, c.dcnt + K_T, c.Kout.p, Kin_of(c), c.e.p,
-                                                          c.snapKo.p, c.snapKi.p, c.snapE.p);
-  CKL("k_snap");
-  k_commit_K<<<g, TPB, 0, c.s>>>(nb, c.bv.p, c.bsrc.p, c.bdst.p, L.kout.p, kin_of(c, r), c.Kout.p, Kin_of(c),
-                                 c.directed);
-  CKL("k_commit_K");
   const int gw = chunk_grid(nb);
   if (r == 0) {
     Adj<int32_t> o = adj_out0(c), i = adj_in0(c);
-    ChunkMap m = chunk_map(c, c.bv.p, c.dcnt + K_B, nb, o.len, i.len);
-    k_commit_e<int32_t><<<gw, TPB, 0, c.s>>>(o, i, m, c.bsrc.p, c.bdst.p, L.lab.p, c.oldlab.p, c.stB.p, epB, c.e.p);
+    ChunkMap m = chunk_map(c, c.bv.p, c.cp[K_B], nb, o.len, i.len);
+    k_commit_e<int32_t><<<gw, TPB, 0, c.s>>>(o, i, m, c.bsrc.p, c.bdst.p, L.lab.p, c.oldlab.p, c.stB.p, epB, c.e.p, nb,
+                                          c.bv.p, L.kout.p, kin_of(c, r), c.Kout.p, Kin_of(c), c.directed);
   } else {
     Adj<int64_t> o = adj_out(c, r), i = adj_in(c, r);
-    ChunkMap m = chunk_map(c, c.bv.p, c.dcnt + K_B, nb, o.len, i.len);
-    k_commit_e<int64_t><<<gw, TPB, 0, c.s>>>(o, i, m, c.bsrc.p, c.bdst.p, L.lab.p, c.oldlab.p, c.stB.p, epB, c.e.p);
+    ChunkMap m = chunk_map(c, c.bv.p, c.cp[K_B], nb, o.len, i.len);
+    k_commit_e<int64_t><<<gw, TPB, 0, c.s>>>(o, i, m, c.bsrc.p, c.bdst.p, L.lab.p, c.oldlab.p, c.stB.p, epB, c.e.p, nb,
+                                          c.bv.p, L.kout.p, kin_of(c, r), c.Kout.p, Kin_of(c), c.directed);
   }
   CKL("k_commit_e");
-  k_commit_dq<<<grid_for(2 * (int64_t)nb, TPB), TPB, 0, c.s>>>(c.lT.p, c.dcnt + K_T, c.Kout.p, Kin_of(c), c.e.p,
+  k_commit_dq<<<grid_for(2 * (int64_t)nb, TPB), TPB, 0, c.s>>>(c.lT.p, c.cp[K_T], c.Kout.p, Kin_of(c), c.e.p,
                                                                c.snapKo.p, c.snapKi.p, c.snapE.p, c.m,
-                                                               c.prm.gamma_num, c.prm.gamma_den, c.d_sc);
+                                                               c.prm.gamma_num, c.prm.gamma_den, c.acc);
   CKL("k_commit_dq");
 }
 
-CommitOut commit_read(ldl_ctx& c, int extra_idx, int32_t* extra) {
+CommitOut commit_expand(ldl_ctx& c, int r, int32_t nb, int32_t ep, int32_t* nU) {
   CommitOut o;
-  I128 dq, dp;
-  const HostRead rr[5] = {{&c.d_sc->dq, &dq, sizeof(I128)}, {&c.d_sc->dp, &dp, sizeof(I128)},
-                          {&c.d_sc->de, &o.de, sizeof(int64_t)}, {c.dcnt + K_T, &o.ntc, sizeof(int32_t)},
-                          {c.dcnt + (extra ? extra_idx : K_T), extra, sizeof(int32_t)}};
-  host_read(c, rr, extra ? 5 : 4);
-  o.dq = i128_of(dq.hi, dq.lo);
-  o.dp = i128_of(dp.hi, dp.lo);
+  CommitAcc a{};
+  const HostRead rr[3] = {{c.acc, &a, sizeof(a)}, {c.cp[K_T], &o.ntc, sizeof(int32_t)}, {c.cp[K_U], nU, sizeof(int32_t)}};
+  expand_tail(c, r, c.bv.p, K_B, c.stS.p, ep, c.lU.p, K_U, nb, tail_begin(c, rr, 3));
+  tail_wait(c, rr, 3);
+  o.dq = i128_of(a.dq.hi, a.dq.lo);
+  o.dp = i128_of(a.dp.hi, a.dp.lo);
+  o.de = a.de;
   return o;
 }
 
 void rollback_move(ldl_ctx& c, int r, int32_t nb, int32_t ntc) {
   LevelState& L = c.lv[r];
   const int64_t m = nb > ntc ? nb : ntc;
-  k_rollback<<<grid_for(m, TPB), TPB, 0, c.s>>>(nb, c.bv.p, c.bsrc.p, L.lab.p, c.lT.p, c.dcnt + K_T, c.Kout.p,
+  k_rollback<<<grid_for(m, TPB), TPB, 0, c.s>>>(nb, c.bv.p, c.bsrc.p, L.lab.p, c.lT.p, c.cp[K_T], c.Kout.p,
                                                 Kin_of(c), c.e.p, c.snapKo.p, c.snapKi.p, c.snapE.p, c.directed);
   CKL("k_rollback");
 }
 
-void mark_moved(ldl_ctx& c, int r, int32_t nb, int32_t epMv, int32_t epM0) {
-  k_mark_moved<<<grid_for(nb, TPB), TPB, 0, c.s>>>(nb, c.bv.p, c.stMv.p, epMv, c.lMv.p, c.dcnt + K_MV,
-                                                   r == 0 ? c.stM0.p : nullptr, epM0, c.lM0.p, c.dcnt + K_M0);
+void mark_moved(ldl_ctx& c, int r, int32_t nb, int32_t epMv, int32_t epM0, int32_t epU, int32_t nU) {
+  k_mark_moved<<<grid_for(std::max(nb, nU), TPB), TPB, 0, c.s>>>(
+      nb, c.bv.p, c.stMv.p, epMv, c.lMv.p, c.cp[K_MV], r == 0 ? c.stM0.p : nullptr, epM0, c.lM0.p, c.cp[K_M0], nU,
+      c.lU.p, c.stU.p, epU, c.lUstar.p, c.cp[K_USTAR]);
   CKL("k_mark_moved");
 }
 
@@ -1681,14 +1715,14 @@ void spexpand(ldl_ctx& c, int r, int32_t nb, int32_t epD, int32_t epR, int32_t* 
   const int g = chunk_grid(nb);
   if (r == 0) {
     Adj<int32_t> o = adj_out0(c), i = adj_in0(c);
-    ChunkMap m = chunk_map(c, c.bv.p, c.dcnt + K_B, nb, o.len, c.directed ? i.len : nullptr);
+    ChunkMap m = chunk_map(c, c.bv.p, c.cp[K_B], nb, o.len, c.directed ? i.len : nullptr);
     k_spexpand<int32_t><<<g, TPB, 0, c.s>>>(o, i, m, L.lab.p, L.par.p, c.lv[r + 1].cnt.p, c.stD.p, epD, c.stR.p,
-                                            epR, lR, c.dcnt + idx_R);
+                                            epR, lR, c.cp[idx_R]);
   } else {
     Adj<int64_t> o = adj_out(c, r), i = adj_in(c, r);
-    ChunkMap m = chunk_map(c, c.bv.p, c.dcnt + K_B, nb, o.len, c.directed ? i.len : nullptr);
+    ChunkMap m = chunk_map(c, c.bv.p, c.cp[K_B], nb, o.len, c.directed ? i.len : nullptr);
     k_spexpand<int64_t><<<g, TPB, 0, c.s>>>(o, i, m, L.lab.p, L.par.p, c.lv[r + 1].cnt.p, c.stD.p, epD, c.stR.p,
-                                            epR, lR, c.dcnt + idx_R);
+                                            epR, lR, c.cp[idx_R]);
   }
   CKL("k_spexpand");
 }
