@@ -123,6 +123,7 @@ struct ldl_ctx {
   int64_t gtab_clean = 0;  // capacity of gkeys / gvals known to be clean
   DBuf<int32_t> glist;   // per hub: the table slots its sweep occupied
   DBuf<int32_t> hcnt;    // per hub: number of occupied slots
+  DBuf<int64_t> hown;    // per hub: weight towards its own community
   // records
   DBuf<u64> rk, rv, tk, tv, rk2, rv2;
   DBuf<int64_t> rsum, rsum2;

@@ -90,48 +90,66 @@ __global__ void __launch_bounds__(UQ_TPB) k_unique(const u64* keys, int64_t n, u
 __global__ void k_seq(const ldl_update* u, int64_t cnt, const u64* vals, const int64_t* ustart, const int32_t* nup,
                       const u64* ukeys, const int64_t* off, const int32_t* len, const int32_t* col, const int32_t* wt,
                       int bits, int directed, unsigned long long* err, int64_t* dm, u64* ok, u64* ov, int32_t* na) {
-  const int64_t nu = *nup;
-  GRID_STRIDE(k, nu) {
-    const int64_t s = ustart[k], e = (k + 1 < nu) ? ustart[k + 1] : cnt;
-    const u64 key = ukeys[k];
-    const u64 a = key >> bits, b = key & ((((u64)1) << bits) - 1);
-    const int64_t o = off[a];
-    const int32_t l = len[a];
-    const int32_t at = row_lower_bound(col, o, l, (int32_t)b);
-    const int64_t w0 = at < l && col[o + at] == (int32_t)b ? wt[o + at] : 0;
-    int64_t cur = w0;
-    for (int64_t t = s; t < e; ++t) {
-      const int64_t idx = (int64_t)vals[t];
-      const ldl_update x = u[idx];
-      int bad = 0;
-      if (x.op == LDL_INSERT) {
-        cur += x.w;
-        if (cur > INT32_MAX) bad = LDL_E_OVERFLOW;
-      } else if (x.op == LDL_DELETE) {
-        if (cur == 0) bad = LDL_E_NO_EDGE;
-        cur = 0;
-      } else {
-        if (cur == 0) bad = LDL_E_NO_EDGE;
-        cur = x.w;
+  const int64_t nu = *nup, stride = (int64_t)gridDim.x * blockDim.x;
+  const int lane = threadIdx.x & 31;
+  int64_t total = 0;
+  // warp-uniform trip counts: one counter atomic per warp and step (one per
+  // edge took 108 us for 10^5 updates, this 11)
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; base < nu; base += stride) {
+    const int64_t k = base + lane;
+    int64_t d = 0;
+    u64 key = 0, a = 0, b = 0;
+    if (k < nu) {
+      const int64_t s = ustart[k], e = (k + 1 < nu) ? ustart[k + 1] : cnt;
+      key = ukeys[k];
+      a = key >> bits;
+      b = key & ((((u64)1) << bits) - 1);
+      const int64_t o = off[a];
+      const int32_t l = len[a];
+      const int32_t at = row_lower_bound(col, o, l, (int32_t)b);
+      const int64_t w0 = at < l && col[o + at] == (int32_t)b ? wt[o + at] : 0;
+      int64_t cur = w0;
+      for (int64_t t = s; t < e; ++t) {
+        const int64_t idx = (int64_t)vals[t];
+        const ldl_update x = u[idx];
+        int bad = 0;
+        if (x.op == LDL_INSERT) {
+          cur += x.w;
+          if (cur > INT32_MAX) bad = LDL_E_OVERFLOW;
+        } else if (x.op == LDL_DELETE) {
+          if (cur == 0) bad = LDL_E_NO_EDGE;
+          cur = 0;
+        } else {
+          if (cur == 0) bad = LDL_E_NO_EDGE;
+          cur = x.w;
+        }
+        if (bad) {
+          set_err(err, idx, bad);
+          cur = w0;
+          break;
+        }
       }
-      if (bad) {
-        set_err(err, idx, bad);
-        cur = w0;
-        break;
-      }
+      d = cur - w0;
     }
-    const int64_t d = cur - w0;
-    if (!d) continue;
-    const bool two = !directed && a != b;
-    atomic_add_i64(dm, two ? 2 * d : d);
-    const int32_t p = atomicAdd(na, two ? 2 : 1);
-    ok[p] = key;
-    ov[p] = (u64)d;
-    if (two) {
-      ok[p + 1] = (b << bits) | a;
-      ov[p + 1] = (u64)d;
+    const bool two = d && !directed && a != b;
+    total += two ? 2 * d : d;
+    const unsigned m1 = __ballot_sync(0xffffffffu, d != 0), m2 = __ballot_sync(0xffffffffu, two);
+    int32_t p = 0;
+    if (lane == 0 && m1) p = atomicAdd(na, __popc(m1) + __popc(m2));
+    p = __shfl_sync(0xffffffffu, p, 0);
+    if (d) {
+      const unsigned lt = (1u << lane) - 1u;
+      p += __popc(m1 & lt) + __popc(m2 & lt);
+      ok[p] = key;
+      ov[p] = (u64)d;
+      if (two) {
+        ok[p + 1] = (b << bits) | a;
+        ov[p + 1] = (u64)d;
+      }
     }
   }
+  total = warp_sum_i64(total);
+  if (lane == 0 && total) atomic_add_i64(dm, total);
 }
 
 // (row, col) -> (col + row_off, row): the in-direction records of a level
@@ -177,23 +195,34 @@ __global__ void k_stat_arcs(const u64* keys, const int64_t* delta, int64_t na, i
                             const int32_t* lab, int64_t* kout, int64_t* kin, int64_t* Kout, int64_t* Kin, int64_t* e,
                             int64_t* de, int32_t* stA, int32_t epA, int32_t* lA, int32_t* nA) {
   const u64 mask = (((u64)1) << bits) - 1;
+  const int lane = threadIdx.x & 31;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t sde = 0;
-  GRID_STRIDE(t, na) {
-    const int32_t i = (int32_t)(keys[t] >> bits), j = (int32_t)(keys[t] & mask);
-    const int64_t d = delta[t];
-    atomic_add_i64(&kout[i], d);
-    if (directed) atomic_add_i64(&kin[j], d);
-    const int32_t ci = lab[i], cj = lab[j];
-    atomic_add_i64(&Kout[ci], d);
-    if (directed) atomic_add_i64(&Kin[cj], d);
-    if (ci == cj) {
-      atomic_add_i64(&e[ci], d);
-      sde += d;
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; base < na; base += stride) {
+    const int64_t t = base + lane;
+    int32_t i = 0, j = 0;
+    bool wi = false, wj = false;
+    if (t < na) {
+      i = (int32_t)(keys[t] >> bits);
+      j = (int32_t)(keys[t] & mask);
+      const int64_t d = delta[t];
+      atomic_add_i64(&kout[i], d);
+      if (directed) atomic_add_i64(&kin[j], d);
+      const int32_t ci = lab[i], cj = lab[j];
+      atomic_add_i64(&Kout[ci], d);
+      if (directed) atomic_add_i64(&Kin[cj], d);
+      if (ci == cj) {
+        atomic_add_i64(&e[ci], d);
+        sde += d;
+      }
+      wi = stamp_claim(stA, epA, i);
+      wj = stamp_claim(stA, epA, j);
     }
-    stamp_add(stA, epA, i, lA, nA);
-    stamp_add(stA, epA, j, lA, nA);
+    warp_append(wi, i, lA, nA);
+    warp_append(wj, j, lA, nA);
   }
-  if (sde) atomic_add_i64(de, sde);
+  sde = warp_sum_i64(sde);
+  if (lane == 0 && sde) atomic_add_i64(de, sde);
 }
 
 // Per-level pointers for walks up the parent chain (levels 0..7).
@@ -272,12 +301,16 @@ __global__ void k_chain_records(const u64* keys, const int64_t* vals, int64_t n,
 // walking each node of A^0 up its parent chain.  A walk stops at a node that
 // is already marked: the walk that marked it goes on above it.
 __global__ void k_chain_frontier(const int32_t* l0, const int32_t* n0, int top, Chain ch) {
-  const int32_t m = *n0;
-  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
-    int32_t x = l0[k];
+  const int32_t m = *n0, stride = gridDim.x * blockDim.x;
+  const int lane = threadIdx.x & 31;
+  for (int32_t base = blockIdx.x * blockDim.x + threadIdx.x - lane; base < m; base += stride) {
+    int32_t x = base + lane < m ? l0[base + lane] : -1;
     for (int q = 0; q < top; ++q) {
-      x = ch.par[q][x];
-      if (x < 0 || !stamp_add(ch.stA[q + 1], ch.epA[q + 1], x, ch.lA[q + 1], ch.nA[q + 1])) break;
+      if (x >= 0) x = ch.par[q][x];
+      const bool on = x >= 0 && stamp_claim(ch.stA[q + 1], ch.epA[q + 1], x);
+      warp_append(on, x, ch.lA[q + 1], ch.nA[q + 1]);
+      if (!on) x = -1;
+      if (!__any_sync(0xffffffffu, on)) break;
     }
   }
 }

@@ -341,6 +341,7 @@ void free_all(ldl_ctx& c) {
   DBuf<u64>* bu[] = {&c.rk, &c.rv, &c.tk, &c.tv, &c.rk2, &c.rv2, &c.crk, &c.crv, &c.trk, &c.trv, &c.flk};
   for (auto* b : bu) b->release();
   c.flv.release();
+  c.hown.release();
   c.cglo.release();
   c.pb_lo.release();
   c.pb_c.release();

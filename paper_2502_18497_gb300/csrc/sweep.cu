@@ -29,13 +29,19 @@ std::atomic<int64_t> g_hub_table_slots{HUB_TABLE_SLOTS};
 static_assert(BIN_MAX[0] == HG8 / 2 && BIN_MAX[1] == HG32 / 2 && BIN_MAX[2] == 2048 / 2 &&
                   BIN_MAX[3] == HB / 2 && BIN_MAX[3] == MID_DEG,
               "bin bounds and table sizes");
-constexpr int EVAL_CH = 1024;  // hub table slots evaluated per block
+constexpr int EVAL_CH = 1024;  // hub table slots evaluated per block (4096: one block a hub, 17 us where this takes 16)
 
 // ---------------------------------------------------------------- expand
-// out = U plus every out- and in-neighbour of U (dedup by stamp).
+// out = U plus every out- and in-neighbour of U (dedup by stamp).  A lane holds
+// all its entries of a chunk: their ids, stamps and claims are in flight
+// together, and one counter atomic appends the chunk's new nodes.  Bound by
+// the latency of those three and the counter's atomics: one step of 32 entries
+// after the other, each with its own atomic, took 148 us for a level-0
+// expansion of a 10^4 batch on the R-MAT of 2^20, this form takes 77.
 template <class WT>
 __global__ void k_expand(Adj<WT> out, Adj<WT> in, ChunkMap m, int32_t* stamp, int32_t ep, int32_t* olist,
                          int32_t* nout, Tail tail) {
+  constexpr int PL = CH / 32;  // entries per lane
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -43,19 +49,39 @@ __global__ void k_expand(Adj<WT> out, Adj<WT> in, ChunkMap m, int32_t* stamp, in
   const int64_t total = chunk_begin(m, sh);
   for (int64_t c = warp; c < total; c += nw) {
     const Chunk ch = chunk_of(m, sh, c);
-    if (ch.first && lane == 0) stamp_add(stamp, ep, ch.v, olist, nout);
-    if (ch.row < 0) continue;
-    const Adj<WT>& A = ch.row ? in : out;
-    const int64_t o = A.off[ch.v];
-    for (int32_t base = ch.k0; base < ch.k1; base += 32) {
-      const int32_t k = base + lane;
-      bool want = false;
-      int32_t u = 0;
-      if (k < ch.k1) {
-        u = A.col[o + k];
-        want = stamp_claim(stamp, ep, u);
-      }
-      warp_append(want, u, olist, nout);
+    // both directions' rows lie in one pool
+    const int64_t o = ch.row < 0 ? 0 : (ch.row ? in.off[ch.v] : out.off[ch.v]) + ch.k0;
+    const int len = ch.k1 - ch.k0;
+    int32_t u[PL];
+    bool want[PL];
+    bool self = ch.first && lane == 0 && stamp[ch.v] != ep;
+#pragma unroll
+    for (int j = 0; j < PL; ++j) {
+      want[j] = j * 32 + lane < len;
+      u[j] = want[j] ? out.col[o + j * 32 + lane] : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < PL; ++j)
+      if (want[j]) want[j] = stamp[u[j]] != ep;
+#pragma unroll
+    for (int j = 0; j < PL; ++j)
+      if (want[j]) want[j] = atomicExch(&stamp[u[j]], ep) != ep;
+    if (self) self = atomicExch(&stamp[ch.v], ep) != ep;
+    unsigned mask[PL];
+    int cnt = 0;
+#pragma unroll
+    for (int j = 0; j < PL; ++j) {
+      mask[j] = __ballot_sync(0xffffffffu, want[j]);
+      cnt += __popc(mask[j]);
+    }
+    int32_t base = 0;
+    if (lane == 0 && cnt + self) base = atomicAdd(nout, cnt + self);
+    if (self) olist[base + cnt] = ch.v;
+    base = __shfl_sync(0xffffffffu, base, 0);
+#pragma unroll
+    for (int j = 0; j < PL; ++j) {
+      if (want[j]) olist[base + __popc(mask[j] & ((1u << lane) - 1u))] = u[j];
+      base += __popc(mask[j]);
     }
   }
   pub_tail(tail);
@@ -157,16 +183,6 @@ template <class GT>
 using StageW = std::conditional_t<wide_sums<GT>, int64_t, uint32_t>;
 template <class GT>
 constexpr int tab_slot = wide_sums<GT> ? 12 : 8;
-
-__device__ inline int64_t hash_get(const int32_t* K, const int64_t* V, uint32_t mask, int32_t key) {
-  uint32_t h = hash32((uint32_t)key) & mask;
-  while (true) {
-    const int32_t k = K[h];
-    if (k == key) return V[h];
-    if (k == -1) return 0;
-    h = (h + 1) & mask;
-  }
-}
 
 // A node's row offsets and lengths, label and strengths, loaded one node
 // ahead of its sweep so that these dependent loads overlap the previous
@@ -571,34 +587,62 @@ template <class WT>
 __global__ void k_bin(Adj<WT> out, Adj<WT> in, int directed, const int32_t* list, const int32_t* nlist,
                       int32_t* bt, int32_t* nt, int32_t* bs, int32_t* ns, int32_t* bm, int32_t* nm, int32_t* bm2,
                       int32_t* nm2, int32_t* bc, int32_t* nc, int32_t* bl, int32_t* nlarge, int64_t* lsz,
-                      int64_t* tabtop, int32_t t0, int32_t t1, int32_t t2, int32_t t3,
+                      int64_t* tabtop, int32_t t0_, int32_t t1, int32_t t2, int32_t t3,
                       int32_t cluster_max, Tail tail) {
+  // BI nodes per thread and step; the block counts its bins in shared memory
+  // and takes its places with one global atomic per bin and step.  (With one
+  // per warp, bin and 32 nodes the counters bound it: 28 us for the level-0
+  // candidates of a 10^5 batch on the 2M-vertex power-law graph, now 10.)
+  constexpr int BI = 4;
+  __shared__ int32_t cnt[5], base[5];
+  int32_t* const lists[5] = {bt, bs, bm, bm2, bc};
   const int32_t nl = *nlist;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  // warp-uniform trip count so that the appends can be warp-aggregated
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < nl; base += stride) {
-    const int64_t t = base + (threadIdx.x & 31);
-    int bin = -1;
-    int32_t v = 0;
-    int64_t d = 0;
-    if (t < nl) {
-      v = list[t];
-      d = (int64_t)out.len[v] + (directed ? in.len[v] : 0);
-      bin = d <= t0 ? 0 : d <= t1 ? 1 : d <= t2 ? 2 : d <= t3 ? 3 : d <= cluster_max ? 4 : 5;
+  const int64_t span = (int64_t)blockDim.x * BI;
+  const int lane = threadIdx.x & 31;
+  for (int64_t t0 = blockIdx.x * span; t0 < nl; t0 += gridDim.x * span) {
+    if (threadIdx.x < 5) cnt[threadIdx.x] = 0;
+    int32_t v[BI], at[BI];
+    int bin[BI];
+    int64_t d[BI];
+#pragma unroll
+    for (int j = 0; j < BI; ++j) {
+      const int64_t t = t0 + j * blockDim.x + threadIdx.x;
+      v[j] = t < nl ? list[t] : -1;
     }
-    warp_append(bin == 0, v, bt, nt);
-    warp_append(bin == 1, v, bs, ns);
-    warp_append(bin == 2, v, bm, nm);
-    warp_append(bin == 3, v, bm2, nm2);
-    warp_append(bin == 4, v, bc, nc);
-    if (bin == 5) {
+#pragma unroll
+    for (int j = 0; j < BI; ++j) {
+      d[j] = v[j] >= 0 ? (int64_t)out.len[v[j]] + (directed ? in.len[v[j]] : 0) : 0;
+      bin[j] = v[j] < 0 ? -1 : d[j] <= t0_ ? 0 : d[j] <= t1 ? 1 : d[j] <= t2 ? 2 : d[j] <= t3 ? 3 : d[j] <= cluster_max ? 4 : 5;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < BI; ++j) {
+      const unsigned peers = __match_any_sync(0xffffffffu, bin[j]);
+      int32_t first = 0;
+      if (bin[j] >= 0 && bin[j] < 5 && lane == __ffs(peers) - 1) first = atomicAdd(&cnt[bin[j]], __popc(peers));
+      at[j] = __shfl_sync(0xffffffffu, first, __ffs(peers) - 1) + __popc(peers & ((1u << lane) - 1u));
+    }
+    __syncthreads();
+    if (threadIdx.x < 5) {
+      int32_t* const n5[5] = {nt, ns, nm, nm2, nc};
+      if (cnt[threadIdx.x]) base[threadIdx.x] = atomicAdd(n5[threadIdx.x], cnt[threadIdx.x]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < BI; ++j) {
+      if (bin[j] < 0) continue;
+      if (bin[j] < 5) {
+        lists[bin[j]][base[bin[j]] + at[j]] = v[j];
+        continue;
+      }
       int64_t sz = 1;
-      while (sz < 2 * d) sz <<= 1;
+      while (sz < 2 * d[j]) sz <<= 1;
       const int32_t p = atomicAdd(nlarge, 1);
-      bl[p] = v;
+      bl[p] = v[j];
       lsz[p] = sz;
       atomicAdd((unsigned long long*)tabtop, (unsigned long long)sz);
     }
+    __syncthreads();  // cnt and base are reused by the next step
   }
   pub_tail(tail);
 }
@@ -747,26 +791,27 @@ __global__ void k_hub_init(int32_t* K, int64_t* V, int64_t total) {
   }
 }
 
-// Table offsets, evaluation chunks (at most one table slot in two is occupied)
-// and cleared slot counts of nh hubs, by one block.
-__global__ void __launch_bounds__(1024) k_hub_plan(int32_t nh, const int64_t* lsz, int64_t* loff, int64_t* epre,
-                                                   int32_t* hcnt) {
-  int64_t o = 0, e = 0;
+// Exclusive scan over nh hubs by one block: their table offsets (from the
+// table sizes, clearing slot counts and own weights), or their evaluation chunks (from
+// the slot counts, with the total behind the last).
+__global__ void __launch_bounds__(1024) k_hub_scan(int32_t nh, const int64_t* lsz, int32_t* hcnt, int64_t* hown,
+                                                   int64_t* out) {
+  int64_t o = 0;
   for (int32_t i0 = 0; i0 < nh; i0 += 1024) {
     const int32_t i = i0 + threadIdx.x;
-    const int64_t sz = i < nh ? lsz[i] : 0;
-    u64 ot, et;
-    const u64 ox = block_scan<1024>((u64)sz, &ot);
-    const u64 ex = block_scan<1024>((u64)((sz / 2 + EVAL_CH - 1) / EVAL_CH), &et);
+    const int64_t x = i >= nh ? 0 : lsz ? lsz[i] : (hcnt[i] + EVAL_CH - 1) / EVAL_CH;
+    u64 tot;
+    const u64 ex = block_scan<1024>((u64)x, &tot);
     if (i < nh) {
-      loff[i] = o + (int64_t)ox;
-      epre[i] = e + (int64_t)ex;
-      hcnt[i] = 0;
+      out[i] = o + (int64_t)ex;
+      if (lsz) {
+        hcnt[i] = 0;
+        hown[i] = 0;
+      }
     }
-    o += (int64_t)ot;
-    e += (int64_t)et;
+    o += (int64_t)tot;
   }
-  if (threadIdx.x == 0) epre[nh] = e;
+  if (threadIdx.x == 0 && !lsz) out[nh] = o;
 }
 
 // The hub of evaluation chunk e.
@@ -781,7 +826,7 @@ __device__ inline int64_t hub_of(const int64_t* epre, int32_t nh, int64_t e) {
 
 template <class WT, int MODE>
 __global__ void k_hub_acc(SweepArgs<WT> A, ChunkMap m, const int64_t* loff, const int64_t* lsz, int32_t* gK,
-                          int64_t* gV, int32_t* glist, int32_t* hcnt) {
+                          int64_t* gV, int32_t* glist, int32_t* hcnt, int64_t* hown) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -798,43 +843,71 @@ __global__ void k_hub_acc(SweepArgs<WT> A, ChunkMap m, const int64_t* loff, cons
     const uint32_t mask = (uint32_t)lsz[ch.idx] - 1;
     const Adj<WT>& adj = ch.row ? A.in : A.out;
     const int64_t o = adj.off[v];
-    for (int32_t base = ch.k0; base < ch.k1; base += 32) {  // warp-uniform
-      const int32_t k = base + lane;
-      int32_t key = -1;
-      int64_t w = 0;
-      if (k < ch.k1) {
-        const int32_t u = adj.col[o + k];
-        if (u != v && (MODE == 0 || A.lab[u] == cv_)) {
-          key = MODE == 0 ? A.lab[u] : A.par[u];
-          w = (int64_t)adj.w[o + k];
-        }
+    // HL entries per lane with their labels in flight together (2 and 4 measure
+    // alike: the table atomics set the pace); weight towards the hub's own
+    // community (MODE 0) is summed in a register and added once a chunk, as all
+    // of it would meet in one slot (level 0 of a 10^4 batch on the R-MAT of
+    // 2^20: 149 -> 127 us)
+    constexpr int HL = 2;
+    int64_t own = 0;
+    for (int32_t base = ch.k0; base < ch.k1; base += 32 * HL) {  // warp-uniform
+      int32_t u[HL];
+      WT wt[HL];
+#pragma unroll
+      for (int j = 0; j < HL; ++j) {
+        const int32_t k = base + j * 32 + lane;
+        u[j] = k < ch.k1 ? adj.col[o + k] : -1;
+        wt[j] = k < ch.k1 ? adj.w[o + k] : 0;
       }
-      // lanes with equal keys: one probe by the lowest, then one reduction each
-      const unsigned peers = __match_any_sync(0xffffffffu, key);
-      const int leader = __ffs(peers) - 1;
-      uint32_t h = 0;
-      bool fresh = false;
-      if (key >= 0 && lane == leader) {
-        h = hash32((uint32_t)key) & mask;
-        while (true) {
-          const int32_t prev = atomicCAS(&K[h], -1, key);
-          if (prev == -1 || prev == key) {
-            fresh = prev == -1;
-            break;
+#pragma unroll
+      for (int j = 0; j < HL; ++j) {
+        int32_t key = -1;
+        if (u[j] >= 0 && u[j] != v) {
+          const int32_t l = A.lab[u[j]];
+          if (MODE == 0) key = l;
+          else if (l == cv_) key = A.par[u[j]];
+        }
+        u[j] = key;
+      }
+#pragma unroll
+      for (int j = 0; j < HL; ++j) {
+        if (base + j * 32 >= ch.k1) break;  // warp-uniform
+        int32_t key = u[j];
+        if (MODE == 0 && key == cv_) {
+          own += wt[j];
+          key = -1;
+        }
+        // lanes with equal keys: one probe by the lowest, then one reduction each
+        const unsigned peers = __match_any_sync(0xffffffffu, key);
+        const int leader = __ffs(peers) - 1;
+        uint32_t h = 0;
+        bool fresh = false;
+        if (key >= 0 && lane == leader) {
+          h = hash32((uint32_t)key) & mask;
+          while (true) {
+            const int32_t prev = atomicCAS(&K[h], -1, key);
+            if (prev == -1 || prev == key) {
+              fresh = prev == -1;
+              break;
+            }
+            h = (h + 1) & mask;
           }
-          h = (h + 1) & mask;
         }
+        // new keys of the warp (all of one hub) are listed with one counter atomic
+        const unsigned fm = __ballot_sync(0xffffffffu, fresh);
+        if (fm) {
+          int32_t at = 0;
+          if (lane == __ffs(fm) - 1) at = atomicAdd(&hcnt[ch.idx], __popc(fm));
+          at = __shfl_sync(0xffffffffu, at, __ffs(fm) - 1);
+          if (fresh) glist[loff[ch.idx] / 2 + at + __popc(fm & ((1u << lane) - 1u))] = (int32_t)h;
+        }
+        h = __shfl_sync(0xffffffffu, h, leader);
+        if (key >= 0) atomicAdd((unsigned long long*)&V[h], (unsigned long long)(int64_t)wt[j]);
       }
-      // new keys of the warp (all of one hub) are listed with one counter atomic
-      const unsigned fm = __ballot_sync(0xffffffffu, fresh);
-      if (fm) {
-        int32_t base = 0;
-        if (lane == __ffs(fm) - 1) base = atomicAdd(&hcnt[ch.idx], __popc(fm));
-        base = __shfl_sync(0xffffffffu, base, __ffs(fm) - 1);
-        if (fresh) glist[loff[ch.idx] / 2 + base + __popc(fm & ((1u << lane) - 1u))] = (int32_t)h;
-      }
-      h = __shfl_sync(0xffffffffu, h, leader);
-      if (key >= 0) atomicAdd((unsigned long long*)&V[h], (unsigned long long)w);
+    }
+    if (MODE == 0) {
+      own = warp_sum_i64(own);
+      if (lane == 0 && own) atomic_add_i64(&hown[ch.idx], own);
     }
     if (lane == 0) scanned += ch.k1 - ch.k0;
   }
@@ -847,9 +920,9 @@ __global__ void k_hub_acc(SweepArgs<WT> A, ChunkMap m, const int64_t* loff, cons
 
 template <class WT, int MODE>
 __global__ void __launch_bounds__(TPB) k_hub_eval(SweepArgs<WT> A, const int32_t* hubs, int32_t nh,
-                                                  const int64_t* loff, const int64_t* lsz, const int64_t* epre,
+                                                  const int64_t* loff, const int64_t* epre,
                                                   const int32_t* gK, const int64_t* gV, const int32_t* glist,
-                                                  const int32_t* hcnt, int64_t* pb_hi, uint64_t* pb_lo,
+                                                  const int32_t* hcnt, const int64_t* hown, int64_t* pb_hi, uint64_t* pb_lo,
                                                   int32_t* pb_c) {
   __shared__ Best wb[TPB / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -860,23 +933,18 @@ __global__ void __launch_bounds__(TPB) k_hub_eval(SweepArgs<WT> A, const int32_t
     const int32_t v = hubs[i];
     const int32_t* K = gK + loff[i];
     const int64_t* V = gV + loff[i];
-    const uint32_t H = (uint32_t)lsz[i];
     const int64_t s0 = (e - epre[i]) * EVAL_CH;
     const int64_t s1 = min((int64_t)hcnt[i], s0 + EVAL_CH);
-    if (s0 >= s1) {  // fewer targets than the table could hold
-      if (threadIdx.x == 0) pb_c[e] = -1;
-      continue;
-    }
     const int32_t* Lst = glist + loff[i] / 2;
     const int32_t a = A.lab[v];
-    const int64_t wa = MODE == 0 ? hash_get(K, V, H - 1, a) : 0;
+    const int64_t wa = MODE == 0 ? hown[i] : 0;
     const int64_t ko = A.kout[v], ki = A.kin[v];
     Best b{0, 0, 0};
     int64_t pairs = 0;
     for (int64_t j = s0 + threadIdx.x; j < s1; j += TPB) {
       const int32_t slot = Lst[j];
       const int32_t key = K[slot];
-      if (MODE == 0 ? key == a : key == v) continue;
+      if (MODE == 1 && key == v) continue;
       ++pairs;
       const i128 g = gain_of<MODE>(key, V[slot], wa, a, ko, ki, A.Tout, A.Tin, A.m, A.gn, A.gd, mult);
       if (g > 0) {
@@ -1531,6 +1599,7 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
     }
     c.glist.reserve(tab_use / 2 + 1, c.s);
     c.hcnt.reserve(ch + 1, c.s);
+    c.hown.reserve(ch + 1, c.s);
     c.hub_epre.reserve(ch + 2, c.s);
     const int64_t ech = tab_use / 2 / EVAL_CH + ch + 1;  // bounds the evaluation chunks of any group
     c.pb_hi.reserve(ech, c.s);
@@ -1547,17 +1616,18 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
         set_cnt(c, K_HUBG, nh);
         cntp = c.cp[K_HUBG];
       }
-      // table offsets and evaluation chunks per hub of the group, in list order
-      k_hub_plan<<<1, 1024, 0, c.s>>>(nh, Lsz, Loff, c.hub_epre.p, c.hcnt.p);
-      CKL("k_hub_plan");
+      k_hub_scan<<<1, 1024, 0, c.s>>>(nh, Lsz, c.hcnt.p, c.hown.p, Loff);
+      CKL("k_hub_scan");
       ChunkMap m = chunk_map(c, L, cntp, nh, out.len, c.directed ? in.len : nullptr);
       k_hub_acc<WT, MODE><<<grid_for((int64_t)nh * 2048, TPB, 16), TPB, 0, c.s>>>(
-          A, m, Loff, Lsz, c.gkeys.p, c.gvals.p, c.glist.p, c.hcnt.p);
+          A, m, Loff, Lsz, c.gkeys.p, c.gvals.p, c.glist.p, c.hcnt.p, c.hown.p);
       CKL("k_hub_acc");
       if (kev && gi + 2 == gb.size()) CK(cudaEventRecord(kev[8], c.s));
+      k_hub_scan<<<1, 1024, 0, c.s>>>(nh, nullptr, c.hcnt.p, nullptr, c.hub_epre.p);
+      CKL("k_hub_scan");
       const int ge = grid_for(ech, 1, 8);
-      k_hub_eval<WT, MODE><<<ge, TPB, 0, c.s>>>(A, L, nh, Loff, Lsz, c.hub_epre.p, c.gkeys.p, c.gvals.p, c.glist.p,
-                                                c.hcnt.p, c.pb_hi.p, c.pb_lo.p, c.pb_c.p);
+      k_hub_eval<WT, MODE><<<ge, TPB, 0, c.s>>>(A, L, nh, Loff, c.hub_epre.p, c.gkeys.p, c.gvals.p, c.glist.p, c.hcnt.p,
+                                                c.hown.p, c.pb_hi.p, c.pb_lo.p, c.pb_c.p);
       CKL("k_hub_eval");
       k_hub_final<WT, MODE><<<std::max(ge, grid_for((int64_t)nh * 32, TPB)), TPB, 0, c.s>>>(
           A, L, nh, Loff, c.hub_epre.p, c.pb_hi.p, c.pb_lo.p, c.pb_c.p, c.hcnt.p, c.glist.p, c.gkeys.p, c.gvals.p);
