@@ -27,6 +27,7 @@ struct LevelState {
   DBuf<int32_t> stA, lA;         // frontier A^r (dedup stamp + list)
   DBuf<int32_t> stK, lK;         // endpoints of arcs deleted since the level was last refined
   int32_t brk_ep = 0;            // epoch of stK
+  int64_t ubA = 0, ubK = 0;      // host bounds on |A^r| and on stK's list
   // weight records of this level not yet applied to its adjacency (levels >= 1
   // of a batch update: unsorted, unreduced; count in cp[K_PEND0 + r])
   DBuf<u64> pk, pv;
@@ -100,6 +101,7 @@ struct ldl_ctx {
   int64_t* sums = nullptr;     // two accumulators of the last sweep or aggregate step
   // whether the last sweep of (level, mode) had hub rows (scheduling only)
   uint8_t hubs_seen[8][2] = {{0}};
+  int64_t ubU = 0;  // host bound on |U*|
   int32_t epoch = 0;
 
   // dedup stamps (one int32 per node id) and lists
@@ -155,11 +157,11 @@ struct ldl_ctx {
   double ks_launch[KS_GROUPS] = {0, 0, 0, 0, 0, 0, 0};
   int64_t syncs = 0;  // host synchronisations in the current batch
   int64_t grow_per_update = 0;  // most device bytes a batch of this context allocated per update
-  // host reads of device values: a pinned, device-mapped page (word 0 is the
-  // sequence number of the last read, the payload follows)
-  volatile int64_t* h_pub = nullptr;
-  int64_t* d_pub = nullptr;
-  int64_t pub_seq = 0;
+  // host reads of device values: a pinned, device-mapped page of tagged words
+  // (scan.cuh), and the number of the last read
+  volatile u64* h_pub = nullptr;
+  u64* d_pub = nullptr;
+  uint32_t pub_seq = 0;
   std::string err;
   bool broken = false;  // a failed rollback left the state unknown
 
@@ -202,9 +204,9 @@ inline Adj<int64_t> adj_in(ldl_ctx& c, int r) {
 inline int64_t* kin_of(ldl_ctx& c, int r) { return c.directed ? c.lv[r].kin.p : c.lv[r].kout.p; }
 inline int64_t* Kin_of(ldl_ctx& c) { return c.directed ? c.Kin.p : c.Kout.p; }
 
-// Copies device values to the host once the context's stream has reached
-// this point: a one-block kernel writes them into the pinned page and then the
-// sequence number, which the host polls (a stream error ends the wait).
+// Copies device values (4-byte multiples) to the host once the context's stream
+// has reached this point: a one-block kernel writes them into the pinned page,
+// which the host polls (a stream error ends the wait).
 void host_read(ldl_ctx& c, const HostRead* r, int n);
 // The same for values that a kernel publishes itself (scan.cuh): the page and
 // the sequence number for it, then the wait for its n payload words.  One

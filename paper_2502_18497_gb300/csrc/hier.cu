@@ -1082,6 +1082,7 @@ static int64_t apply_records(ldl_ctx& c, int r, const u64* keys, const int64_t* 
                                                 c.d_sc, &trk)
                            : csr_apply<int64_t>(c.lv[r].out, keys, vals, mul * nr, n_dev, mul, c.bits, c.CS, c.P, c.s,
                                                 c.d_sc, &trk);
+  Lr.ubK = std::min<int64_t>(c.n, Lr.ubK + 2 * m / mul);
   return m / mul;
 }
 
@@ -1284,15 +1285,14 @@ int32_t split(ldl_ctx& c, int r, int32_t epD, int32_t epX) {
   zero_cnt(c, K_X);
   const int32_t epF = c.next_epoch();  // communities whose connectivity is in doubt
   // The level's deleted-arc endpoints and U* stay on the device: both kernels
-  // stride over their lists' counts with a grid bounded by the node count.
-  const int gs = grid_for(c.n, TPB, 4);
-  k_brk_check<<<gs, TPB, 0, c.s>>>(L.lK.p, c.cp[K_BRK0 + r], L.alive.p, L.par.p, c.stX.p, epX, c.lX.p,
+  // stride over their lists' counts with grids sized by the host's bounds.
+  k_brk_check<<<grid_for(L.ubK, TPB, 4), TPB, 0, c.s>>>(L.lK.p, c.cp[K_BRK0 + r], L.alive.p, L.par.p, c.stX.p, epX, c.lX.p,
                                    c.cp[K_X], c.ckf.p, epF);
   CKL("k_brk_check");
   const int32_t epL = c.next_epoch();
   int32_t cnt2[2] = {0, 0};
   const HostRead rd[2] = {{c.cp[K_D], &cnt2[0], sizeof(int32_t)}, {c.cp[K_X], &cnt2[1], sizeof(int32_t)}};
-  k_leave<<<gs, TPB, 0, c.s>>>(c.lUstar.p, c.cp[K_USTAR], L.alive.p, L.lab.p, N.lab.p, L.par.p, c.par_old.p,
+  k_leave<<<grid_for(c.ubU, TPB, 4), TPB, 0, c.s>>>(c.lUstar.p, c.cp[K_USTAR], L.alive.p, L.lab.p, N.lab.p, L.par.p, c.par_old.p,
                                L.kout.p, kin_of(c, r), N.kout.p, kin_of(c, r + 1), N.cnt.p, c.directed, c.stL.p, epL,
                                c.stD.p, epD, c.lD.p, c.cp[K_D], c.stX.p, epX, c.lX.p, c.cp[K_X], c.nbr.p,
                                tail_begin(c, rd, 2));
@@ -1330,6 +1330,7 @@ int32_t split(ldl_ctx& c, int r, int32_t epD, int32_t epX) {
   }
   // the deletions of this level are consumed
   L.brk_ep = c.next_epoch();
+  L.ubK = 0;
   zero_cnt(c, K_BRK0 + r);
   return nD;
 }
@@ -1458,9 +1459,10 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
     sub_end(c, SU_AGG_EMIT);
     sub_begin(c);
   }
-  // |U*| stays on the device: the grid is bounded by two blocks per SM
+  if (!build) N.ubA = std::min<int64_t>(c.n, N.ubA + c.ubU + 2 * (int64_t)nD + 2 * nr);
+  // |U*| stays on the device
   const bool recs = nC > 0 && epA_next;
-  k_next_level<<<device_sms() * 2, TPB, 0, c.s>>>(c.lUstar.p, c.cp[K_USTAR], c.lD.p, c.cp[K_D], L.par.p,
+  k_next_level<<<grid_for(build ? c.n : c.ubU + nD + nr, TPB, 2), TPB, 0, c.s>>>(c.lUstar.p, c.cp[K_USTAR], c.lD.p, c.cp[K_D], L.par.p,
                                                   c.par_old.p, L.lab.p, N.lab.p, recs ? c.rk.p : nullptr,
                                                   c.cp[K_NR], nr, c.bits, N.alive.p, epA_next ? N.stA.p : nullptr,
                                                   epA_next, N.lA.p, c.cp[K_A0 + r + 1], &c.d_sc->agg_recs);

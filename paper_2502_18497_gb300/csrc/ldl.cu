@@ -81,23 +81,10 @@ DeviceScope::~DeviceScope() {
 }
 
 namespace {
-constexpr int PUB_MAX = 8;        // values per read
-constexpr int PUB_BYTES = 4000;   // payload bytes per read
-struct PubReq {
-  const unsigned char* src[PUB_MAX];
-  int32_t off[PUB_MAX], bytes[PUB_MAX];
-  int32_t n;
-};
+constexpr int PAGE_WORDS = 500;  // payload words per read
 
-__global__ void k_publish(PubReq q, unsigned char* payload, int64_t* seq_word, int64_t seq) {
-  for (int i = 0; i < q.n; ++i)
-    for (int b = threadIdx.x; b < q.bytes[i]; b += blockDim.x) payload[q.off[i] + b] = q.src[i][b];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence_system();  // the payload is visible to the host before the sequence number
-    *(volatile int64_t*)seq_word = seq;
-  }
-}
+// hands values of earlier kernels to the host (one block)
+__global__ void k_publish(Tail t) { put_tail(t); }
 
 __global__ void k_set_i32(int32_t* p, int32_t v) { *p = v; }
 
@@ -142,52 +129,43 @@ __global__ void __launch_bounds__(256) k_snapshot(SnapList l, unsigned char* dst
 
 }  // namespace
 
-// Polls the mapped sequence word until the read `seq` has arrived.  Every so
-// often it asks the stream: an error ends the wait with that error; an idle
-// stream whose write is still not seen falls back to a full synchronisation
-// before failing.
-static void wait_page(ldl_ctx& c, int64_t seq) {
-  for (uint64_t spins = 1; c.h_pub[0] != seq; ++spins) {
-    if ((spins & 4095) == 0) {
+// Waits for n payload words of the read under way.  Every so often it asks the
+// stream: an error ends the wait with that error; an idle stream whose write is
+// still not seen falls back to a full synchronisation before failing.
+static void wait_words(ldl_ctx& c, int n) {
+  const uint32_t seq = c.pub_seq;
+  uint64_t spins = 0;
+  for (int w = 0; w < n; ++w)
+    while ((uint32_t)(c.h_pub[w] >> 32) != seq) {
+      if ((++spins & 4095) != 0) continue;
       const cudaError_t e = cudaStreamQuery(c.s);
       if (e == cudaErrorNotReady) continue;
       CK(e);
       CK(cudaStreamSynchronize(c.s));
-      if (c.h_pub[0] != seq) ldl_throw(LDL_E_CUDA, "internal: a published value never reached the host");
+      if ((uint32_t)(c.h_pub[w] >> 32) != seq) ldl_throw(LDL_E_CUDA, "internal: a published value never reached the host");
     }
-  }
   std::atomic_thread_fence(std::memory_order_acquire);
 }
 
 Pub pub_begin(ldl_ctx& c) {
   ++c.syncs;
-  return Pub{c.d_pub, ++c.pub_seq};
+  if (++c.pub_seq == 0) {  // all numbers used: no word of the page may match a new one
+    for (int w = 0; w < PAGE_WORDS; ++w) c.h_pub[w] = 0;
+    c.pub_seq = 1;  // 0 marks a tail without a read
+  }
+  return Pub{c.d_pub, c.pub_seq};
 }
 
 void pub_wait(ldl_ctx& c, int64_t* out, int n) {
-  wait_page(c, c.pub_seq);
-  for (int i = 0; i < n; ++i) out[i] = c.h_pub[1 + i];
+  wait_words(c, 2 * n);
+  for (int i = 0; i < n; ++i) out[i] = (int64_t)((c.h_pub[2 * i] & 0xffffffffu) | (c.h_pub[2 * i + 1] << 32));
 }
 
 void host_read(ldl_ctx& c, const HostRead* r, int n) {
-  ++c.syncs;
-  PubReq q{};
-  int32_t off = 0;
-  if (n > PUB_MAX) ldl_throw(LDL_E_INVALID, "internal: host read of too many values");
-  for (int i = 0; i < n; ++i) {
-    q.src[i] = (const unsigned char*)r[i].src;
-    q.off[i] = off;
-    q.bytes[i] = r[i].bytes;
-    off += (r[i].bytes + 7) & ~7;
-  }
-  if (off > PUB_BYTES) ldl_throw(LDL_E_INVALID, "internal: host read too large");
-  q.n = n;
-  const int64_t seq = ++c.pub_seq;
-  k_publish<<<1, 64, 0, c.s>>>(q, (unsigned char*)(c.d_pub + 1), c.d_pub, seq);
+  const Tail t = tail_begin(c, r, n);
+  k_publish<<<1, 64, 0, c.s>>>(t);
   CKL("k_publish");
-  wait_page(c, seq);
-  const unsigned char* pay = (const unsigned char*)(c.h_pub + 1);
-  for (int i = 0; i < n; ++i) memcpy(r[i].dst, pay + q.off[i], (size_t)r[i].bytes);
+  tail_wait(c, r, n);
 }
 
 int32_t rd_cnt(ldl_ctx& c, int idx) {
@@ -226,7 +204,7 @@ Tail tail_begin(ldl_ctx& c, const HostRead* r, int n) {
     t.words[i] = r[i].bytes / 4;
     off += t.words[i];
   }
-  if (off * 4 > PUB_BYTES) ldl_throw(LDL_E_INVALID, "internal: host read too large");
+  if (off > PAGE_WORDS) ldl_throw(LDL_E_INVALID, "internal: host read too large");
   t.n = n;
   zero_cnt(c, K_TICKET);
   t.ticket = c.cp[K_TICKET];
@@ -237,12 +215,15 @@ Tail tail_begin(ldl_ctx& c, const HostRead* r, int n) {
 }
 
 void tail_wait(ldl_ctx& c, const HostRead* r, int n) {
-  wait_page(c, c.pub_seq);
-  const unsigned char* pay = (const unsigned char*)(c.h_pub + 1);
-  for (int i = 0; i < n; ++i) {
-    memcpy(r[i].dst, pay, (size_t)r[i].bytes);
-    pay += r[i].bytes;
-  }
+  int words = 0;
+  for (int i = 0; i < n; ++i) words += r[i].bytes / 4;
+  wait_words(c, words);
+  int at = 0;
+  for (int i = 0; i < n; ++i)
+    for (int w = 0; w < r[i].bytes / 4; ++w) {
+      const uint32_t v = (uint32_t)c.h_pub[at++];
+      memcpy((unsigned char*)r[i].dst + 4 * w, &v, 4);
+    }
 }
 
 void set_cnt(ldl_ctx& c, int idx, int32_t v) {
@@ -374,8 +355,9 @@ void free_all(ldl_ctx& c) {
 // lUstar / stU (epoch epU) hold U*.  Moved nodes go to lMv (epMv) and, at
 // level 0, to lM0 (epM0).
 static int64_t move_loop(ldl_ctx& c, int r, int rounds, int32_t epU, int32_t epMv, int32_t epM0, int32_t epCh,
-                         int32_t nU) {
+                         int32_t nU, int64_t s_max) {
   // nU = |U| on entry; later rounds take it from the end of the previous one.
+  // s_max bounds the first round's candidate set.
   // Returns the committed moves, an upper bound of the distinct moved nodes
   // (lMv), which is empty exactly when it is 0.
   int64_t committed = 0;
@@ -391,7 +373,7 @@ static int64_t move_loop(ldl_ctx& c, int r, int rounds, int32_t epU, int32_t epM
     stage_end(c, ST_EXPAND);
     // |S| stays on the device: the sweep's kernels stride over it (n bounds
     // their grids) and it comes back with the candidates (β test)
-    const SweepOut so = sweep(c, r, 0, c.lS.p, K_S, c.n);
+    const SweepOut so = sweep(c, r, 0, c.lS.p, K_S, j == 0 ? std::min(c.n, s_max) : c.n);
     const int32_t nS = so.nlist, nc = so.nc, nb = so.nb;
     if (nc == 0) break;
     c.res.rejected += nc - nb;
@@ -477,7 +459,7 @@ static void static_build(ldl_ctx& c) {
     zero_cnt(c, K_MV);
     zero_cnt(c, K_M0);
     zero_cnt(c, K_CH);
-    const int64_t mv = move_loop(c, r, c.prm.M_static, epU, epMv, epM0, epCh, nU);
+    const int64_t mv = move_loop(c, r, c.prm.M_static, epU, epMv, epM0, epCh, nU, c.n);
     if (r > 0) pushdown(c, r, epCh, mv);
     if (r == L) break;
     level_alloc(c, r + 1);
@@ -627,6 +609,8 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
   for (int r = 0; r <= T; ++r) {
     epA[r] = c.next_epoch();  // the lists' counters were cleared at the start of ingest
     c.lv[r].brk_ep = c.next_epoch();
+    c.lv[r].ubA = std::min(c.n, 2 * na);
+    c.lv[r].ubK = 0;
   }
   stage_begin(c);
   const int32_t epT = c.next_epoch();
@@ -647,23 +631,27 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
     for (int r = 0; r <= T; ++r) {
       // |A^r| stays on the device: the kernel strides over it with a grid of
       // two blocks per SM, and one read returns |U|, the level's pending
-      // record count for its flush and, from level 1 on, |M0| (on the first
-      // visit: the statistic repair's sums)
+      // record count for its flush, the entries of U's rows and, from level 1
+      // on, |M0| (on the first visit: the statistic repair's sums)
       const int32_t epU = c.next_epoch();
       zero_cnt(c, K_U);
       zero_cnt(c, K_USTAR);
+      c.sums = (int64_t*)fresh(c, 2, c.d_sc->sums);
       int32_t nU = 0, nP = 0, m0 = 0;
+      int64_t deg = 0;
       RepairAcc ra{};
       const bool first = pass == 0 && r == 0;
-      HostRead rr[3] = {{c.cp[K_U], &nU, sizeof(int32_t)},
+      HostRead rr[4] = {{c.cp[K_U], &nU, sizeof(int32_t)},
                         {c.cp[K_PEND0 + r], &nP, sizeof(int32_t)},
-                        {c.cp[K_M0], &m0, sizeof(int32_t)}};
+                        {c.cp[K_M0], &m0, sizeof(int32_t)},
+                        {c.sums, &deg, sizeof(int64_t)}};
       if (first) {
         rr[2].src = c.racc;
         rr[2].dst = &ra;
         rr[2].bytes = (int32_t)sizeof(ra);
       }
-      frontier(c, r, epU, rr, 3);
+      frontier(c, r, epU, rr, 4);
+      c.ubU = nU;
       if (first) {
         repair_done(c, ra, dm);
         Qpass = qnum(c);
@@ -676,7 +664,9 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
       stage_begin(c);
       flush_level(c, r, nP);  // the level's weights are read from here on
       stage_end(c, ST_AGG);
-      const int64_t mv = move_loop(c, r, c.prm.M, epU, epMv, epM0, epCh, nU);
+      // U and every row entry bound the first candidate set (a flush adds at
+      // most one entry per record and row)
+      const int64_t mv = move_loop(c, r, c.prm.M, epU, epMv, epM0, epCh, nU, nU + deg + 2 * (int64_t)nP);
       if (r > 0) {
         stage_begin(c);
         pushdown(c, r, epCh, mv);
@@ -708,6 +698,7 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
     for (int r = 0; r <= T; ++r) {
       epA[r] = c.next_epoch();
       zero_cnt(c, K_A0 + r);
+      c.lv[r].ubA = r == 0 ? c.n : 0;
     }
     expand_set(c, 0, c.lM0.p, K_M0, c.lv[0].stA.p, epA[0], c.lv[0].lA.p, K_A0, nM0);
   }
@@ -807,11 +798,11 @@ ldl_status ctx_new(const ldl_params& p, int64_t n, ldl_ctx** out) {
     {
       void* hp = nullptr;
       CK(cudaHostAlloc(&hp, 4096, cudaHostAllocMapped));
-      c->h_pub = (volatile int64_t*)hp;
-      c->h_pub[0] = 0;
+      memset(hp, 0, 4096);
+      c->h_pub = (volatile u64*)hp;
       void* dp = nullptr;
       CK(cudaHostGetDevicePointer(&dp, hp, 0));
-      c->d_pub = (int64_t*)dp;
+      c->d_pub = (u64*)dp;
     }
     CK(cudaEventCreate(&c->ev0));
     CK(cudaEventCreate(&c->ev1));

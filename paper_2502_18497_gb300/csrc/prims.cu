@@ -377,24 +377,67 @@ __global__ void __launch_bounds__(RS_THREADS, 4) k_rs_coop(u64* keys, u64* vals,
 // contiguous sub-tile (rounds of 32, stable), the block turns the per-warp
 // digit counts into positions, the pairs are placed in shared memory in
 // digit order and read back in the same warp-contiguous layout.
+// Up to RK_MAX pairs are placed by counting instead: a thread compares its key
+// with all others (a few pairs: 2.1 us instead of 5.4, with sums 4.3 instead
+// of 7.9; some hundred 3.3 instead of 6.4).
+constexpr int SM_THREADS = 512;
+constexpr int SM_ITEMS = RS_TILE / SM_THREADS;
+constexpr int SM_WARPS = SM_THREADS / WARP;
+constexpr int RK_MAX = 256;
 struct RsSmall {
-  int32_t whist[RS_THREADS / WARP][256];
+  int32_t whist[SM_WARPS][256];
   int32_t tstart[256];
   u64 sk[RS_TILE];
   u64 sv[RS_TILE];
 };
 
-__device__ inline void rs_small_passes(RsSmall& m, u64 (&key)[RS_ITEMS], u64 (&val)[RS_ITEMS], int n, int lo_bit,
-                                       int bits) {
-  constexpr int NW = RS_THREADS / WARP;
+// place of pair k of this thread: contiguous per warp
+__device__ inline int sm_at(int k) { return (threadIdx.x >> 5) * (SM_ITEMS * 32) + k * 32 + (threadIdx.x & 31); }
+
+__device__ inline void rs_small_sort(RsSmall& m, u64 (&key)[SM_ITEMS], u64 (&val)[SM_ITEMS], int n, int lo_bit,
+                                     int bits) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (n <= RK_MAX) {
+    // the pairs are in the first warps: pair i belongs to warp i / (SM_ITEMS * 32)
+    const u64 mask = bits >= 64 ? ~(u64)0 : (((u64)1) << bits) - 1;
+    for (int k = 0; k < SM_ITEMS; ++k)
+      if (sm_at(k) < n) {
+        m.sk[sm_at(k)] = key[k];
+        m.sv[sm_at(k)] = val[k];
+      }
+    __syncthreads();
+    u64 mk = 0, mv = 0;
+    int rank = 0;
+    if (tid < n) {
+      mk = m.sk[tid];
+      mv = m.sv[tid];
+      const u64 x = (mk & mask) >> lo_bit;
+#pragma unroll 4
+      for (int j = 0; j < n; ++j) {
+        const u64 y = (m.sk[j] & mask) >> lo_bit;
+        rank += y < x || (y == x && j < tid);
+      }
+    }
+    __syncthreads();
+    if (tid < n) {
+      m.sk[rank] = mk;
+      m.sv[rank] = mv;
+    }
+    __syncthreads();
+    for (int k = 0; k < SM_ITEMS; ++k)
+      if (sm_at(k) < n) {
+        key[k] = m.sk[sm_at(k)];
+        val[k] = m.sv[sm_at(k)];
+      }
+    __syncthreads();
+    return;
+  }
   for (int shift = lo_bit; shift < bits; shift += 8) {
     for (int d = lane; d < 256; d += 32) m.whist[wid][d] = 0;
     __syncwarp();
-    int rk[RS_ITEMS];
-    for (int k = 0; k < RS_ITEMS; ++k) {
-      const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
-      const int d = li < n ? (int)((key[k] >> shift) & 255) : 256;
+    int rk[SM_ITEMS];
+    for (int k = 0; k < SM_ITEMS; ++k) {
+      const int d = sm_at(k) < n ? (int)((key[k] >> shift) & 255) : 256;
       const unsigned peers = __match_any_sync(0xffffffffu, d);
       const int before = d < 256 ? m.whist[wid][d] : 0;
       rk[k] = before + __popc(peers & ((1u << lane) - 1u));
@@ -404,17 +447,18 @@ __device__ inline void rs_small_passes(RsSmall& m, u64 (&key)[RS_ITEMS], u64 (&v
     }
     __syncthreads();
     int cnt = 0;
-    for (int w = 0; w < NW; ++w) {  // thread = digit (RS_THREADS == 256)
-      const int c = m.whist[w][tid];
-      m.whist[w][tid] = cnt;
-      cnt += c;
-    }
-    int64_t total;
-    m.tstart[tid] = (int32_t)block_excl_scan_i64(cnt, &total);
+    if (tid < 256)
+      for (int w = 0; w < SM_WARPS; ++w) {  // thread = digit
+        const int c = m.whist[w][tid];
+        m.whist[w][tid] = cnt;
+        cnt += c;
+      }
+    u64 total;
+    const u64 start = block_scan<SM_THREADS>((u64)cnt, &total);
+    if (tid < 256) m.tstart[tid] = (int32_t)start;
     __syncthreads();
-    for (int k = 0; k < RS_ITEMS; ++k) {
-      const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
-      if (li < n) {
+    for (int k = 0; k < SM_ITEMS; ++k) {
+      if (sm_at(k) < n) {
         const int d = (int)((key[k] >> shift) & 255);
         const int p = m.tstart[d] + m.whist[wid][d] + rk[k];
         m.sk[p] = key[k];
@@ -422,66 +466,63 @@ __device__ inline void rs_small_passes(RsSmall& m, u64 (&key)[RS_ITEMS], u64 (&v
       }
     }
     __syncthreads();
-    for (int k = 0; k < RS_ITEMS; ++k) {
-      const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
-      if (li < n) {
-        key[k] = m.sk[li];
-        val[k] = m.sv[li];
+    for (int k = 0; k < SM_ITEMS; ++k) {
+      if (sm_at(k) < n) {
+        key[k] = m.sk[sm_at(k)];
+        val[k] = m.sv[sm_at(k)];
       }
     }
     __syncthreads();  // whist, tstart and the staging buffers are rewritten next pass
   }
 }
 
-__global__ void __launch_bounds__(RS_THREADS) k_rs_small(u64* keys, u64* vals, int n, const int32_t* n_dev, int lo_bit,
+extern __shared__ __align__(16) unsigned char small_smem[];
+
+__global__ void __launch_bounds__(SM_THREADS) k_rs_small(u64* keys, u64* vals, int n, const int32_t* n_dev, int lo_bit,
                                                          int bits) {
-  __shared__ RsSmall m;
+  RsSmall& m = *(RsSmall*)small_smem;
   if (n_dev) n = min(n, *n_dev);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  u64 key[RS_ITEMS], val[RS_ITEMS];
-  for (int k = 0; k < RS_ITEMS; ++k) {
-    const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
-    key[k] = li < n ? keys[li] : 0;
-    val[k] = li < n ? vals[li] : 0;
+  u64 key[SM_ITEMS], val[SM_ITEMS];
+  for (int k = 0; k < SM_ITEMS; ++k) {
+    key[k] = sm_at(k) < n ? keys[sm_at(k)] : 0;
+    val[k] = sm_at(k) < n ? vals[sm_at(k)] : 0;
   }
-  rs_small_passes(m, key, val, n, lo_bit, bits);
-  for (int k = 0; k < RS_ITEMS; ++k) {
-    const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
-    if (li < n) {
-      keys[li] = key[k];
-      vals[li] = val[k];
+  rs_small_sort(m, key, val, n, lo_bit, bits);
+  for (int k = 0; k < SM_ITEMS; ++k)
+    if (sm_at(k) < n) {
+      keys[sm_at(k)] = key[k];
+      vals[sm_at(k)] = val[k];
     }
-  }
 }
 
 // Sort by the low 2 * bits key bits, sum per key with zero sums dropped, and
 // with `both` the same records transposed behind them, in (row, col) order
 // (rows from row_off): sort_reduce() for n <= RS_TILE in one launch.
-__global__ void __launch_bounds__(RS_THREADS) k_rs_small_reduce(const u64* keys, const u64* vals, int n,
+__global__ void __launch_bounds__(SM_THREADS) k_rs_small_reduce(const u64* keys, const u64* vals, int n,
                                                                 const int32_t* n_dev, int bits, int both,
                                                                 int64_t row_off, u64* okeys, int64_t* ovals,
                                                                 int32_t* nr) {
-  __shared__ RsSmall m;
+  RsSmall& m = *(RsSmall*)small_smem;
   if (n_dev) n = min(n, *n_dev);
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  u64 key[RS_ITEMS], val[RS_ITEMS];
-  for (int k = 0; k < RS_ITEMS; ++k) {
-    const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
+  const int tid = threadIdx.x;
+  u64 key[SM_ITEMS], val[SM_ITEMS];
+  for (int k = 0; k < SM_ITEMS; ++k) {
+    const int li = sm_at(k);
     key[k] = li < n ? keys[li] : 0;
     val[k] = li < n ? vals[li] : 0;
   }
-  rs_small_passes(m, key, val, n, 0, 2 * bits);
-  // sorted pairs into shared memory, RS_ITEMS consecutive ones per thread
-  for (int k = 0; k < RS_ITEMS; ++k) {
-    const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
+  rs_small_sort(m, key, val, n, 0, 2 * bits);
+  // sorted pairs into shared memory, SM_ITEMS consecutive ones per thread
+  for (int k = 0; k < SM_ITEMS; ++k) {
+    const int li = sm_at(k);
     m.sk[li] = key[k];
     m.sv[li] = val[k];
   }
   __syncthreads();
-  const int i0 = tid * RS_ITEMS;
+  const int i0 = tid * SM_ITEMS;
   int heads = 0;
   int64_t sum = 0;
-  for (int k = 0; k < RS_ITEMS; ++k) {
+  for (int k = 0; k < SM_ITEMS; ++k) {
     const int i = i0 + k;
     key[k] = m.sk[i];
     heads += i < n && (i == 0 || key[k] != m.sk[i - 1]);
@@ -489,14 +530,15 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_small_reduce(const u64* keys,
   }
   // segment numbers, and running sums whose differences at the segments' ends
   // are the segment sums (both modulo 2^64)
-  int64_t nseg64, all;
-  int seg = (int)block_excl_scan_i64(heads, &nseg64);
-  int64_t run = block_excl_scan_i64(sum, &all);
+  u64 nseg64, all64;
+  int seg = (int)block_scan<SM_THREADS>((u64)heads, &nseg64);
+  int64_t run = (int64_t)block_scan<SM_THREADS>((u64)sum, &all64);
   const int nseg = (int)nseg64;
-  u64 hk[RS_ITEMS];
-  int64_t hr[RS_ITEMS];
+  const int64_t all = (int64_t)all64;
+  u64 hk[SM_ITEMS];
+  int64_t hr[SM_ITEMS];
   int hs = 0;
-  for (int k = 0; k < RS_ITEMS; ++k) {
+  for (int k = 0; k < SM_ITEMS; ++k) {
     const int i = i0 + k;
     if (i < n && (i == 0 || key[k] != m.sk[i - 1])) {
       hk[hs] = key[k];
@@ -512,15 +554,15 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_small_reduce(const u64* keys,
   }
   __syncthreads();
   int live = 0;
-  for (int k = 0; k < RS_ITEMS; ++k) {
+  for (int k = 0; k < SM_ITEMS; ++k) {
     const int s = i0 + k;
     hk[k] = s < nseg ? m.sk[s] : 0;
     hr[k] = s < nseg ? (s + 1 < nseg ? (int64_t)m.sv[s + 1] : all) - (int64_t)m.sv[s] : 0;
     live += hr[k] != 0;
   }
-  int64_t nlive;
-  int p = (int)block_excl_scan_i64(live, &nlive);  // its barriers also end the reads above
-  for (int k = 0; k < RS_ITEMS; ++k)
+  u64 nlive;
+  int p = (int)block_scan<SM_THREADS>((u64)live, &nlive);  // its barriers also end the reads above
+  for (int k = 0; k < SM_ITEMS; ++k)
     if (hr[k] != 0) {
       okeys[p] = hk[k];
       ovals[p] = hr[k];
@@ -532,16 +574,16 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_small_reduce(const u64* keys,
   if (!both) return;
   __syncthreads();
   n = (int)nlive;
-  for (int k = 0; k < RS_ITEMS; ++k) {
-    const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
+  for (int k = 0; k < SM_ITEMS; ++k) {
+    const int li = sm_at(k);
     key[k] = li < n ? m.sk[li] : 0;
     val[k] = li < n ? m.sv[li] : 0;
   }
   __syncthreads();
   // the records are in (row, col) order: a stable sort on the new row alone
-  rs_small_passes(m, key, val, n, bits, 2 * bits + 1);
-  for (int k = 0; k < RS_ITEMS; ++k) {
-    const int li = wid * (RS_ITEMS * 32) + k * 32 + lane;
+  rs_small_sort(m, key, val, n, bits, 2 * bits + 1);
+  for (int k = 0; k < SM_ITEMS; ++k) {
+    const int li = sm_at(k);
     if (li < n) {
       okeys[n + li] = key[k];
       ovals[n + li] = (int64_t)val[k];
@@ -872,6 +914,20 @@ bool scan_wait_gives_up(cudaStream_t s) {
   return bad != 0;
 }
 
+// The one-block sorts use 49 KB of shared memory: opted in once per device,
+// thread and kernel.
+static void small_smem_opt_in(const void* f) {
+  static thread_local const void* done[2] = {nullptr, nullptr};
+  static thread_local int done_dev = -1;
+  int dev = 0;
+  CK(cudaGetDevice(&dev));
+  if (done_dev != dev) done[0] = done[1] = nullptr;
+  done_dev = dev;
+  if (done[0] == f || done[1] == f) return;
+  CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RsSmall)));
+  done[done[0] ? 1 : 0] = f;
+}
+
 // Launches the sort of n pairs (an upper bound with x.n_dev).  A plain sort's
 // result is in (keys, vals) afterwards, which may have been swapped with (tk,
 // tv); a transposing one's lies behind its input.
@@ -945,7 +1001,8 @@ void radix_sort_pairs(u64*& keys, u64*& vals, u64*& tk, u64*& tv, int64_t n, int
                       int lo_bit, const int32_t* n_dev) {
   if (n <= 1 || bits <= lo_bit) return;
   if (n <= RS_TILE) {
-    k_rs_small<<<1, RS_THREADS, 0, s>>>(keys, vals, (int)n, n_dev, lo_bit, bits);
+    small_smem_opt_in((const void*)k_rs_small);
+    k_rs_small<<<1, SM_THREADS, sizeof(RsSmall), s>>>(keys, vals, (int)n, n_dev, lo_bit, bits);
     CKL("k_rs_small");
     return;
   }
@@ -955,10 +1012,11 @@ void radix_sort_pairs(u64*& keys, u64*& vals, u64*& tk, u64*& tv, int64_t n, int
 void sort_reduce(DBuf<u64>& k, DBuf<u64>& v, DBuf<u64>& tk, DBuf<u64>& tv, int64_t n, const int32_t* n_dev, int bits,
                  bool both, int64_t row_off, u64* okeys, int64_t* ovals, int32_t* nr, Prims& P, cudaStream_t s) {
   if (n <= RS_TILE) {
-    // one block sorts, sums and transposes: 7.6 us for a few records and 11.4
+    // one block sorts, sums and transposes: 4.3 us for a few records and 8.8
     // for some hundred, where the launches of the larger sizes take 16.4 and
     // 23.5 and the gaps between them
-    k_rs_small_reduce<<<1, RS_THREADS, 0, s>>>(k.p, v.p, (int)n, n_dev, bits, both ? 1 : 0, row_off, okeys, ovals, nr);
+    small_smem_opt_in((const void*)k_rs_small_reduce);
+    k_rs_small_reduce<<<1, SM_THREADS, sizeof(RsSmall), s>>>(k.p, v.p, (int)n, n_dev, bits, both ? 1 : 0, row_off, okeys, ovals, nr);
     CKL("k_rs_small_reduce");
     return;
   }

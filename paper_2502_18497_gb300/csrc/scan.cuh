@@ -94,50 +94,60 @@ __device__ inline void look_back(u64* st, int64_t tile, const int64_t (&agg)[NC]
     if (lane == k) atomicExch((unsigned long long*)&st[tile * NC + k], ((u64)(pre[k] + agg[k]) << 10) | tag | 2u);
 }
 
-// A kernel's result for the host: 64-bit words into the mapped page, then the
-// read's sequence number (written by one thread).
+// A kernel's result for the host: each 32-bit word goes into the mapped page
+// as one 64-bit store of (sequence number << 32 | word), so that a word tells
+// by itself whether it belongs to this read.  The host waits for every word;
+// nothing has to order them (a fence to the host between the payload and a
+// sequence number cost 1.5 us a read).
 struct Pub {
-  int64_t* page;  // word 0: sequence number, then the payload
-  int64_t seq;
+  u64* page;
+  uint32_t seq;
 };
+
+__device__ inline void put_word(u64* page, uint32_t seq, int w, uint32_t v) {
+  *(volatile u64*)(page + w) = ((u64)seq << 32) | v;
+}
 
 template <int N>
 __device__ inline void publish(const Pub& p, const int64_t (&v)[N]) {
 #pragma unroll
-  for (int i = 0; i < N; ++i) p.page[1 + i] = v[i];
-  __threadfence_system();  // the payload is visible to the host before the sequence number
-  *(volatile int64_t*)p.page = p.seq;
+  for (int i = 0; i < N; ++i) {
+    put_word(p.page, p.seq, 2 * i, (uint32_t)(u64)v[i]);
+    put_word(p.page, p.seq, 2 * i + 1, (uint32_t)((u64)v[i] >> 32));
+  }
 }
 
 // Values that a kernel hands to the host when its last block is done: device
-// words (4-byte multiples) copied into the mapped page, then the sequence
-// number.  The ticket counts the blocks that are through (zero before the
-// launch).  seq = 0: nothing to hand over.
+// words (4-byte multiples).  The ticket counts the blocks that are through
+// (zero before the launch).  seq = 0: nothing to hand over.
 constexpr int TAIL_MAX = 8;
 struct Tail {
   const uint32_t* src[TAIL_MAX];
   int32_t off[TAIL_MAX], words[TAIL_MAX];  // in 4-byte words of the payload
   int32_t n;
-  int64_t* page;
-  int64_t seq;
+  u64* page;
+  uint32_t seq;
   int32_t* ticket;
 };
+
+__device__ inline void put_tail(const Tail& t) {
+  for (int i = 0; i < t.n; ++i)
+    for (int w = threadIdx.x; w < t.words[i]; w += blockDim.x)
+      put_word(t.page, t.seq, t.off[i] + w, __ldcg(t.src[i] + w));
+}
 
 // Called by every thread of every block as the kernel's last step: a separate
 // one-block kernel for the copy costs 2.6 us and the gap in front of it.
 __device__ inline void pub_tail(const Tail& t) {
   if (t.seq == 0) return;
-  __shared__ int s_last;
   __threadfence();  // this thread's writes, before its block's ticket
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(t.ticket, 1) == (int)gridDim.x - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  uint32_t* pay = (uint32_t*)(t.page + 1);
-  for (int i = 0; i < t.n; ++i)
-    for (int w = threadIdx.x; w < t.words[i]; w += blockDim.x) pay[t.off[i] + w] = __ldcg(t.src[i] + w);
-  __threadfence_system();  // the payload is visible to the host before the sequence number
-  __syncthreads();
-  if (threadIdx.x == 0) *(volatile int64_t*)t.page = t.seq;
+  if (gridDim.x > 1) {
+    __shared__ int s_last;
+    if (threadIdx.x == 0) s_last = atomicAdd(t.ticket, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+  }
+  put_tail(t);
 }

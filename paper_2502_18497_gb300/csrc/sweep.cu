@@ -29,6 +29,10 @@ std::atomic<int64_t> g_hub_table_slots{HUB_TABLE_SLOTS};
 static_assert(BIN_MAX[0] == HG8 / 2 && BIN_MAX[1] == HG32 / 2 && BIN_MAX[2] == 2048 / 2 &&
                   BIN_MAX[3] == HB / 2 && BIN_MAX[3] == MID_DEG,
               "bin bounds and table sizes");
+// Nodes up to which a sweep uses one kernel for all degrees: one edge on 10k
+// vertices took 621 us a batch with a launch per bin, 531 with one; with 4096
+// here, batches of 100 to 1000 measure the same as with 1024 (within 1%).
+constexpr int SWEEP_FEW = 1024;
 constexpr int EVAL_CH = 1024;  // hub table slots evaluated per block (4096: one block a hub, 17 us where this takes 16)
 
 // ---------------------------------------------------------------- expand
@@ -87,20 +91,28 @@ __global__ void k_expand(Adj<WT> out, Adj<WT> in, ChunkMap m, int32_t* stamp, in
   pub_tail(tail);
 }
 
-// U = U* = the existing nodes of a frontier list (each listed once).
+// U = U* = the existing nodes of a frontier list (each listed once), and the
+// entries of their rows (which bound the first candidate set).
 __global__ void k_frontier(const int32_t* list, const int32_t* nlist, const uint8_t* alive, int32_t* lU, int32_t* nU,
-                           int32_t* stU, int32_t epU, int32_t* lUs, int32_t* nUs, Tail tail) {
+                           int32_t* stU, int32_t epU, int32_t* lUs, int32_t* nUs, const int32_t* len_out,
+                           const int32_t* len_in, int64_t* deg, Tail tail) {
   const int32_t nl = *nlist;
+  int64_t sum = 0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   // warp-uniform trip counts, so that appends aggregate over the warp
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < nl; base += stride) {
     const int64_t t = base + (threadIdx.x & 31);
     const int32_t v = t < nl ? list[t] : 0;
     const bool on = t < nl && (!alive || alive[v]);
-    if (on) stU[v] = epU;
+    if (on) {
+      stU[v] = epU;
+      sum += (int64_t)len_out[v] + (len_in ? len_in[v] : 0);
+    }
     warp_append(on, v, lU, nU);
     warp_append(on, v, lUs, nUs);
   }
+  sum = warp_sum_i64(sum);
+  if ((threadIdx.x & 31) == 0 && sum) atomic_add_i64(deg, sum);
   pub_tail(tail);
 }
 
@@ -1430,8 +1442,11 @@ void expand_set(ldl_ctx& c, int r, const int32_t* list, int idx_n, int32_t* stam
 
 void frontier(ldl_ctx& c, int r, int32_t epU, const HostRead* rr, int n) {
   LevelState& L = c.lv[r];
-  k_frontier<<<grid_for(c.n, TPB, 2), TPB, 0, c.s>>>(L.lA.p, c.cp[K_A0 + r], r ? L.alive.p : nullptr, c.lU.p, c.cp[K_U],
-                                                     c.stU.p, epU, c.lUstar.p, c.cp[K_USTAR], tail_begin(c, rr, n));
+  const int32_t* lo = r == 0 ? adj_out0(c).len : adj_out(c, r).len;
+  const int32_t* li = !c.directed ? nullptr : r == 0 ? adj_in0(c).len : adj_in(c, r).len;
+  k_frontier<<<grid_for(L.ubA, TPB, 2), TPB, 0, c.s>>>(L.lA.p, c.cp[K_A0 + r], r ? L.alive.p : nullptr, c.lU.p,
+                                                       c.cp[K_U], c.stU.p, epU, c.lUstar.p, c.cp[K_USTAR], lo, li,
+                                                       c.sums, tail_begin(c, rr, n));
   CKL("k_frontier");
   tail_wait(c, rr, n);
 }
@@ -1454,7 +1469,8 @@ static bool sweep_gain_fits_i64(const ldl_ctx& c) {
 
 // The bins of nodes with at most 2048 entries, in the gain type GT.
 template <class WT, int MODE, class GT>
-static void sweep_bins(ldl_ctx& c, const SweepArgs<WT>& A, int64_t n_hint, cudaEvent_t* kev) {
+static void sweep_bins(ldl_ctx& c, const SweepArgs<WT>& A, int64_t n_hint, bool few, cudaEvent_t* kev) {
+  if (!few) {
   k_sweep_group<WT, MODE, 8, GT><<<grid_for(n_hint * 8, TPB, 6), TPB, 0, c.s>>>(A, c.binT.p, c.cp[K_TINY]);
   CKL("k_sweep_group<8>");
   if (kev) CK(cudaEventRecord(kev[1], c.s));
@@ -1467,6 +1483,7 @@ static void sweep_bins(ldl_ctx& c, const SweepArgs<WT>& A, int64_t n_hint, cudaE
     CKL("k_sweep_block(mid1)");
   }
   if (kev) CK(cudaEventRecord(kev[3], c.s));
+  }
   {
     const size_t sm = (size_t)tab_slot<GT> * HB;
     CK(cudaFuncSetAttribute(k_sweep_block<WT, MODE, 256, HB, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1533,12 +1550,16 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   // count; should there be hubs after all, they are swept and the filter,
   // which leaves its scratch as it found it, runs again on all candidates.
   uint8_t& expect = c.hubs_seen[r][MODE];
+  // Few nodes are all swept by one block each, whatever their degree: a launch
+  // per degree bin costs more than it saves (see SWEEP_FEW).
+  const bool few = n_hint <= SWEEP_FEW && !c.kstats;
   const bool early = expect || c.kstats;
   k_bin<WT><<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(out, in, c.directed, list, c.cp[idx_n], c.binT.p, c.cp[K_TINY],
                                                      c.binS.p, c.cp[K_SMALL], c.binM.p, c.cp[K_MID], c.binM2.p,
                                                      c.cp[K_MID2], c.binC.p, c.cp[K_CLU], c.binL.p, c.cp[K_LARGE],
-                                                     c.binLsz.p, c.sums, c.bin_deg[0], c.bin_deg[1], c.bin_deg[2],
-                                                     c.bin_deg[3], std::min(c.prm.cluster_max_deg, CLUSTER_DEG),
+                                                     c.binLsz.p, c.sums, few ? -1 : c.bin_deg[0],
+                                                     few ? -1 : c.bin_deg[1], few ? -1 : c.bin_deg[2],
+                                                     few ? MID_DEG : c.bin_deg[3], std::min(c.prm.cluster_max_deg, CLUSTER_DEG),
                                                      early ? tail_begin(c, rb, 8) : Tail{});
   CKL("k_bin");
   // Every bin but the hubs is swept by a grid-stride kernel that reads its
@@ -1546,8 +1567,8 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   // and the host's wait below overlaps them.  n_hint bounds every bin.
   cudaEvent_t* kev = c.kstats ? kstats_events(c) : nullptr;
   if (kev) CK(cudaEventRecord(kev[0], c.s));
-  if (sweep_gain_fits_i64(c)) sweep_bins<WT, MODE, int64_t>(c, A, n_hint, kev);
-  else sweep_bins<WT, MODE, i128>(c, A, n_hint, kev);
+  if (sweep_gain_fits_i64(c)) sweep_bins<WT, MODE, int64_t>(c, A, n_hint, few, kev);
+  else sweep_bins<WT, MODE, i128>(c, A, n_hint, few, kev);
   if (kev) CK(cudaEventRecord(kev[4], c.s));
   if (c.prm.cluster_max_deg > c.bin_deg[3]) {
     const size_t sm = (sizeof(int64_t) + sizeof(int32_t)) * CL_SLOTS;
@@ -1766,6 +1787,7 @@ void rollback_move(ldl_ctx& c, int r, int32_t nb, int32_t ntc) {
 }
 
 void mark_moved(ldl_ctx& c, int r, int32_t nb, int32_t epMv, int32_t epM0, int32_t epU, int32_t nU) {
+  c.ubU = std::min<int64_t>(c.n, c.ubU + nU);
   k_mark_moved<<<grid_for(std::max(nb, nU), TPB), TPB, 0, c.s>>>(
       nb, c.bv.p, c.stMv.p, epMv, c.lMv.p, c.cp[K_MV], r == 0 ? c.stM0.p : nullptr, epM0, c.lM0.p, c.cp[K_M0], nU,
       c.lU.p, c.stU.p, epU, c.lUstar.p, c.cp[K_USTAR]);
