@@ -325,6 +325,9 @@ struct DevScalars {
   int64_t agg_recs;  // aggregate records of the batch
   int64_t seg_n;     // CSR update: segments
   int64_t plan_bad;  // last CSR update that met an impossible record
+  // names its totals in a host read (pool slots, segments, scratch, rebuild,
+  // records, whether one was impossible); they go there from registers
+  int64_t plan[6];
   int64_t sw_entries[KS_GROUPS];  // per sweep kernel group: adjacency entries read since statistics
                                   // were enabled
   int64_t sw_bytes[KS_GROUPS];    // algorithmic bytes of the same sweeps

@@ -21,12 +21,17 @@ namespace {
 constexpr int TPB = 256;
 
 // ---- planning an update: records -> rows (segments) -> what each row needs
-// A record list: n records, or mul * *n_dev of them with n an upper bound.
+// A record list: n records, or mul * *n_dev of them with n an upper bound; none
+// where the gate is given and zero.
 struct RecN {
   int64_t n;
   const int32_t* n_dev;
   int mul;
-  __device__ int64_t count() const { return n_dev ? min(n, (int64_t)mul * *n_dev) : n; }
+  const int32_t* gate;
+  __device__ int64_t count() const {
+    if (gate && *gate == 0) return 0;
+    return n_dev ? min(n, (int64_t)mul * *n_dev) : n;
+  }
 };
 
 // Per-record and per-segment arrays of an update (see CsrScratch).
@@ -39,6 +44,7 @@ struct PlanOut {
   int64_t* nseg;  // device: number of segments
   u64* bad;       // device: the last plan number that met an impossible record
   u64 plan;       // this plan's number
+  const void* totals;  // DevScalars::plan: names the totals in a tail
 };
 
 struct Rec {
@@ -107,10 +113,12 @@ __device__ inline SegNeed plan_segment(const PlanOut& o, int64_t s, int64_t a, i
   return q;
 }
 
-__device__ inline void publish_plan(const Pub& pub, const PlanOut& o, int64_t need, int64_t nseg, int64_t stot,
-                                    int64_t wtot, int64_t nrec) {
+// The plan's totals straight into the tail's entry for them (its other values
+// are of earlier kernels).
+__device__ inline void put_totals(const Tail& t, const PlanOut& o, int64_t need, int64_t nseg, int64_t stot,
+                                  int64_t wtot, int64_t nrec) {
   const int64_t v[6] = {need, nseg, stot, wtot, nrec, (int64_t)(*(volatile u64*)o.bad == o.plan)};
-  publish<6>(pub, v);
+  put_values(t, o.totals, v);
 }
 
 constexpr int PL_TPB = 512;  // records (segments) per tile: one each per thread, as a match is a chain of loads
@@ -156,10 +164,10 @@ __global__ void __launch_bounds__(PL_TPB) k_plan_records(const int64_t* off, con
   }
 }
 
-// Segments: scratch, rebuild and pool offsets by one pass; the last tile
-// publishes the totals to the host.
+// Segments: scratch, rebuild and pool offsets by one pass; the last tile hands
+// the totals to the host.
 __global__ void __launch_bounds__(PL_TPB) k_plan_segments(const int32_t* len, const int32_t* cap, RecN rn, PlanOut o,
-                                                          LookBack q, Pub pub) {
+                                                          LookBack q, Tail tail) {
   __shared__ int64_t s_tile, s_pre[3];
   __shared__ int64_t s_sum[3];
   if (threadIdx.x == 0) s_tile = atomicAdd(q.ctr, 1);
@@ -189,10 +197,13 @@ __global__ void __launch_bounds__(PL_TPB) k_plan_segments(const int32_t* len, co
     o.woff[s] = s_pre[1] + (int64_t)ex[1];
     o.noff[s] = s_pre[2] + (int64_t)ex[2];
   }
-  if (threadIdx.x == 0 && (tile + 1) * PL_TPB >= nseg) {
-    o.soff[nseg] = s_sum[0];
-    o.woff[nseg] = s_sum[1];
-    publish_plan(pub, o, s_sum[2], nseg, s_sum[0], s_sum[1], n);
+  if ((tile + 1) * PL_TPB >= nseg) {
+    if (threadIdx.x == 0) {
+      o.soff[nseg] = s_sum[0];
+      o.woff[nseg] = s_sum[1];
+      put_totals(tail, o, s_sum[2], nseg, s_sum[0], s_sum[1], n);
+    }
+    put_tail(tail, o.totals);
   }
 }
 
@@ -202,7 +213,7 @@ template <class WT>
 __global__ void __launch_bounds__(PS_TPB) k_plan_small(const int64_t* off, const int32_t* len, const int32_t* cap,
                                                        const int32_t* col, const WT* w, const u64* keys,
                                                        const int64_t* delta, RecN rn, int bshift, PlanOut o,
-                                                       DelTrack t, Pub pub) {
+                                                       DelTrack t, Tail tail) {
   const int64_t n = rn.count(), i = threadIdx.x;
   Rec r{0, 0, 0};
   if (i < n) r = match_record<WT>(off, len, col, w, keys, delta, i, bshift, o, t);
@@ -239,8 +250,9 @@ __global__ void __launch_bounds__(PS_TPB) k_plan_small(const int64_t* off, const
   if (i == 0) {
     o.soff[nseg] = (int64_t)ts;
     o.woff[nseg] = (int64_t)tw;
-    publish_plan(pub, o, (int64_t)tp, nseg, (int64_t)ts, (int64_t)tw, n);
+    put_totals(tail, o, (int64_t)tp, nseg, (int64_t)ts, (int64_t)tw, n);
   }
+  put_tail(tail, o.totals);
 }
 
 // ---- undo log (batches that may be rolled back)
@@ -539,10 +551,16 @@ static void compact_pool(SlackCSR<WT>& g, int64_t extra, CsrScratch& S, Prims& P
   g.pool_top = total;
 }
 
+static PlanOut plan_out(CsrScratch& S, DevScalars* d_sc) {
+  return PlanOut{S.pos.p,    S.lb.p,     S.segid.p, S.pins.p, S.pdel.p, S.oldw.p,     S.seg.p,
+                 S.segrow.p, S.newcap.p, S.soff.p,  S.woff.p, S.noff.p, &d_sc->seg_n, (u64*)&d_sc->plan_bad,
+                 S.plans,    d_sc->plan};
+}
+
 template <class WT>
-int64_t csr_apply(SlackCSR<WT>& g, const u64* keys, const int64_t* delta, int64_t n_max, const int32_t* n_dev, int mul,
-                  int bshift, CsrScratch& S, Prims& P, cudaStream_t s, DevScalars* d_sc, const DelTrack* trk) {
-  if (n_max <= 0) return 0;
+void csr_plan(const SlackCSR<WT>& g, const CsrRecords& r, CsrScratch& S, Prims& P, cudaStream_t s, DevScalars* d_sc,
+              const DelTrack* trk, const Tail& tail) {
+  const int64_t n_max = r.n_max;
   S.pos.reserve(n_max + 1, s);
   S.lb.reserve(n_max + 1, s);
   S.oldw.reserve(n_max + 1, s);
@@ -556,31 +574,48 @@ int64_t csr_apply(SlackCSR<WT>& g, const u64* keys, const int64_t* delta, int64_
   S.soff.reserve(n_max + 2, s);
   S.woff.reserve(n_max + 2, s);
   S.noff.reserve(n_max + 2, s);
-  const RecN rn{n_max, n_dev, mul};
-  const PlanOut o{S.pos.p,  S.lb.p,     S.segid.p,  S.pins.p, S.pdel.p, S.oldw.p,     S.seg.p,
-                  S.segrow.p, S.newcap.p, S.soff.p, S.woff.p, S.noff.p, &d_sc->seg_n, (u64*)&d_sc->plan_bad,
-                  ++S.plans};
+  const RecN rn{n_max, r.n_dev, r.mul, r.gate};
+  ++S.plans;
+  const PlanOut o = plan_out(S, d_sc);
   const DelTrack t = trk ? *trk : DelTrack{};
   // Up to one record per thread of a block, one launch plans the update: 6.2 us
   // for a few records and 7.5 for some hundred, where the two tiled launches
   // take 8.9 and 9.9 and the gap between them.  Beyond, one block would match
   // several records per thread one after the other.
-  const Pub pub = P.pub_begin(P.rd_owner);
   if (n_max <= PS_TPB) {
-    k_plan_small<WT><<<1, PS_TPB, 0, s>>>(g.off.p, g.len.p, g.cap.p, g.col.p, g.w.p, keys, delta, rn, bshift, o, t,
-                                          pub);
+    k_plan_small<WT><<<1, PS_TPB, 0, s>>>(g.off.p, g.len.p, g.cap.p, g.col.p, g.w.p, r.keys, r.delta, rn, r.bshift, o,
+                                          t, tail);
     CKL("k_plan_small");
   } else {
     const int tiles = div_up(n_max, PL_TPB);
     const LookBack q1 = look_back_begin(P, 3 * (int64_t)tiles, s);
-    k_plan_records<WT><<<tiles, PL_TPB, 0, s>>>(g.off.p, g.len.p, g.col.p, g.w.p, keys, delta, rn, bshift, o, t, q1);
+    k_plan_records<WT><<<tiles, PL_TPB, 0, s>>>(g.off.p, g.len.p, g.col.p, g.w.p, r.keys, r.delta, rn, r.bshift, o, t,
+                                                q1);
     CKL("k_plan_records");
     const LookBack q2 = look_back_begin(P, 3 * (int64_t)tiles, s);
-    k_plan_segments<<<tiles, PL_TPB, 0, s>>>(g.len.p, g.cap.p, rn, o, q2, pub);
+    k_plan_segments<<<tiles, PL_TPB, 0, s>>>(g.len.p, g.cap.p, rn, o, q2, tail);
     CKL("k_plan_segments");
   }
+}
+
+template <class WT>
+int64_t csr_apply(SlackCSR<WT>& g, const CsrRecords& r, CsrScratch& S, Prims& P, cudaStream_t s, DevScalars* d_sc,
+                  const DelTrack* trk) {
+  if (r.n_max <= 0) return 0;
   int64_t tot[6];
-  P.pub_wait(P.rd_owner, tot, 6);
+  const HostRead rr{d_sc->plan, tot, sizeof(tot)};
+  csr_plan<WT>(g, r, S, P, s, d_sc, trk, P.tail_begin(P.rd_owner, &rr, 1));
+  P.tail_wait(P.rd_owner, &rr, 1);
+  return csr_finish<WT>(g, r, tot, S, P, s, d_sc);
+}
+
+template <class WT>
+int64_t csr_finish(SlackCSR<WT>& g, const CsrRecords& r, const int64_t (&tot)[6], CsrScratch& S, Prims& P,
+                   cudaStream_t s, DevScalars* d_sc) {
+  const u64* keys = r.keys;
+  const int64_t* delta = r.delta;
+  const int bshift = r.bshift;
+  const PlanOut o = plan_out(S, d_sc);
   const int64_t need = tot[0], nseg = tot[1], stotal = tot[2], wtotal = tot[3], nrec = tot[4];
   if (tot[5]) ldl_throw(LDL_E_INVALID, "internal: adjacency update would make a weight negative");
   if (nrec <= 0) return 0;
@@ -709,7 +744,15 @@ template void csr_build<int32_t>(SlackCSR<int32_t>&, int64_t, const u64*, const 
                                  CsrScratch&, Prims&, cudaStream_t);
 template void csr_build<int64_t>(SlackCSR<int64_t>&, int64_t, const u64*, const int64_t*, int64_t, int, int,
                                  CsrScratch&, Prims&, cudaStream_t);
-template int64_t csr_apply<int32_t>(SlackCSR<int32_t>&, const u64*, const int64_t*, int64_t, const int32_t*, int, int,
-                                    CsrScratch&, Prims&, cudaStream_t, DevScalars*, const DelTrack*);
-template int64_t csr_apply<int64_t>(SlackCSR<int64_t>&, const u64*, const int64_t*, int64_t, const int32_t*, int, int,
-                                    CsrScratch&, Prims&, cudaStream_t, DevScalars*, const DelTrack*);
+template void csr_plan<int32_t>(const SlackCSR<int32_t>&, const CsrRecords&, CsrScratch&, Prims&, cudaStream_t, DevScalars*,
+                                const DelTrack*, const Tail&);
+template int64_t csr_finish<int32_t>(SlackCSR<int32_t>&, const CsrRecords&, const int64_t (&)[6], CsrScratch&, Prims&,
+                                     cudaStream_t, DevScalars*);
+template int64_t csr_apply<int32_t>(SlackCSR<int32_t>&, const CsrRecords&, CsrScratch&, Prims&, cudaStream_t, DevScalars*,
+                                    const DelTrack*);
+template void csr_plan<int64_t>(const SlackCSR<int64_t>&, const CsrRecords&, CsrScratch&, Prims&, cudaStream_t, DevScalars*,
+                                const DelTrack*, const Tail&);
+template int64_t csr_finish<int64_t>(SlackCSR<int64_t>&, const CsrRecords&, const int64_t (&)[6], CsrScratch&, Prims&,
+                                     cudaStream_t, DevScalars*);
+template int64_t csr_apply<int64_t>(SlackCSR<int64_t>&, const CsrRecords&, CsrScratch&, Prims&, cudaStream_t, DevScalars*,
+                                    const DelTrack*);

@@ -60,11 +60,32 @@ void csr_txn_commit(SlackCSR<WT>& g, cudaStream_t s);
 template <class WT>
 cudaError_t csr_txn_rollback(SlackCSR<WT>& g, cudaStream_t s);
 
+// Records of an update, key (row << bshift | col) and delta, sorted by key and
+// unique: n_max of them, or mul * *n_dev (device count, n_max an upper bound);
+// none where the gate is given and *gate is zero when the update is planned.
+struct CsrRecords {
+  const u64* keys;
+  const int64_t* delta;
+  int64_t n_max;
+  const int32_t* n_dev;
+  int mul;
+  int bshift;
+  const int32_t* gate = nullptr;
+};
+
 // Add delta to each record's entry: absent entries are inserted, entries that
-// reach zero are removed (their endpoints go to *trk when given).  n_max
-// records, or mul * *n_dev of them (device count, n_max an upper bound).
-// Waits for the host once (pool growth decision) and returns the number of
-// records.
+// reach zero are removed (their endpoints go to *trk when given).  In two
+// halves: csr_plan launches the planning, whose last kernel hands over `tail`
+// (the caller reads d_sc->plan with it and waits), and csr_finish, given those
+// totals, applies the update and returns the number of records.  No other
+// update is planned in between.
 template <class WT>
-int64_t csr_apply(SlackCSR<WT>& g, const u64* keys, const int64_t* delta, int64_t n_max, const int32_t* n_dev, int mul,
-                  int bshift, CsrScratch& S, Prims& P, cudaStream_t s, DevScalars* d_sc, const DelTrack* trk = nullptr);
+void csr_plan(const SlackCSR<WT>& g, const CsrRecords& r, CsrScratch& S, Prims& P, cudaStream_t s, DevScalars* d_sc,
+              const DelTrack* trk, const Tail& tail);
+template <class WT>
+int64_t csr_finish(SlackCSR<WT>& g, const CsrRecords& r, const int64_t (&tot)[6], CsrScratch& S, Prims& P,
+                   cudaStream_t s, DevScalars* d_sc);
+// both, with the wait between them
+template <class WT>
+int64_t csr_apply(SlackCSR<WT>& g, const CsrRecords& r, CsrScratch& S, Prims& P, cudaStream_t s, DevScalars* d_sc,
+                  const DelTrack* trk = nullptr);

@@ -208,11 +208,6 @@ inline int64_t* Kin_of(ldl_ctx& c) { return c.directed ? c.Kin.p : c.Kout.p; }
 // has reached this point: a one-block kernel writes them into the pinned page,
 // which the host polls (a stream error ends the wait).
 void host_read(ldl_ctx& c, const HostRead* r, int n);
-// The same for values that a kernel publishes itself (scan.cuh): the page and
-// the sequence number for it, then the wait for its n payload words.  One
-// read at a time: nothing else is read between the two.
-Pub pub_begin(ldl_ctx& c);
-void pub_wait(ldl_ctx& c, int64_t* out, int n);
 int32_t rd_cnt(ldl_ctx& c, int idx);
 void zero_cnt(ldl_ctx& c, int idx);
 // `words` zeroed words, 16-byte aligned: from the arena, else `home` cleared.

@@ -387,12 +387,21 @@ __global__ void k_reset_par(const int32_t* lD, int32_t nD, int32_t* par, int64_t
 }
 
 // ---------------------------------------------------------------- split
+// The split may be launched behind a sweep before the host knows whether the
+// sweep ends the level's moves.  It runs only if it does: no move was accepted,
+// no hub row is still to be swept and the filter finished.
+struct SplitGate {
+  const int32_t *nb, *hubs, *stat;  // null: open
+  __device__ bool open() const { return !nb || (*nb == 0 && (!hubs || *hubs == 0) && *stat != -2); }
+};
+
 // TouchedRefined of a batch update (see split()).  The refined communities
 // holding an endpoint of a deleted level-r arc are re-checked (before any
 // node leaves, so with their current parents).
 __global__ void k_brk_check(const int32_t* lK, const int32_t* nK, const uint8_t* alive, const int32_t* par,
-                            int32_t* stX, int32_t epX, int32_t* lX, int32_t* nX, int32_t* ckf, int32_t epF) {
-  const int32_t n = *nK;
+                            int32_t* stX, int32_t epX, int32_t* lX, int32_t* nX, int32_t* ckf, int32_t epF,
+                            SplitGate gate) {
+  const int32_t n = gate.open() ? *nK : 0;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t z = lK[k];
     if (alive[z] && par[z] >= 0) {
@@ -409,8 +418,8 @@ __global__ void k_leave(const int32_t* lU, const int32_t* nU, const uint8_t* ali
                         const int32_t* labN, int32_t* par, int32_t* par_old, const int64_t* kout, const int64_t* kin,
                         int64_t* kout1, int64_t* kin1, int32_t* cnt1, int directed, int32_t* stL, int32_t epL,
                         int32_t* stD, int32_t epD, int32_t* lD, int32_t* nD, int32_t* stX, int32_t epX, int32_t* lX,
-                        int32_t* nX, int32_t* nbr, Tail tail) {
-  const int32_t n = *nU;
+                        int32_t* nX, int32_t* nbr, SplitGate gate, Tail tail) {
+  const int32_t n = gate.open() ? *nU : 0;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t u = lU[k];
     if (!alive[u]) continue;
@@ -1066,24 +1075,33 @@ static void combine_in_out(ldl_ctx& c, const u64* keys, const u64* vals, int64_t
   CK(cudaMemcpyAsync(c.rv2.p + nr, c.trv.p, sizeof(u64) * (size_t)nr, cudaMemcpyDeviceToDevice, c.s));
 }
 
+// Where level r's update records the endpoints of arcs that disappear.  A
+// deleted arc can only disconnect the refined community holding both of its
+// endpoints (refined communities are connected); until the level's next split
+// its parents change only where a node empties and leaves its parent.
+static DelTrack del_track(ldl_ctx& c, int r) {
+  LevelState& L = c.lv[r];
+  return DelTrack{L.stK.p, L.brk_ep, L.lK.p, c.cp[K_BRK0 + r], c.n, r < c.T ? L.par.p : nullptr};
+}
+
+// m records (both directions of a directed level) were applied: arcs
+static int64_t applied(ldl_ctx& c, int r, int64_t m) {
+  if (c.directed) m /= 2;
+  c.lv[r].ubK = std::min<int64_t>(c.n, c.lv[r].ubK + 2 * m);
+  return m;
+}
+
 // Applies sorted unique records (directed: followed by their in-direction
 // copies) to a level's adjacency; the endpoints of arcs that disappear are
 // recorded for the level's next refinement.  nr records, or *n_dev of them
 // with nr an upper bound; returns their number.
 static int64_t apply_records(ldl_ctx& c, int r, const u64* keys, const int64_t* vals, int64_t nr,
                              const int32_t* n_dev) {
-  LevelState& Lr = c.lv[r];
-  // a deleted arc can only disconnect the refined community holding both of
-  // its endpoints (refined communities are connected); until the level's next
-  // split its parents change only where a node empties and leaves its parent
-  const DelTrack trk{Lr.stK.p, Lr.brk_ep, Lr.lK.p, c.cp[K_BRK0 + r], c.n, r < c.T ? Lr.par.p : nullptr};
-  const int mul = c.directed ? 2 : 1;
-  const int64_t m = r == 0 ? csr_apply<int32_t>(c.lv[0].out0, keys, vals, mul * nr, n_dev, mul, c.bits, c.CS, c.P, c.s,
-                                                c.d_sc, &trk)
-                           : csr_apply<int64_t>(c.lv[r].out, keys, vals, mul * nr, n_dev, mul, c.bits, c.CS, c.P, c.s,
-                                                c.d_sc, &trk);
-  Lr.ubK = std::min<int64_t>(c.n, Lr.ubK + 2 * m / mul);
-  return m / mul;
+  const CsrRecords rec{keys, vals, (c.directed ? 2 : 1) * nr, n_dev, c.directed ? 2 : 1, c.bits};
+  const DelTrack trk = del_track(c, r);
+  const int64_t m = r == 0 ? csr_apply<int32_t>(c.lv[0].out0, rec, c.CS, c.P, c.s, c.d_sc, &trk)
+                           : csr_apply<int64_t>(c.lv[r].out, rec, c.CS, c.P, c.s, c.d_sc, &trk);
+  return applied(c, r, m);
 }
 
 static Chain chain_of(ldl_ctx& c, const int32_t* epA) {
@@ -1145,6 +1163,36 @@ void flush_level(ldl_ctx& c, int q, int64_t known) {
   sort_reduce(L.pk, L.pv, c.tk, c.tv, n, nullptr, c.bits, c.directed, c.n, c.flk.p, c.flv.p, nr, c.P, c.s);
   c.res.pending_records += n;
   c.res.pending_applied += apply_records(c, q, c.flk.p, c.flv.p, n, nr);
+}
+
+static CsrRecords flush_records(ldl_ctx& c, int64_t n, const int32_t* gate) {
+  const int mul = c.directed ? 2 : 1;
+  return CsrRecords{c.flk.p, c.flv.p, mul * n, c.cp[K_FL], mul, c.bits, gate};
+}
+
+void flush_plan(ldl_ctx& c, int q, const int32_t* gate, HostRead* rr, int n, int64_t (&tot)[6]) {
+  LevelState& L = c.lv[q];
+  const int64_t ub = L.pend_ub;
+  c.flk.reserve((c.directed ? 2 : 1) * ub + 1, c.s);
+  c.flv.reserve((c.directed ? 2 : 1) * ub + 1, c.s);
+  zero_cnt(c, K_FL);
+  // sorting the list changes its order only: it stays valid if the gate is shut
+  sort_reduce(L.pk, L.pv, c.tk, c.tv, ub, c.cp[K_PEND0 + q], c.bits, c.directed, c.n, c.flk.p, c.flv.p, c.cp[K_FL], c.P,
+              c.s);
+  rr[n] = {c.d_sc->plan, tot, sizeof(tot)};
+  const DelTrack trk = del_track(c, q);
+  csr_plan<int64_t>(c.lv[q].out, flush_records(c, ub, gate), c.CS, c.P, c.s, c.d_sc, &trk, tail_begin(c, rr, n + 1));
+  tail_wait(c, rr, n + 1);
+}
+
+void flush_finish(ldl_ctx& c, int q, int64_t n, const int64_t (&tot)[6]) {
+  LevelState& L = c.lv[q];
+  const int64_t ub = L.pend_ub;
+  L.pend_ub = 0;
+  zero_cnt(c, K_PEND0 + q);
+  c.res.pending_records += n;
+  c.res.pending_applied +=
+      applied(c, q, csr_finish<int64_t>(c.lv[q].out, flush_records(c, ub, nullptr), tot, c.CS, c.P, c.s, c.d_sc));
 }
 
 void repair_done(ldl_ctx& c, const RepairAcc& a, int64_t dm) {
@@ -1278,27 +1326,40 @@ static void union_find(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t nG, i
 // lowest member.  Returns |D|, the nodes whose refined community changed
 // (list lD, stamp epD, old parents in par_old); the level's deletion list is
 // consumed.
-int32_t split(ldl_ctx& c, int r, int32_t epD, int32_t epX) {
+void split_launch(ldl_ctx& c, int r, SplitRun& sr, bool gated, bool hubs, HostRead* rr, int n) {
   LevelState& L = c.lv[r];
   LevelState& N = c.lv[r + 1];
   zero_cnt(c, K_D);
   zero_cnt(c, K_X);
-  const int32_t epF = c.next_epoch();  // communities whose connectivity is in doubt
+  sr.epD = c.next_epoch();
+  sr.epF = c.next_epoch();  // communities whose connectivity is in doubt
+  sr.epL = c.next_epoch();
+  const int32_t epX = c.next_epoch();
+  const SplitGate gate{gated ? c.cp[K_B] : nullptr, hubs ? c.cp[K_LARGE] : nullptr, c.cp[K_UNDEC]};
   // The level's deleted-arc endpoints and U* stay on the device: both kernels
   // stride over their lists' counts with grids sized by the host's bounds.
-  k_brk_check<<<grid_for(L.ubK, TPB, 4), TPB, 0, c.s>>>(L.lK.p, c.cp[K_BRK0 + r], L.alive.p, L.par.p, c.stX.p, epX, c.lX.p,
-                                   c.cp[K_X], c.ckf.p, epF);
+  k_brk_check<<<grid_for(L.ubK, TPB, 4), TPB, 0, c.s>>>(L.lK.p, c.cp[K_BRK0 + r], L.alive.p, L.par.p, c.stX.p, epX,
+                                                        c.lX.p, c.cp[K_X], c.ckf.p, sr.epF, gate);
   CKL("k_brk_check");
-  const int32_t epL = c.next_epoch();
-  int32_t cnt2[2] = {0, 0};
-  const HostRead rd[2] = {{c.cp[K_D], &cnt2[0], sizeof(int32_t)}, {c.cp[K_X], &cnt2[1], sizeof(int32_t)}};
-  k_leave<<<grid_for(c.ubU, TPB, 4), TPB, 0, c.s>>>(c.lUstar.p, c.cp[K_USTAR], L.alive.p, L.lab.p, N.lab.p, L.par.p, c.par_old.p,
-                               L.kout.p, kin_of(c, r), N.kout.p, kin_of(c, r + 1), N.cnt.p, c.directed, c.stL.p, epL,
-                               c.stD.p, epD, c.lD.p, c.cp[K_D], c.stX.p, epX, c.lX.p, c.cp[K_X], c.nbr.p,
-                               tail_begin(c, rd, 2));
+  rr[n] = {c.cp[K_D], &sr.nleft, sizeof(int32_t)};
+  rr[n + 1] = {c.cp[K_X], &sr.nx, sizeof(int32_t)};
+  k_leave<<<grid_for(c.ubU, TPB, 4), TPB, 0, c.s>>>(c.lUstar.p, c.cp[K_USTAR], L.alive.p, L.lab.p, N.lab.p, L.par.p,
+                                                    c.par_old.p, L.kout.p, kin_of(c, r), N.kout.p, kin_of(c, r + 1),
+                                                    N.cnt.p, c.directed, c.stL.p, sr.epL, c.stD.p, sr.epD, c.lD.p,
+                                                    c.cp[K_D], c.stX.p, epX, c.lX.p, c.cp[K_X], c.nbr.p, gate,
+                                                    tail_begin(c, rr, n + 2));
   CKL("k_leave");
-  tail_wait(c, rd, 2);
-  const int32_t nleft = cnt2[0], nx = cnt2[1];
+}
+
+int32_t split(ldl_ctx& c, int r, SplitRun& sr) {
+  LevelState& L = c.lv[r];
+  LevelState& N = c.lv[r + 1];
+  if (!sr.done) {
+    HostRead rr[2];
+    split_launch(c, r, sr, false, false, rr, 0);
+    tail_wait(c, rr, 2);
+  }
+  const int32_t nleft = sr.nleft, nx = sr.nx, epL = sr.epL, epF = sr.epF, epD = sr.epD;
   int32_t nD = nleft;  // k_rename appends to lD
   if (nx > 0) {
     if (nleft > 0) {
@@ -1438,8 +1499,9 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
       // current parents, the lists of the levels above
       chain_records(c, c.rk.p, c.rsum.p, nr, c.cp[K_NR], r + 1, true, false);
       sort_pairs(c.crk, c.crv, c.tk, c.tv, 2 * (int64_t)nC, 2 * c.bits, c.P, c.s, 0, c.cp[K_CREC]);
-      csr_apply<int32_t>(L.children, c.crk.p, (const int64_t*)c.crv.p, 2 * (int64_t)nC, c.cp[K_CREC], 1, c.bits,
-                         c.CS, c.P, c.s, c.d_sc);
+      csr_apply<int32_t>(L.children,
+                         CsrRecords{c.crk.p, (const int64_t*)c.crv.p, 2 * (int64_t)nC, c.cp[K_CREC], 1, c.bits}, c.CS,
+                         c.P, c.s, c.d_sc);
     }
     sub_end(c, SU_AGG_APPLY);
     sub_begin(c);

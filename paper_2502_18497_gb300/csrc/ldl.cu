@@ -147,20 +147,6 @@ static void wait_words(ldl_ctx& c, int n) {
   std::atomic_thread_fence(std::memory_order_acquire);
 }
 
-Pub pub_begin(ldl_ctx& c) {
-  ++c.syncs;
-  if (++c.pub_seq == 0) {  // all numbers used: no word of the page may match a new one
-    for (int w = 0; w < PAGE_WORDS; ++w) c.h_pub[w] = 0;
-    c.pub_seq = 1;  // 0 marks a tail without a read
-  }
-  return Pub{c.d_pub, c.pub_seq};
-}
-
-void pub_wait(ldl_ctx& c, int64_t* out, int n) {
-  wait_words(c, 2 * n);
-  for (int i = 0; i < n; ++i) out[i] = (int64_t)((c.h_pub[2 * i] & 0xffffffffu) | (c.h_pub[2 * i + 1] << 32));
-}
-
 void host_read(ldl_ctx& c, const HostRead* r, int n) {
   const Tail t = tail_begin(c, r, n);
   k_publish<<<1, 64, 0, c.s>>>(t);
@@ -208,9 +194,13 @@ Tail tail_begin(ldl_ctx& c, const HostRead* r, int n) {
   t.n = n;
   zero_cnt(c, K_TICKET);
   t.ticket = c.cp[K_TICKET];
-  const Pub p = pub_begin(c);
-  t.page = p.page;
-  t.seq = p.seq;
+  ++c.syncs;
+  if (++c.pub_seq == 0) {  // all numbers used: no word of the page may match a new one
+    for (int w = 0; w < PAGE_WORDS; ++w) c.h_pub[w] = 0;
+    c.pub_seq = 1;  // 0 marks a tail without a read
+  }
+  t.page = c.d_pub;
+  t.seq = c.pub_seq;
   return t;
 }
 
@@ -301,8 +291,8 @@ void alloc_globals(ldl_ctx& c) {
   for (int k = 0; k < K_COUNT; ++k) c.cp[k] = c.dcnt + k;
   c.P.rd = [](void* owner, const HostRead* r, int n) { host_read(*(ldl_ctx*)owner, r, n); };
   c.P.rd_owner = &c;
-  c.P.pub_begin = [](void* owner) { return pub_begin(*(ldl_ctx*)owner); };
-  c.P.pub_wait = [](void* owner, int64_t* out, int n) { pub_wait(*(ldl_ctx*)owner, out, n); };
+  c.P.tail_begin = [](void* owner, const HostRead* r, int n) { return tail_begin(*(ldl_ctx*)owner, r, n); };
+  c.P.tail_wait = [](void* owner, const HostRead* r, int n) { tail_wait(*(ldl_ctx*)owner, r, n); };
 }
 
 void free_all(ldl_ctx& c) {
@@ -355,9 +345,10 @@ void free_all(ldl_ctx& c) {
 // lUstar / stU (epoch epU) hold U*.  Moved nodes go to lMv (epMv) and, at
 // level 0, to lM0 (epM0).
 static int64_t move_loop(ldl_ctx& c, int r, int rounds, int32_t epU, int32_t epMv, int32_t epM0, int32_t epCh,
-                         int32_t nU, int64_t s_max) {
+                         int32_t nU, int64_t s_max, SplitRun* spec) {
   // nU = |U| on entry; later rounds take it from the end of the previous one.
-  // s_max bounds the first round's candidate set.
+  // s_max bounds the first round's candidate set.  With spec the level's split
+  // may start behind the last sweep.
   // Returns the committed moves, an upper bound of the distinct moved nodes
   // (lMv), which is empty exactly when it is 0.
   int64_t committed = 0;
@@ -373,7 +364,7 @@ static int64_t move_loop(ldl_ctx& c, int r, int rounds, int32_t epU, int32_t epM
     stage_end(c, ST_EXPAND);
     // |S| stays on the device: the sweep's kernels stride over it (n bounds
     // their grids) and it comes back with the candidates (β test)
-    const SweepOut so = sweep(c, r, 0, c.lS.p, K_S, j == 0 ? std::min(c.n, s_max) : c.n);
+    const SweepOut so = sweep(c, r, 0, c.lS.p, K_S, j == 0 ? std::min(c.n, s_max) : c.n, spec);
     const int32_t nS = so.nlist, nc = so.nc, nb = so.nb;
     if (nc == 0) break;
     c.res.rejected += nc - nb;
@@ -459,7 +450,7 @@ static void static_build(ldl_ctx& c) {
     zero_cnt(c, K_MV);
     zero_cnt(c, K_M0);
     zero_cnt(c, K_CH);
-    const int64_t mv = move_loop(c, r, c.prm.M_static, epU, epMv, epM0, epCh, nU, c.n);
+    const int64_t mv = move_loop(c, r, c.prm.M_static, epU, epMv, epM0, epCh, nU, c.n, nullptr);
     if (r > 0) pushdown(c, r, epCh, mv);
     if (r == L) break;
     level_alloc(c, r + 1);
@@ -590,6 +581,10 @@ static void txn_rollback(ldl_ctx& c) {
 }
 
 // ---------------------------------------------------------------- batch update
+// Longest pending list (by its bound) planned ahead of the frontier's count:
+// what one block sorts.  Longer ones are worth the wait for their exact count.
+constexpr int64_t FLUSH_EAGER = 2048;
+
 static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on_device) {
   memset(&c.res, 0, sizeof(c.res));
   c.syncs = 0;
@@ -641,7 +636,7 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
       int64_t deg = 0;
       RepairAcc ra{};
       const bool first = pass == 0 && r == 0;
-      HostRead rr[4] = {{c.cp[K_U], &nU, sizeof(int32_t)},
+      HostRead rr[5] = {{c.cp[K_U], &nU, sizeof(int32_t)},
                         {c.cp[K_PEND0 + r], &nP, sizeof(int32_t)},
                         {c.cp[K_M0], &m0, sizeof(int32_t)},
                         {c.sums, &deg, sizeof(int64_t)}};
@@ -650,7 +645,17 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
         rr[2].dst = &ra;
         rr[2].bytes = (int32_t)sizeof(ra);
       }
-      frontier(c, r, epU, rr, 4);
+      // A short pending list of the level is planned before
+      // |U| is known: one wait for both (the plan does nothing if U is empty).
+      const bool eager = c.lv[r].pend_ub > 0 && c.lv[r].pend_ub <= FLUSH_EAGER;
+      int64_t tot[6];
+      if (eager) {
+        frontier(c, r, epU, Tail{});
+        flush_plan(c, r, c.cp[K_U], rr, 4, tot);
+      } else {
+        frontier(c, r, epU, tail_begin(c, rr, 4));
+        tail_wait(c, rr, 4);
+      }
       c.ubU = nU;
       if (first) {
         repair_done(c, ra, dm);
@@ -659,14 +664,18 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
       if (r > 0) nM0 = m0;
       if (nU == 0) continue;
       if (r < 8) c.res.frontier_nodes[r] += nU;
+      SplitRun sr;
       const int32_t epMv = c.next_epoch();
       zero_cnt(c, K_MV);
       stage_begin(c);
-      flush_level(c, r, nP);  // the level's weights are read from here on
+      // the level's weights are read from here on
+      if (eager) flush_finish(c, r, nP, tot);
+      else flush_level(c, r, nP);
       stage_end(c, ST_AGG);
       // U and every row entry bound the first candidate set (a flush adds at
       // most one entry per record and row)
-      const int64_t mv = move_loop(c, r, c.prm.M, epU, epMv, epM0, epCh, nU, nU + deg + 2 * (int64_t)nP);
+      const int64_t mv = move_loop(c, r, c.prm.M, epU, epMv, epM0, epCh, nU, nU + deg + 2 * (int64_t)nP,
+                                   r < T ? &sr : nullptr);
       if (r > 0) {
         stage_begin(c);
         pushdown(c, r, epCh, mv);
@@ -674,9 +683,9 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
       }
       if (r < T) {
         stage_begin(c);
-        const int32_t epD = c.next_epoch(), epX = c.next_epoch();
         sub_begin(c);
-        const int32_t nD = split(c, r, epD, epX);
+        const int32_t nD = split(c, r, sr);
+        const int32_t epD = sr.epD;
         sub_end(c, SU_REF_DISSOLVE);
         sub_begin(c);
         refine_loop(c, r, c.prm.M, epD, nD);

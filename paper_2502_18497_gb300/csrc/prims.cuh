@@ -11,10 +11,9 @@ struct Prims {  // scratch owned by a context
   // how totals reach the host (nullptr: a copy and a stream synchronisation)
   HostReadFn rd = nullptr;
   void* rd_owner = nullptr;
-  // a read whose values a kernel publishes itself: begin hands out the page
-  // and the next sequence number, wait returns the payload words
-  Pub (*pub_begin)(void* owner) = nullptr;
-  void (*pub_wait)(void* owner, int64_t* out, int n) = nullptr;
+  // a read that a kernel hands over itself (scan.cuh)
+  Tail (*tail_begin)(void* owner, const HostRead* r, int n) = nullptr;
+  void (*tail_wait)(void* owner, const HostRead* r, int n) = nullptr;
   void read(const HostRead* r, int n, cudaStream_t s) {
     if (rd) {
       rd(rd_owner, r, n);

@@ -99,22 +99,8 @@ __device__ inline void look_back(u64* st, int64_t tile, const int64_t (&agg)[NC]
 // by itself whether it belongs to this read.  The host waits for every word;
 // nothing has to order them (a fence to the host between the payload and a
 // sequence number cost 1.5 us a read).
-struct Pub {
-  u64* page;
-  uint32_t seq;
-};
-
 __device__ inline void put_word(u64* page, uint32_t seq, int w, uint32_t v) {
   *(volatile u64*)(page + w) = ((u64)seq << 32) | v;
-}
-
-template <int N>
-__device__ inline void publish(const Pub& p, const int64_t (&v)[N]) {
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-    put_word(p.page, p.seq, 2 * i, (uint32_t)(u64)v[i]);
-    put_word(p.page, p.seq, 2 * i + 1, (uint32_t)((u64)v[i] >> 32));
-  }
 }
 
 // Values that a kernel hands to the host when its last block is done: device
@@ -130,10 +116,26 @@ struct Tail {
   int32_t* ticket;
 };
 
-__device__ inline void put_tail(const Tail& t) {
-  for (int i = 0; i < t.n; ++i)
+// (except values whose source is `skip`: the kernel puts those itself)
+__device__ inline void put_tail(const Tail& t, const void* skip = nullptr) {
+  for (int i = 0; i < t.n; ++i) {
+    if (skip && t.src[i] == skip) continue;
     for (int w = threadIdx.x; w < t.words[i]; w += blockDim.x)
       put_word(t.page, t.seq, t.off[i] + w, __ldcg(t.src[i] + w));
+  }
+}
+
+// Entry `src` of the tail from N values of the calling thread.
+template <int N>
+__device__ inline void put_values(const Tail& t, const void* src, const int64_t (&v)[N]) {
+  for (int i = 0; i < t.n; ++i) {
+    if (t.src[i] != src) continue;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      put_word(t.page, t.seq, t.off[i] + 2 * k, (uint32_t)(u64)v[k]);
+      put_word(t.page, t.seq, t.off[i] + 2 * k + 1, (uint32_t)((u64)v[k] >> 32));
+    }
+  }
 }
 
 // Called by every thread of every block as the kernel's last step: a separate

@@ -1440,15 +1440,14 @@ void expand_set(ldl_ctx& c, int r, const int32_t* list, int idx_n, int32_t* stam
   expand_tail(c, r, list, idx_n, stamp, ep, olist, idx_out, n_hint, Tail{});
 }
 
-void frontier(ldl_ctx& c, int r, int32_t epU, const HostRead* rr, int n) {
+void frontier(ldl_ctx& c, int r, int32_t epU, const Tail& tail) {
   LevelState& L = c.lv[r];
   const int32_t* lo = r == 0 ? adj_out0(c).len : adj_out(c, r).len;
   const int32_t* li = !c.directed ? nullptr : r == 0 ? adj_in0(c).len : adj_in(c, r).len;
   k_frontier<<<grid_for(L.ubA, TPB, 2), TPB, 0, c.s>>>(L.lA.p, c.cp[K_A0 + r], r ? L.alive.p : nullptr, c.lU.p,
                                                        c.cp[K_U], c.stU.p, epU, c.lUstar.p, c.cp[K_USTAR], lo, li,
-                                                       c.sums, tail_begin(c, rr, n));
+                                                       c.sums, tail);
   CKL("k_frontier");
-  tail_wait(c, rr, n);
 }
 
 void union_into(ldl_ctx& c, const int32_t* list, int idx_n, int32_t* stamp, int32_t ep, int32_t* olist, int idx_out,
@@ -1506,7 +1505,7 @@ static cudaEvent_t* kstats_events(ldl_ctx& c) {
 
 template <class WT, int MODE>
 static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_t* list, int idx_n,
-                        int64_t n_hint) {
+                        int64_t n_hint, SplitRun* spec) {
   if (MODE == 0) stage_begin(c);  // refinement is timed as a whole
   for (int k : {K_CAND, K_TINY, K_SMALL, K_MID, K_MID2, K_CLU, K_LARGE}) zero_cnt(c, k);
   c.sums = (int64_t*)fresh(c, 2, c.d_sc->sums);
@@ -1553,6 +1552,12 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   // Few nodes are all swept by one block each, whatever their degree: a launch
   // per degree bin costs more than it saves (see SWEEP_FEW).
   const bool few = n_hint <= SWEEP_FEW && !c.kstats;
+  // The split is only launched ahead behind such short sweeps: they mostly end
+  // the level's moves, and where moves are accepted its two launches are lost
+  // (one edge on 10k vertices 508 -> 486 us a batch; with it behind every sweep,
+  // batches of 10^3 and more on the R-MAT graphs lost up to 1%).
+  if (spec) spec->done = false;
+  if (!few) spec = nullptr;
   const bool early = expect || c.kstats;
   k_bin<WT><<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(out, in, c.directed, list, c.cp[idx_n], c.binT.p, c.cp[K_TINY],
                                                      c.binS.p, c.cp[K_SMALL], c.binM.p, c.cp[K_MID], c.binM2.p,
@@ -1582,7 +1587,7 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   if (early) tail_wait(c, rb, 8);
   else {
     const HostRead ro[3] = {rb[5], rb[6], rb[7]};
-    dd = decouple(c, ro, 3);
+    dd = decouple(c, ro, 3, spec, r, true);
   }
   if (kev) CK(cudaEventRecord(kev[6], c.s));  // the wait above is charged to no kernel
   if (ch > 0) {
@@ -1674,7 +1679,7 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   expect = ch > 0;
   if (early || ch > 0) {
     if (MODE == 0) stage_begin(c);
-    dd = decouple(c);
+    dd = decouple(c, nullptr, 0, spec, r, false);
     if (MODE == 0) stage_end(c, ST_DECOUPLE);
   }
   c.res.decouple_rounds += dd.rounds;
@@ -1685,16 +1690,16 @@ extern "C" void ldl_debug_hub_table_slots(int64_t slots) {
   g_hub_table_slots.store(slots > 0 ? slots : HUB_TABLE_SLOTS);
 }
 
-SweepOut sweep(ldl_ctx& c, int r, int mode, const int32_t* list, int idx_n, int64_t n_hint) {
+SweepOut sweep(ldl_ctx& c, int r, int mode, const int32_t* list, int idx_n, int64_t n_hint, SplitRun* spec) {
   if (r == 0) {
-    if (mode == 0) return sweep_t<int32_t, 0>(c, r, adj_out0(c), adj_in0(c), list, idx_n, n_hint);
-    return sweep_t<int32_t, 1>(c, r, adj_out0(c), adj_in0(c), list, idx_n, n_hint);
+    if (mode == 0) return sweep_t<int32_t, 0>(c, r, adj_out0(c), adj_in0(c), list, idx_n, n_hint, spec);
+    return sweep_t<int32_t, 1>(c, r, adj_out0(c), adj_in0(c), list, idx_n, n_hint, spec);
   }
-  if (mode == 0) return sweep_t<int64_t, 0>(c, r, adj_out(c, r), adj_in(c, r), list, idx_n, n_hint);
-  return sweep_t<int64_t, 1>(c, r, adj_out(c, r), adj_in(c, r), list, idx_n, n_hint);
+  if (mode == 0) return sweep_t<int64_t, 0>(c, r, adj_out(c, r), adj_in(c, r), list, idx_n, n_hint, spec);
+  return sweep_t<int64_t, 1>(c, r, adj_out(c, r), adj_in(c, r), list, idx_n, n_hint, spec);
 }
 
-DecoupleOut decouple(ldl_ctx& c, const HostRead* extra, int n_extra) {
+DecoupleOut decouple(ldl_ctx& c, const HostRead* extra, int n_extra, SplitRun* spec, int r, bool hubs) {
   // The single-block filter runs first and reads the candidate count on the
   // device; one read then returns the count, the accepted number and the
   // filter's status (-2: too many candidates for one block).
@@ -1706,9 +1711,12 @@ DecoupleOut decouple(ldl_ctx& c, const HostRead* extra, int n_extra) {
   CK(cudaFuncSetAttribute(k_dec_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DEC_SMEM));
   k_dec_block<<<1, DEC_THREADS, DEC_SMEM, c.s>>>(c.cp[K_CAND], c.cv.p, c.csrc.p, c.cdst.p, c.cghi.p, c.cglo.p,
                                                  c.role.p, c.best.p, c.bv.p, c.bsrc.p, c.bdst.p, c.cp[K_B],
-                                                 c.cp[K_UNDEC], tail_begin(c, rr, 3 + n_extra));
+                                                 c.cp[K_UNDEC], spec ? Tail{} : tail_begin(c, rr, 3 + n_extra));
   CKL("k_dec_block");
-  tail_wait(c, rr, 3 + n_extra);
+  if (spec) split_launch(c, r, *spec, true, hubs, rr, 3 + n_extra);
+  tail_wait(c, rr, 3 + n_extra + (spec ? 2 : 0));
+  // the gate's own test (the first extra value is the hub count)
+  if (spec) spec->done = nb == 0 && stat != -2 && !(hubs && *(const int32_t*)extra[0].dst != 0);
   if (nc <= 0) return {0, 0, 0};
   if (stat != -2) {
     if (stat < 0) ldl_throw(LDL_E_INVALID, "internal: decoupling did not converge");
