@@ -40,30 +40,75 @@ template <class T>
 struct DBuf {
   T* p = nullptr;
   int64_t cap = 0;
+  bool own = true;  // false: part of a Slab
   void reserve(int64_t n, cudaStream_t s, bool keep = false) {
     if (n <= cap) return;
     int64_t nc = cap ? cap : 1024;
     while (nc < n) nc = nc * 3 / 2 + 1024;
     T* q = (T*)dalloc((size_t)nc * sizeof(T));
     if (keep && p && cap) CK(cudaMemcpyAsync(q, p, (size_t)cap * sizeof(T), cudaMemcpyDeviceToDevice, s));
-    if (p) {
+    if (p && own) {
       CK(cudaStreamSynchronize(s));
       dfree(p);
     }
     p = q;
     cap = nc;
+    own = true;
   }
   void exact(int64_t n) {  // allocate exactly n (no growth policy)
     if (n <= cap) return;
     T* q = (T*)dalloc((size_t)(n > 0 ? n : 1) * sizeof(T));
-    if (p) dfree(p);
+    if (p && own) dfree(p);
     p = q;
     cap = n;
+    own = true;
   }
   void release() {
-    if (p) dfree(p);
+    if (p && own) dfree(p);
     p = nullptr;
     cap = 0;
+    own = true;
+  }
+};
+
+// Buffers of fixed size that live and die together, in one allocation: a
+// cudaMalloc of some MB takes about 35 us and its cudaFree 30 or more, and a
+// context has some 80 arrays of n entries and 10 more per level.
+struct Slab {
+  unsigned char* base = nullptr;
+  struct Part {
+    void** p;
+    int64_t* cap;
+    bool* own;
+    int64_t n;
+    size_t bytes;
+  };
+  std::vector<Part> parts;
+  template <class T>
+  void add(DBuf<T>& b, int64_t n) {
+    parts.push_back({(void**)&b.p, &b.cap, &b.own, n, (size_t)(n > 0 ? n : 1) * sizeof(T)});
+  }
+  static size_t round(size_t b) { return (b + 255) & ~(size_t)255; }
+  // Bytes of the parts from part `from` on, as laid out.
+  size_t span(size_t from, size_t to) const {
+    size_t b = 0;
+    for (size_t i = from; i < to; ++i) b += round(parts[i].bytes);
+    return b;
+  }
+  void alloc() {  // places every added buffer
+    base = (unsigned char*)dalloc(span(0, parts.size()));
+    size_t at = 0;
+    for (auto& x : parts) {
+      *x.p = base + at;
+      *x.cap = x.n;
+      *x.own = false;
+      at += round(x.bytes);
+    }
+  }
+  void release() {  // after the buffers' own release()
+    if (base) dfree(base);
+    base = nullptr;
+    parts.clear();
   }
 };
 
@@ -261,6 +306,7 @@ struct SlackCSR {
   int64_t n = 0;
   DBuf<int64_t> off;
   DBuf<int32_t> len, cap;
+  Slab tables;           // off, len and cap
   DBuf<int32_t> col;
   DBuf<WT> w;
   int64_t pool_top = 0;  // host mirror of the first free pool slot
@@ -288,7 +334,7 @@ struct SlackCSR {
   DBuf<int32_t> llen, lcap, lcol;
   DBuf<WT> lw, lold;
   void release() {
-    off.release(); len.release(); cap.release(); col.release(); w.release();
+    off.release(); len.release(); cap.release(); tables.release(); col.release(); w.release();
     for (auto& x : retired) {
       if (x.first != col.p) dfree(x.first);
       if (x.second != w.p) dfree(x.second);

@@ -292,41 +292,6 @@ __global__ void k_undo_weights(int64_t nw, const int64_t* lpos, const WT* lold, 
   }
 }
 
-__device__ inline int64_t find_seg(const int64_t* pre, int64_t nseg, int64_t t) {
-  // last s with pre[s] <= t (pre is an exclusive scan, pre[0] = 0)
-  int64_t lo = 0, hi = nseg;
-  while (hi - lo > 1) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (pre[mid] <= t) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
-// last s in [lo, hi] with pre[s] <= t
-__device__ inline int64_t seg_in(const int64_t* pre, int64_t lo, int64_t hi, int64_t t) {
-  while (lo < hi) {
-    const int64_t mid = (lo + hi + 1) >> 1;
-    if (pre[mid] <= t) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-// Items [0, total) split into segments by the exclusive scan pre.  Each warp
-// takes runs of SEG_RUN consecutive items: two warp-uniform searches bound the
-// run's segments, and each item then searches only that narrow range.
-constexpr int SEG_RUN = 256;
-#define FOR_SEG_ITEMS(t, s, pre, nseg, total)                                                       \
-  const int64_t warp_ = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;                     \
-  const int64_t nwarps_ = ((int64_t)gridDim.x * blockDim.x) >> 5;                                   \
-  for (int64_t c0_ = warp_ * SEG_RUN; c0_ < (total); c0_ += nwarps_ * SEG_RUN) {                   \
-    const int64_t c1_ = min(c0_ + SEG_RUN, (int64_t)(total)) - 1;                                   \
-    const int64_t slo_ = find_seg(pre, nseg, c0_), shi_ = find_seg(pre, nseg, c1_);                 \
-    for (int64_t t = c0_ + (threadIdx.x & 31); t <= c1_; t += 32) {                                 \
-      const int64_t s = seg_in(pre, slo_, shi_, t);
-#define END_SEG_ITEMS \
-  }                   \
-  }
-
 // First half of an update: the weights of rows that keep their entries change
 // in place, and the rows to rebuild are copied out as they are (into the undo
 // log while a batch is logged).  With a log also: per row its old offset,
@@ -444,8 +409,18 @@ __global__ void k_compact_rows(int64_t n, const int64_t* off, const int64_t* lpr
 }
 
 // ---------------------------------------------------------------- build
-__global__ void k_count_rows(const u64* keys, int64_t nrec, int bshift, int32_t* cnt) {
-  GRID_STRIDE(i, nrec) atomicAdd(&cnt[keys[i] >> bshift], 1);
+// Row lengths (cleared before) and first records of sorted records: a row's
+// first and last record each add their share, where an atomic per record took
+// 220 us for 16M records (neighbouring threads meet in one counter).
+__global__ void k_row_bounds(const u64* keys, int64_t nrec, int bshift, int32_t* len, int64_t* start) {
+  GRID_STRIDE(i, nrec) {
+    const int64_t row = (int64_t)(keys[i] >> bshift);
+    if (i == 0 || (int64_t)(keys[i - 1] >> bshift) != row) {
+      start[row] = i;
+      atomicAdd((unsigned*)&len[row], 0u - (unsigned)i);  // modulo 2^32, as the length fits
+    }
+    if (i + 1 == nrec || (int64_t)(keys[i + 1] >> bshift) != row) atomicAdd((unsigned*)&len[row], (unsigned)(i + 1));
+  }
 }
 
 __global__ void k_caps(const int32_t* cnt, int64_t n, int32_t* cap, int slack_pct) {
@@ -480,24 +455,22 @@ template <class WT>
 void csr_build(SlackCSR<WT>& g, int64_t n, const u64* keys, const int64_t* vals, int64_t nrec, int bshift,
                int slack_pct, CsrScratch& S, Prims& P, cudaStream_t s) {
   g.n = n;
-  g.off.exact(n + 1);
-  g.len.exact(n + 1);
-  g.cap.exact(n + 1);
+  if (g.off.cap < n + 1) {
+    g.off.release(); g.len.release(); g.cap.release(); g.tables.release();
+    g.tables.add(g.off, n + 1);
+    g.tables.add(g.len, n + 1);
+    g.tables.add(g.cap, n + 1);
+    g.tables.alloc();
+  }
   CK(cudaMemsetAsync(g.len.p, 0, sizeof(int32_t) * (size_t)(n + 1), s));
+  S.rs.reserve(n + 1, s);
   if (nrec > 0) {
-    k_count_rows<<<grid_for(nrec, TPB), TPB, 0, s>>>(keys, nrec, bshift, g.len.p);
-    CKL("k_count_rows");
+    k_row_bounds<<<grid_for(nrec, TPB), TPB, 0, s>>>(keys, nrec, bshift, g.len.p, S.rs.p);
+    CKL("k_row_bounds");
   }
   k_caps<<<grid_for(n, TPB), TPB, 0, s>>>(g.len.p, n, g.cap.p, slack_pct);
   CKL("k_caps");
-  S.rs.reserve(n + 1, s);
-  S.tmp64.reserve(n + 1, s);
-  k_i32_to_i64<<<grid_for(n, TPB), TPB, 0, s>>>(g.len.p, S.tmp64.p, n);
-  CKL("k_i32_to_i64");
-  scan_exclusive(S.tmp64.p, S.rs.p, n, P, s, false);
-  k_i32_to_i64<<<grid_for(n, TPB), TPB, 0, s>>>(g.cap.p, S.tmp64.p, n);
-  CKL("k_i32_to_i64");
-  const int64_t total = scan_exclusive(S.tmp64.p, g.off.p, n, P, s, true);
+  const int64_t total = scan_exclusive_i32(g.cap.p, g.off.p, n, P, s, true);
   const int64_t pool = total + total / 8 + 1024;
   g.col.release();
   g.w.release();
@@ -561,19 +534,7 @@ template <class WT>
 void csr_plan(const SlackCSR<WT>& g, const CsrRecords& r, CsrScratch& S, Prims& P, cudaStream_t s, DevScalars* d_sc,
               const DelTrack* trk, const Tail& tail) {
   const int64_t n_max = r.n_max;
-  S.pos.reserve(n_max + 1, s);
-  S.lb.reserve(n_max + 1, s);
-  S.oldw.reserve(n_max + 1, s);
-  S.pins.reserve(n_max + 1, s);
-  S.pdel.reserve(n_max + 1, s);
-  S.segid.reserve(n_max + 1, s);
-  // the segment count stays on the device: one segment per record bounds it
-  S.seg.reserve(n_max + 1, s);
-  S.segrow.reserve(n_max + 1, s);
-  S.newcap.reserve(n_max + 1, s);
-  S.soff.reserve(n_max + 2, s);
-  S.woff.reserve(n_max + 2, s);
-  S.noff.reserve(n_max + 2, s);
+  S.reserve_recs(n_max, s);  // the segment count stays on the device: one segment per record bounds it
   const RecN rn{n_max, r.n_dev, r.mul, r.gate};
   ++S.plans;
   const PlanOut o = plan_out(S, d_sc);

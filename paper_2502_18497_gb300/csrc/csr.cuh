@@ -3,18 +3,73 @@
 #include "common.cuh"
 #include "prims.cuh"
 
+__device__ inline int64_t find_seg(const int64_t* pre, int64_t nseg, int64_t t) {
+  // last s with pre[s] <= t (pre is an exclusive scan, pre[0] = 0)
+  int64_t lo = 0, hi = nseg;
+  while (hi - lo > 1) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (pre[mid] <= t) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
+// last s in [lo, hi] with pre[s] <= t
+__device__ inline int64_t seg_in(const int64_t* pre, int64_t lo, int64_t hi, int64_t t) {
+  while (lo < hi) {
+    const int64_t mid = (lo + hi + 1) >> 1;
+    if (pre[mid] <= t) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+// Items [0, total) split into segments by the exclusive scan pre.  Each warp
+// takes runs of SEG_RUN consecutive items: two warp-uniform searches bound the
+// run's segments, and each item then searches only that narrow range.
+constexpr int SEG_RUN = 256;
+#define FOR_SEG_ITEMS(t, s, pre, nseg, total)                                                       \
+  const int64_t warp_ = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;                     \
+  const int64_t nwarps_ = ((int64_t)gridDim.x * blockDim.x) >> 5;                                   \
+  for (int64_t c0_ = warp_ * SEG_RUN; c0_ < (total); c0_ += nwarps_ * SEG_RUN) {                   \
+    const int64_t c1_ = min(c0_ + SEG_RUN, (int64_t)(total)) - 1;                                   \
+    const int64_t slo_ = find_seg(pre, nseg, c0_), shi_ = find_seg(pre, nseg, c1_);                 \
+    for (int64_t t = c0_ + (threadIdx.x & 31); t <= c1_; t += 32) {                                 \
+      const int64_t s = seg_in(pre, slo_, shi_, t);
+#define END_SEG_ITEMS \
+  }                   \
+  }
+
 struct CsrScratch {
-  DBuf<int64_t> seg, segrow, oldw, rs, tmp64, soff, woff, noff;
-  DBuf<int32_t> pos, lb, newcap, pins, pdel, segid, scol, sw32;
-  DBuf<int64_t> sw64;
+  // per record and per segment of an update (for max_rec of them, in one slab)
+  DBuf<int64_t> seg, segrow, oldw, soff, woff, noff;
+  DBuf<int32_t> pos, lb, newcap, pins, pdel, segid;
+  Slab recs;
+  int64_t max_rec = 0;
+  DBuf<int64_t> rs, tmp64, sw64;
+  DBuf<int32_t> scol, sw32;
   u64 plans = 0;  // updates planned so far
   template <class WT>
   DBuf<WT>& sw_of();
+  void drop_recs() {
+    for (auto* b : {&seg, &segrow, &oldw, &soff, &woff, &noff}) b->release();
+    for (auto* b : {&pos, &lb, &newcap, &pins, &pdel, &segid}) b->release();
+    recs.release();
+    max_rec = 0;
+  }
+  void reserve_recs(int64_t n, cudaStream_t s) {
+    if (n <= max_rec) return;
+    int64_t nc = max_rec ? max_rec : 1024;
+    while (nc < n) nc = nc * 3 / 2 + 1024;
+    CK(cudaStreamSynchronize(s));
+    drop_recs();
+    for (auto* b : {&seg, &segrow, &oldw, &soff, &woff, &noff}) recs.add(*b, nc + 2);
+    for (auto* b : {&pos, &lb, &newcap, &pins, &pdel, &segid}) recs.add(*b, nc + 2);
+    recs.alloc();
+    max_rec = nc;
+  }
   void release() {
-    DBuf<int64_t>* a[] = {&seg, &segrow, &oldw, &rs, &tmp64, &soff, &woff, &noff, &sw64};
-    for (auto* b : a) b->release();
-    DBuf<int32_t>* c[] = {&pos, &lb, &newcap, &pins, &pdel, &segid, &scol, &sw32};
-    for (auto* b : c) b->release();
+    drop_recs();
+    for (auto* b : {&rs, &tmp64, &sw64}) b->release();
+    for (auto* b : {&scol, &sw32}) b->release();
   }
 };
 template <>

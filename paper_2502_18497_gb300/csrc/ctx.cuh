@@ -33,10 +33,12 @@ struct LevelState {
   DBuf<u64> pk, pv;
   int64_t pend_ub = 0;           // host bound on the pending count
   bool allocated = false;
+  Slab nodes;            // the node arrays
   void release() {
     out0.release(); in0.release(); out.release(); in.release(); children.release();
     lab.release(); par.release(); cnt.release(); kout.release(); kin.release(); alive.release();
     stA.release(); lA.release(); stK.release(); lK.release(); pk.release(); pv.release();
+    nodes.release();
     pend_ub = 0;
     allocated = false;
   }
@@ -139,6 +141,7 @@ struct ldl_ctx {
   DBuf<ldl_update> upd;
   Prims P;
   CsrScratch CS;
+  Slab globals;  // the arrays of n entries
 
   // counters of the last batch
   ldl_result res{};

@@ -867,30 +867,25 @@ __global__ void k_next_level(const int32_t* lU, const int32_t* nU, const int32_t
 }
 
 // ---------------------------------------------------------------- static set-up
-__global__ void k_csr_records(const int64_t* rp, const int32_t* col, const int32_t* w, int64_t n, int bits,
-                              u64* rk, u64* rv, unsigned long long* err) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t v = warp; v < n; v += nw) {
-    const int64_t s = rp[v], e = rp[v + 1];
-    if (e < s) {
-      if (lane == 0) set_err(err, 0, LDL_E_INVALID);
-      continue;
-    }
-    for (int64_t k = s + lane; k < e; k += 32) {
-      const int32_t c = col[k];
-      if (c < 0 || c >= n) {
-        set_err(err, 0, LDL_E_RANGE);
-        rk[k] = 0;
-        rv[k] = 0;
-        continue;
-      }
-      if (w[k] < 1) set_err(err, 0, LDL_E_INVALID);
-      rk[k] = ((u64)v << bits) | (u64)c;
-      rv[k] = (u64)(int64_t)w[k];
-    }
+// Records of a CSR snapshot (nnz entries, rp[0] = 0, rp[n] = nnz), entry by
+// entry so that a hub row spreads over the GPU (a warp per row took 2.1 ms on
+// the R-MAT of 2^20, all of it the longest row).  *unsorted is set where a
+// row's columns are not strictly increasing.
+__global__ void k_csr_records(const int64_t* rp, const int32_t* col, const int32_t* w, int64_t n, int64_t nnz, int bits,
+                              u64* rk, u64* rv, unsigned long long* err, int32_t* unsorted) {
+  GRID_STRIDE(v, n) {
+    if (rp[v + 1] < rp[v]) set_err(err, 0, LDL_E_INVALID);
   }
+  bool bad = false;
+  FOR_SEG_ITEMS(t, v, rp, n, nnz)
+    const int32_t c = col[t], x = w[t];
+    if (c < 0 || c >= n) set_err(err, 0, LDL_E_RANGE);
+    if (x < 1) set_err(err, 0, LDL_E_INVALID);
+    bad |= t > 0 && t > rp[v] && col[t - 1] >= c;
+    rk[t] = ((u64)v << bits) | (u64)(uint32_t)c;
+    rv[t] = (u64)(int64_t)x;
+  END_SEG_ITEMS
+  if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicExch(unsorted, 1);
 }
 
 __global__ void k_check_max(const int64_t* s, int64_t n, unsigned long long* err) {
@@ -906,30 +901,33 @@ __global__ void k_compare(const u64* a, const int64_t* av, const u64* b, const u
   }
 }
 
-template <class WT>
-__global__ void k_row_sums(Adj<WT> a, int64_t n, int64_t* out, int64_t* self, int64_t* total) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+// Row sums (cleared before) of sorted records, rows counted from row0, the
+// weight on the diagonal and the sum of all.  A thread sums RS_RUN consecutive
+// records and adds once per row it meets, so a hub row is no longer than others
+// (a warp per row took 337 us on the R-MAT of 2^20).
+constexpr int RS_RUN = 8;
+__global__ void k_row_sums(const u64* keys, const int64_t* w, int64_t nrec, int bits, int64_t row0, int64_t* out,
+                           int64_t* self, int64_t* total) {
+  const u64 mask = (((u64)1) << bits) - 1;
   int64_t tot = 0;
-  for (int64_t v = warp; v < n; v += nw) {
-    const int64_t o = a.off[v];
-    const int32_t l = a.len[v];
-    int64_t s = 0, sl = 0;
-    for (int32_t k = lane; k < l; k += 32) {
-      const int64_t w = (int64_t)a.w[o + k];
-      s += w;
-      if (a.col[o + k] == v) sl += w;
+  GRID_STRIDE(r, (nrec + RS_RUN - 1) / RS_RUN) {
+    int64_t row = -1, s = 0;
+    for (int64_t i = r * RS_RUN; i < min(nrec, (r + 1) * RS_RUN); ++i) {
+      const int64_t v = (int64_t)(keys[i] >> bits) - row0;
+      if (v != row && row >= 0) {
+        atomic_add_i64(&out[row], s);
+        tot += s;
+        s = 0;
+      }
+      row = v;
+      s += w[i];
+      if (self && (int64_t)(keys[i] & mask) == v) atomic_add_i64(&self[v], w[i]);
     }
-    s = warp_sum_i64(s);
-    sl = warp_sum_i64(sl);
-    if (lane == 0) {
-      out[v] = s;
-      if (self) self[v] = sl;
-      tot += s;
-    }
+    if (row >= 0) atomic_add_i64(&out[row], s);
+    tot += s;
   }
-  if (lane == 0 && total && tot) atomic_add_i64(total, tot);
+  tot = warp_sum_i64(tot);
+  if ((threadIdx.x & 31) == 0 && total && tot) atomic_add_i64(total, tot);
 }
 
 __global__ void k_iota(int32_t* a, int64_t n) {
@@ -1408,7 +1406,8 @@ static int64_t emit_records(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t 
   if (cap > INT32_MAX) ldl_throw(LDL_E_OVERFLOW, "aggregate records beyond the 32-bit record counter");
   c.rk2.reserve(cap, c.s);
   c.rv2.reserve(cap, c.s);
-  ChunkMap m = chunk_map(c, c.lC.p, c.cp[K_C], nC, out.len, in.len);
+  // (in the static build the in-rows would be walked for nothing)
+  ChunkMap m = chunk_map(c, c.lC.p, c.cp[K_C], nC, out.len, build ? nullptr : in.len);
   k_emit<WT><<<chunk_grid(nC), TPB, 0, c.s>>>(out, in, m, c.lv[r].par.p, c.par_old.p,
                                                                           c.stC.p, epC, c.bits, c.rk2.p, c.rv2.p,
                                                                           c.cp[K_REC], cap, c.cp[K_ERR]);
@@ -1536,24 +1535,22 @@ void level_alloc(ldl_ctx& c, int r) {
   LevelState& L = c.lv[r];
   if (L.allocated) return;
   const int64_t n = c.n;
-  L.lab.exact(n);
-  L.par.exact(n);
-  L.cnt.exact(n);
-  L.kout.exact(n);
-  if (c.directed) L.kin.exact(n);
-  L.alive.exact(n);
-  L.stA.exact(n);
-  L.lA.exact(n);
-  L.stK.exact(n);
-  L.lK.exact(n);
-  CK(cudaMemsetAsync(L.stK.p, 0, sizeof(int32_t) * (size_t)n, c.s));
-  CK(cudaMemsetAsync(L.lab.p, 0, sizeof(int32_t) * (size_t)n, c.s));
+  // (the cleared arrays first: one clear)
+  Slab& S = L.nodes;
+  S.add(L.stK, n);
+  S.add(L.lab, n);
+  S.add(L.cnt, n);
+  S.add(L.kout, n);
+  if (c.directed) S.add(L.kin, n);
+  S.add(L.alive, n);
+  S.add(L.stA, n);
+  const size_t cleared = S.parts.size();
+  S.add(L.par, n);
+  S.add(L.lA, n);
+  S.add(L.lK, n);
+  S.alloc();
+  CK(cudaMemsetAsync(S.base, 0, S.span(0, cleared), c.s));
   CK(cudaMemsetAsync(L.par.p, 0xff, sizeof(int32_t) * (size_t)n, c.s));
-  CK(cudaMemsetAsync(L.cnt.p, 0, sizeof(int32_t) * (size_t)n, c.s));
-  CK(cudaMemsetAsync(L.kout.p, 0, sizeof(int64_t) * (size_t)n, c.s));
-  if (c.directed) CK(cudaMemsetAsync(L.kin.p, 0, sizeof(int64_t) * (size_t)n, c.s));
-  CK(cudaMemsetAsync(L.alive.p, 0, (size_t)n, c.s));
-  CK(cudaMemsetAsync(L.stA.p, 0, sizeof(int32_t) * (size_t)n, c.s));
   L.allocated = true;
 }
 
@@ -1589,24 +1586,30 @@ void upload_graph(ldl_ctx& c, int64_t nnz, const int64_t* row_ptr, const int32_t
   c.rk.reserve(nnz + 1, c.s);
   c.rv.reserve(nnz + 1, c.s);
   reset_err(c);
-  k_csr_records<<<grid_for(n * 32, TPB), TPB, 0, c.s>>>(drp.p, dcol.p, dw.p, n, c.bits, c.rk.p, c.rv.p, err_ptr(c));
+  zero_cnt(c, K_TMP);
+  k_csr_records<<<grid_for(std::max(n, nnz / 8), TPB), TPB, 0, c.s>>>(drp.p, dcol.p, dw.p, n, nnz, c.bits, c.rk.p,
+                                                                      c.rv.p, err_ptr(c), c.cp[K_TMP]);
   CKL("k_csr_records");
   CK(cudaStreamSynchronize(c.s));
   drp.release();
   dcol.release();
   dw.release();
   throw_err(c, err_ptr(c), "invalid CSR");
-  sort_pairs(c.rk, c.rv, c.tk, c.tv, nnz, 2 * c.bits, c.P, c.s);
-  c.rk2.reserve(nnz + 1, c.s);
-  c.rsum.reserve(nnz + 1, c.s);
-  const int64_t na = reduce_by_key(c.rk.p, c.rv.p, nnz, c.rk2.p, c.rsum.p, c.P, c.s);
-  reset_err(c);
-  k_check_max<<<grid_for(na, TPB), TPB, 0, c.s>>>(c.rsum.p, na, err_ptr(c));
-  CKL("k_check_max");
-  throw_err(c, err_ptr(c), "summed weight above INT32_MAX");
-  // (rk2, rsum) = unique arcs
-  CK(cudaMemcpyAsync(c.rk.p, c.rk2.p, sizeof(u64) * (size_t)na, cudaMemcpyDeviceToDevice, c.s));
-  CK(cudaMemcpyAsync(c.rv.p, c.rsum.p, sizeof(int64_t) * (size_t)na, cudaMemcpyDeviceToDevice, c.s));
+  int64_t na = nnz;
+  // rows in strictly increasing column order are unique sorted arcs already
+  if (rd_cnt(c, K_TMP)) {
+    sort_pairs(c.rk, c.rv, c.tk, c.tv, nnz, 2 * c.bits, c.P, c.s);
+    c.rk2.reserve(nnz + 1, c.s);
+    c.rsum.reserve(nnz + 1, c.s);
+    na = reduce_by_key(c.rk.p, c.rv.p, nnz, c.rk2.p, c.rsum.p, c.P, c.s);
+    reset_err(c);
+    k_check_max<<<grid_for(na, TPB), TPB, 0, c.s>>>(c.rsum.p, na, err_ptr(c));
+    CKL("k_check_max");
+    throw_err(c, err_ptr(c), "summed weight above INT32_MAX");
+    // (rk2, rsum) = unique arcs
+    CK(cudaMemcpyAsync(c.rk.p, c.rk2.p, sizeof(u64) * (size_t)na, cudaMemcpyDeviceToDevice, c.s));
+    CK(cudaMemcpyAsync(c.rv.p, c.rsum.p, sizeof(int64_t) * (size_t)na, cudaMemcpyDeviceToDevice, c.s));
+  }
   if (na) {
     c.rk2.reserve(na + 1, c.s);
     c.rv2.reserve(na + 1, c.s);
@@ -1630,11 +1633,15 @@ void upload_graph(ldl_ctx& c, int64_t nnz, const int64_t* row_ptr, const int32_t
   }
   // strengths, m, labels, community totals
   CK(cudaMemsetAsync(&c.d_sc->dm, 0, sizeof(int64_t), c.s));
-  const int gw = grid_for(n * 32, TPB);
-  k_row_sums<int32_t><<<gw, TPB, 0, c.s>>>(adj_out0(c), n, L0.kout.p, c.e.p, &c.d_sc->dm);
+  CK(cudaMemsetAsync(L0.kout.p, 0, sizeof(int64_t) * (size_t)n, c.s));
+  CK(cudaMemsetAsync(c.e.p, 0, sizeof(int64_t) * (size_t)n, c.s));
+  const int gr = grid_for((na + RS_RUN - 1) / RS_RUN, TPB);
+  k_row_sums<<<gr, TPB, 0, c.s>>>(c.rk.p, (const int64_t*)c.rv.p, na, c.bits, 0, L0.kout.p, c.e.p, &c.d_sc->dm);
   CKL("k_row_sums");
   if (c.directed) {
-    k_row_sums<int32_t><<<gw, TPB, 0, c.s>>>(adj_in0(c), n, L0.kin.p, nullptr, nullptr);
+    CK(cudaMemsetAsync(L0.kin.p, 0, sizeof(int64_t) * (size_t)n, c.s));
+    k_row_sums<<<gr, TPB, 0, c.s>>>(c.rk2.p + na, (const int64_t*)c.rv2.p + na, na, c.bits, n, L0.kin.p, nullptr,
+                                    nullptr);
     CKL("k_row_sums(in)");
   }
   k_iota<<<grid_for(n, TPB), TPB, 0, c.s>>>(L0.lab.p, n);

@@ -257,30 +257,30 @@ static i128 qnum(const ldl_ctx& c) {
 // ---------------------------------------------------------------- allocation
 void alloc_globals(ldl_ctx& c) {
   const int64_t n = c.n;
-  c.Kout.exact(n);
-  if (c.directed) c.Kin.exact(n);
-  c.e.exact(n);
+  Slab& S = c.globals;
+  // (the cleared arrays first: one clear)
   DBuf<int32_t>* st[] = {&c.stS, &c.stU, &c.stMv, &c.stB, &c.stM0, &c.stD, &c.stC, &c.stR, &c.stX, &c.stT, &c.stE,
-                         &c.stCh, &c.stL, &c.ckf};
-  for (auto* b : st) {
-    b->exact(n);
-    CK(cudaMemsetAsync(b->p, 0, sizeof(int32_t) * (size_t)n, c.s));
-  }
+                         &c.stCh, &c.stL, &c.ckf, &c.role};
+  for (auto* b : st) S.add(*b, n);
+  const size_t cleared = S.parts.size();
   DBuf<int32_t>* ls[] = {&c.lU, &c.lS, &c.lUstar, &c.lMv, &c.lM0, &c.lD, &c.lC, &c.lR, &c.lR2, &c.lX, &c.lT,
                          &c.lE2, &c.lCh, &c.lChg, &c.lTmp, &c.lG, &c.comp, &c.nbr, &c.cv, &c.csrc, &c.cdst, &c.cst, &c.bv,
-                         &c.bsrc, &c.bdst, &c.oldlab, &c.par_old, &c.lab_before, &c.binT, &c.binS, &c.binM, &c.binM2, &c.binC, &c.binL};
-  for (auto* b : ls) b->exact(n);
-  c.best.exact(n);
+                         &c.bsrc, &c.bdst, &c.oldlab, &c.par_old, &c.lab_before, &c.binT, &c.binS, &c.binM, &c.binM2, &c.binC, &c.binL,
+                         &c.best};
+  for (auto* b : ls) S.add(*b, n);
+  S.add(c.Kout, n);
+  if (c.directed) S.add(c.Kin, n);
+  S.add(c.e, n);
+  S.add(c.cghi, n);
+  S.add(c.cglo, n);
+  S.add(c.snapKo, 2 * n);
+  S.add(c.snapKi, 2 * n);
+  S.add(c.snapE, 2 * n);
+  S.add(c.binLoff, n + 1);
+  S.add(c.binLsz, n + 1);
+  S.alloc();
+  CK(cudaMemsetAsync(S.base, 0, S.span(0, cleared), c.s));
   CK(cudaMemsetAsync(c.best.p, 0xff, sizeof(int32_t) * (size_t)n, c.s));
-  c.role.exact(n);
-  CK(cudaMemsetAsync(c.role.p, 0, sizeof(int32_t) * (size_t)n, c.s));
-  c.cghi.exact(n);
-  c.cglo.exact(n);
-  c.snapKo.exact(2 * n);
-  c.snapKi.exact(2 * n);
-  c.snapE.exact(2 * n);
-  c.binLoff.exact(n + 1);
-  c.binLsz.exact(n + 1);
   c.d_sc = (DevScalars*)dalloc(sizeof(DevScalars));
   CK(cudaMemsetAsync(c.d_sc, 0, sizeof(DevScalars), c.s));
   c.dcnt = (int32_t*)dalloc(sizeof(int32_t) * K_COUNT);
@@ -316,6 +316,7 @@ void free_all(ldl_ctx& c) {
   c.cglo.release();
   c.pb_lo.release();
   c.pb_c.release();
+  c.globals.release();
   c.gtab_clean = 0;
   c.upd.release();
   c.snap.release();
@@ -345,10 +346,10 @@ void free_all(ldl_ctx& c) {
 // lUstar / stU (epoch epU) hold U*.  Moved nodes go to lMv (epMv) and, at
 // level 0, to lM0 (epM0).
 static int64_t move_loop(ldl_ctx& c, int r, int rounds, int32_t epU, int32_t epMv, int32_t epM0, int32_t epCh,
-                         int32_t nU, int64_t s_max, SplitRun* spec) {
+                         int32_t nU, int64_t s_max, SplitRun* spec, bool whole = false) {
   // nU = |U| on entry; later rounds take it from the end of the previous one.
   // s_max bounds the first round's candidate set.  With spec the level's split
-  // may start behind the last sweep.
+  // may start behind the last sweep.  whole: U holds every node of the level.
   // Returns the committed moves, an upper bound of the distinct moved nodes
   // (lMv), which is empty exactly when it is 0.
   int64_t committed = 0;
@@ -359,12 +360,18 @@ static int64_t move_loop(ldl_ctx& c, int r, int rounds, int32_t epU, int32_t epM
     c.res.rounds++;
     stage_begin(c);
     const int32_t epS = c.next_epoch();
-    zero_cnt(c, K_S);
-    expand_set(c, r, c.lU.p, K_U, c.stS.p, epS, c.lS.p, K_S, nU);
+    // (with U every node of the level, as in a static level's first round,
+    // S = U)
+    const bool all = j == 0 && whole;
+    if (!all) {
+      zero_cnt(c, K_S);
+      expand_set(c, r, c.lU.p, K_U, c.stS.p, epS, c.lS.p, K_S, nU);
+    }
     stage_end(c, ST_EXPAND);
     // |S| stays on the device: the sweep's kernels stride over it (n bounds
     // their grids) and it comes back with the candidates (β test)
-    const SweepOut so = sweep(c, r, 0, c.lS.p, K_S, j == 0 ? std::min(c.n, s_max) : c.n, spec);
+    const SweepOut so = all ? sweep(c, r, 0, c.lU.p, K_U, nU)
+                            : sweep(c, r, 0, c.lS.p, K_S, j == 0 ? std::min(c.n, s_max) : c.n, spec);
     const int32_t nS = so.nlist, nc = so.nc, nb = so.nb;
     if (nc == 0) break;
     c.res.rejected += nc - nb;
@@ -450,7 +457,7 @@ static void static_build(ldl_ctx& c) {
     zero_cnt(c, K_MV);
     zero_cnt(c, K_M0);
     zero_cnt(c, K_CH);
-    const int64_t mv = move_loop(c, r, c.prm.M_static, epU, epMv, epM0, epCh, nU, c.n, nullptr);
+    const int64_t mv = move_loop(c, r, c.prm.M_static, epU, epMv, epM0, epCh, nU, c.n, nullptr, true);
     if (r > 0) pushdown(c, r, epCh, mv);
     if (r == L) break;
     level_alloc(c, r + 1);

@@ -1050,7 +1050,8 @@ __device__ inline void claim(int32_t* best, int32_t c, int32_t i, const int64_t*
 // next round's slot is cleared while the current one is still being read).
 // Every block reads the same count after the barrier, so all leave together;
 // at most nc + 1 rounds (each decides the earliest undecided candidate).
-__global__ void __launch_bounds__(TPB) k_dec_grid(int32_t nc, int32_t* cst, const int32_t* cv, const int32_t* src,
+constexpr int DG_TPB = 1024;
+__global__ void __launch_bounds__(DG_TPB) k_dec_grid(int32_t nc, int32_t* cst, const int32_t* cv, const int32_t* src,
                                                   const int32_t* dst, const int64_t* ghi, const uint64_t* glo,
                                                   int32_t* role, int32_t* best, int32_t* bv, int32_t* bsrc,
                                                   int32_t* bdst, int32_t* nb, int32_t* undecided, int32_t* stat) {
@@ -1723,10 +1724,9 @@ DecoupleOut decouple(ldl_ctx& c, const HostRead* extra, int n_extra, SplitRun* s
     return {nc, nb, stat};
   }
   // many candidates: one cooperative launch of co-resident blocks runs all rounds
-  int per_sm = 0;
-  const int sms = device_sms();
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dec_grid, TPB, 0));
-  const int g = std::max(1, std::min(grid_for(nc, TPB), sms * per_sm));
+  // (at most one large block per SM: the grid barriers, three a round, take
+  // longer with more blocks)
+  const int g = std::min(div_up(nc, DG_TPB), device_sms());
   zero_cnt(c, K_B);
   int32_t ncv = nc;
   int32_t* cst = c.cst.p;
@@ -1738,7 +1738,7 @@ DecoupleOut decouple(ldl_ctx& c, const HostRead* extra, int n_extra, SplitRun* s
   int32_t* undec = (int32_t*)fresh(c, 2, c.d_sc->home);  // the two round counters
   int32_t* statp = c.cp[K_UNDEC];
   void* args[] = {&ncv, &cst, &cvp, &srcp, &dstp, &ghi, &glo, &role, &best, &bv, &bsrc, &bdst, &nbp, &undec, &statp};
-  CK(cudaLaunchCooperativeKernel((const void*)k_dec_grid, dim3(g), dim3(TPB), args, 0, c.s));
+  CK(cudaLaunchCooperativeKernel((const void*)k_dec_grid, dim3(g), dim3(DG_TPB), args, 0, c.s));
   CKL("k_dec_grid");
   const HostRead rf[2] = {{c.cp[K_B], &nb, sizeof(int32_t)}, {c.cp[K_UNDEC], &stat, sizeof(int32_t)}};
   host_read(c, rf, 2);
