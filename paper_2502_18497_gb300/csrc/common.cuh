@@ -333,6 +333,35 @@ struct SlackCSR {
   DBuf<int64_t> lrow, loff, lsrc, lpos, lofs;
   DBuf<int32_t> llen, lcap, lcol;
   DBuf<WT> lw, lold;
+  Slab log;              // all of them but lofs
+  int64_t rcap = 0, wcap = 0, ccap = 0;  // row, weight and content entries it holds
+  // Room in the log for this many entries in all, its contents kept.
+  void reserve_log(int64_t nr, int64_t nw, int64_t nc, cudaStream_t s) {
+    if (nr <= rcap && nw <= wcap && nc <= ccap) return;
+    auto grown = [](int64_t have, int64_t want) { return want <= have ? have : want + want / 2 + 256; };
+    const int64_t r2 = grown(rcap, nr), w2 = grown(wcap, nw), c2 = grown(ccap, nc);
+    Slab fresh;
+    DBuf<int64_t> row2, off2, src2, pos2;
+    DBuf<int32_t> len2, cap2, col2;
+    DBuf<WT> w_2, old2;
+    fresh.add(row2, r2); fresh.add(off2, r2); fresh.add(src2, r2); fresh.add(len2, r2); fresh.add(cap2, r2);
+    fresh.add(pos2, w2); fresh.add(old2, w2);
+    fresh.add(col2, c2); fresh.add(w_2, c2);
+    fresh.alloc();
+    auto move = [&](auto& to, auto& from, int64_t used) {
+      if (used) CK(cudaMemcpyAsync(to.p, from.p, (size_t)used * sizeof(*to.p), cudaMemcpyDeviceToDevice, s));
+    };
+    move(row2, lrow, rtop); move(off2, loff, rtop); move(src2, lsrc, rtop); move(len2, llen, rtop);
+    move(cap2, lcap, rtop);
+    move(pos2, lpos, wtop); move(old2, lold, wtop);
+    move(col2, lcol, ctop); move(w_2, lw, ctop);
+    CK(cudaStreamSynchronize(s));
+    if (log.base) dfree(log.base);
+    log.base = fresh.base;
+    lrow = row2; loff = off2; lsrc = src2; lpos = pos2;
+    llen = len2; lcap = cap2; lcol = col2; lw = w_2; lold = old2;
+    rcap = r2; wcap = w2; ccap = c2;
+  }
   void release() {
     off.release(); len.release(); cap.release(); tables.release(); col.release(); w.release();
     for (auto& x : retired) {
@@ -342,6 +371,8 @@ struct SlackCSR {
     retired.clear();
     lrow.release(); loff.release(); lsrc.release(); lpos.release(); lofs.release();
     llen.release(); lcap.release(); lcol.release(); lw.release(); lold.release();
+    log.release();
+    rcap = wcap = ccap = 0;
     events.clear();
     logging = false;
     pool_top = 0;

@@ -587,15 +587,7 @@ int64_t csr_finish(SlackCSR<WT>& g, const CsrRecords& r, const int64_t (&tot)[6]
   WT* swp = nullptr;
   if (g.logging) {
     // everything a rollback needs, reserved before any change
-    g.lrow.reserve(g.rtop + nseg + 1, s, true);
-    g.loff.reserve(g.rtop + nseg + 1, s, true);
-    g.lsrc.reserve(g.rtop + nseg + 1, s, true);
-    g.llen.reserve(g.rtop + nseg + 1, s, true);
-    g.lcap.reserve(g.rtop + nseg + 1, s, true);
-    g.lpos.reserve(g.wtop + nrec + 1, s, true);
-    g.lold.reserve(g.wtop + nrec + 1, s, true);
-    g.lcol.reserve(g.ctop + stotal + 1, s, true);
-    g.lw.reserve(g.ctop + stotal + 1, s, true);
+    g.reserve_log(g.rtop + nseg + 1, g.wtop + nrec + 1, g.ctop + stotal + 1, s);
     u = {g.lrow.p + g.rtop, g.loff.p + g.rtop, g.lsrc.p + g.rtop, g.lpos.p + g.wtop,
          g.llen.p + g.rtop, g.lcap.p + g.rtop, g.lold.p + g.wtop, g.ctop};
     scol = g.lcol.p + g.ctop;

@@ -591,25 +591,25 @@ __global__ void __launch_bounds__(SM_THREADS) k_rs_small_reduce(const u64* keys,
   }
 }
 
-// Whole sort in one thread-block cluster of CS_CL blocks (n <= CS_CL *
-// CS_TILE): block c holds the pairs at positions [c * CS_TILE, (c+1) *
-// CS_TILE), CS_ITEMS per thread in registers.  Per 8-bit pass every warp
-// ranks its contiguous sub-tile (stable), each block publishes its digit
-// counts in shared memory, and after a cluster barrier every block reads all
-// blocks' counts (distributed shared memory) to place each of its pairs at
-// its global position: digit start + counts of lower blocks + counts of
-// lower warps + rank.  The pair is stored into the shared memory of the block
-// that owns that position; after a second barrier each block reloads its
-// slice.  The pairs never leave the chip between passes.
+// Whole sort in one thread-block cluster of CL blocks (n <= CL * CS_TILE):
+// the pairs are cut into CL tiles of T (a multiple of the block's threads, so
+// that short lists spread over the cluster too), block c holds the pairs at
+// positions [c * T, (c+1) * T), up to CS_ITEMS per thread in registers.  Per
+// 8-bit pass every warp ranks its contiguous sub-tile (stable), each block
+// publishes its digit counts in shared memory, and after a cluster barrier
+// every block reads all blocks' counts (distributed shared memory) to place
+// each of its pairs at its global position: digit start + counts of lower
+// blocks + counts of lower warps + rank.  The pair is stored into the shared
+// memory of the block that owns that position; after a second barrier each
+// block reloads its slice.  The pairs never leave the chip between passes.
 constexpr int CS_THREADS = 512;
 constexpr int CS_ITEMS = 12;
 constexpr int CS_TILE = CS_THREADS * CS_ITEMS;  // 6144 pairs, 96 KB per block
-constexpr int CS_CL = 8;
 constexpr int CS_NW = CS_THREADS / WARP;
-constexpr int CS_MAX = CS_CL * CS_TILE;
 
-__global__ void __cluster_dims__(CS_CL, 1, 1) __launch_bounds__(CS_THREADS, 1)
-    k_rs_cluster(u64* keys, u64* vals, int n, int lo_bit, int bits, RsExt x) {
+template <int CL>
+__global__ void __launch_bounds__(CS_THREADS, 1) k_rs_cluster(u64* keys, u64* vals, int n, int lo_bit, int bits,
+                                                              RsExt x) {
   extern __shared__ u64 cs_smem[];
   u64* sk = cs_smem;
   u64* sv = cs_smem + CS_TILE;
@@ -620,16 +620,19 @@ __global__ void __cluster_dims__(CS_CL, 1, 1) __launch_bounds__(CS_THREADS, 1)
   cg::cluster_group cl = cg::this_cluster();
   const int c = (int)cl.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int base = c * CS_TILE;
   if (x.n_dev) n = min(n, *x.n_dev);
-  const int tile_n = max(0, min(CS_TILE, n - base));
+  const int items = max(1, (n + CL * CS_THREADS - 1) / (CL * CS_THREADS));  // per thread
+  const int T = items * CS_THREADS, base = c * T;
+  const int tile_n = max(0, min(T, n - base));
+  const uint32_t magic = (uint32_t)((((u64)1 << 32) + T - 1) / T);  // p / T = p * magic >> 32 for p < 2^17
   u64 key[CS_ITEMS], val[CS_ITEMS];
   for (int k = 0; k < CS_ITEMS; ++k) {
-    const int li = wid * (CS_ITEMS * 32) + k * 32 + lane;
-    key[k] = li < tile_n ? keys[base + li] : 0;
-    val[k] = li < tile_n ? vals[base + li] : 0;
+    const int li = wid * (items * 32) + k * 32 + lane;
+    const bool on = k < items && li < tile_n;
+    key[k] = on ? keys[base + li] : 0;
+    val[k] = on ? vals[base + li] : 0;
     if (x.tbits) key[k] = transposed(key[k], x.tbits, x.row_off);
-    if (x.zero && li < tile_n) x.zero[base + li] = 0;
+    if (x.zero && on) x.zero[base + li] = 0;
   }
   if (x.tbits) {  // the result goes behind the input
     keys += n;
@@ -639,8 +642,10 @@ __global__ void __cluster_dims__(CS_CL, 1, 1) __launch_bounds__(CS_THREADS, 1)
     for (int d = lane; d < 256; d += 32) whist[wid][d] = 0;
     __syncwarp();
     int rk[CS_ITEMS];
+#pragma unroll
     for (int k = 0; k < CS_ITEMS; ++k) {
-      const int li = wid * (CS_ITEMS * 32) + k * 32 + lane;
+      if (k >= items) break;  // the same in every thread
+      const int li = wid * (items * 32) + k * 32 + lane;
       const int d = li < tile_n ? (int)((key[k] >> shift) & 255) : 256;
       const unsigned peers = __match_any_sync(0xffffffffu, d);
       const int before = d < 256 ? whist[wid][d] : 0;
@@ -662,7 +667,7 @@ __global__ void __cluster_dims__(CS_CL, 1, 1) __launch_bounds__(CS_THREADS, 1)
     cl.sync();  // every block's counts are published
     if (tid < 256) {
       int tot = 0, lower = 0;
-      for (int b = 0; b < CS_CL; ++b) {
+      for (int b = 0; b < CL; ++b) {
         const int x = cl.map_shared_rank(hist, b)[tid];
         tot += x;
         if (b < c) lower += x;
@@ -690,27 +695,27 @@ __global__ void __cluster_dims__(CS_CL, 1, 1) __launch_bounds__(CS_THREADS, 1)
     }
     __syncthreads();
     for (int k = 0; k < CS_ITEMS; ++k) {
-      const int li = wid * (CS_ITEMS * 32) + k * 32 + lane;
-      if (li < tile_n) {
+      const int li = wid * (items * 32) + k * 32 + lane;
+      if (k < items && li < tile_n) {
         const int d = (int)((key[k] >> shift) & 255);
         const int p = tpos[d] + whist[wid][d] + rk[k];
-        const int owner = p / CS_TILE, slot = p - owner * CS_TILE;
+        const int owner = (int)__umulhi((uint32_t)p, magic), slot = p - owner * T;
         cl.map_shared_rank(sk, owner)[slot] = key[k];
         cl.map_shared_rank(sv, owner)[slot] = val[k];
       }
     }
     cl.sync();  // every pair is in place; counts and staging are reused next pass
     for (int k = 0; k < CS_ITEMS; ++k) {
-      const int li = wid * (CS_ITEMS * 32) + k * 32 + lane;
-      if (li < tile_n) {
+      const int li = wid * (items * 32) + k * 32 + lane;
+      if (k < items && li < tile_n) {
         key[k] = sk[li];
         val[k] = sv[li];
       }
     }
   }
   for (int k = 0; k < CS_ITEMS; ++k) {
-    const int li = wid * (CS_ITEMS * 32) + k * 32 + lane;
-    if (li < tile_n) {
+    const int li = wid * (items * 32) + k * 32 + lane;
+    if (k < items && li < tile_n) {
       keys[base + li] = key[k];
       vals[base + li] = val[k];
     }
@@ -928,21 +933,56 @@ static void small_smem_opt_in(const void* f) {
   done[done[0] ? 1 : 0] = f;
 }
 
+// Blocks of a sorting cluster: 16 where the device can place such a cluster
+// (it is beyond the portable size), else 8.  Asked once per device and thread.
+constexpr int CS_SMEM = 2 * CS_TILE * (int)sizeof(u64);
+static int cluster_size() {
+  static thread_local int size = 0, at_dev = -1;
+  int dev = 0;
+  CK(cudaGetDevice(&dev));
+  if (at_dev == dev) return size;
+  CK(cudaFuncSetAttribute(k_rs_cluster<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, CS_SMEM));
+  CK(cudaFuncSetAttribute(k_rs_cluster<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, CS_SMEM));
+  CK(cudaFuncSetAttribute(k_rs_cluster<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(16);
+  cfg.blockDim = dim3(CS_THREADS);
+  cfg.dynamicSmemBytes = CS_SMEM;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 16;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, k_rs_cluster<16>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    clusters = 0;
+  }
+  size = clusters > 0 ? 16 : 8;
+  at_dev = dev;
+  return size;
+}
+
 // Launches the sort of n pairs (an upper bound with x.n_dev).  A plain sort's
 // result is in (keys, vals) afterwards, which may have been swapped with (tk,
 // tv); a transposing one's lies behind its input.
 static void sort_launch(u64*& keys, u64*& vals, u64*& tk, u64*& tv, int64_t n, int bits, Prims& P, cudaStream_t s,
                         int lo_bit, const RsExt& x) {
-  if (n <= CS_MAX) {  // one cluster, the pairs kept on chip
-    const int smem = 2 * CS_TILE * (int)sizeof(u64);
-    static thread_local int cs_attr_dev = -1;
-    int dev = 0;
-    CK(cudaGetDevice(&dev));
-    if (cs_attr_dev != dev) {
-      CK(cudaFuncSetAttribute(k_rs_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-      cs_attr_dev = dev;
-    }
-    k_rs_cluster<<<CS_CL, CS_THREADS, smem, s>>>(keys, vals, (int)n, lo_bit, bits, x);
+  const int cl = cluster_size();
+  if (n <= (int64_t)cl * CS_TILE) {  // one cluster, the pairs kept on chip
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(cl);
+    cfg.blockDim = dim3(CS_THREADS);
+    cfg.dynamicSmemBytes = CS_SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cl;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    CK(cudaLaunchKernelEx(&cfg, cl == 16 ? k_rs_cluster<16> : k_rs_cluster<8>, keys, vals, (int)n, lo_bit, bits, x));
     CKL("k_rs_cluster");
     return;
   }

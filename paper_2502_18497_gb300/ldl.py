@@ -301,7 +301,9 @@ class LDL:
         return Level(*a)
 
     def labels(self) -> np.ndarray:
-        return self.level(0).lab
+        lab = np.empty(self.n, np.int32)
+        self._check(load().ldl_get_level(self._h, 0, _ptr(lab), None, None, None, None, None))
+        return lab
 
     def level_adj(self, r: int):
         nnz = C.c_int64()
