@@ -332,21 +332,43 @@ __global__ void __launch_bounds__(RS_THREADS, 4) k_rs_scatter(const u64* keys, c
                   out_off ? ovals + n : ovals, n, shift, nb, goff, dtot, blockIdx.x, first ? x.tbits : 0, x.row_off);
 }
 
-// The whole multi-tile sort in one cooperative launch (all nb tiles'
-// blocks co-resident): per 8-bit pass the tile histograms, the per-digit
-// scans over tiles and the scatter, separated by grid barriers, ping-ponging
-// between (keys, vals) and (tk, tv).  Replaces three launches per pass.  A
-// transposing sort ping-pongs between the place behind its input and (tk,
-// tv) such that the last pass ends there.
-__global__ void __launch_bounds__(RS_THREADS, 4) k_rs_coop(u64* keys, u64* vals, u64* tk, u64* tv, int64_t n,
-                                                           int lo_bit, int bits, int64_t* ghist, int64_t* dtot,
+// The whole multi-tile sort in one cooperative launch, one block per SM and one
+// tile per block: the tiles are T pairs, a multiple of the block's threads, so
+// that any list up to CO_ITEMS pairs per thread is one wave.  Per 8-bit pass a
+// block loads its tile into registers once, ranks it per warp (stable) and
+// publishes its digit counts; warps scan the digits over the tiles; the tile
+// goes through shared memory in digit order to its global places.  A grid
+// barrier after each.  Bound by the barriers and the passes' latency: 82 us for
+// six passes over some 10^5 pairs (2M-vertex power-law graph), 113 with four
+// small blocks per SM, a second load and a scan block per digit.  A transposing sort ping-pongs between the place
+// behind its input and (tk, tv) such that the last pass ends there.
+constexpr int CO_THREADS = 512;
+constexpr int CO_ITEMS = 16;
+constexpr int CO_TILE = CO_THREADS * CO_ITEMS;
+constexpr int CO_NW = CO_THREADS / WARP;
+struct CoShared {
+  int32_t whist[CO_NW][256];
+  int32_t tstart[256];
+  int64_t gstart[256];
+  u64 sk[CO_TILE];
+  u64 sv[CO_TILE];
+};
+
+__global__ void __launch_bounds__(CO_THREADS, 1) k_rs_coop(u64* keys, u64* vals, u64* tk, u64* tv, int64_t n,
+                                                           int lo_bit, int bits, int32_t* ghist, int32_t* dtot,
                                                            RsExt x) {
+  extern __shared__ __align__(16) unsigned char co_smem[];
+  CoShared& m = *(CoShared*)co_smem;
   cg::grid_group grid = cg::this_grid();
   if (x.n_dev) n = min(n, (int64_t)*x.n_dev);
-  const int64_t nb = (n + RS_TILE - 1) / RS_TILE;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int items = (int)max((int64_t)1, (n + (int64_t)gridDim.x * CO_THREADS - 1) / ((int64_t)gridDim.x * CO_THREADS));
+  const int T = items * CO_THREADS;
+  const int nb = (int)((n + T - 1) / T), b = blockIdx.x;  // nb <= gridDim.x
+  const int64_t base = (int64_t)b * T;
+  const int tile_n = (int)max((int64_t)0, min((int64_t)T, n - base));
   if (x.zero)
-    for (int64_t i = (int64_t)blockIdx.x * RS_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * RS_THREADS)
-      x.zero[i] = 0;
+    for (int64_t i = (int64_t)b * CO_THREADS + tid; i < n; i += (int64_t)gridDim.x * CO_THREADS) x.zero[i] = 0;
   u64 *ik = keys, *iv = vals, *ok = tk, *ov = tv;
   u64 *nk = keys, *nv = vals;  // written by the pass after the first
   if (x.tbits) {
@@ -358,13 +380,81 @@ __global__ void __launch_bounds__(RS_THREADS, 4) k_rs_coop(u64* keys, u64* vals,
     }
   }
   for (int shift = lo_bit; shift < bits; shift += 8) {
-    const int tb = shift == lo_bit ? x.tbits : 0;
-    for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) rs_hist_tile(ik, n, shift, nb, ghist, b, tb, x.row_off);
+    u64 key[CO_ITEMS], val[CO_ITEMS];
+    int rk[CO_ITEMS];
+#pragma unroll
+    for (int k = 0; k < CO_ITEMS; ++k) {
+      const int li = wid * (items * 32) + k * 32 + lane;
+      const bool on = k < items && li < tile_n;
+      key[k] = on ? ik[base + li] : 0;
+      val[k] = on ? iv[base + li] : 0;
+      if (x.tbits && shift == lo_bit) key[k] = transposed(key[k], x.tbits, x.row_off);
+    }
+    for (int d = lane; d < 256; d += 32) m.whist[wid][d] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < CO_ITEMS; ++k) {
+      if (k >= items) break;  // the same in every thread
+      const int li = wid * (items * 32) + k * 32 + lane;
+      const int d = li < tile_n ? (int)((key[k] >> shift) & 255) : 256;
+      const unsigned peers = __match_any_sync(0xffffffffu, d);
+      const int before = d < 256 ? m.whist[wid][d] : 0;
+      rk[k] = before + __popc(peers & ((1u << lane) - 1u));
+      __syncwarp();
+      if (d < 256 && lane == __ffs(peers) - 1) m.whist[wid][d] = before + __popc(peers);
+      __syncwarp();
+    }
+    __syncthreads();
+    int cnt = 0;
+    if (tid < 256) {
+      for (int w = 0; w < CO_NW; ++w) {  // thread = digit
+        const int c = m.whist[w][tid];
+        m.whist[w][tid] = cnt;
+        cnt += c;
+      }
+      if (b < nb) ghist[tid * nb + b] = cnt;
+    }
+    u64 total;
+    const u64 ts = block_scan<CO_THREADS>((u64)cnt, &total);
+    if (tid < 256) m.tstart[tid] = (int32_t)ts;
     grid.sync();
-    for (int d = blockIdx.x; d < 256; d += gridDim.x) rs_dscan_digit(ghist, nb, dtot, d);
+    for (int d = b * CO_NW + wid; d < 256; d += gridDim.x * CO_NW) {  // a warp per digit
+      int32_t* row = ghist + (int64_t)d * nb;
+      int carry = 0;
+      for (int c0 = 0; c0 < nb; c0 += 32) {
+        const int v = c0 + lane < nb ? row[c0 + lane] : 0;
+        int incl = v;
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += y;
+        }
+        if (c0 + lane < nb) row[c0 + lane] = carry + incl - v;
+        carry += __shfl_sync(0xffffffffu, incl, 31);
+      }
+      if (lane == 0) dtot[d] = carry;
+    }
     grid.sync();
-    for (int64_t b = blockIdx.x; b < nb; b += gridDim.x)
-      rs_scatter_tile(ik, iv, ok, ov, n, shift, nb, ghist, dtot, b, tb, x.row_off);
+    const u64 dbase = block_scan<CO_THREADS>(tid < 256 ? (u64)dtot[tid] : 0, &total);
+    if (tid < 256 && b < nb) m.gstart[tid] = (int64_t)dbase + ghist[tid * nb + b];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < CO_ITEMS; ++k) {
+      const int li = wid * (items * 32) + k * 32 + lane;
+      if (k < items && li < tile_n) {
+        const int d = (int)((key[k] >> shift) & 255);
+        const int p = m.tstart[d] + m.whist[wid][d] + rk[k];
+        m.sk[p] = key[k];
+        m.sv[p] = val[k];
+      }
+    }
+    __syncthreads();
+    for (int j = tid; j < tile_n; j += CO_THREADS) {
+      const u64 k = m.sk[j];
+      const int d = (int)((k >> shift) & 255);
+      const int64_t p = m.gstart[d] + (j - m.tstart[d]);
+      ok[p] = k;
+      ov[p] = m.sv[j];
+    }
     grid.sync();
     ik = ok; iv = ov;
     u64* t = ok; ok = nk; nk = t;
@@ -987,20 +1077,24 @@ static void sort_launch(u64*& keys, u64*& vals, u64*& tk, u64*& tv, int64_t n, i
     return;
   }
   const int64_t nb = (n + RS_TILE - 1) / RS_TILE;
-  P.hist.reserve(256 * nb + 1, s);
+  P.hist.reserve(std::max<int64_t>(256 * nb + 1, 128 * (int64_t)device_sms() + 1), s);
   P.bsum.reserve(256, s);
-  // up to a few hundred tiles: one cooperative launch for all passes
-  static thread_local int coop_per_sm = -1;
-  if (coop_per_sm < 0) CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&coop_per_sm, k_rs_coop, RS_THREADS, 0));
-  const int64_t coop_max = (int64_t)coop_per_sm * device_sms();
-  if (nb <= coop_max && nb <= 1024) {
-    const int grid = (int)std::max<int64_t>(nb, std::min<int64_t>(256, coop_max));
+  // up to one tile per SM: one cooperative launch for all passes
+  if (n <= (int64_t)device_sms() * CO_TILE) {
+    static thread_local int co_attr_dev = -1;
+    int dev = 0;
+    CK(cudaGetDevice(&dev));
+    if (co_attr_dev != dev) {
+      CK(cudaFuncSetAttribute(k_rs_coop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CoShared)));
+      co_attr_dev = dev;
+    }
     int64_t n_ = n;
     int lo_ = lo_bit, bits_ = bits;
-    int64_t *gh = P.hist.p, *dt = P.bsum.p;
+    int32_t *gh = (int32_t*)P.hist.p, *dt = (int32_t*)P.bsum.p;
     RsExt x_ = x;
     void* args[] = {&keys, &vals, &tk, &tv, &n_, &lo_, &bits_, &gh, &dt, &x_};
-    CK(cudaLaunchCooperativeKernel((const void*)k_rs_coop, dim3(grid), dim3(RS_THREADS), args, 0, s));
+    CK(cudaLaunchCooperativeKernel((const void*)k_rs_coop, dim3(device_sms()), dim3(CO_THREADS), args, sizeof(CoShared),
+                                   s));
     CKL("k_rs_coop");
     if (!x.tbits)
       for (int shift = lo_bit; shift < bits; shift += 8) {  // where the result ended up
