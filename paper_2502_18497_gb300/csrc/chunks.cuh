@@ -75,23 +75,6 @@ __device__ inline int64_t chunk_begin(const ChunkMap& m, ChunkPre& sh) {
   return base;
 }
 
-// Last i in [0, n) with pre[i] <= c, by the whole warp (c the same in every
-// lane): 32 pivots a step, so three dependent loads for 10^4 nodes instead of
-// fourteen.
-template <class T>
-__device__ inline int64_t warp_find(const T* pre, int64_t n, int64_t c) {
-  const int lane = threadIdx.x & 31;
-  int64_t lo = 0, hi = n;
-  __syncwarp();
-  while (hi - lo > 1) {
-    const int64_t step = (hi - lo + 31) >> 5, at = lo + (lane + 1) * step;
-    const int k = __popc(__ballot_sync(0xffffffffu, at < hi && pre[at] <= c));
-    lo += k * step;
-    hi = min(hi, lo + step);
-  }
-  return lo;
-}
-
 // Chunk c, the same in every lane of a warp that calls it together.
 __device__ inline Chunk chunk_of(const ChunkMap& m, const ChunkPre& sh, int64_t c) {
   const int64_t lo = m.pre ? warp_find(m.pre, m.n_hint, c) : warp_find(sh.pre, min(m.n_hint, (int64_t)*m.nlist), c);

@@ -3,16 +3,6 @@
 #include "common.cuh"
 #include "prims.cuh"
 
-__device__ inline int64_t find_seg(const int64_t* pre, int64_t nseg, int64_t t) {
-  // last s with pre[s] <= t (pre is an exclusive scan, pre[0] = 0)
-  int64_t lo = 0, hi = nseg;
-  while (hi - lo > 1) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (pre[mid] <= t) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
 // last s in [lo, hi] with pre[s] <= t
 __device__ inline int64_t seg_in(const int64_t* pre, int64_t lo, int64_t hi, int64_t t) {
   while (lo < hi) {
@@ -23,20 +13,29 @@ __device__ inline int64_t seg_in(const int64_t* pre, int64_t lo, int64_t hi, int
 }
 
 // Items [0, total) split into segments by the exclusive scan pre.  Each warp
-// takes runs of SEG_RUN consecutive items: two warp-uniform searches bound the
-// run's segments, and each item then searches only that narrow range.
+// takes runs of SEG_RUN consecutive items: two warp-wide searches bound the
+// run's segments.  f(t0, n, slo, shi) is called by the whole warp for the n
+// items from t0 on, whose segments are slo .. shi; lane l's items are t0 + l,
+// t0 + l + 32, ...
 constexpr int SEG_RUN = 256;
-#define FOR_SEG_ITEMS(t, s, pre, nseg, total)                                                       \
-  const int64_t warp_ = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;                     \
-  const int64_t nwarps_ = ((int64_t)gridDim.x * blockDim.x) >> 5;                                   \
-  for (int64_t c0_ = warp_ * SEG_RUN; c0_ < (total); c0_ += nwarps_ * SEG_RUN) {                   \
-    const int64_t c1_ = min(c0_ + SEG_RUN, (int64_t)(total)) - 1;                                   \
-    const int64_t slo_ = find_seg(pre, nseg, c0_), shi_ = find_seg(pre, nseg, c1_);                 \
-    for (int64_t t = c0_ + (threadIdx.x & 31); t <= c1_; t += 32) {                                 \
-      const int64_t s = seg_in(pre, slo_, shi_, t);
-#define END_SEG_ITEMS \
-  }                   \
+constexpr int SEG_PL = SEG_RUN / 32;  // items per lane
+template <class F>
+__device__ inline void for_seg_runs(const int64_t* pre, int64_t nseg, int64_t total, F f) {
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t t0 = warp * SEG_RUN; t0 < total; t0 += nwarps * SEG_RUN) {
+    const int n = (int)min((int64_t)SEG_RUN, total - t0);
+    const int64_t slo = warp_find(pre, nseg, t0);
+    const int64_t shi =
+        slo + 1 >= nseg || pre[slo + 1] > t0 + n - 1 ? slo : warp_find(pre, nseg, t0 + n - 1, slo + 1);
+    f(t0, n, slo, shi);
   }
+}
+
+// The segment of item t of such a run.
+__device__ inline int64_t seg_of(const int64_t* pre, int64_t slo, int64_t shi, int64_t t) {
+  return slo == shi ? slo : seg_in(pre, slo, shi, t);
+}
 
 struct CsrScratch {
   // per record and per segment of an update (for max_rec of them, in one slab)

@@ -877,14 +877,17 @@ __global__ void k_csr_records(const int64_t* rp, const int32_t* col, const int32
     if (rp[v + 1] < rp[v]) set_err(err, 0, LDL_E_INVALID);
   }
   bool bad = false;
-  FOR_SEG_ITEMS(t, v, rp, n, nnz)
-    const int32_t c = col[t], x = w[t];
-    if (c < 0 || c >= n) set_err(err, 0, LDL_E_RANGE);
-    if (x < 1) set_err(err, 0, LDL_E_INVALID);
-    bad |= t > 0 && t > rp[v] && col[t - 1] >= c;
-    rk[t] = ((u64)v << bits) | (u64)(uint32_t)c;
-    rv[t] = (u64)(int64_t)x;
-  END_SEG_ITEMS
+  for_seg_runs(rp, n, nnz, [&](int64_t t0, int cnt, int64_t slo, int64_t shi) {
+    for (int64_t t = t0 + (threadIdx.x & 31); t < t0 + cnt; t += 32) {
+      const int64_t v = seg_of(rp, slo, shi, t);
+      const int32_t c = col[t], x = w[t];
+      if (c < 0 || c >= n) set_err(err, 0, LDL_E_RANGE);
+      if (x < 1) set_err(err, 0, LDL_E_INVALID);
+      bad |= t > 0 && t > rp[v] && col[t - 1] >= c;
+      rk[t] = ((u64)v << bits) | (u64)(uint32_t)c;
+      rv[t] = (u64)(int64_t)x;
+    }
+  });
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicExch(unsorted, 1);
 }
 

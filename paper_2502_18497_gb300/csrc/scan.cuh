@@ -32,6 +32,23 @@ __device__ inline u64 block_scan(u64 v, u64* total) {
   return before + x - v;
 }
 
+// Last i in [lo, n) with pre[i] <= c, by the whole warp (c the same in every
+// lane, pre[lo] <= c): 32 pivots a step, so three dependent loads for 10^4 nodes instead of
+// fourteen.
+template <class T>
+__device__ inline int64_t warp_find(const T* pre, int64_t n, int64_t c, int64_t lo = 0) {
+  const int lane = threadIdx.x & 31;
+  int64_t hi = n;
+  __syncwarp();
+  while (hi - lo > 1) {
+    const int64_t step = (hi - lo + 31) >> 5, at = lo + (lane + 1) * step;
+    const int k = __popc(__ballot_sync(0xffffffffu, at < hi && pre[at] <= c));
+    lo += k * step;
+    hi = min(hi, lo + step);
+  }
+  return lo;
+}
+
 // Decoupled look-back over tiles for NC sums at once (see k_scan_lb for the
 // scheme and why the waits end): tile t's words are st[t * NC ..], each
 // (value << 10 | epoch << 2 | status) with status 1 = the tile's own sum and
