@@ -39,28 +39,11 @@ __device__ inline int64_t block_excl_scan_i64(int64_t v, int64_t* total) {
   return before + x - v;
 }
 
-// Scan inputs: an array, or the chunk count of each node of a list
-// (chunks.cuh: ceil(len / chunk) per row, at least 1 per listed node, 0 past
-// the list's device-side count).
+// Scan input: an array.
 template <class T>
 struct ArrayIn {
   const T* p;
   __device__ int64_t operator()(int64_t i) const { return (int64_t)p[i]; }
-};
-
-struct ChunkCountIn {
-  const int32_t* list;
-  const int32_t* nlist;
-  int64_t n_hint;
-  const int32_t* la;
-  const int32_t* lb;
-  int32_t chunk;
-  __device__ int64_t operator()(int64_t i) const {
-    if (i >= n_hint || i >= *nlist) return 0;
-    const int32_t v = list[i];
-    const int64_t c = (la[v] + chunk - 1) / chunk + (lb ? (lb[v] + chunk - 1) / chunk : 0);
-    return c > 0 ? c : 1;
-  }
 };
 
 // whole input in one tile: scan and total in one launch
@@ -160,6 +143,36 @@ __global__ void __launch_bounds__(SC_THREADS) k_scan_lb(In in, int64_t* out, int
     if (i < n) out[i] = p;
     p += loc[k];
   }
+}
+
+// Scan of the chunk counts of a node list (chunks.cuh: ceil(len / chunk) per
+// row, at least 1 per listed node, 0 past the list's device-side count).  One
+// node per thread: the counts hang on two dependent loads each (5 us for some
+// 10^4 nodes; 10 with eight nodes per thread).
+constexpr int CC_TPB = 512;
+__global__ void __launch_bounds__(CC_TPB) k_scan_chunks(const int32_t* list, const int32_t* nlist, int64_t n_hint,
+                                                        const int32_t* la, const int32_t* lb, int32_t chunk,
+                                                        int64_t* out, LookBack q) {
+  __shared__ int64_t s_tile, s_pre;
+  if (threadIdx.x == 0) s_tile = atomicAdd(q.ctr, 1);
+  __syncthreads();
+  const int64_t tile = s_tile, i = tile * CC_TPB + threadIdx.x;
+  int64_t c = 0;
+  if (i < n_hint && i < *nlist) {
+    const int32_t v = list[i];
+    c = (la[v] + chunk - 1) / chunk + (lb ? (lb[v] + chunk - 1) / chunk : 0);
+    if (c == 0) c = 1;
+  }
+  u64 tot;
+  const u64 ex = block_scan<CC_TPB>((u64)c, &tot);
+  if (threadIdx.x < 32) {
+    const int64_t agg[1] = {(int64_t)tot};
+    int64_t pre[1];
+    look_back<1>(q.st, tile, agg, pre, q.ep, q.err);
+    if (threadIdx.x == 0) s_pre = pre[0];
+  }
+  __syncthreads();
+  if (i <= n_hint) out[i] = s_pre + (int64_t)ex;
 }
 
 // ---------------------------------------------------------------- radix sort
@@ -973,7 +986,10 @@ int64_t scan_exclusive_i32(const int32_t* in, int64_t* out, int64_t n, Prims& P,
 
 void scan_chunk_counts(const int32_t* list, const int32_t* nlist, int64_t n_hint, const int32_t* la,
                        const int32_t* lb, int32_t chunk, int64_t* out, Prims& P, cudaStream_t s) {
-  scan_launch(ChunkCountIn{list, nlist, n_hint, la, lb, chunk}, out, n_hint + 1, nullptr, P, s);
+  const int tiles = div_up(n_hint + 1, CC_TPB);
+  const LookBack q = look_back_begin(P, tiles, s);
+  k_scan_chunks<<<tiles, CC_TPB, 0, s>>>(list, nlist, n_hint, la, lb, chunk, out, q);
+  CKL("k_scan_chunks");
 }
 
 int32_t* scan_error_flag(Prims& P) { return P.lb_ctl.cap ? P.lb_ctl.p + 256 : nullptr; }

@@ -455,32 +455,39 @@ __global__ void __launch_bounds__(TPB, wide_sums<GT> ? 4 : 6) k_sweep_group(Swee
 // Entries of a node's rows staged in registers: entry k of the node is its
 // out-row entry k (k < lo) or its in-row entry k - lo; thread tid holds the
 // entries tid + j * NT.  First the neighbour ids and weights ...
-template <class WT, int NT, int ACC, class SW>
+// Steps in which a warp has no entry are skipped by the whole warp: most rows
+// of a bin are far shorter than its longest.
+template <class WT, int NT, bool DIR, int ACC, class SW>
 __device__ inline void stage_rows(const SweepArgs<WT>& A, const NodeMeta& m, int32_t (&u)[ACC], SW (&w)[ACC]) {
-  if (A.directed) {
+  const int32_t l = DIR ? m.lo + m.li : m.lo, w0 = (int32_t)threadIdx.x & ~31;
 #pragma unroll
-    for (int j = 0; j < ACC; ++j) {
+  for (int j = 0; j < ACC; ++j) {
+    u[j] = -1;
+    if (w0 + j * NT < l) {
       const int32_t k = (int32_t)threadIdx.x + j * NT;
-      const int64_t at = (k < m.lo ? m.oo : m.oi - m.lo) + k;
-      u[j] = k < m.lo + m.li ? A.out.col[at] : -1;
-      w[j] = k < m.lo + m.li ? (SW)A.out.w[at] : 0;
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < ACC; ++j) {
-      const int32_t k = (int32_t)threadIdx.x + j * NT;
-      u[j] = k < m.lo ? A.out.col[m.oo + k] : -1;
-      w[j] = k < m.lo ? (SW)A.out.w[m.oo + k] : 0;
+      const int64_t at = (!DIR || k < m.lo ? m.oo : m.oi - m.lo) + k;
+      if (k < l) {
+        u[j] = A.out.col[at];
+        w[j] = (SW)A.out.w[at];
+      }
     }
   }
 }
 
+template <class WT, int NT, int ACC, class SW>
+__device__ inline void stage_rows(const SweepArgs<WT>& A, const NodeMeta& m, int32_t (&u)[ACC], SW (&w)[ACC]) {
+  if (A.directed) stage_rows<WT, NT, true>(A, m, u, w);
+  else stage_rows<WT, NT, false>(A, m, u, w);
+}
+
 // ... then each id becomes its hash key (neighbour label, or for BestRef the
 // neighbour's refined community when it shares v's label; -1: skipped).
-template <class WT, int MODE, int ACC>
-__device__ inline void stage_keys(const SweepArgs<WT>& A, int32_t v, int32_t a, int32_t (&u)[ACC]) {
+template <class WT, int MODE, int NT, int ACC>
+__device__ inline void stage_keys(const SweepArgs<WT>& A, int32_t v, int32_t a, int32_t l, int32_t (&u)[ACC]) {
+  const int32_t w0 = (int32_t)threadIdx.x & ~31;
 #pragma unroll
   for (int j = 0; j < ACC; ++j) {
+    if (w0 + j * NT >= l) continue;  // the whole warp
     const int32_t x = u[j];
     int32_t key = -1;
     if (x >= 0 && x != v) {
@@ -521,7 +528,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, 
   if (blockIdx.x < nl) {
     cur = node_meta(A, list[blockIdx.x]);
     stage_rows<WT, NT>(A, cur, ek, ew);
-    stage_keys<WT, MODE, ACC>(A, cur.v, cur.a, ek);
+    stage_keys<WT, MODE, NT>(A, cur.v, cur.a, cur.lo + cur.li, ek);
   }
   if (blockIdx.x + gridDim.x < nl) nxt = node_meta(A, list[blockIdx.x + gridDim.x]);
   if (blockIdx.x < nl)
@@ -536,6 +543,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, 
     StageW<GT> own = 0;
 #pragma unroll
     for (int j = 0; j < ACC; ++j) {
+      if ((int)(threadIdx.x & ~31u) + j * NT >= d) continue;  // the whole warp
       if (MODE == 0 && ek[j] == a) own += ew[j];
       else if (ek[j] >= 0) T.add(H - 1, ek[j], ew[j]);
     }
@@ -544,7 +552,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, 
         const int64_t at = (k < cur.lo ? cur.oo : cur.oi - cur.lo) + k;
         const int64_t wx = (int64_t)A.out.w[at];
         int32_t kx[1] = {A.out.col[at]};
-        stage_keys<WT, MODE, 1>(A, v, a, kx);
+        stage_keys<WT, MODE, 0>(A, v, a, INT32_MAX, kx);
         if (MODE == 0 && kx[0] == a) own += (StageW<GT>)wx;
         else if (kx[0] >= 0) T.add(H - 1, kx[0], wx);
       }
@@ -567,7 +575,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, 
     int64_t pairs = 0;
     eval_slots<MODE, GT>(T, H, threadIdx.x, NT, MODE == 0 ? a : v, a, wa, ko, ki, A.directed, A.Tout, A.Tin, A.m, A.gn, A.gd,
                          mult, b, pairs);
-    if (has_next) stage_keys<WT, MODE, ACC>(A, nxt.v, nxt.a, ek);  // label gathers overlap the argmax
+    if (has_next) stage_keys<WT, MODE, NT>(A, nxt.v, nxt.a, nxt.lo + nxt.li, ek);  // label gathers overlap the argmax
     if (__any_sync(0xffffffffu, b.have)) b = seg_best<GT, 32>(b);
     if (lane == 0) wb[wid] = b;
     pairs_all += pairs;
