@@ -30,6 +30,35 @@ void ldl_cuda_check(cudaError_t e, const char* what, const char* file, int line)
 extern std::atomic<int64_t> g_launches;  // kernels launched by this library
 #define CKL(name) (g_launches.fetch_add(1, std::memory_order_relaxed), ldl_cuda_check(cudaGetLastError(), name, __FILE__, __LINE__))
 
+// ---------------------------------------------------------------- launches
+// Every kernel of the library begins with this: it waits until the kernel
+// before it in the stream is done and its writes are visible, and lets the
+// kernel after it be placed meanwhile (that one waits here in turn).
+__device__ __forceinline__ void pdl_enter() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launches a kernel that begins with pdl_enter() so that its blocks may be
+// placed while the kernel before it still runs.  With plain launches the gap
+// between two short kernels was about 2 us: one edge on 10k vertices took 511
+// us a batch (70 launches), now 400; a batch of 10^4 on the R-MAT of 2^20
+// (267 launches) 4.79 ms, now 4.31.
+template <class... P, class... A>
+inline void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  CK(cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...));
+}
+
 // ---------------------------------------------------------------- device memory
 // All device allocations of a context go through dalloc/dfree so that a test
 // can make the k-th one fail.

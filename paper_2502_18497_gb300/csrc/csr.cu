@@ -129,6 +129,7 @@ template <class WT>
 __global__ void __launch_bounds__(PL_TPB) k_plan_records(const int64_t* off, const int32_t* len, const int32_t* col,
                                                          const WT* w, const u64* keys, const int64_t* delta, RecN rn,
                                                          int bshift, PlanOut o, DelTrack t, LookBack q) {
+  pdl_enter();
   __shared__ int64_t s_tile, s_pre[3];
   if (threadIdx.x == 0) s_tile = atomicAdd(q.ctr, 1);
   __syncthreads();
@@ -168,6 +169,7 @@ __global__ void __launch_bounds__(PL_TPB) k_plan_records(const int64_t* off, con
 // the totals to the host.
 __global__ void __launch_bounds__(PL_TPB) k_plan_segments(const int32_t* len, const int32_t* cap, RecN rn, PlanOut o,
                                                           LookBack q, Tail tail) {
+  pdl_enter();
   __shared__ int64_t s_tile, s_pre[3];
   __shared__ int64_t s_sum[3];
   if (threadIdx.x == 0) s_tile = atomicAdd(q.ctr, 1);
@@ -214,6 +216,7 @@ __global__ void __launch_bounds__(PS_TPB) k_plan_small(const int64_t* off, const
                                                        const int32_t* col, const WT* w, const u64* keys,
                                                        const int64_t* delta, RecN rn, int bshift, PlanOut o,
                                                        DelTrack t, Tail tail) {
+  pdl_enter();
   const int64_t n = rn.count(), i = threadIdx.x;
   Rec r{0, 0, 0};
   if (i < n) r = match_record<WT>(off, len, col, w, keys, delta, i, bshift, o, t);
@@ -265,6 +268,7 @@ __global__ void k_undo_rows(int64_t nr, const int64_t* lrow, const int64_t* loff
                             const int32_t* lcap, const int64_t* lsrc, const int32_t* lcol, const WT* lw,
                             int64_t* off, int32_t* len, int32_t* cap, int32_t* col, WT* w, int restore_content,
                             int64_t top0) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -286,6 +290,7 @@ __global__ void k_undo_rows(int64_t nr, const int64_t* lrow, const int64_t* loff
 
 template <class WT>
 __global__ void k_undo_weights(int64_t nw, const int64_t* lpos, const WT* lold, WT* w, int64_t top0) {
+  pdl_enter();
   GRID_STRIDE(i, nw) {
     const int64_t p = lpos[i];
     if (p >= 0 && p < top0) w[p] = lold[i];
@@ -310,6 +315,7 @@ template <class WT>
 __global__ void k_apply(int64_t nrec, int64_t nseg, int64_t stotal, const u64* keys, const int64_t* delta, int bshift,
                         PlanOut o, const int64_t* off, const int32_t* len, const int32_t* cap, const int32_t* col,
                         WT* w, int32_t* scol, WT* sw, UndoOut<WT> u) {
+  pdl_enter();
   GRID_STRIDE(i, nrec) {
     const int32_t p = o.pos[i];
     const int64_t at = p >= 0 ? off[(int64_t)(keys[i] >> bshift)] + p : -1;
@@ -369,6 +375,7 @@ template <class WT>
 __global__ void k_rebuild(int64_t nrec, int64_t nseg, int64_t total, int64_t base, PlanOut o, const int32_t* scol,
                           const WT* sw, const u64* keys, const int64_t* delta, int bshift, int64_t* off, int32_t* len,
                           int32_t* cap, int32_t* col, WT* w) {
+  pdl_enter();
   const u64 cmask = (((u64)1) << bshift) - 1;
   GRID_STRIDE(s, nseg) {
     if (o.woff[s + 1] == o.woff[s]) continue;
@@ -468,6 +475,7 @@ __global__ void k_rebuild(int64_t nrec, int64_t nseg, int64_t total, int64_t bas
 template <class WT>
 __global__ void k_compact_rows(int64_t n, const int64_t* off, const int64_t* lpre, int64_t total,
                                const int64_t* noff, const int32_t* col, const WT* w, int32_t* ncol, WT* nw) {
+  pdl_enter();
   for_seg_runs(lpre, n, total, [&](int64_t t0, int cnt, int64_t slo, int64_t shi) {
     for (int64_t t = t0 + (threadIdx.x & 31); t < t0 + cnt; t += 32) {
       const int64_t v = seg_of(lpre, slo, shi, t), k = t - lpre[v];
@@ -482,6 +490,7 @@ __global__ void k_compact_rows(int64_t n, const int64_t* off, const int64_t* lpr
 // first and last record each add their share, where an atomic per record took
 // 220 us for 16M records (neighbouring threads meet in one counter).
 __global__ void k_row_bounds(const u64* keys, int64_t nrec, int bshift, int32_t* len, int64_t* start) {
+  pdl_enter();
   GRID_STRIDE(i, nrec) {
     const int64_t row = (int64_t)(keys[i] >> bshift);
     if (i == 0 || (int64_t)(keys[i - 1] >> bshift) != row) {
@@ -493,6 +502,7 @@ __global__ void k_row_bounds(const u64* keys, int64_t nrec, int bshift, int32_t*
 }
 
 __global__ void k_caps(const int32_t* cnt, int64_t n, int32_t* cap, int slack_pct) {
+  pdl_enter();
   GRID_STRIDE(v, n) {
     const int64_t d = cnt[v];
     int64_t c = d + (d * slack_pct) / 100 + (d ? 2 : 0);
@@ -504,6 +514,7 @@ __global__ void k_caps(const int32_t* cnt, int64_t n, int32_t* cap, int slack_pc
 template <class WT>
 __global__ void k_scatter_build(const u64* keys, const int64_t* vals, int64_t nrec, int bshift, const int64_t* rs,
                                 const int64_t* off, int32_t* col, WT* w) {
+  pdl_enter();
   const u64 cmask = (((u64)1) << bshift) - 1;
   GRID_STRIDE(i, nrec) {
     const int64_t row = (int64_t)(keys[i] >> bshift);
@@ -514,6 +525,7 @@ __global__ void k_scatter_build(const u64* keys, const int64_t* vals, int64_t nr
 }
 
 __global__ void k_i32_to_i64(const int32_t* a, int64_t* b, int64_t n) {
+  pdl_enter();
   GRID_STRIDE(i, n) b[i] = a[i];
 }
 
@@ -534,10 +546,10 @@ void csr_build(SlackCSR<WT>& g, int64_t n, const u64* keys, const int64_t* vals,
   CK(cudaMemsetAsync(g.len.p, 0, sizeof(int32_t) * (size_t)(n + 1), s));
   S.rs.reserve(n + 1, s);
   if (nrec > 0) {
-    k_row_bounds<<<grid_for(nrec, TPB), TPB, 0, s>>>(keys, nrec, bshift, g.len.p, S.rs.p);
+    launch(k_row_bounds, grid_for(nrec, TPB), TPB, 0, s, keys, nrec, bshift, g.len.p, S.rs.p);
     CKL("k_row_bounds");
   }
-  k_caps<<<grid_for(n, TPB), TPB, 0, s>>>(g.len.p, n, g.cap.p, slack_pct);
+  launch(k_caps, grid_for(n, TPB), TPB, 0, s, g.len.p, n, g.cap.p, slack_pct);
   CKL("k_caps");
   const int64_t total = scan_exclusive_i32(g.cap.p, g.off.p, n, P, s, true);
   const int64_t pool = total + total / 8 + 1024;
@@ -547,7 +559,7 @@ void csr_build(SlackCSR<WT>& g, int64_t n, const u64* keys, const int64_t* vals,
   g.w.exact(pool);
   g.pool_top = total;
   if (nrec > 0) {
-    k_scatter_build<WT><<<grid_for(nrec, TPB), TPB, 0, s>>>(keys, vals, nrec, bshift, S.rs.p, g.off.p, g.col.p, g.w.p);
+    launch(k_scatter_build<WT>, grid_for(nrec, TPB), TPB, 0, s, keys, vals, nrec, bshift, S.rs.p, g.off.p, g.col.p, g.w.p);
     CKL("k_scatter_build");
   }
 }
@@ -558,7 +570,7 @@ static void compact_pool(SlackCSR<WT>& g, int64_t extra, CsrScratch& S, Prims& P
   const int64_t n = g.n;
   S.tmp64.reserve(n + 1, s);
   S.rs.reserve(n + 1, s);
-  k_i32_to_i64<<<grid_for(n, TPB), TPB, 0, s>>>(g.cap.p, S.tmp64.p, n);
+  launch(k_i32_to_i64, grid_for(n, TPB), TPB, 0, s, g.cap.p, S.tmp64.p, n);
   CKL("k_i32_to_i64");
   const int64_t total = scan_exclusive(S.tmp64.p, S.rs.p, n, P, s, true);  // new offsets
   // the same headroom again: rows that outgrow their slack move to the pool's
@@ -568,7 +580,7 @@ static void compact_pool(SlackCSR<WT>& g, int64_t extra, CsrScratch& S, Prims& P
   WT* w2 = (WT*)dalloc(sizeof(WT) * (size_t)pool);
   const int64_t live = scan_exclusive_i32(g.len.p, S.tmp64.p, n, P, s, true);
   if (live > 0) {
-    k_compact_rows<WT><<<grid_for((live + 7) / 8, TPB), TPB, 0, s>>>(n, g.off.p, S.tmp64.p, live, S.rs.p, g.col.p,
+    launch(k_compact_rows<WT>, grid_for((live + 7) / 8, TPB), TPB, 0, s, n, g.off.p, S.tmp64.p, live, S.rs.p, g.col.p,
                                                                      g.w.p, c2, w2);
     CKL("k_compact_rows");
   }
@@ -613,17 +625,17 @@ void csr_plan(const SlackCSR<WT>& g, const CsrRecords& r, CsrScratch& S, Prims& 
   // take 8.9 and 9.9 and the gap between them.  Beyond, one block would match
   // several records per thread one after the other.
   if (n_max <= PS_TPB) {
-    k_plan_small<WT><<<1, PS_TPB, 0, s>>>(g.off.p, g.len.p, g.cap.p, g.col.p, g.w.p, r.keys, r.delta, rn, r.bshift, o,
+    launch(k_plan_small<WT>, 1, PS_TPB, 0, s, g.off.p, g.len.p, g.cap.p, g.col.p, g.w.p, r.keys, r.delta, rn, r.bshift, o,
                                           t, tail);
     CKL("k_plan_small");
   } else {
     const int tiles = div_up(n_max, PL_TPB);
     const LookBack q1 = look_back_begin(P, 3 * (int64_t)tiles, s);
-    k_plan_records<WT><<<tiles, PL_TPB, 0, s>>>(g.off.p, g.len.p, g.col.p, g.w.p, r.keys, r.delta, rn, r.bshift, o, t,
+    launch(k_plan_records<WT>, tiles, PL_TPB, 0, s, g.off.p, g.len.p, g.col.p, g.w.p, r.keys, r.delta, rn, r.bshift, o, t,
                                                 q1);
     CKL("k_plan_records");
     const LookBack q2 = look_back_begin(P, 3 * (int64_t)tiles, s);
-    k_plan_segments<<<tiles, PL_TPB, 0, s>>>(g.len.p, g.cap.p, rn, o, q2, tail);
+    launch(k_plan_segments, tiles, PL_TPB, 0, s, g.len.p, g.cap.p, rn, o, q2, tail);
     CKL("k_plan_segments");
   }
 }
@@ -667,7 +679,7 @@ int64_t csr_finish(SlackCSR<WT>& g, const CsrRecords& r, const int64_t (&tot)[6]
     scol = S.scol.p;
     swp = sw.p;
   }
-  k_apply<WT><<<grid_for(std::max(nrec, (stotal + 7) / 8), TPB), TPB, 0, s>>>(
+  launch(k_apply<WT>, grid_for(std::max(nrec, (stotal + 7) / 8), TPB), TPB, 0, s,
       nrec, nseg, stotal, keys, delta, bshift, o, g.off.p, g.len.p, g.cap.p, g.col.p, g.w.p, scol, swp, u);
   CKL("k_apply");
   if (g.logging) {
@@ -677,7 +689,7 @@ int64_t csr_finish(SlackCSR<WT>& g, const CsrRecords& r, const int64_t (&tot)[6]
     g.ctop += stotal;
   }
   if (wtotal > 0) {
-    k_rebuild<WT><<<grid_for(std::max(nseg, (wtotal + 7) / 8), TPB), TPB, 0, s>>>(
+    launch(k_rebuild<WT>, grid_for(std::max(nseg, (wtotal + 7) / 8), TPB), TPB, 0, s,
         nrec, nseg, wtotal, g.pool_top, o, scol, swp, keys, delta, bshift, g.off.p, g.len.p, g.cap.p, g.col.p, g.w.p);
     CKL("k_rebuild");
     g.pool_top += need;
@@ -724,7 +736,7 @@ cudaError_t csr_txn_rollback(SlackCSR<WT>& g, cudaStream_t s) {
     const int restore = ev.col == g.col0 ? 1 : 0;
     if (ev.nr > 0) {
       const int grid = (int)std::min<int64_t>((ev.nr + 7) / 8, 4096);
-      k_undo_rows<WT><<<grid, TPB, 0, s>>>(ev.nr, g.lrow.p + ev.r0, g.loff.p + ev.r0, g.llen.p + ev.r0,
+      launch(k_undo_rows<WT>, grid, TPB, 0, s, ev.nr, g.lrow.p + ev.r0, g.loff.p + ev.r0, g.llen.p + ev.r0,
                                            g.lcap.p + ev.r0, g.lsrc.p + ev.r0, g.lcol.p, g.lw.p, g.off.p, g.len.p,
                                            g.cap.p, g.col0, g.w0, restore, g.top0);
       g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -732,7 +744,7 @@ cudaError_t csr_txn_rollback(SlackCSR<WT>& g, cudaStream_t s) {
     }
     if (e == cudaSuccess && restore && ev.nw > 0) {
       const int grid = (int)std::min<int64_t>((ev.nw + TPB - 1) / TPB, 4096);
-      k_undo_weights<WT><<<grid, TPB, 0, s>>>(ev.nw, g.lpos.p + ev.w0, g.lold.p + ev.w0, g.w0, g.top0);
+      launch(k_undo_weights<WT>, grid, TPB, 0, s, ev.nw, g.lpos.p + ev.w0, g.lold.p + ev.w0, g.w0, g.top0);
       g_launches.fetch_add(1, std::memory_order_relaxed);
       e = cudaGetLastError();
     }

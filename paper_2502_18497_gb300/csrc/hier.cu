@@ -20,6 +20,7 @@ __device__ inline void set_err(unsigned long long* err, int64_t idx, int code) {
 
 // Start of a batch: every counter, and the scalars that ingest adds to.
 __global__ void k_batch_begin(int32_t* dcnt, int32_t* arena, DevScalars* sc) {
+  pdl_enter();
   const int t = threadIdx.x;
   if (t < K_COUNT) dcnt[t] = 0;
   for (int i = t; i < ARENA_WORDS / 4; i += blockDim.x) ((int4*)arena)[i] = make_int4(0, 0, 0, 0);
@@ -36,6 +37,7 @@ __global__ void k_batch_begin(int32_t* dcnt, int32_t* arena, DevScalars* sc) {
 // gets key 0: the batch is rejected before anything uses it).
 __global__ void k_upd_keys(const ldl_update* u, int64_t cnt, int64_t n, int bits, int directed, u64* keys, u64* vals,
                            unsigned long long* err) {
+  pdl_enter();
   GRID_STRIDE(i, cnt) {
     const ldl_update x = u[i];
     int code = 0;
@@ -61,6 +63,7 @@ __global__ void k_upd_keys(const ldl_update* u, int64_t cnt, int64_t n, int bits
 constexpr int UQ_TPB = 512;
 __global__ void __launch_bounds__(UQ_TPB) k_unique(const u64* keys, int64_t n, u64* ukeys, int64_t* ustart,
                                                    int32_t* nu, LookBack q) {
+  pdl_enter();
   __shared__ int64_t s_tile, s_pre;
   if (threadIdx.x == 0) s_tile = atomicAdd(q.ctr, 1);
   __syncthreads();
@@ -90,6 +93,7 @@ __global__ void __launch_bounds__(UQ_TPB) k_unique(const u64* keys, int64_t n, u
 __global__ void k_seq(const ldl_update* u, int64_t cnt, const u64* vals, const int64_t* ustart, const int32_t* nup,
                       const u64* ukeys, const int64_t* off, const int32_t* len, const int32_t* col, const int32_t* wt,
                       int bits, int directed, unsigned long long* err, int64_t* dm, u64* ok, u64* ov, int32_t* na) {
+  pdl_enter();
   const int64_t nu = *nup, stride = (int64_t)gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31;
   int64_t total = 0;
@@ -155,6 +159,7 @@ __global__ void k_seq(const ldl_update* u, int64_t cnt, const u64* vals, const i
 // (row, col) -> (col + row_off, row): the in-direction records of a level
 // whose in-rows live at row_off (directed graphs keep both in one CSR).
 __global__ void k_transpose(const u64* k, const u64* v, int64_t n, int bits, u64* ok, u64* ov, int64_t row_off) {
+  pdl_enter();
   const u64 mask = (((u64)1) << bits) - 1;
   GRID_STRIDE(i, n) {
     ok[i] = (((k[i] & mask) + (u64)row_off) << bits) | (k[i] >> bits);
@@ -167,6 +172,7 @@ __global__ void k_transpose(const u64* k, const u64* v, int64_t n, int bits, u64
 // K_in as it is (the totals change in k_stat_arcs).
 __global__ void k_dirty(const u64* keys, int64_t na, int bits, const int32_t* lab, int32_t* stT, int32_t epT,
                         int32_t* lT, int32_t* nT, const int64_t* Kout, const int64_t* Kin, I128* acc) {
+  pdl_enter();
   const u64 mask = (((u64)1) << bits) - 1;
   i128 s = 0;
   GRID_STRIDE(i, na) {
@@ -181,6 +187,7 @@ __global__ void k_dirty(const u64* keys, int64_t na, int bits, const int32_t* la
 // sum over listed communities of K_out * K_in into an int128 accumulator
 __global__ void k_psum(const int32_t* list, const int32_t* nlist, const int64_t* Kout, const int64_t* Kin,
                        I128* acc) {
+  pdl_enter();
   const int32_t n = *nlist;
   i128 s = 0;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -194,6 +201,7 @@ __global__ void k_psum(const int32_t* list, const int32_t* nlist, const int64_t*
 __global__ void k_stat_arcs(const u64* keys, const int64_t* delta, int64_t na, int bits, int directed,
                             const int32_t* lab, int64_t* kout, int64_t* kin, int64_t* Kout, int64_t* Kin, int64_t* e,
                             int64_t* de, int32_t* stA, int32_t epA, int32_t* lA, int32_t* nA) {
+  pdl_enter();
   const u64 mask = (((u64)1) << bits) - 1;
   const int lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -265,6 +273,7 @@ __device__ inline void warp_append_rec(bool want, u64 key, int64_t v, u64* pk, u
 
 __global__ void k_chain_records(const u64* keys, const int64_t* vals, int64_t n, const int32_t* n_dev, int bits, int q0, int top, int self,
                                 int add_k, int directed, Chain ch) {
+  pdl_enter();
   if (n_dev) n = min(n, (int64_t)*n_dev);
   const u64 mask = (((u64)1) << bits) - 1;
   const int lane = threadIdx.x & 31;
@@ -301,6 +310,7 @@ __global__ void k_chain_records(const u64* keys, const int64_t* vals, int64_t n,
 // walking each node of A^0 up its parent chain.  A walk stops at a node that
 // is already marked: the walk that marked it goes on above it.
 __global__ void k_chain_frontier(const int32_t* l0, const int32_t* n0, int top, Chain ch) {
+  pdl_enter();
   const int32_t m = *n0, stride = gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31;
   for (int32_t base = blockIdx.x * blockDim.x + threadIdx.x - lane; base < m; base += stride) {
@@ -320,6 +330,7 @@ __global__ void k_chain_frontier(const int32_t* l0, const int32_t* n0, int top, 
 __global__ void k_push(ChunkMap m, const int32_t* lab_up, Adj<int32_t> ch_adj, const int32_t* par, int32_t* lab,
                        int32_t* olist, int32_t* nout, int32_t* stCh, int32_t epCh, int32_t* lCh, int32_t* nCh,
                        int32_t* lab_before, Tail tail) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -351,6 +362,7 @@ __global__ void k_push(ChunkMap m, const int32_t* lab_up, Adj<int32_t> ch_adj, c
 
 // ---------------------------------------------------------------- dissolve
 __global__ void k_stamp_list(const int32_t* l, const int32_t* n, int32_t* st, int32_t ep) {
+  pdl_enter();
   const int32_t m = *n;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) st[l[k]] = ep;
 }
@@ -358,6 +370,7 @@ __global__ void k_stamp_list(const int32_t* l, const int32_t* n, int32_t* st, in
 __global__ void k_dissolve(const int32_t* lD, const int32_t* nD, int32_t* par, int32_t* par_old,
                            const int64_t* kout, const int64_t* kin, int64_t* kout1, int64_t* kin1, int32_t* cnt1,
                            int directed) {
+  pdl_enter();
   const int32_t n = *nD;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t u = lD[k];
@@ -377,6 +390,7 @@ __global__ void k_dissolve(const int32_t* lD, const int32_t* nD, int32_t* par, i
 
 __global__ void k_reset_par(const int32_t* lD, int32_t nD, int32_t* par, int64_t* kout1, int64_t* kin1,
                             int32_t* cnt1, int directed) {
+  pdl_enter();
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < nD; k += gridDim.x * blockDim.x) {
     const int32_t u = lD[k];
     par[u] = -1;
@@ -401,6 +415,7 @@ struct SplitGate {
 __global__ void k_brk_check(const int32_t* lK, const int32_t* nK, const uint8_t* alive, const int32_t* par,
                             int32_t* stX, int32_t epX, int32_t* lX, int32_t* nX, int32_t* ckf, int32_t epF,
                             SplitGate gate) {
+  pdl_enter();
   const int32_t n = gate.open() ? *nK : 0;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t z = lK[k];
@@ -419,6 +434,7 @@ __global__ void k_leave(const int32_t* lU, const int32_t* nU, const uint8_t* ali
                         int64_t* kout1, int64_t* kin1, int32_t* cnt1, int directed, int32_t* stL, int32_t epL,
                         int32_t* stD, int32_t epD, int32_t* lD, int32_t* nD, int32_t* stX, int32_t epX, int32_t* lX,
                         int32_t* nX, int32_t* nbr, SplitGate gate, Tail tail) {
+  pdl_enter();
   const int32_t n = gate.open() ? *nU : 0;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t u = lU[k];
@@ -452,6 +468,7 @@ __global__ void k_leave(const int32_t* lU, const int32_t* nU, const uint8_t* ali
 template <class WT>
 __global__ void k_leave_degree(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* par, const int32_t* par_old,
                                const int32_t* stL, int32_t epL, int32_t* nbr, int32_t* ckf, int32_t epF) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -479,6 +496,7 @@ __global__ void k_leave_degree(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_
 // component.
 __global__ void k_members(Adj<int32_t> ch_adj, ChunkMap m, const int32_t* par, const int32_t* stL, int32_t epL,
                           const int32_t* ckf, int32_t epF, int32_t* comp, int32_t* lG, int32_t* nG, Tail tail) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -551,6 +569,7 @@ constexpr int UF_SAMPLE = 2;
 template <class WT>
 __global__ void k_uf_sample(Adj<WT> out, Adj<WT> in, int directed, const int32_t* lG, const int32_t* nG,
                             const int32_t* par, const int32_t* stL, int32_t epL, int32_t* comp) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -579,6 +598,7 @@ __global__ void k_uf_sample(Adj<WT> out, Adj<WT> in, int directed, const int32_t
 template <class WT>
 __global__ void k_uf(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* par, const uint8_t* alive,
                      const int32_t* stL, int32_t epL, int32_t* comp) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -610,6 +630,7 @@ __global__ void k_uf(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* par, co
 // component (the root, or before it an ancestor), so other threads' finds
 // still end at the root.
 __global__ void k_uf_final(const int32_t* lG, const int32_t* nG, int32_t* comp) {
+  pdl_enter();
   const int32_t n = *nG;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t u = lG[k];
@@ -624,6 +645,7 @@ __global__ void k_rename(const int32_t* lG, const int32_t* nG, const int32_t* co
                          const int32_t* stL, int32_t epL, int32_t* par, int32_t* par_old, const int64_t* kout,
                          const int64_t* kin, int64_t* kout1, int64_t* kin1, int32_t* cnt1, int directed,
                          int32_t* stD, int32_t epD, int32_t* lD, int32_t* nD, Tail tail) {
+  pdl_enter();
   const int32_t n = *nG;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t u = lG[k];
@@ -647,6 +669,7 @@ __global__ void k_rename(const int32_t* lG, const int32_t* nG, const int32_t* co
 // the listed nodes that are singleton refined communities
 __global__ void k_singletons(const int32_t* l, const int32_t* n, const int32_t* par, const int32_t* cnt1, int32_t* out,
                              int32_t* nout) {
+  pdl_enter();
   const int32_t m = *n;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < m; base += stride) {
@@ -666,6 +689,7 @@ __global__ void k_singletons(const int32_t* l, const int32_t* n, const int32_t* 
 __global__ void k_changed(const int32_t* lD, const int32_t* nD, const int32_t* par, const int32_t* par_old,
                           int32_t* stC, int32_t epC, int32_t* lC, int32_t* nC, const int32_t* len_out,
                           const int32_t* len_in, int64_t* acc_out, int64_t* acc_in, Tail tail) {
+  pdl_enter();
   const int32_t n = *nD;
   int64_t so = 0, si = 0;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -689,6 +713,7 @@ template <class WT>
 __global__ void k_emit(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* par, const int32_t* par_old,
                        const int32_t* stC, int32_t epC, int bits, u64* rk, u64* rv, int32_t* cnt, int64_t cap,
                        int32_t* err) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -764,6 +789,7 @@ __global__ void k_emit(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* par, 
 __global__ void k_emit_nodes(const int32_t* lC, const int32_t* nC, const int32_t* par, const int32_t* par_old,
                              const int64_t* kout, const int64_t* kin, int bits, int q0, int top, int directed,
                              Chain ch, u64* ck, u64* cv, int32_t* ncr) {
+  pdl_enter();
   const int32_t n = *nC;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t u = lC[k];
@@ -805,6 +831,7 @@ struct ExistChain {
 
 __global__ void k_exist_chain(const int32_t* lC, const int32_t* nC, const int32_t* par, const int32_t* par_old,
                               int32_t* stE, int32_t epE, int q0, int top, ExistChain ch, int32_t* err) {
+  pdl_enter();
   const int32_t n = *nC;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < 2 * n; k += gridDim.x * blockDim.x) {
     const int32_t u = lC[k >> 1];
@@ -842,6 +869,7 @@ __global__ void k_next_level(const int32_t* lU, const int32_t* nU, const int32_t
                              const int32_t* par, const int32_t* par_old, const int32_t* lab, int32_t* lab_up,
                              const u64* keys, const int32_t* nr, int64_t nr_max, int bits, const uint8_t* alive,
                              int32_t* stA, int32_t epA, int32_t* lA, int32_t* nA, int64_t* agg_recs) {
+  pdl_enter();
   const int64_t mu = *nU, md = *nD;
   const int64_t mr = keys ? min((int64_t)*nr, nr_max) : 0;
   const u64 mask = (((u64)1) << bits) - 1;
@@ -873,6 +901,7 @@ __global__ void k_next_level(const int32_t* lU, const int32_t* nU, const int32_t
 // row's columns are not strictly increasing.
 __global__ void k_csr_records(const int64_t* rp, const int32_t* col, const int32_t* w, int64_t n, int64_t nnz, int bits,
                               u64* rk, u64* rv, unsigned long long* err, int32_t* unsorted) {
+  pdl_enter();
   GRID_STRIDE(v, n) {
     if (rp[v + 1] < rp[v]) set_err(err, 0, LDL_E_INVALID);
   }
@@ -892,6 +921,7 @@ __global__ void k_csr_records(const int64_t* rp, const int32_t* col, const int32
 }
 
 __global__ void k_check_max(const int64_t* s, int64_t n, unsigned long long* err) {
+  pdl_enter();
   GRID_STRIDE(i, n) {
     if (s[i] > INT32_MAX) set_err(err, 0, LDL_E_OVERFLOW);
   }
@@ -899,6 +929,7 @@ __global__ void k_check_max(const int64_t* s, int64_t n, unsigned long long* err
 
 __global__ void k_compare(const u64* a, const int64_t* av, const u64* b, const u64* bv, int64_t n,
                           unsigned long long* err) {
+  pdl_enter();
   GRID_STRIDE(i, n) {
     if (a[i] != b[i] || (u64)av[i] != bv[i]) set_err(err, 0, LDL_E_INVALID);
   }
@@ -911,6 +942,7 @@ __global__ void k_compare(const u64* a, const int64_t* av, const u64* b, const u
 constexpr int RS_RUN = 8;
 __global__ void k_row_sums(const u64* keys, const int64_t* w, int64_t nrec, int bits, int64_t row0, int64_t* out,
                            int64_t* self, int64_t* total) {
+  pdl_enter();
   const u64 mask = (((u64)1) << bits) - 1;
   int64_t tot = 0;
   GRID_STRIDE(r, (nrec + RS_RUN - 1) / RS_RUN) {
@@ -934,14 +966,17 @@ __global__ void k_row_sums(const u64* keys, const int64_t* w, int64_t nrec, int 
 }
 
 __global__ void k_iota(int32_t* a, int64_t n) {
+  pdl_enter();
   GRID_STRIDE(i, n) a[i] = (int32_t)i;
 }
 
 __global__ void k_fill_i32(int32_t* a, int64_t n, int32_t v) {
+  pdl_enter();
   GRID_STRIDE(i, n) a[i] = v;
 }
 
 __global__ void k_alive_list(const uint8_t* alive, int64_t n, int32_t* l, int32_t* cnt) {
+  pdl_enter();
   GRID_STRIDE(i, n) {
     if (!alive || alive[i]) l[atomicAdd(cnt, 1)] = (int32_t)i;
   }
@@ -949,6 +984,7 @@ __global__ void k_alive_list(const uint8_t* alive, int64_t n, int32_t* l, int32_
 
 
 __global__ void k_esum(const int64_t* e, const int64_t* Kout, const int64_t* Kin, int64_t n, int64_t* E, I128* P) {
+  pdl_enter();
   int64_t se = 0;
   i128 sp = 0;
   GRID_STRIDE(i, n) {
@@ -965,6 +1001,7 @@ __global__ void k_esum(const int64_t* e, const int64_t* Kout, const int64_t* Kin
 
 __global__ void k_changed_final(const int32_t* lCh, const int32_t* nCh, const int32_t* lab,
                                 const int32_t* lab_before, int32_t* out, int32_t* nout, Tail tail) {
+  pdl_enter();
   const int32_t n = *nCh;
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     const int32_t u = lCh[k];
@@ -974,6 +1011,7 @@ __global__ void k_changed_final(const int32_t* lCh, const int32_t* nCh, const in
 }
 
 __global__ void k_gather(const int32_t* ids, int32_t k, const int32_t* lab, int32_t* out) {
+  pdl_enter();
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < k; i += gridDim.x * blockDim.x) out[i] = lab[ids[i]];
 }
 
@@ -982,7 +1020,7 @@ __global__ void k_gather(const int32_t* ids, int32_t k, const int32_t* lab, int3
 // ================================================================== host side
 void gather_labels(ldl_ctx& c, const int32_t* ids, int32_t k, int32_t* out) {
   if (k <= 0) return;
-  k_gather<<<grid_for(k, TPB), TPB, 0, c.s>>>(ids, k, c.lv[0].lab.p, out);
+  launch(k_gather, grid_for(k, TPB), TPB, 0, c.s, ids, k, c.lv[0].lab.p, out);
   CKL("k_gather");
 }
 static void throw_err(ldl_ctx& c, unsigned long long* d_err, const char* what) {
@@ -1014,7 +1052,7 @@ int64_t ingest(ldl_ctx& c, const ldl_update* upd, int64_t count, int on_device, 
   *dm = 0;
   c.arena_top = 0;
   for (int k = 0; k < K_COUNT; ++k) c.cp[k] = c.dcnt + k;
-  k_batch_begin<<<1, 1024, 0, c.s>>>(c.dcnt, c.arena, c.d_sc);
+  launch(k_batch_begin, 1, 1024, 0, c.s, c.dcnt, c.arena, c.d_sc);
   CKL("k_batch_begin");
   if (count <= 0) return 0;
   const ldl_update* du = upd;
@@ -1032,15 +1070,15 @@ int64_t ingest(ldl_ctx& c, const ldl_update* upd, int64_t count, int on_device, 
   unsigned long long* err = (unsigned long long*)&c.d_sc->err_key;
   unsigned long long* err_seq = (unsigned long long*)&c.d_sc->err_seq;
   const int g = grid_for(count, TPB);
-  k_upd_keys<<<g, TPB, 0, c.s>>>(du, count, c.n, c.bits, c.directed, c.rk.p, c.rv.p, err);
+  launch(k_upd_keys, g, TPB, 0, c.s, du, count, c.n, c.bits, c.directed, c.rk.p, c.rv.p, err);
   CKL("k_upd_keys");
   sort_pairs(c.rk, c.rv, c.tk, c.tv, count, 2 * c.bits, c.P, c.s);
   const int tiles = div_up(count, UQ_TPB);
   const LookBack q = look_back_begin(c.P, tiles, c.s);
-  k_unique<<<tiles, UQ_TPB, 0, c.s>>>(c.rk.p, count, c.rk2.p, c.rsum.p, c.cp[K_NU], q);
+  launch(k_unique, tiles, UQ_TPB, 0, c.s, c.rk.p, count, c.rk2.p, c.rsum.p, c.cp[K_NU], q);
   CKL("k_unique");
   const auto& g0 = c.lv[0].out0;
-  k_seq<<<g, TPB, 0, c.s>>>(du, count, c.rv.p, c.rsum.p, c.cp[K_NU], c.rk2.p, g0.off.p, g0.len.p, g0.col.p, g0.w.p,
+  launch(k_seq, g, TPB, 0, c.s, du, count, c.rv.p, c.rsum.p, c.cp[K_NU], c.rk2.p, g0.off.p, g0.len.p, g0.col.p, g0.w.p,
                             c.bits, c.directed, err_seq, &c.d_sc->dm, c.trk.p, c.trv.p, c.cp[K_REC]);
   CKL("k_seq");
   // the changed arcs in order (each once, no change zero), on directed graphs
@@ -1065,7 +1103,7 @@ static void combine_in_out(ldl_ctx& c, const u64* keys, const u64* vals, int64_t
   c.rv2.reserve(2 * nr + 1, c.s);
   c.trk.reserve(nr + 1, c.s);
   c.trv.reserve(nr + 1, c.s);
-  k_transpose<<<grid_for(nr, TPB), TPB, 0, c.s>>>(keys, vals, nr, c.bits, c.trk.p, c.trv.p, c.n);
+  launch(k_transpose, grid_for(nr, TPB), TPB, 0, c.s, keys, vals, nr, c.bits, c.trk.p, c.trv.p, c.n);
   CKL("k_transpose");
   // the out-records are ordered by row, so a stable sort on the new row alone
   // gives (in-row, col) order
@@ -1138,7 +1176,7 @@ static void chain_records(ldl_ctx& c, const u64* keys, const int64_t* vals, int6
     L.pv.reserve(L.pend_ub + n + 1, c.s, true);
     L.pend_ub += n;
   }
-  k_chain_records<<<grid_for(n, TPB), TPB, 0, c.s>>>(keys, vals, n, n_dev, c.bits, q0, c.T, self ? 1 : 0, add_k ? 1 : 0,
+  launch(k_chain_records, grid_for(n, TPB), TPB, 0, c.s, keys, vals, n, n_dev, c.bits, q0, c.T, self ? 1 : 0, add_k ? 1 : 0,
                                                      c.directed, chain_of(c, nullptr));
   CKL("k_chain_records");
 }
@@ -1210,18 +1248,18 @@ void repair_batch(ldl_ctx& c, int64_t na, const int32_t* epA, int32_t epT) {
   LevelState& L0 = c.lv[0];
   zero_cnt(c, K_T);
   c.racc = (RepairAcc*)fresh(c, sizeof(RepairAcc) / 4, c.d_sc->home2);
-  k_dirty<<<grid_for(na, TPB), TPB, 0, c.s>>>(c.rk.p, na, c.bits, L0.lab.p, c.stT.p, epT, c.lT.p, c.cp[K_T], c.Kout.p,
+  launch(k_dirty, grid_for(na, TPB), TPB, 0, c.s, c.rk.p, na, c.bits, L0.lab.p, c.stT.p, epT, c.lT.p, c.cp[K_T], c.Kout.p,
                                               Kin_of(c), &c.racc->p_old);
   CKL("k_dirty");
-  k_stat_arcs<<<grid_for(na, TPB), TPB, 0, c.s>>>(c.rk.p, (const int64_t*)c.rv.p, na, c.bits, c.directed, L0.lab.p,
+  launch(k_stat_arcs, grid_for(na, TPB), TPB, 0, c.s, c.rk.p, (const int64_t*)c.rv.p, na, c.bits, c.directed, L0.lab.p,
                                                   L0.kout.p, kin_of(c, 0), c.Kout.p, Kin_of(c), c.e.p, &c.racc->de,
                                                   L0.stA.p, epA[0], L0.lA.p, c.cp[K_A0]);
   CKL("k_stat_arcs");
-  k_psum<<<grid_for(2 * na, TPB), TPB, 0, c.s>>>(c.lT.p, c.cp[K_T], c.Kout.p, Kin_of(c), &c.racc->p_new);
+  launch(k_psum, grid_for(2 * na, TPB), TPB, 0, c.s, c.lT.p, c.cp[K_T], c.Kout.p, Kin_of(c), &c.racc->p_new);
   CKL("k_psum");
   if (c.T == 0) return;
   // InitFrontier: A^{q+1} = pi_q(A^q) along the chain
-  k_chain_frontier<<<grid_for(2 * na, TPB), TPB, 0, c.s>>>(L0.lA.p, c.cp[K_A0], c.T, chain_of(c, epA));
+  launch(k_chain_frontier, grid_for(2 * na, TPB), TPB, 0, c.s, L0.lA.p, c.cp[K_A0], c.T, chain_of(c, epA));
   CKL("k_chain_frontier");
   // the aggregate chain: W_q(anc(i), anc(j)) += delta and the strengths of
   // every level above 0; the weights are applied when each level is next read
@@ -1245,7 +1283,7 @@ void pushdown(ldl_ctx& c, int r, int32_t epCh, int64_t moved_ub) {
     ChunkMap m = chunk_map(c, src, c.cp[idx], n, L.children.len.p, nullptr);
     int32_t nn = 0;
     const HostRead rr{c.cp[idxs[flip]], &nn, sizeof(int32_t)};
-    k_push<<<chunk_grid(n), TPB, 0, c.s>>>(
+    launch(k_push, chunk_grid(n), TPB, 0, c.s,
         m, c.lv[q + 1].lab.p, ch, L.par.p, L.lab.p, dst, c.cp[idxs[flip]], q == 0 ? c.stCh.p : nullptr, epCh,
         c.lCh.p, c.cp[K_CH], c.lab_before.p, q > 0 ? tail_begin(c, &rr, 1) : Tail{});
     CKL("k_push");
@@ -1265,13 +1303,13 @@ int32_t dissolve_all(ldl_ctx& c, int r, int32_t epD) {
   LevelState& L = c.lv[r];
   LevelState& N = c.lv[r + 1];
   zero_cnt(c, K_D);
-  k_alive_list<<<grid_for(c.n, TPB), TPB, 0, c.s>>>(r ? L.alive.p : nullptr, c.n, c.lD.p, c.cp[K_D]);
+  launch(k_alive_list, grid_for(c.n, TPB), TPB, 0, c.s, r ? L.alive.p : nullptr, c.n, c.lD.p, c.cp[K_D]);
   CKL("k_alive_list");
-  k_stamp_list<<<grid_for(c.n, TPB), TPB, 0, c.s>>>(c.lD.p, c.cp[K_D], c.stD.p, epD);
+  launch(k_stamp_list, grid_for(c.n, TPB), TPB, 0, c.s, c.lD.p, c.cp[K_D], c.stD.p, epD);
   CKL("k_stamp_list");
   const int32_t nd = rd_cnt(c, K_D);
   if (nd > 0) {
-    k_dissolve<<<grid_for(nd, TPB), TPB, 0, c.s>>>(c.lD.p, c.cp[K_D], L.par.p, c.par_old.p, L.kout.p,
+    launch(k_dissolve, grid_for(nd, TPB), TPB, 0, c.s, c.lD.p, c.cp[K_D], L.par.p, c.par_old.p, L.kout.p,
                                                    kin_of(c, r), N.kout.p, kin_of(c, r + 1), N.cnt.p, c.directed);
     CKL("k_dissolve");
   }
@@ -1281,7 +1319,7 @@ int32_t dissolve_all(ldl_ctx& c, int r, int32_t epD) {
 void singletons_of(ldl_ctx& c, int r, const int32_t* list, int idx_n, int64_t n_hint, int32_t* out, int idx_out) {
   zero_cnt(c, idx_out);
   if (n_hint > 0) {
-    k_singletons<<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(list, c.cp[idx_n], c.lv[r].par.p, c.lv[r + 1].cnt.p, out,
+    launch(k_singletons, grid_for(n_hint, TPB), TPB, 0, c.s, list, c.cp[idx_n], c.lv[r].par.p, c.lv[r + 1].cnt.p, out,
                                                          c.cp[idx_out]);
     CKL("k_singletons");
   }
@@ -1289,7 +1327,7 @@ void singletons_of(ldl_ctx& c, int r, const int32_t* list, int idx_n, int64_t n_
 
 void reset_par(ldl_ctx& c, int r, int32_t nD) {
   if (nD <= 0) return;
-  k_reset_par<<<grid_for(nD, TPB), TPB, 0, c.s>>>(c.lD.p, nD, c.lv[r].par.p, c.lv[r + 1].kout.p,
+  launch(k_reset_par, grid_for(nD, TPB), TPB, 0, c.s, c.lD.p, nD, c.lv[r].par.p, c.lv[r + 1].kout.p,
                                                   kin_of(c, r + 1), c.lv[r + 1].cnt.p, c.directed);
   CKL("k_reset_par");
 }
@@ -1297,7 +1335,7 @@ void reset_par(ldl_ctx& c, int r, int32_t nD) {
 template <class WT>
 static void leave_degree(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t nD, int32_t epL, int32_t epF) {
   ChunkMap m = chunk_map(c, c.lD.p, c.cp[K_D], nD, out.len, c.directed ? in.len : nullptr);
-  k_leave_degree<WT><<<chunk_grid(nD), TPB, 0, c.s>>>(out, in, m, c.lv[r].par.p, c.par_old.p,
+  launch(k_leave_degree<WT>, chunk_grid(nD), TPB, 0, c.s, out, in, m, c.lv[r].par.p, c.par_old.p,
                                                                            c.stL.p, epL, c.nbr.p, c.ckf.p, epF);
   CKL("k_leave_degree");
 }
@@ -1305,11 +1343,11 @@ static void leave_degree(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t nD,
 template <class WT>
 static void union_find(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t nG, int32_t epL) {
   LevelState& L = c.lv[r];
-  k_uf_sample<WT><<<grid_for((int64_t)nG * 32, TPB, 16), TPB, 0, c.s>>>(out, in, c.directed, c.lG.p, c.cp[K_G],
+  launch(k_uf_sample<WT>, grid_for((int64_t)nG * 32, TPB, 16), TPB, 0, c.s, out, in, c.directed, c.lG.p, c.cp[K_G],
                                                                        L.par.p, c.stL.p, epL, c.comp.p);
   CKL("k_uf_sample");
   ChunkMap m = chunk_map(c, c.lG.p, c.cp[K_G], nG, out.len, c.directed ? in.len : nullptr);
-  k_uf<WT><<<chunk_grid(nG), TPB, 0, c.s>>>(out, in, m, L.par.p, L.alive.p, c.stL.p, epL,
+  launch(k_uf<WT>, chunk_grid(nG), TPB, 0, c.s, out, in, m, L.par.p, L.alive.p, c.stL.p, epL,
                                                                   c.comp.p);
   CKL("k_uf");
 }
@@ -1339,12 +1377,12 @@ void split_launch(ldl_ctx& c, int r, SplitRun& sr, bool gated, bool hubs, HostRe
   const SplitGate gate{gated ? c.cp[K_B] : nullptr, hubs ? c.cp[K_LARGE] : nullptr, c.cp[K_UNDEC]};
   // The level's deleted-arc endpoints and U* stay on the device: both kernels
   // stride over their lists' counts with grids sized by the host's bounds.
-  k_brk_check<<<grid_for(L.ubK, TPB, 4), TPB, 0, c.s>>>(L.lK.p, c.cp[K_BRK0 + r], L.alive.p, L.par.p, c.stX.p, epX,
+  launch(k_brk_check, grid_for(L.ubK, TPB, 4), TPB, 0, c.s, L.lK.p, c.cp[K_BRK0 + r], L.alive.p, L.par.p, c.stX.p, epX,
                                                         c.lX.p, c.cp[K_X], c.ckf.p, sr.epF, gate);
   CKL("k_brk_check");
   rr[n] = {c.cp[K_D], &sr.nleft, sizeof(int32_t)};
   rr[n + 1] = {c.cp[K_X], &sr.nx, sizeof(int32_t)};
-  k_leave<<<grid_for(c.ubU, TPB, 4), TPB, 0, c.s>>>(c.lUstar.p, c.cp[K_USTAR], L.alive.p, L.lab.p, N.lab.p, L.par.p,
+  launch(k_leave, grid_for(c.ubU, TPB, 4), TPB, 0, c.s, c.lUstar.p, c.cp[K_USTAR], L.alive.p, L.lab.p, N.lab.p, L.par.p,
                                                     c.par_old.p, L.kout.p, kin_of(c, r), N.kout.p, kin_of(c, r + 1),
                                                     N.cnt.p, c.directed, c.stL.p, sr.epL, c.stD.p, sr.epD, c.lD.p,
                                                     c.cp[K_D], c.stX.p, epX, c.lX.p, c.cp[K_X], c.nbr.p, gate,
@@ -1372,7 +1410,7 @@ int32_t split(ldl_ctx& c, int r, SplitRun& sr) {
     const HostRead rg{c.cp[K_G], &nG, sizeof(int32_t)};
     Adj<int32_t> ch{L.children.off.p, L.children.len.p, L.children.col.p, L.children.w.p};
     ChunkMap m = chunk_map(c, c.lX.p, c.cp[K_X], nx, L.children.len.p, nullptr);
-    k_members<<<chunk_grid(nx), TPB, 0, c.s>>>(ch, m, L.par.p, c.stL.p, epL, c.ckf.p, epF,
+    launch(k_members, chunk_grid(nx), TPB, 0, c.s, ch, m, L.par.p, c.stL.p, epL, c.ckf.p, epF,
                                                                    c.comp.p, c.lG.p, c.cp[K_G], tail_begin(c, &rg, 1));
     CKL("k_members");
     tail_wait(c, &rg, 1);
@@ -1380,10 +1418,10 @@ int32_t split(ldl_ctx& c, int r, SplitRun& sr) {
     if (nG > 0) {
       if (r == 0) union_find<int32_t>(c, r, adj_out0(c), adj_in0(c), nG, epL);
       else union_find<int64_t>(c, r, adj_out(c, r), adj_in(c, r), nG, epL);
-      k_uf_final<<<grid_for(nG, TPB), TPB, 0, c.s>>>(c.lG.p, c.cp[K_G], c.comp.p);
+      launch(k_uf_final, grid_for(nG, TPB), TPB, 0, c.s, c.lG.p, c.cp[K_G], c.comp.p);
       CKL("k_uf_final");
       const HostRead rn{c.cp[K_D], &nD, sizeof(int32_t)};
-      k_rename<<<grid_for(nG, TPB), TPB, 0, c.s>>>(c.lG.p, c.cp[K_G], c.comp.p, L.alive.p, c.stL.p, epL, L.par.p,
+      launch(k_rename, grid_for(nG, TPB), TPB, 0, c.s, c.lG.p, c.cp[K_G], c.comp.p, L.alive.p, c.stL.p, epL, L.par.p,
                                                    c.par_old.p, L.kout.p, kin_of(c, r), N.kout.p, kin_of(c, r + 1),
                                                    N.cnt.p, c.directed, c.stD.p, epD, c.lD.p, c.cp[K_D], tail_begin(c, &rn, 1));
       CKL("k_rename");
@@ -1411,7 +1449,7 @@ static int64_t emit_records(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t 
   c.rv2.reserve(cap, c.s);
   // (in the static build the in-rows would be walked for nothing)
   ChunkMap m = chunk_map(c, c.lC.p, c.cp[K_C], nC, out.len, build ? nullptr : in.len);
-  k_emit<WT><<<chunk_grid(nC), TPB, 0, c.s>>>(out, in, m, c.lv[r].par.p, c.par_old.p,
+  launch(k_emit<WT>, chunk_grid(nC), TPB, 0, c.s, out, in, m, c.lv[r].par.p, c.par_old.p,
                                                                           c.stC.p, epC, c.bits, c.rk2.p, c.rv2.p,
                                                                           c.cp[K_REC], cap, c.cp[K_ERR]);
   CKL("k_emit");
@@ -1438,7 +1476,7 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
     const int32_t* lo = r == 0 ? adj_out0(c).len : adj_out(c, r).len;
     const int32_t* li = r == 0 ? adj_in0(c).len : adj_in(c, r).len;
     const HostRead rr[2] = {{c.cp[K_C], &nC, sizeof(int32_t)}, {c.sums, deg, 2 * sizeof(int64_t)}};
-    k_changed<<<grid_for(nD, TPB), TPB, 0, c.s>>>(c.lD.p, c.cp[K_D], L.par.p, c.par_old.p, c.stC.p, epC, c.lC.p,
+    launch(k_changed, grid_for(nD, TPB), TPB, 0, c.s, c.lD.p, c.cp[K_D], L.par.p, c.par_old.p, c.stC.p, epC, c.lC.p,
                                                   c.cp[K_C], lo, li, c.sums, c.sums + 1, tail_begin(c, rr, 2));
     CKL("k_changed");
     tail_wait(c, rr, 2);
@@ -1449,7 +1487,7 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
                           : emit_records<int64_t>(c, r, adj_out(c, r), adj_in(c, r), nC, epC, build, deg);
     c.crk.reserve(2 * (int64_t)nC + 2, c.s);
     c.crv.reserve(2 * (int64_t)nC + 2, c.s);
-    k_emit_nodes<<<grid_for(nC, TPB), TPB, 0, c.s>>>(c.lC.p, c.cp[K_C], L.par.p, c.par_old.p, L.kout.p,
+    launch(k_emit_nodes, grid_for(nC, TPB), TPB, 0, c.s, c.lC.p, c.cp[K_C], L.par.p, c.par_old.p, L.kout.p,
                                                      kin_of(c, r), c.bits, r + 1, build ? r + 1 : c.T, c.directed,
                                                      chain_of(c, nullptr), c.crk.p, c.crv.p, c.cp[K_CREC]);
     CKL("k_emit_nodes");
@@ -1514,7 +1552,7 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
       ech.alive[q] = c.lv[q].alive.p;
       ech.par[q] = c.lv[q].par.p;
     }
-    k_exist_chain<<<grid_for(2 * (int64_t)nC, TPB), TPB, 0, c.s>>>(c.lC.p, c.cp[K_C], L.par.p, c.par_old.p,
+    launch(k_exist_chain, grid_for(2 * (int64_t)nC, TPB), TPB, 0, c.s, c.lC.p, c.cp[K_C], L.par.p, c.par_old.p,
                                                                     c.stE.p, c.next_epoch(), r + 1, c.T, ech,
                                                                     c.cp[K_ERR]);
     CKL("k_exist_chain");
@@ -1526,7 +1564,7 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
   if (!build) N.ubA = std::min<int64_t>(c.n, N.ubA + c.ubU + 2 * (int64_t)nD + 2 * nr);
   // |U*| stays on the device
   const bool recs = nC > 0 && epA_next;
-  k_next_level<<<grid_for(build ? c.n : c.ubU + nD + nr, TPB, 2), TPB, 0, c.s>>>(c.lUstar.p, c.cp[K_USTAR], c.lD.p, c.cp[K_D], L.par.p,
+  launch(k_next_level, grid_for(build ? c.n : c.ubU + nD + nr, TPB, 2), TPB, 0, c.s, c.lUstar.p, c.cp[K_USTAR], c.lD.p, c.cp[K_D], L.par.p,
                                                   c.par_old.p, L.lab.p, N.lab.p, recs ? c.rk.p : nullptr,
                                                   c.cp[K_NR], nr, c.bits, N.alive.p, epA_next ? N.stA.p : nullptr,
                                                   epA_next, N.lA.p, c.cp[K_A0 + r + 1], &c.d_sc->agg_recs);
@@ -1561,14 +1599,14 @@ void level_free(ldl_ctx& c, int r) { c.lv[r].release(); }
 
 int32_t alive_list(ldl_ctx& c, int r, int32_t* list, int idx) {
   zero_cnt(c, idx);
-  k_alive_list<<<grid_for(c.n, TPB), TPB, 0, c.s>>>(r ? c.lv[r].alive.p : nullptr, c.n, list, c.cp[idx]);
+  launch(k_alive_list, grid_for(c.n, TPB), TPB, 0, c.s, r ? c.lv[r].alive.p : nullptr, c.n, list, c.cp[idx]);
   CKL("k_alive_list");
   return rd_cnt(c, idx);
 }
 
 void changed_labels(ldl_ctx& c, const HostRead* rr, int n) {
   // strides over the candidates' device count with a grid bounded by the node count
-  k_changed_final<<<grid_for(c.n, TPB, 2), TPB, 0, c.s>>>(c.lCh.p, c.cp[K_CH], c.lv[0].lab.p, c.lab_before.p, c.lChg.p,
+  launch(k_changed_final, grid_for(c.n, TPB, 2), TPB, 0, c.s, c.lCh.p, c.cp[K_CH], c.lv[0].lab.p, c.lab_before.p, c.lChg.p,
                                                           c.cp[K_CHG], tail_begin(c, rr, n));
   CKL("k_changed_final");
   tail_wait(c, rr, n);
@@ -1590,7 +1628,7 @@ void upload_graph(ldl_ctx& c, int64_t nnz, const int64_t* row_ptr, const int32_t
   c.rv.reserve(nnz + 1, c.s);
   reset_err(c);
   zero_cnt(c, K_TMP);
-  k_csr_records<<<grid_for(std::max(n, nnz / 8), TPB), TPB, 0, c.s>>>(drp.p, dcol.p, dw.p, n, nnz, c.bits, c.rk.p,
+  launch(k_csr_records, grid_for(std::max(n, nnz / 8), TPB), TPB, 0, c.s, drp.p, dcol.p, dw.p, n, nnz, c.bits, c.rk.p,
                                                                       c.rv.p, err_ptr(c), c.cp[K_TMP]);
   CKL("k_csr_records");
   CK(cudaStreamSynchronize(c.s));
@@ -1606,7 +1644,7 @@ void upload_graph(ldl_ctx& c, int64_t nnz, const int64_t* row_ptr, const int32_t
     c.rsum.reserve(nnz + 1, c.s);
     na = reduce_by_key(c.rk.p, c.rv.p, nnz, c.rk2.p, c.rsum.p, c.P, c.s);
     reset_err(c);
-    k_check_max<<<grid_for(na, TPB), TPB, 0, c.s>>>(c.rsum.p, na, err_ptr(c));
+    launch(k_check_max, grid_for(na, TPB), TPB, 0, c.s, c.rsum.p, na, err_ptr(c));
     CKL("k_check_max");
     throw_err(c, err_ptr(c), "summed weight above INT32_MAX");
     // (rk2, rsum) = unique arcs
@@ -1617,11 +1655,11 @@ void upload_graph(ldl_ctx& c, int64_t nnz, const int64_t* row_ptr, const int32_t
     c.rk2.reserve(na + 1, c.s);
     c.rv2.reserve(na + 1, c.s);
     if (!c.directed) {
-      k_transpose<<<grid_for(na, TPB), TPB, 0, c.s>>>(c.rk.p, c.rv.p, na, c.bits, c.rk2.p, c.rv2.p, 0);
+      launch(k_transpose, grid_for(na, TPB), TPB, 0, c.s, c.rk.p, c.rv.p, na, c.bits, c.rk2.p, c.rv2.p, 0);
       CKL("k_transpose");
       sort_pairs(c.rk2, c.rv2, c.tk, c.tv, na, 2 * c.bits, c.P, c.s, c.bits);  // rows already ordered
       reset_err(c);
-      k_compare<<<grid_for(na, TPB), TPB, 0, c.s>>>(c.rk.p, (const int64_t*)c.rv.p, c.rk2.p, c.rv2.p, na,
+      launch(k_compare, grid_for(na, TPB), TPB, 0, c.s, c.rk.p, (const int64_t*)c.rv.p, c.rk2.p, c.rv2.p, na,
                                                     err_ptr(c));
       CKL("k_compare");
       throw_err(c, err_ptr(c), "undirected CSR is not symmetric");
@@ -1639,24 +1677,24 @@ void upload_graph(ldl_ctx& c, int64_t nnz, const int64_t* row_ptr, const int32_t
   CK(cudaMemsetAsync(L0.kout.p, 0, sizeof(int64_t) * (size_t)n, c.s));
   CK(cudaMemsetAsync(c.e.p, 0, sizeof(int64_t) * (size_t)n, c.s));
   const int gr = grid_for((na + RS_RUN - 1) / RS_RUN, TPB);
-  k_row_sums<<<gr, TPB, 0, c.s>>>(c.rk.p, (const int64_t*)c.rv.p, na, c.bits, 0, L0.kout.p, c.e.p, &c.d_sc->dm);
+  launch(k_row_sums, gr, TPB, 0, c.s, c.rk.p, (const int64_t*)c.rv.p, na, c.bits, 0, L0.kout.p, c.e.p, &c.d_sc->dm);
   CKL("k_row_sums");
   if (c.directed) {
     CK(cudaMemsetAsync(L0.kin.p, 0, sizeof(int64_t) * (size_t)n, c.s));
-    k_row_sums<<<gr, TPB, 0, c.s>>>(c.rk2.p + na, (const int64_t*)c.rv2.p + na, na, c.bits, n, L0.kin.p, nullptr,
+    launch(k_row_sums, gr, TPB, 0, c.s, c.rk2.p + na, (const int64_t*)c.rv2.p + na, na, c.bits, n, L0.kin.p, nullptr,
                                     nullptr);
     CKL("k_row_sums(in)");
   }
-  k_iota<<<grid_for(n, TPB), TPB, 0, c.s>>>(L0.lab.p, n);
+  launch(k_iota, grid_for(n, TPB), TPB, 0, c.s, L0.lab.p, n);
   CKL("k_iota");
-  k_fill_i32<<<grid_for(n, TPB), TPB, 0, c.s>>>(L0.cnt.p, n, 1);
+  launch(k_fill_i32, grid_for(n, TPB), TPB, 0, c.s, L0.cnt.p, n, 1);
   CKL("k_fill_i32");
   CK(cudaMemsetAsync(L0.alive.p, 1, (size_t)n, c.s));
   CK(cudaMemcpyAsync(c.Kout.p, L0.kout.p, sizeof(int64_t) * (size_t)n, cudaMemcpyDeviceToDevice, c.s));
   if (c.directed) CK(cudaMemcpyAsync(c.Kin.p, L0.kin.p, sizeof(int64_t) * (size_t)n, cudaMemcpyDeviceToDevice, c.s));
   c.racc = (RepairAcc*)c.d_sc->home2;
   CK(cudaMemsetAsync(c.racc, 0, sizeof(RepairAcc), c.s));
-  k_esum<<<grid_for(n, TPB), TPB, 0, c.s>>>(c.e.p, c.Kout.p, Kin_of(c), n, &c.racc->de, &c.racc->p_new);
+  launch(k_esum, grid_for(n, TPB), TPB, 0, c.s, c.e.p, c.Kout.p, Kin_of(c), n, &c.racc->de, &c.racc->p_new);
   CKL("k_esum");
   DevScalars h;
   CK(cudaMemcpyAsync(&h, c.d_sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, c.s));

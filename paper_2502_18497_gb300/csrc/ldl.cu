@@ -84,9 +84,9 @@ namespace {
 constexpr int PAGE_WORDS = 500;  // payload words per read
 
 // hands values of earlier kernels to the host (one block)
-__global__ void k_publish(Tail t) { put_tail(t); }
+__global__ void k_publish(Tail t) { pdl_enter(); put_tail(t); }
 
-__global__ void k_set_i32(int32_t* p, int32_t v) { *p = v; }
+__global__ void k_set_i32(int32_t* p, int32_t v) { pdl_enter(); *p = v; }
 
 // Copies byte ranges into one buffer (16 bytes per access; every range and its
 // place start 256-byte aligned).  One launch for all arrays of a snapshot,
@@ -102,6 +102,7 @@ struct SnapList {
 };
 
 __global__ void __launch_bounds__(256) k_snapshot(SnapList l, unsigned char* dst) {
+  pdl_enter();
   constexpr int U = 4;  // units in flight per thread
   const int64_t total = l.unit[l.n], span = (int64_t)gridDim.x * 256 * U;
   int i = 0;
@@ -149,7 +150,7 @@ static void wait_words(ldl_ctx& c, int n) {
 
 void host_read(ldl_ctx& c, const HostRead* r, int n) {
   const Tail t = tail_begin(c, r, n);
-  k_publish<<<1, 64, 0, c.s>>>(t);
+  launch(k_publish, 1, 64, 0, c.s, t);
   CKL("k_publish");
   tail_wait(c, r, n);
 }
@@ -217,7 +218,7 @@ void tail_wait(ldl_ctx& c, const HostRead* r, int n) {
 }
 
 void set_cnt(ldl_ctx& c, int idx, int32_t v) {
-  k_set_i32<<<1, 1, 0, c.s>>>(c.cp[idx], v);
+  launch(k_set_i32, 1, 1, 0, c.s, c.cp[idx], v);
   CKL("k_set_i32");
 }
 
@@ -544,7 +545,7 @@ static void txn_begin(ldl_ctx& c) {
     l.unit[l.n + 1] = l.unit[l.n] + (int64_t)(sg.bytes / 16);
     ++l.n;
   }
-  k_snapshot<<<grid_for((l.unit[l.n] + 3) / 4, 256, 8), 256, 0, c.s>>>(l, c.snap.p);
+  launch(k_snapshot, grid_for((l.unit[l.n] + 3) / 4, 256, 8), 256, 0, c.s, l, c.snap.p);
   CKL("k_snapshot");
   for_each_csr(c, [&](auto& g) { csr_txn_begin(g); });
   c.snap_m = c.m;

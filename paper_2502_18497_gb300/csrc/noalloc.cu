@@ -32,6 +32,7 @@ int32_t* g_ptr[kMaxDevices] = {nullptr};
 cudaError_t g_ptr_err[kMaxDevices] = {cudaSuccess};
 
 __global__ void k_gather_noalloc(const int32_t* ids, int32_t k, const int32_t* lab, int32_t* out) {
+  pdl_enter();
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < k; i += gridDim.x * blockDim.x) out[i] = lab[ids[i]];
 }
 
@@ -81,7 +82,7 @@ extern "C" ldl_status ldl_copy_changed_noalloc(const ldl_ctx* cc, int32_t* ids, 
   int32_t* scratch = g_ptr[dev];
   const int32_t kk = (int32_t)k;
   const int grid = (int)std::min<int64_t>(((int64_t)kk + 255) / 256, 4096);
-  k_gather_noalloc<<<grid, 256, 0, c.s>>>(c.lChg.p, kk, c.lv[0].lab.p, scratch);
+  launch(k_gather_noalloc, grid, 256, 0, c.s, c.lChg.p, kk, c.lv[0].lab.p, scratch);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(ids, c.lChg.p, sizeof(int32_t) * (size_t)kk, cudaMemcpyDeviceToHost, c.s);

@@ -49,6 +49,7 @@ struct ArrayIn {
 // whole input in one tile: scan and total in one launch
 template <class In>
 __global__ void k_scan_one(In in, int64_t* out, int64_t n, int64_t* total) {
+  pdl_enter();
   const int64_t base = (int64_t)threadIdx.x * SC_ITEMS;
   int64_t loc[SC_ITEMS];
   int64_t s = 0;
@@ -81,6 +82,7 @@ constexpr int LB_TILE = SC_THREADS * LB_ITEMS;
 template <class In>
 __global__ void __launch_bounds__(SC_THREADS) k_scan_lb(In in, int64_t* out, int64_t n, u64* st, int32_t* ctr,
                                                         uint32_t ep, int64_t* total, int32_t* err) {
+  pdl_enter();
   __shared__ int64_t s_tile, s_pre;
   if (threadIdx.x == 0) s_tile = atomicAdd(ctr, 1);
   __syncthreads();
@@ -153,6 +155,7 @@ constexpr int CC_TPB = 512;
 __global__ void __launch_bounds__(CC_TPB) k_scan_chunks(const int32_t* list, const int32_t* nlist, int64_t n_hint,
                                                         const int32_t* la, const int32_t* lb, int32_t chunk,
                                                         int64_t* out, LookBack q) {
+  pdl_enter();
   __shared__ int64_t s_tile, s_pre;
   if (threadIdx.x == 0) s_tile = atomicAdd(q.ctr, 1);
   __syncthreads();
@@ -221,6 +224,7 @@ __device__ inline void rs_hist_tile(const u64* keys, int64_t n, int shift, int64
 
 __global__ void k_rs_hist(const u64* keys, int64_t n, int shift, int64_t nb, int64_t* ghist, RsExt x, int first,
                           int in_off) {
+  pdl_enter();
   if (x.n_dev) n = min(n, (int64_t)*x.n_dev);
   if (x.zero && first)
     for (int64_t i = (int64_t)blockIdx.x * RS_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * RS_THREADS)
@@ -254,6 +258,7 @@ __device__ inline void rs_dscan_digit(int64_t* ghist, int64_t nb, int64_t* dtot,
 }
 
 __global__ void __launch_bounds__(SC_THREADS) k_rs_dscan(int64_t* ghist, int64_t nb, int64_t* dtot) {
+  pdl_enter();
   rs_dscan_digit(ghist, nb, dtot, blockIdx.x);
 }
 
@@ -340,6 +345,7 @@ __global__ void __launch_bounds__(RS_THREADS, 4) k_rs_scatter(const u64* keys, c
                                                               u64* ovals, int64_t n, int shift, int64_t nb,
                                                               const int64_t* goff, const int64_t* dtot, RsExt x,
                                                               int first, int in_off, int out_off) {
+  pdl_enter();
   if (x.n_dev) n = min(n, (int64_t)*x.n_dev);
   rs_scatter_tile(in_off ? keys + n : keys, in_off ? vals + n : vals, out_off ? okeys + n : okeys,
                   out_off ? ovals + n : ovals, n, shift, nb, goff, dtot, blockIdx.x, first ? x.tbits : 0, x.row_off);
@@ -370,6 +376,7 @@ struct CoShared {
 __global__ void __launch_bounds__(CO_THREADS, 1) k_rs_coop(u64* keys, u64* vals, u64* tk, u64* tv, int64_t n,
                                                            int lo_bit, int bits, int32_t* ghist, int32_t* dtot,
                                                            RsExt x) {
+  pdl_enter();
   extern __shared__ __align__(16) unsigned char co_smem[];
   CoShared& m = *(CoShared*)co_smem;
   cg::grid_group grid = cg::this_grid();
@@ -583,6 +590,7 @@ extern __shared__ __align__(16) unsigned char small_smem[];
 
 __global__ void __launch_bounds__(SM_THREADS) k_rs_small(u64* keys, u64* vals, int n, const int32_t* n_dev, int lo_bit,
                                                          int bits) {
+  pdl_enter();
   RsSmall& m = *(RsSmall*)small_smem;
   if (n_dev) n = min(n, *n_dev);
   u64 key[SM_ITEMS], val[SM_ITEMS];
@@ -605,6 +613,7 @@ __global__ void __launch_bounds__(SM_THREADS) k_rs_small_reduce(const u64* keys,
                                                                 const int32_t* n_dev, int bits, int both,
                                                                 int64_t row_off, u64* okeys, int64_t* ovals,
                                                                 int32_t* nr) {
+  pdl_enter();
   RsSmall& m = *(RsSmall*)small_smem;
   if (n_dev) n = min(n, *n_dev);
   const int tid = threadIdx.x;
@@ -713,6 +722,7 @@ constexpr int CS_NW = CS_THREADS / WARP;
 template <int CL>
 __global__ void __launch_bounds__(CS_THREADS, 1) k_rs_cluster(u64* keys, u64* vals, int n, int lo_bit, int bits,
                                                               RsExt x) {
+  pdl_enter();
   extern __shared__ u64 cs_smem[];
   u64* sk = cs_smem;
   u64* sv = cs_smem + CS_TILE;
@@ -833,6 +843,7 @@ __global__ void __launch_bounds__(CS_THREADS, 1) k_rs_cluster(u64* keys, u64* va
 // search for the first equal key.
 constexpr int RBK_RUN = 8;
 __global__ void k_segsum(const u64* keys, const u64* vals, int64_t n, const int32_t* n_dev, int64_t* usum) {
+  pdl_enter();
   if (n_dev) n = min(n, (int64_t)*n_dev);
   const int64_t nt = (n + RBK_RUN - 1) / RBK_RUN;
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nt; r += (int64_t)gridDim.x * blockDim.x) {
@@ -868,6 +879,7 @@ __global__ void k_segsum(const u64* keys, const u64* vals, int64_t n, const int3
 __global__ void __launch_bounds__(SC_THREADS) k_reduce_out(const u64* keys, const int64_t* usum, int64_t n,
                                                            const int32_t* n_dev, u64* okeys, int64_t* ovals,
                                                            int32_t* nr, int64_t* nr64, LookBack q) {
+  pdl_enter();
   __shared__ int64_t s_tile, s_pre;
   if (n_dev) n = min(n, (int64_t)*n_dev);
   if (threadIdx.x == 0) s_tile = atomicAdd(q.ctr, 1);
@@ -953,12 +965,12 @@ LookBack look_back_begin(Prims& P, int64_t words, cudaStream_t s) {
 template <class In>
 static void scan_launch(In in, int64_t* out, int64_t n, int64_t* total_dev, Prims& P, cudaStream_t s) {
   if (n <= SC_TILE) {
-    k_scan_one<In><<<1, SC_THREADS, 0, s>>>(in, out, n, total_dev);
+    launch(k_scan_one<In>, 1, SC_THREADS, 0, s, in, out, n, total_dev);
     CKL("k_scan_one");
   } else {
     const uint32_t ep = lb_begin(P, n, s);
     const int64_t tiles = (n + LB_TILE - 1) / LB_TILE;
-    k_scan_lb<In><<<(unsigned)tiles, SC_THREADS, 0, s>>>(in, out, n, P.lb_st.p, P.lb_ctl.p + ep, ep, total_dev,
+    launch(k_scan_lb<In>, (unsigned)tiles, SC_THREADS, 0, s, in, out, n, P.lb_st.p, P.lb_ctl.p + ep, ep, total_dev,
                                                          P.lb_ctl.p + 256);
     CKL("k_scan_lb");
   }
@@ -988,7 +1000,7 @@ void scan_chunk_counts(const int32_t* list, const int32_t* nlist, int64_t n_hint
                        const int32_t* lb, int32_t chunk, int64_t* out, Prims& P, cudaStream_t s) {
   const int tiles = div_up(n_hint + 1, CC_TPB);
   const LookBack q = look_back_begin(P, tiles, s);
-  k_scan_chunks<<<tiles, CC_TPB, 0, s>>>(list, nlist, n_hint, la, lb, chunk, out, q);
+  launch(k_scan_chunks, tiles, CC_TPB, 0, s, list, nlist, n_hint, la, lb, chunk, out, q);
   CKL("k_scan_chunks");
 }
 
@@ -1008,7 +1020,7 @@ bool scan_wait_gives_up(cudaStream_t s) {
     const uint32_t ep = lb_begin(P, n, s);
     const int32_t one = 1;
     CK(cudaMemcpyAsync(P.lb_ctl.p + ep, &one, sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    k_scan_lb<ArrayIn<int64_t>><<<1, SC_THREADS, 0, s>>>(ArrayIn<int64_t>{in}, out, n, P.lb_st.p, P.lb_ctl.p + ep, ep,
+    launch(k_scan_lb<ArrayIn<int64_t>>, 1, SC_THREADS, 0, s, ArrayIn<int64_t>{in}, out, n, P.lb_st.p, P.lb_ctl.p + ep, ep,
                                                           out + n, P.lb_ctl.p + 256);
     CKL("k_scan_lb");
     CK(cudaMemcpyAsync(&bad, P.lb_ctl.p + 256, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
@@ -1082,12 +1094,14 @@ static void sort_launch(u64*& keys, u64*& vals, u64*& tk, u64*& tv, int64_t n, i
     cfg.blockDim = dim3(CS_THREADS);
     cfg.dynamicSmemBytes = CS_SMEM;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = cl;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     CK(cudaLaunchKernelEx(&cfg, cl == 16 ? k_rs_cluster<16> : k_rs_cluster<8>, keys, vals, (int)n, lo_bit, bits, x));
     CKL("k_rs_cluster");
     return;
@@ -1131,11 +1145,11 @@ static void sort_launch(u64*& keys, u64*& vals, u64*& tk, u64*& tv, int64_t n, i
   }
   for (int shift = lo_bit; shift < bits; shift += 8) {
     const int first = shift == lo_bit;
-    k_rs_hist<<<(unsigned)nb, RS_THREADS, 0, s>>>(in.k, n, shift, nb, P.hist.p, x, first, in.off);
+    launch(k_rs_hist, (unsigned)nb, RS_THREADS, 0, s, in.k, n, shift, nb, P.hist.p, x, first, in.off);
     CKL("k_rs_hist");
-    k_rs_dscan<<<256, SC_THREADS, 0, s>>>(P.hist.p, nb, P.bsum.p);
+    launch(k_rs_dscan, 256, SC_THREADS, 0, s, P.hist.p, nb, P.bsum.p);
     CKL("k_rs_dscan");
-    k_rs_scatter<<<(unsigned)nb, RS_THREADS, 0, s>>>(in.k, in.v, out.k, out.v, n, shift, nb, P.hist.p, P.bsum.p, x,
+    launch(k_rs_scatter, (unsigned)nb, RS_THREADS, 0, s, in.k, in.v, out.k, out.v, n, shift, nb, P.hist.p, P.bsum.p, x,
                                                      first, in.off, out.off);
     CKL("k_rs_scatter");
     in = out;
@@ -1152,7 +1166,7 @@ void radix_sort_pairs(u64*& keys, u64*& vals, u64*& tk, u64*& tv, int64_t n, int
   if (n <= 1 || bits <= lo_bit) return;
   if (n <= RS_TILE) {
     small_smem_opt_in((const void*)k_rs_small);
-    k_rs_small<<<1, SM_THREADS, sizeof(RsSmall), s>>>(keys, vals, (int)n, n_dev, lo_bit, bits);
+    launch(k_rs_small, 1, SM_THREADS, sizeof(RsSmall), s, keys, vals, (int)n, n_dev, lo_bit, bits);
     CKL("k_rs_small");
     return;
   }
@@ -1166,7 +1180,7 @@ void sort_reduce(DBuf<u64>& k, DBuf<u64>& v, DBuf<u64>& tk, DBuf<u64>& tv, int64
     // for some hundred, where the launches of the larger sizes take 16.4 and
     // 23.5 and the gaps between them
     small_smem_opt_in((const void*)k_rs_small_reduce);
-    k_rs_small_reduce<<<1, SM_THREADS, sizeof(RsSmall), s>>>(k.p, v.p, (int)n, n_dev, bits, both ? 1 : 0, row_off, okeys, ovals, nr);
+    launch(k_rs_small_reduce, 1, SM_THREADS, sizeof(RsSmall), s, k.p, v.p, (int)n, n_dev, bits, both ? 1 : 0, row_off, okeys, ovals, nr);
     CKL("k_rs_small_reduce");
     return;
   }
@@ -1180,11 +1194,11 @@ void sort_reduce(DBuf<u64>& k, DBuf<u64>& v, DBuf<u64>& tk, DBuf<u64>& tv, int64
     swap_buf(k, tk);
     swap_buf(v, tv);
   }
-  k_segsum<<<grid_for((n + RBK_RUN - 1) / RBK_RUN, 256), 256, 0, s>>>(k.p, v.p, n, n_dev, P.usum.p);
+  launch(k_segsum, grid_for((n + RBK_RUN - 1) / RBK_RUN, 256), 256, 0, s, k.p, v.p, n, n_dev, P.usum.p);
   CKL("k_segsum");
   const int tiles = div_up(n, LB_TILE);
   const LookBack q = look_back_begin(P, tiles, s);
-  k_reduce_out<<<tiles, SC_THREADS, 0, s>>>(k.p, P.usum.p, n, n_dev, okeys, ovals, nr, nullptr, q);
+  launch(k_reduce_out, tiles, SC_THREADS, 0, s, k.p, P.usum.p, n, n_dev, okeys, ovals, nr, nullptr, q);
   CKL("k_reduce_out");
   if (both) {
     // in (row, col) order already: a stable sort on the new row alone
@@ -1199,12 +1213,12 @@ int64_t reduce_by_key(const u64* keys, const u64* vals, int64_t n, u64* okeys, i
   P.usum.reserve(n + 1, s);
   // a segment crossing a run boundary is summed atomically into a zeroed slot
   CK(cudaMemsetAsync(P.usum.p, 0, sizeof(int64_t) * (size_t)n, s));
-  k_segsum<<<grid_for((n + RBK_RUN - 1) / RBK_RUN, 256), 256, 0, s>>>(keys, vals, n, nullptr, P.usum.p);
+  launch(k_segsum, grid_for((n + RBK_RUN - 1) / RBK_RUN, 256), 256, 0, s, keys, vals, n, nullptr, P.usum.p);
   CKL("k_segsum");
   const int tiles = div_up(n, LB_TILE);
   const LookBack q = look_back_begin(P, tiles, s);
   P.bsum.reserve(2, s);
-  k_reduce_out<<<tiles, SC_THREADS, 0, s>>>(keys, P.usum.p, n, nullptr, okeys, ovals, nullptr, P.bsum.p, q);
+  launch(k_reduce_out, tiles, SC_THREADS, 0, s, keys, P.usum.p, n, nullptr, okeys, ovals, nullptr, P.bsum.p, q);
   CKL("k_reduce_out");
   int64_t nz = 0;
   const HostRead r{P.bsum.p, &nz, sizeof(int64_t)};

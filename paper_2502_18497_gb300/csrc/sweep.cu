@@ -45,6 +45,7 @@ constexpr int EVAL_CH = 1024;  // hub table slots evaluated per block (4096: one
 template <class WT>
 __global__ void k_expand(Adj<WT> out, Adj<WT> in, ChunkMap m, int32_t* stamp, int32_t ep, int32_t* olist,
                          int32_t* nout, Tail tail) {
+  pdl_enter();
   constexpr int PL = CH / 32;  // entries per lane
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -96,6 +97,7 @@ __global__ void k_expand(Adj<WT> out, Adj<WT> in, ChunkMap m, int32_t* stamp, in
 __global__ void k_frontier(const int32_t* list, const int32_t* nlist, const uint8_t* alive, int32_t* lU, int32_t* nU,
                            int32_t* stU, int32_t epU, int32_t* lUs, int32_t* nUs, const int32_t* len_out,
                            const int32_t* len_in, int64_t* deg, Tail tail) {
+  pdl_enter();
   const int32_t nl = *nlist;
   int64_t sum = 0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -118,6 +120,7 @@ __global__ void k_frontier(const int32_t* list, const int32_t* nlist, const uint
 
 __global__ void k_union(const int32_t* list, const int32_t* nlist, int32_t* stamp, int32_t ep, int32_t* olist,
                         int32_t* nout) {
+  pdl_enter();
   const int32_t nl = *nlist;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nl; t += (int64_t)gridDim.x * blockDim.x)
     stamp_add(stamp, ep, list[t], olist, nout);
@@ -392,6 +395,7 @@ __device__ inline void emit_cand(const SweepArgs<WT>& A, int32_t v, int32_t src,
 template <class WT, int MODE, int G, class GT>
 __global__ void __launch_bounds__(TPB, wide_sums<GT> ? 4 : 6) k_sweep_group(SweepArgs<WT> A, const int32_t* list,
                                                                              const int32_t* nlist) {
+  pdl_enter();
   constexpr int HG = G == 8 ? HG8 : HG32;
   constexpr int GPW = 32 / G;  // groups per warp
   constexpr bool WIDE = wide_sums<GT>;
@@ -512,6 +516,7 @@ __device__ inline void stage_keys(const SweepArgs<WT>& A, int32_t v, int32_t a, 
 template <class WT, int MODE, int NT, int HMAX, class GT>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, const int32_t* list,
                                                                const int32_t* nlist) {
+  pdl_enter();
   extern __shared__ unsigned char smem[];
   constexpr bool WIDE = wide_sums<GT>;
   __shared__ BestG<GT> wb[NT / 32];
@@ -609,6 +614,7 @@ __global__ void k_bin(Adj<WT> out, Adj<WT> in, int directed, const int32_t* list
                       int32_t* nm2, int32_t* bc, int32_t* nc, int32_t* bl, int32_t* nlarge, int64_t* lsz,
                       int64_t* tabtop, int32_t t0_, int32_t t1, int32_t t2, int32_t t3,
                       int32_t cluster_max, Tail tail) {
+  pdl_enter();
   // BI nodes per thread and step; the block counts its bins in shared memory
   // and takes its places with one global atomic per bin and step.  (With one
   // per warp, bin and 32 nodes the counters bound it: 28 us for the level-0
@@ -678,6 +684,7 @@ __global__ void k_bin(Adj<WT> out, Adj<WT> in, int directed, const int32_t* list
 template <class WT, int MODE>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(TPB)
     k_sweep_cluster(SweepArgs<WT> A, const int32_t* list, const int32_t* nlist) {
+  pdl_enter();
   extern __shared__ unsigned char smem[];
   int64_t* V = (int64_t*)smem;
   int32_t* K = (int32_t*)(smem + sizeof(int64_t) * CL_SLOTS);
@@ -805,6 +812,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(TPB)
 // evaluated, in chunks whose partial bests are reduced per hub, and then
 // cleared, so the tables stay clean between sweeps without a full re-fill.
 __global__ void k_hub_init(int32_t* K, int64_t* V, int64_t total) {
+  pdl_enter();
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     K[t] = -1;
     V[t] = 0;
@@ -816,6 +824,7 @@ __global__ void k_hub_init(int32_t* K, int64_t* V, int64_t total) {
 // the slot counts, with the total behind the last).
 __global__ void __launch_bounds__(1024) k_hub_scan(int32_t nh, const int64_t* lsz, int32_t* hcnt, int64_t* hown,
                                                    int64_t* out) {
+  pdl_enter();
   int64_t o = 0;
   for (int32_t i0 = 0; i0 < nh; i0 += 1024) {
     const int32_t i = i0 + threadIdx.x;
@@ -847,6 +856,7 @@ __device__ inline int64_t hub_of(const int64_t* epre, int32_t nh, int64_t e) {
 template <class WT, int MODE>
 __global__ void k_hub_acc(SweepArgs<WT> A, ChunkMap m, const int64_t* loff, const int64_t* lsz, int32_t* gK,
                           int64_t* gV, int32_t* glist, int32_t* hcnt, int64_t* hown) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -944,6 +954,7 @@ __global__ void __launch_bounds__(TPB) k_hub_eval(SweepArgs<WT> A, const int32_t
                                                   const int32_t* gK, const int64_t* gV, const int32_t* glist,
                                                   const int32_t* hcnt, const int64_t* hown, int64_t* pb_hi, uint64_t* pb_lo,
                                                   int32_t* pb_c) {
+  pdl_enter();
   __shared__ Best wb[TPB / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t mult = A.directed ? 1 : 2;
@@ -996,6 +1007,7 @@ template <class WT, int MODE>
 __global__ void k_hub_final(SweepArgs<WT> A, const int32_t* hubs, int32_t nh, const int64_t* loff,
                             const int64_t* epre, const int64_t* pb_hi, const uint64_t* pb_lo, const int32_t* pb_c,
                             const int32_t* hcnt, const int32_t* glist, int32_t* gK, int64_t* gV) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1063,6 +1075,7 @@ __global__ void __launch_bounds__(DG_TPB) k_dec_grid(int32_t nc, int32_t* cst, c
                                                   const int32_t* dst, const int64_t* ghi, const uint64_t* glo,
                                                   int32_t* role, int32_t* best, int32_t* bv, int32_t* bsrc,
                                                   int32_t* bdst, int32_t* nb, int32_t* undecided, int32_t* stat) {
+  pdl_enter();
   cg::grid_group grid = cg::this_grid();
   const int32_t tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
   for (int32_t i = tid; i < nc; i += nth) cst[i] = 0;
@@ -1143,6 +1156,7 @@ __global__ void __launch_bounds__(DEC_THREADS) k_dec_block(const int32_t* ncp, c
                                                            const uint64_t* glo, int32_t* role, int32_t* best,
                                                            int32_t* bv, int32_t* bsrc, int32_t* bdst, int32_t* nb,
                                                            int32_t* stat, Tail tail) {
+  pdl_enter();
   extern __shared__ unsigned char dsm[];
   int64_t* sghi = (int64_t*)dsm;
   uint64_t* sglo = (uint64_t*)(dsm + sizeof(int64_t) * DEC_SMALL);
@@ -1252,6 +1266,7 @@ __global__ void k_commit_mark(int32_t nb, const int32_t* bv, const int32_t* bsrc
                               int32_t* lT, int32_t* nT, int32_t* stCh, int32_t epCh, int32_t* lCh, int32_t* nCh,
                               int32_t* lab_before, int level0, const int64_t* Kout, const int64_t* Kin,
                               const int64_t* e, int64_t* sko, int64_t* ski, int64_t* se) {
+  pdl_enter();
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) {
     const int32_t v = bv[i];
     oldlab[v] = bsrc[i];
@@ -1272,6 +1287,7 @@ __global__ void k_commit_e(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* b
                            const int32_t* lab, const int32_t* oldlab, const int32_t* stB, int32_t epB, int64_t* e,
                            int32_t nb, const int32_t* bv, const int64_t* kout, const int64_t* kin, int64_t* Kout,
                            int64_t* Kin, int directed) {
+  pdl_enter();
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) {
     const int32_t v = bv[i];
     atomic_add_i64(&Kout[bsrc[i]], -kout[v]);
@@ -1326,6 +1342,7 @@ __global__ void k_commit_e(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* b
 __global__ void k_commit_dq(const int32_t* lT, const int32_t* nT, const int64_t* Kout, const int64_t* Kin,
                             const int64_t* e, const int64_t* sko, const int64_t* ski, const int64_t* se, int64_t m,
                             int64_t gn, int64_t gd, CommitAcc* sc) {
+  pdl_enter();
   const int32_t n = *nT;
   i128 dq = 0, dp = 0;
   int64_t de = 0;
@@ -1350,6 +1367,7 @@ __global__ void k_commit_dq(const int32_t* lT, const int32_t* nT, const int64_t*
 __global__ void k_rollback(int32_t nb, const int32_t* bv, const int32_t* bsrc, int32_t* lab, const int32_t* lT,
                            const int32_t* nT, int64_t* Kout, int64_t* Kin, int64_t* e, const int64_t* sko,
                            const int64_t* ski, const int64_t* se, int directed) {
+  pdl_enter();
   const int32_t n = *nT;
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) lab[bv[i]] = bsrc[i];
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -1365,6 +1383,7 @@ __global__ void k_rollback(int32_t nb, const int32_t* bv, const int32_t* bsrc, i
 __global__ void k_mark_moved(int32_t nb, const int32_t* bv, int32_t* stMv, int32_t epMv, int32_t* lMv, int32_t* nMv,
                              int32_t* stM0, int32_t epM0, int32_t* lM0, int32_t* nM0, int32_t nU, const int32_t* lU,
                              int32_t* stU, int32_t epU, int32_t* lUs, int32_t* nUs) {
+  pdl_enter();
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) {
     stamp_add(stMv, epMv, bv[i], lMv, nMv);
     if (stM0) stamp_add(stM0, epM0, bv[i], lM0, nM0);
@@ -1380,6 +1399,7 @@ __global__ void k_mark_moved(int32_t nb, const int32_t* bv, int32_t* stMv, int32
 // ---------------------------------------------------------------- refine commit
 __global__ void k_commit_ref(int32_t nb, const int32_t* bv, const int32_t* bdst, int32_t* par, const int64_t* kout,
                              const int64_t* kin, int64_t* kout1, int64_t* kin1, int32_t* cnt1, int directed) {
+  pdl_enter();
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) {
     const int32_t v = bv[i], X = bdst[i];
     par[v] = X;
@@ -1400,6 +1420,7 @@ template <class WT>
 __global__ void k_spexpand(Adj<WT> out, Adj<WT> in, ChunkMap m, const int32_t* lab, const int32_t* par,
                            const int32_t* cnt1, const int32_t* stD, int32_t epD, int32_t* stR, int32_t epR,
                            int32_t* lR, int32_t* nR) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1434,11 +1455,11 @@ static void expand_tail(ldl_ctx& c, int r, const int32_t* list, int idx_n, int32
   if (r == 0) {
     Adj<int32_t> o = adj_out0(c), i = adj_in0(c);
     ChunkMap m = chunk_map(c, list, c.cp[idx_n], n_hint, o.len, c.directed ? i.len : nullptr);
-    k_expand<int32_t><<<g, TPB, 0, c.s>>>(o, i, m, stamp, ep, olist, c.cp[idx_out], tail);
+    launch(k_expand<int32_t>, g, TPB, 0, c.s, o, i, m, stamp, ep, olist, c.cp[idx_out], tail);
   } else {
     Adj<int64_t> o = adj_out(c, r), i = adj_in(c, r);
     ChunkMap m = chunk_map(c, list, c.cp[idx_n], n_hint, o.len, c.directed ? i.len : nullptr);
-    k_expand<int64_t><<<g, TPB, 0, c.s>>>(o, i, m, stamp, ep, olist, c.cp[idx_out], tail);
+    launch(k_expand<int64_t>, g, TPB, 0, c.s, o, i, m, stamp, ep, olist, c.cp[idx_out], tail);
   }
   CKL("k_expand");
 }
@@ -1453,7 +1474,7 @@ void frontier(ldl_ctx& c, int r, int32_t epU, const Tail& tail) {
   LevelState& L = c.lv[r];
   const int32_t* lo = r == 0 ? adj_out0(c).len : adj_out(c, r).len;
   const int32_t* li = !c.directed ? nullptr : r == 0 ? adj_in0(c).len : adj_in(c, r).len;
-  k_frontier<<<grid_for(L.ubA, TPB, 2), TPB, 0, c.s>>>(L.lA.p, c.cp[K_A0 + r], r ? L.alive.p : nullptr, c.lU.p,
+  launch(k_frontier, grid_for(L.ubA, TPB, 2), TPB, 0, c.s, L.lA.p, c.cp[K_A0 + r], r ? L.alive.p : nullptr, c.lU.p,
                                                        c.cp[K_U], c.stU.p, epU, c.lUstar.p, c.cp[K_USTAR], lo, li,
                                                        c.sums, tail);
   CKL("k_frontier");
@@ -1461,7 +1482,7 @@ void frontier(ldl_ctx& c, int r, int32_t epU, const Tail& tail) {
 
 void union_into(ldl_ctx& c, const int32_t* list, int idx_n, int32_t* stamp, int32_t ep, int32_t* olist, int idx_out,
                 int64_t n_hint) {
-  k_union<<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(list, c.cp[idx_n], stamp, ep, olist, c.cp[idx_out]);
+  launch(k_union, grid_for(n_hint, TPB), TPB, 0, c.s, list, c.cp[idx_n], stamp, ep, olist, c.cp[idx_out]);
   CKL("k_union");
 }
 
@@ -1479,15 +1500,15 @@ static bool sweep_gain_fits_i64(const ldl_ctx& c) {
 template <class WT, int MODE, class GT>
 static void sweep_bins(ldl_ctx& c, const SweepArgs<WT>& A, int64_t n_hint, bool few, cudaEvent_t* kev) {
   if (!few) {
-  k_sweep_group<WT, MODE, 8, GT><<<grid_for(n_hint * 8, TPB, 6), TPB, 0, c.s>>>(A, c.binT.p, c.cp[K_TINY]);
+  launch(k_sweep_group<WT, MODE, 8, GT>, grid_for(n_hint * 8, TPB, 6), TPB, 0, c.s, A, c.binT.p, c.cp[K_TINY]);
   CKL("k_sweep_group<8>");
   if (kev) CK(cudaEventRecord(kev[1], c.s));
-  k_sweep_group<WT, MODE, 32, GT><<<grid_for(n_hint * 32, TPB, 6), TPB, 0, c.s>>>(A, c.binS.p, c.cp[K_SMALL]);
+  launch(k_sweep_group<WT, MODE, 32, GT>, grid_for(n_hint * 32, TPB, 6), TPB, 0, c.s, A, c.binS.p, c.cp[K_SMALL]);
   CKL("k_sweep_group<32>");
   if (kev) CK(cudaEventRecord(kev[2], c.s));
   {
     const size_t sm = (size_t)tab_slot<GT> * 2048;
-    k_sweep_block<WT, MODE, 128, 2048, GT><<<grid_for(n_hint, 1, 16), 128, sm, c.s>>>(A, c.binM.p, c.cp[K_MID]);
+    launch(k_sweep_block<WT, MODE, 128, 2048, GT>, grid_for(n_hint, 1, 16), 128, sm, c.s, A, c.binM.p, c.cp[K_MID]);
     CKL("k_sweep_block(mid1)");
   }
   if (kev) CK(cudaEventRecord(kev[3], c.s));
@@ -1496,7 +1517,7 @@ static void sweep_bins(ldl_ctx& c, const SweepArgs<WT>& A, int64_t n_hint, bool 
     const size_t sm = (size_t)tab_slot<GT> * HB;
     CK(cudaFuncSetAttribute(k_sweep_block<WT, MODE, 256, HB, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)sm));
-    k_sweep_block<WT, MODE, 256, HB, GT><<<grid_for(n_hint, 1, 4), 256, sm, c.s>>>(A, c.binM2.p, c.cp[K_MID2]);
+    launch(k_sweep_block<WT, MODE, 256, HB, GT>, grid_for(n_hint, 1, 4), 256, sm, c.s, A, c.binM2.p, c.cp[K_MID2]);
     CKL("k_sweep_block(mid2)");
   }
 }
@@ -1568,7 +1589,7 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   if (spec) spec->done = false;
   if (!few) spec = nullptr;
   const bool early = expect || c.kstats;
-  k_bin<WT><<<grid_for(n_hint, TPB), TPB, 0, c.s>>>(out, in, c.directed, list, c.cp[idx_n], c.binT.p, c.cp[K_TINY],
+  launch(k_bin<WT>, grid_for(n_hint, TPB), TPB, 0, c.s, out, in, c.directed, list, c.cp[idx_n], c.binT.p, c.cp[K_TINY],
                                                      c.binS.p, c.cp[K_SMALL], c.binM.p, c.cp[K_MID], c.binM2.p,
                                                      c.cp[K_MID2], c.binC.p, c.cp[K_CLU], c.binL.p, c.cp[K_LARGE],
                                                      c.binLsz.p, c.sums, few ? -1 : c.bin_deg[0],
@@ -1588,7 +1609,7 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
     const size_t sm = (sizeof(int64_t) + sizeof(int32_t)) * CL_SLOTS;
     CK(cudaFuncSetAttribute(k_sweep_cluster<WT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     const int ncl = (int)std::min<int64_t>(n_hint, std::max(1, device_sms() * 2 / CL));
-    k_sweep_cluster<WT, MODE><<<ncl * CL, TPB, sm, c.s>>>(A, c.binC.p, c.cp[K_CLU]);
+    launch(k_sweep_cluster<WT, MODE>, ncl * CL, TPB, sm, c.s, A, c.binC.p, c.cp[K_CLU]);
     CKL("k_sweep_cluster");
   }
   if (kev) CK(cudaEventRecord(kev[5], c.s));
@@ -1628,7 +1649,7 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
     c.gkeys.reserve(tab_use, c.s);
     c.gvals.reserve(tab_use, c.s);
     if (c.gtab_clean != c.gkeys.cap || c.gvals.cap != c.gkeys.cap) {  // fresh tables: fill once
-      k_hub_init<<<grid_for(c.gkeys.cap, TPB), TPB, 0, c.s>>>(c.gkeys.p, c.gvals.p, c.gkeys.cap);
+      launch(k_hub_init, grid_for(c.gkeys.cap, TPB), TPB, 0, c.s, c.gkeys.p, c.gvals.p, c.gkeys.cap);
       CKL("k_hub_init");
       c.gtab_clean = c.gkeys.cap;
     }
@@ -1651,20 +1672,20 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
         set_cnt(c, K_HUBG, nh);
         cntp = c.cp[K_HUBG];
       }
-      k_hub_scan<<<1, 1024, 0, c.s>>>(nh, Lsz, c.hcnt.p, c.hown.p, Loff);
+      launch(k_hub_scan, 1, 1024, 0, c.s, nh, Lsz, c.hcnt.p, c.hown.p, Loff);
       CKL("k_hub_scan");
       ChunkMap m = chunk_map(c, L, cntp, nh, out.len, c.directed ? in.len : nullptr);
-      k_hub_acc<WT, MODE><<<grid_for((int64_t)nh * 2048, TPB, 16), TPB, 0, c.s>>>(
+      launch(k_hub_acc<WT, MODE>, grid_for((int64_t)nh * 2048, TPB, 16), TPB, 0, c.s,
           A, m, Loff, Lsz, c.gkeys.p, c.gvals.p, c.glist.p, c.hcnt.p, c.hown.p);
       CKL("k_hub_acc");
       if (kev && gi + 2 == gb.size()) CK(cudaEventRecord(kev[8], c.s));
-      k_hub_scan<<<1, 1024, 0, c.s>>>(nh, nullptr, c.hcnt.p, nullptr, c.hub_epre.p);
+      launch(k_hub_scan, 1, 1024, 0, c.s, nh, nullptr, c.hcnt.p, nullptr, c.hub_epre.p);
       CKL("k_hub_scan");
       const int ge = grid_for(ech, 1, 8);
-      k_hub_eval<WT, MODE><<<ge, TPB, 0, c.s>>>(A, L, nh, Loff, c.hub_epre.p, c.gkeys.p, c.gvals.p, c.glist.p, c.hcnt.p,
+      launch(k_hub_eval<WT, MODE>, ge, TPB, 0, c.s, A, L, nh, Loff, c.hub_epre.p, c.gkeys.p, c.gvals.p, c.glist.p, c.hcnt.p,
                                                 c.hown.p, c.pb_hi.p, c.pb_lo.p, c.pb_c.p);
       CKL("k_hub_eval");
-      k_hub_final<WT, MODE><<<std::max(ge, grid_for((int64_t)nh * 32, TPB)), TPB, 0, c.s>>>(
+      launch(k_hub_final<WT, MODE>, std::max(ge, grid_for((int64_t)nh * 32, TPB)), TPB, 0, c.s,
           A, L, nh, Loff, c.hub_epre.p, c.pb_hi.p, c.pb_lo.p, c.pb_c.p, c.hcnt.p, c.glist.p, c.gkeys.p, c.gvals.p);
       CKL("k_hub_final");
     }
@@ -1718,7 +1739,7 @@ DecoupleOut decouple(ldl_ctx& c, const HostRead* extra, int n_extra, SplitRun* s
                            {c.cp[K_UNDEC], &stat, sizeof(int32_t)}};
   for (int i = 0; i < n_extra; ++i) rr[3 + i] = extra[i];
   CK(cudaFuncSetAttribute(k_dec_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DEC_SMEM));
-  k_dec_block<<<1, DEC_THREADS, DEC_SMEM, c.s>>>(c.cp[K_CAND], c.cv.p, c.csrc.p, c.cdst.p, c.cghi.p, c.cglo.p,
+  launch(k_dec_block, 1, DEC_THREADS, DEC_SMEM, c.s, c.cp[K_CAND], c.cv.p, c.csrc.p, c.cdst.p, c.cghi.p, c.cglo.p,
                                                  c.role.p, c.best.p, c.bv.p, c.bsrc.p, c.bdst.p, c.cp[K_B],
                                                  c.cp[K_UNDEC], spec ? Tail{} : tail_begin(c, rr, 3 + n_extra));
   CKL("k_dec_block");
@@ -1759,7 +1780,7 @@ void commit_move(ldl_ctx& c, int r, int32_t nb, int32_t epB, int32_t epT, int32_
   const int g = grid_for(nb, TPB);
   zero_cnt(c, K_T);
   c.acc = (CommitAcc*)fresh(c, sizeof(CommitAcc) / 4, c.d_sc->home);
-  k_commit_mark<<<g, TPB, 0, c.s>>>(nb, c.bv.p, c.bsrc.p, c.bdst.p, L.lab.p, c.oldlab.p, c.stB.p, epB, c.stT.p, epT,
+  launch(k_commit_mark, g, TPB, 0, c.s, nb, c.bv.p, c.bsrc.p, c.bdst.p, L.lab.p, c.oldlab.p, c.stB.p, epB, c.stT.p, epT,
                                     c.lT.p, c.cp[K_T], c.stCh.p, epCh, c.lCh.p, c.cp[K_CH], c.lab_before.p, r == 0,
                                     c.Kout.p, Kin_of(c), c.e.p, c.snapKo.p, c.snapKi.p, c.snapE.p);
   CKL("k_commit_mark");
@@ -1767,16 +1788,16 @@ void commit_move(ldl_ctx& c, int r, int32_t nb, int32_t epB, int32_t epT, int32_
   if (r == 0) {
     Adj<int32_t> o = adj_out0(c), i = adj_in0(c);
     ChunkMap m = chunk_map(c, c.bv.p, c.cp[K_B], nb, o.len, i.len);
-    k_commit_e<int32_t><<<gw, TPB, 0, c.s>>>(o, i, m, c.bsrc.p, c.bdst.p, L.lab.p, c.oldlab.p, c.stB.p, epB, c.e.p, nb,
+    launch(k_commit_e<int32_t>, gw, TPB, 0, c.s, o, i, m, c.bsrc.p, c.bdst.p, L.lab.p, c.oldlab.p, c.stB.p, epB, c.e.p, nb,
                                           c.bv.p, L.kout.p, kin_of(c, r), c.Kout.p, Kin_of(c), c.directed);
   } else {
     Adj<int64_t> o = adj_out(c, r), i = adj_in(c, r);
     ChunkMap m = chunk_map(c, c.bv.p, c.cp[K_B], nb, o.len, i.len);
-    k_commit_e<int64_t><<<gw, TPB, 0, c.s>>>(o, i, m, c.bsrc.p, c.bdst.p, L.lab.p, c.oldlab.p, c.stB.p, epB, c.e.p, nb,
+    launch(k_commit_e<int64_t>, gw, TPB, 0, c.s, o, i, m, c.bsrc.p, c.bdst.p, L.lab.p, c.oldlab.p, c.stB.p, epB, c.e.p, nb,
                                           c.bv.p, L.kout.p, kin_of(c, r), c.Kout.p, Kin_of(c), c.directed);
   }
   CKL("k_commit_e");
-  k_commit_dq<<<grid_for(2 * (int64_t)nb, TPB), TPB, 0, c.s>>>(c.lT.p, c.cp[K_T], c.Kout.p, Kin_of(c), c.e.p,
+  launch(k_commit_dq, grid_for(2 * (int64_t)nb, TPB), TPB, 0, c.s, c.lT.p, c.cp[K_T], c.Kout.p, Kin_of(c), c.e.p,
                                                                c.snapKo.p, c.snapKi.p, c.snapE.p, c.m,
                                                                c.prm.gamma_num, c.prm.gamma_den, c.acc);
   CKL("k_commit_dq");
@@ -1797,14 +1818,14 @@ CommitOut commit_expand(ldl_ctx& c, int r, int32_t nb, int32_t ep, int32_t* nU) 
 void rollback_move(ldl_ctx& c, int r, int32_t nb, int32_t ntc) {
   LevelState& L = c.lv[r];
   const int64_t m = nb > ntc ? nb : ntc;
-  k_rollback<<<grid_for(m, TPB), TPB, 0, c.s>>>(nb, c.bv.p, c.bsrc.p, L.lab.p, c.lT.p, c.cp[K_T], c.Kout.p,
+  launch(k_rollback, grid_for(m, TPB), TPB, 0, c.s, nb, c.bv.p, c.bsrc.p, L.lab.p, c.lT.p, c.cp[K_T], c.Kout.p,
                                                 Kin_of(c), c.e.p, c.snapKo.p, c.snapKi.p, c.snapE.p, c.directed);
   CKL("k_rollback");
 }
 
 void mark_moved(ldl_ctx& c, int r, int32_t nb, int32_t epMv, int32_t epM0, int32_t epU, int32_t nU) {
   c.ubU = std::min<int64_t>(c.n, c.ubU + nU);
-  k_mark_moved<<<grid_for(std::max(nb, nU), TPB), TPB, 0, c.s>>>(
+  launch(k_mark_moved, grid_for(std::max(nb, nU), TPB), TPB, 0, c.s,
       nb, c.bv.p, c.stMv.p, epMv, c.lMv.p, c.cp[K_MV], r == 0 ? c.stM0.p : nullptr, epM0, c.lM0.p, c.cp[K_M0], nU,
       c.lU.p, c.stU.p, epU, c.lUstar.p, c.cp[K_USTAR]);
   CKL("k_mark_moved");
@@ -1813,7 +1834,7 @@ void mark_moved(ldl_ctx& c, int r, int32_t nb, int32_t epMv, int32_t epM0, int32
 void commit_ref(ldl_ctx& c, int r, int32_t nb) {
   LevelState& L = c.lv[r];
   LevelState& N = c.lv[r + 1];
-  k_commit_ref<<<grid_for(nb, TPB), TPB, 0, c.s>>>(nb, c.bv.p, c.bdst.p, L.par.p, L.kout.p, kin_of(c, r), N.kout.p,
+  launch(k_commit_ref, grid_for(nb, TPB), TPB, 0, c.s, nb, c.bv.p, c.bdst.p, L.par.p, L.kout.p, kin_of(c, r), N.kout.p,
                                                    kin_of(c, r + 1), N.cnt.p, c.directed);
   CKL("k_commit_ref");
 }
@@ -1824,12 +1845,12 @@ void spexpand(ldl_ctx& c, int r, int32_t nb, int32_t epD, int32_t epR, int32_t* 
   if (r == 0) {
     Adj<int32_t> o = adj_out0(c), i = adj_in0(c);
     ChunkMap m = chunk_map(c, c.bv.p, c.cp[K_B], nb, o.len, c.directed ? i.len : nullptr);
-    k_spexpand<int32_t><<<g, TPB, 0, c.s>>>(o, i, m, L.lab.p, L.par.p, c.lv[r + 1].cnt.p, c.stD.p, epD, c.stR.p,
+    launch(k_spexpand<int32_t>, g, TPB, 0, c.s, o, i, m, L.lab.p, L.par.p, c.lv[r + 1].cnt.p, c.stD.p, epD, c.stR.p,
                                             epR, lR, c.cp[idx_R]);
   } else {
     Adj<int64_t> o = adj_out(c, r), i = adj_in(c, r);
     ChunkMap m = chunk_map(c, c.bv.p, c.cp[K_B], nb, o.len, c.directed ? i.len : nullptr);
-    k_spexpand<int64_t><<<g, TPB, 0, c.s>>>(o, i, m, L.lab.p, L.par.p, c.lv[r + 1].cnt.p, c.stD.p, epD, c.stR.p,
+    launch(k_spexpand<int64_t>, g, TPB, 0, c.s, o, i, m, L.lab.p, L.par.p, c.lv[r + 1].cnt.p, c.stD.p, epD, c.stR.p,
                                             epR, lR, c.cp[idx_R]);
   }
   CKL("k_spexpand");
