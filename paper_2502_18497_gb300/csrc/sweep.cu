@@ -33,6 +33,12 @@ static_assert(BIN_MAX[0] == HG8 / 2 && BIN_MAX[1] == HG32 / 2 && BIN_MAX[2] == 2
 // vertices took 621 us a batch with a launch per bin, 531 with one; with 4096
 // here, batches of 100 to 1000 measure the same as with 1024 (within 1%).
 constexpr int SWEEP_FEW = 1024;
+// Hub entries per block of the accumulation (four chunks for its eight warps).
+// The grid follows the tables' size, which is 2..4 slots an entry; with eight
+// blocks per hub a few rows of 10^5 entries were walked by 64 warps each, one
+// chunk after the other (batches on the 2M-vertex power-law graph: 10^5 updates
+// 4473 -> 4417 us, 100 updates 1642 -> 1621 us; 2 * TPB here measures the same).
+constexpr int HUB_ACC = 4 * 256;
 constexpr int EVAL_CH = 1024;  // hub table slots evaluated per block (4096: one block a hub, 17 us where this takes 16)
 
 // ---------------------------------------------------------------- expand
@@ -1675,7 +1681,7 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
       launch(k_hub_scan, 1, 1024, 0, c.s, nh, Lsz, c.hcnt.p, c.hown.p, Loff);
       CKL("k_hub_scan");
       ChunkMap m = chunk_map(c, L, cntp, nh, out.len, c.directed ? in.len : nullptr);
-      launch(k_hub_acc<WT, MODE>, grid_for((int64_t)nh * 2048, TPB, 16), TPB, 0, c.s,
+      launch(k_hub_acc<WT, MODE>, grid_for(tab_use / 4, HUB_ACC, 16), TPB, 0, c.s,
           A, m, Loff, Lsz, c.gkeys.p, c.gvals.p, c.glist.p, c.hcnt.p, c.hown.p);
       CKL("k_hub_acc");
       if (kev && gi + 2 == gb.size()) CK(cudaEventRecord(kev[8], c.s));
