@@ -33,12 +33,21 @@ static_assert(BIN_MAX[0] == HG8 / 2 && BIN_MAX[1] == HG32 / 2 && BIN_MAX[2] == 2
 // vertices took 621 us a batch with a launch per bin, 531 with one; with 4096
 // here, batches of 100 to 1000 measure the same as with 1024 (within 1%).
 constexpr int SWEEP_FEW = 1024;
+// Nodes up to which a sweep runs all four bins in one launch (k_sweep_bins), so
+// that short bins fill one another's idle blocks instead of waiting for one
+// another.  Against a launch per bin: a batch of 100 on 10k vertices 673 -> 626
+// us, 500 on 131k 1040 -> 994, 10^3 on the R-MAT of 131k 1782 -> 1730.  Above,
+// the groups' own kernel pays with its 6 blocks an SM to 4: with every sweep in
+// one launch a batch of 10^4 on the R-MAT of 2^20 took 4490-4600 us where this
+// bound takes 4310-4350, and one of 10^5 on the 2M-vertex power-law graph
+// 4740-4900 where it takes 4410-4650.
+constexpr int64_t SWEEP_FUSE = 131072;
 // Hub entries per block of the accumulation (four chunks for its eight warps).
 // The grid follows the tables' size, which is 2..4 slots an entry; with eight
 // blocks per hub a few rows of 10^5 entries were walked by 64 warps each, one
 // chunk after the other (batches on the 2M-vertex power-law graph: 10^5 updates
-// 4473 -> 4417 us, 100 updates 1642 -> 1621 us; 2 * TPB here measures the same).
-constexpr int HUB_ACC = 4 * 256;
+// 4473 -> 4417 us, 100 updates 1571 -> 1563 us; 2 * TPB here measures the same).
+constexpr int HUB_ACC = 4 * TPB;
 constexpr int EVAL_CH = 1024;  // hub table slots evaluated per block (4096: one block a hub, 17 us where this takes 16)
 
 // ---------------------------------------------------------------- expand
@@ -398,28 +407,31 @@ __device__ inline void emit_cand(const SweepArgs<WT>& A, int32_t v, int32_t src,
 // 206 us and groups to 176 (2M-vertex power-law graph, batch of 10^5): one
 // multiply to hash, the target-independent terms of the gain collected, keys
 // read four at a time, no separate clearing, no argmax without a candidate.
+// Sweeps list[0..nl) as block blk of gridDim.x blocks of TPB threads.  A warp's
+// tables take the same GROUP_SMEM / (TPB / 32) bytes of smem for both G.
+template <class GT>
+constexpr int GROUP_SMEM = TPB / 32 * HG32 * tab_slot<GT>;
+static_assert(HG32 == 4 * HG8 && TPB / 32 * HG32 <= HB);
+
 template <class WT, int MODE, int G, class GT>
-__global__ void __launch_bounds__(TPB, wide_sums<GT> ? 4 : 6) k_sweep_group(SweepArgs<WT> A, const int32_t* list,
-                                                                             const int32_t* nlist) {
-  pdl_enter();
+__device__ inline void sweep_groups(const SweepArgs<WT>& A, const int32_t* list, uint32_t nl, unsigned char* smem,
+                                    uint32_t blk) {
   constexpr int HG = G == 8 ? HG8 : HG32;
   constexpr int GPW = 32 / G;  // groups per warp
   constexpr bool WIDE = wide_sums<GT>;
-  __shared__ __align__(16) int32_t hk[TPB / G][HG];
-  __shared__ __align__(16) uint32_t hv[WIDE ? 2 : 1][TPB / G][HG];
   const int lane = threadIdx.x & 31, gl = threadIdx.x & (G - 1);
-  const Tab<WIDE> T{hk[threadIdx.x / G], hv[0][threadIdx.x / G], WIDE ? hv[WIDE ? 1 : 0][threadIdx.x / G] : nullptr};
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t ngroups = ((int64_t)gridDim.x * blockDim.x) / G;
-  const int32_t nl = *nlist;
+  int32_t* const hk = (int32_t*)(smem + (size_t)(threadIdx.x / G) * HG * tab_slot<GT>);
+  const Tab<WIDE> T{hk, (uint32_t*)hk + HG, WIDE ? (uint32_t*)hk + 2 * HG : nullptr};
+  const uint32_t warp = blk * (TPB / 32) + threadIdx.x / 32;
+  const uint32_t ngroups = gridDim.x * (TPB / G);
   const int64_t mult = A.directed ? 1 : 2;
   uint32_t entries = 0, pairs = 0, nodes = 0;
   // the list is read one node ahead, off the chain of dependent loads
-  int64_t t = warp * GPW + lane / G;
+  uint32_t t = warp * GPW + lane / G;
   int32_t v_next = t < nl ? list[t] : 0;
   for (uint32_t k = 4 * gl; k < HG; k += 4 * G) T.clear4(k);
   __syncwarp();
-  for (int64_t base = warp * GPW; base < nl; base += ngroups, t += ngroups) {
+  for (uint32_t base = warp * GPW; base < nl; base += ngroups, t += ngroups) {
     const bool act = t < nl;
     const int32_t v = v_next;
     v_next = t + ngroups < nl ? list[t + ngroups] : 0;
@@ -460,6 +472,14 @@ __global__ void __launch_bounds__(TPB, wide_sums<GT> ? 4 : 6) k_sweep_group(Swee
   }
 }
 
+template <class WT, int MODE, int G, class GT>
+__global__ void __launch_bounds__(TPB, wide_sums<GT> ? 4 : 6) k_sweep_group(SweepArgs<WT> A, const int32_t* list,
+                                                                             const int32_t* nlist) {
+  pdl_enter();
+  __shared__ __align__(16) unsigned char smem[GROUP_SMEM<GT>];
+  sweep_groups<WT, MODE, G, GT>(A, list, *nlist, smem, blockIdx.x);
+}
+
 // one block per node; the hash lives in dynamic shared memory (mid degrees)
 // or in a global-memory slice (hubs, table != nullptr)
 // Entries of a node's rows staged in registers: entry k of the node is its
@@ -467,14 +487,21 @@ __global__ void __launch_bounds__(TPB, wide_sums<GT> ? 4 : 6) k_sweep_group(Swee
 // entries tid + j * NT.  First the neighbour ids and weights ...
 // Steps in which a warp has no entry are skipped by the whole warp: most rows
 // of a bin are far shorter than its longest.
+// Barrier of a block of NT threads, or of half `bar` of a block of 2 * NT.
+template <int NT>
+__device__ inline void sub_sync(int bar) {
+  if (NT == TPB) __syncthreads();
+  else asm volatile("bar.sync %0, %1;" ::"r"(bar + 1), "r"(NT) : "memory");
+}
+
 template <class WT, int NT, bool DIR, int ACC, class SW>
-__device__ inline void stage_rows(const SweepArgs<WT>& A, const NodeMeta& m, int32_t (&u)[ACC], SW (&w)[ACC]) {
-  const int32_t l = DIR ? m.lo + m.li : m.lo, w0 = (int32_t)threadIdx.x & ~31;
+__device__ inline void stage_rows(const SweepArgs<WT>& A, const NodeMeta& m, int tid, int32_t (&u)[ACC], SW (&w)[ACC]) {
+  const int32_t l = DIR ? m.lo + m.li : m.lo, w0 = tid & ~31;
 #pragma unroll
   for (int j = 0; j < ACC; ++j) {
     u[j] = -1;
     if (w0 + j * NT < l) {
-      const int32_t k = (int32_t)threadIdx.x + j * NT;
+      const int32_t k = tid + j * NT;
       const int64_t at = (!DIR || k < m.lo ? m.oo : m.oi - m.lo) + k;
       if (k < l) {
         u[j] = A.out.col[at];
@@ -485,16 +512,16 @@ __device__ inline void stage_rows(const SweepArgs<WT>& A, const NodeMeta& m, int
 }
 
 template <class WT, int NT, int ACC, class SW>
-__device__ inline void stage_rows(const SweepArgs<WT>& A, const NodeMeta& m, int32_t (&u)[ACC], SW (&w)[ACC]) {
-  if (A.directed) stage_rows<WT, NT, true>(A, m, u, w);
-  else stage_rows<WT, NT, false>(A, m, u, w);
+__device__ inline void stage_rows(const SweepArgs<WT>& A, const NodeMeta& m, int tid, int32_t (&u)[ACC], SW (&w)[ACC]) {
+  if (A.directed) stage_rows<WT, NT, true>(A, m, tid, u, w);
+  else stage_rows<WT, NT, false>(A, m, tid, u, w);
 }
 
 // ... then each id becomes its hash key (neighbour label, or for BestRef the
 // neighbour's refined community when it shares v's label; -1: skipped).
 template <class WT, int MODE, int NT, int ACC>
-__device__ inline void stage_keys(const SweepArgs<WT>& A, int32_t v, int32_t a, int32_t l, int32_t (&u)[ACC]) {
-  const int32_t w0 = (int32_t)threadIdx.x & ~31;
+__device__ inline void stage_keys(const SweepArgs<WT>& A, int32_t v, int32_t a, int32_t l, int tid, int32_t (&u)[ACC]) {
+  const int32_t w0 = tid & ~31;
 #pragma unroll
   for (int j = 0; j < ACC; ++j) {
     if (w0 + j * NT >= l) continue;  // the whole warp
@@ -519,33 +546,33 @@ __device__ inline void stage_keys(const SweepArgs<WT>& A, int32_t v, int32_t a, 
 // With the evaluation emptying the table, two barriers a node instead of
 // four: 263 -> 215 us for the rows of 97..1024 entries of a 10^5 batch on the
 // 2M-vertex power-law graph, 249 -> 214 us for 10^4 on the R-MAT of 2^20.
+// The caller may reuse smem right away: nothing reads it after the last barrier.
 template <class WT, int MODE, int NT, int HMAX, class GT>
-__global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, const int32_t* list,
-                                                               const int32_t* nlist) {
-  pdl_enter();
-  extern __shared__ unsigned char smem[];
+__device__ inline void sweep_blocks(const SweepArgs<WT>& A, const int32_t* list, uint32_t nl, unsigned char* smem,
+                                    int tid, int bar, uint32_t blk, uint32_t nblk) {
   constexpr bool WIDE = wide_sums<GT>;
-  __shared__ BestG<GT> wb[NT / 32];
-  __shared__ int64_t wown[NT / 32];
+  __shared__ BestG<GT> wb_[2][NT / 32];
+  __shared__ int64_t wown_[2][NT / 32];
+  BestG<GT>* const wb = wb_[bar];
+  int64_t* const wown = wown_[bar];
   constexpr int ACC = HMAX / (2 * NT);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = tid & 31, wid = tid >> 5;
   const Tab<WIDE> T{(int32_t*)smem, (uint32_t*)smem + HMAX, WIDE ? (uint32_t*)smem + 2 * HMAX : nullptr};
-  const int32_t nl = *nlist;
   const int64_t mult = A.directed ? 1 : 2;
   int64_t ent_all = 0, nodes = 0, pairs_all = 0;
   NodeMeta cur{}, nxt{};
   int32_t ek[ACC];
   StageW<GT> ew[ACC];
-  if (blockIdx.x < nl) {
-    cur = node_meta(A, list[blockIdx.x]);
-    stage_rows<WT, NT>(A, cur, ek, ew);
-    stage_keys<WT, MODE, NT>(A, cur.v, cur.a, cur.lo + cur.li, ek);
+  if (blk < nl) {
+    cur = node_meta(A, list[blk]);
+    stage_rows<WT, NT>(A, cur, tid, ek, ew);
+    stage_keys<WT, MODE, NT>(A, cur.v, cur.a, cur.lo + cur.li, tid, ek);
   }
-  if (blockIdx.x + gridDim.x < nl) nxt = node_meta(A, list[blockIdx.x + gridDim.x]);
-  if (blockIdx.x < nl)
-    for (uint32_t k = 4 * threadIdx.x; k < HMAX; k += 4 * NT) T.clear4(k);
-  __syncthreads();
-  for (int64_t t = blockIdx.x; t < nl; t += gridDim.x) {
+  if (blk + nblk < nl) nxt = node_meta(A, list[blk + nblk]);
+  if (blk < nl)
+    for (uint32_t k = 4 * tid; k < HMAX; k += 4 * NT) T.clear4(k);
+  sub_sync<NT>(bar);
+  for (uint32_t t = blk; t < nl; t += nblk) {
     const int32_t v = cur.v;
     const int64_t d = (int64_t)cur.lo + cur.li;
     uint32_t H = 256;
@@ -554,16 +581,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, 
     StageW<GT> own = 0;
 #pragma unroll
     for (int j = 0; j < ACC; ++j) {
-      if ((int)(threadIdx.x & ~31u) + j * NT >= d) continue;  // the whole warp
+      if ((tid & ~31) + j * NT >= d) continue;  // the whole warp
       if (MODE == 0 && ek[j] == a) own += ew[j];
       else if (ek[j] >= 0) T.add(H - 1, ek[j], ew[j]);
     }
     if (d > ACC * NT) {  // entries beyond the staged ones
-      for (int64_t k = ACC * NT + threadIdx.x; k < d; k += NT) {
+      for (int64_t k = ACC * NT + tid; k < d; k += NT) {
         const int64_t at = (k < cur.lo ? cur.oo : cur.oi - cur.lo) + k;
         const int64_t wx = (int64_t)A.out.w[at];
         int32_t kx[1] = {A.out.col[at]};
-        stage_keys<WT, MODE, 0>(A, v, a, INT32_MAX, kx);
+        stage_keys<WT, MODE, 0>(A, v, a, INT32_MAX, tid, kx);
         if (MODE == 0 && kx[0] == a) own += (StageW<GT>)wx;
         else if (kx[0] >= 0) T.add(H - 1, kx[0], wx);
       }
@@ -573,9 +600,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, 
       else own = __reduce_add_sync(0xffffffffu, own);
       if (lane == 0) wown[wid] = own;
     }
-    __syncthreads();
-    const bool has_next = t + gridDim.x < nl;
-    if (has_next) stage_rows<WT, NT>(A, nxt, ek, ew);  // in flight during the evaluation
+    sub_sync<NT>(bar);
+    const bool has_next = t + nblk < nl;
+    if (has_next) stage_rows<WT, NT>(A, nxt, tid, ek, ew);  // in flight during the evaluation
     int64_t wa = 0;
     if (MODE == 0) {
 #pragma unroll
@@ -584,17 +611,17 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, 
     const int64_t ko = cur.ko, ki = cur.ki;
     BestG<GT> b{0, 0, 0};
     int64_t pairs = 0;
-    eval_slots<MODE, GT>(T, H, threadIdx.x, NT, MODE == 0 ? a : v, a, wa, ko, ki, A.directed, A.Tout, A.Tin, A.m, A.gn, A.gd,
+    eval_slots<MODE, GT>(T, H, (uint32_t)tid, (uint32_t)NT, MODE == 0 ? a : v, a, wa, ko, ki, A.directed, A.Tout, A.Tin, A.m, A.gn, A.gd,
                          mult, b, pairs);
-    if (has_next) stage_keys<WT, MODE, NT>(A, nxt.v, nxt.a, nxt.lo + nxt.li, ek);  // label gathers overlap the argmax
+    if (has_next) stage_keys<WT, MODE, NT>(A, nxt.v, nxt.a, nxt.lo + nxt.li, tid, ek);  // label gathers overlap the argmax
     if (__any_sync(0xffffffffu, b.have)) b = seg_best<GT, 32>(b);
     if (lane == 0) wb[wid] = b;
     pairs_all += pairs;
     // two barriers a node: this one also separates the evaluation (which
     // empties the table) from the next node's inserts, and the next node's
     // barrier separates thread 0's reads of wb from their next writes
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    sub_sync<NT>(bar);
+    if (tid == 0) {
       BestG<GT> r = wb[0];
       for (int w = 1; w < NT / 32; ++w)
         if (better(wb[w], r)) r = wb[w];
@@ -603,15 +630,55 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, 
       ++nodes;
     }
     cur = nxt;
-    if (t + 2 * (int64_t)gridDim.x < nl) nxt = node_meta(A, list[t + 2 * (int64_t)gridDim.x]);
+    if (t + 2 * nblk < nl) nxt = node_meta(A, list[t + 2 * nblk]);
   }
   // statistics once per block
   const int64_t bytes = warp_sum_i64(sweep_bytes<WT, MODE>(A.directed, ent_all, nodes, pairs_all));
   if (lane == 0 && bytes) atomic_add_i64(&A.stats->sw_bytes[NT == 128 ? 2 : 3], bytes);
-  if (threadIdx.x == 0 && ent_all) {
+  if (tid == 0 && ent_all) {
     atomic_add_i64(A.scanned, ent_all);
     atomic_add_i64(&A.stats->sw_entries[NT == 128 ? 2 : 3], ent_all);
   }
+}
+
+template <class WT, int MODE, int NT, int HMAX, class GT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_sweep_block(SweepArgs<WT> A, const int32_t* list,
+                                                               const int32_t* nlist) {
+  pdl_enter();
+  extern __shared__ __align__(16) unsigned char smem[];
+  sweep_blocks<WT, MODE, NT, HMAX, GT>(A, list, *nlist, smem, threadIdx.x, 0, blockIdx.x, gridDim.x);
+}
+
+// The four bins in one launch (see SWEEP_FUSE), each going on at the block
+// where the one before it ended, the longest nodes first; the two halves of a
+// block sweep the nodes of the lower mid bin on their own (as nodes of whole
+// blocks they cost the 2M-vertex power-law graph 10%).  Bound by the longest
+// chain of dependent loads of any block.
+template <class WT, int MODE, class GT>
+__global__ void __launch_bounds__(TPB, 4) k_sweep_bins(SweepArgs<WT> A, const int32_t* bt, const int32_t* nt,
+                                                       const int32_t* bs, const int32_t* ns, const int32_t* bm,
+                                                       const int32_t* nm, const int32_t* bm2, const int32_t* nm2) {
+  pdl_enter();
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int HALF = TPB / 2;
+  const int half = threadIdx.x / HALF;
+  uint32_t blk = blockIdx.x;
+  int32_t n = *nm2;
+  sweep_blocks<WT, MODE, TPB, HB, GT>(A, bm2, n, smem, threadIdx.x, 0, blk, gridDim.x);
+  // the next bin starts at the block after this one's last node
+  const auto turn = [&](uint32_t used) { blk = (blk + gridDim.x - used % gridDim.x) % gridDim.x; };
+  turn(n);
+  n = *nm;
+  sweep_blocks<WT, MODE, HALF, HB / 2, GT>(A, bm, n, smem + (size_t)half * (HB / 2) * tab_slot<GT>,
+                                           threadIdx.x % HALF, half, 2 * blk + half, 2 * gridDim.x);
+  // a warp's tables lie in its half's part of smem, which the other half may still be using
+  unsigned char* const sw = smem + (size_t)half * (HB / 2 * tab_slot<GT> - GROUP_SMEM<GT> / 2);
+  turn((uint32_t)(n + 1) / 2);
+  n = *ns;
+  sweep_groups<WT, MODE, 32, GT>(A, bs, n, sw, blk);
+  turn((uint32_t)(n + TPB / 32 - 1) / (TPB / 32));
+  __syncwarp();
+  sweep_groups<WT, MODE, 8, GT>(A, bt, *nt, sw, blk);
 }
 
 template <class WT>
@@ -1504,20 +1571,27 @@ static bool sweep_gain_fits_i64(const ldl_ctx& c) {
 
 // The bins of nodes with at most 2048 entries, in the gain type GT.
 template <class WT, int MODE, class GT>
-static void sweep_bins(ldl_ctx& c, const SweepArgs<WT>& A, int64_t n_hint, bool few, cudaEvent_t* kev) {
-  if (!few) {
-  launch(k_sweep_group<WT, MODE, 8, GT>, grid_for(n_hint * 8, TPB, 6), TPB, 0, c.s, A, c.binT.p, c.cp[K_TINY]);
-  CKL("k_sweep_group<8>");
-  if (kev) CK(cudaEventRecord(kev[1], c.s));
-  launch(k_sweep_group<WT, MODE, 32, GT>, grid_for(n_hint * 32, TPB, 6), TPB, 0, c.s, A, c.binS.p, c.cp[K_SMALL]);
-  CKL("k_sweep_group<32>");
-  if (kev) CK(cudaEventRecord(kev[2], c.s));
-  {
-    const size_t sm = (size_t)tab_slot<GT> * 2048;
-    launch(k_sweep_block<WT, MODE, 128, 2048, GT>, grid_for(n_hint, 1, 16), 128, sm, c.s, A, c.binM.p, c.cp[K_MID]);
-    CKL("k_sweep_block(mid1)");
+static void sweep_bins(ldl_ctx& c, const SweepArgs<WT>& A, int64_t n_hint, bool few, bool fused, cudaEvent_t* kev) {
+  if (fused) {
+    const size_t sm = (size_t)tab_slot<GT> * HB;
+    CK(cudaFuncSetAttribute(k_sweep_bins<WT, MODE, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    launch(k_sweep_bins<WT, MODE, GT>, grid_for(n_hint, 1, 4), TPB, sm, c.s, A, c.binT.p, c.cp[K_TINY], c.binS.p,
+           c.cp[K_SMALL], c.binM.p, c.cp[K_MID], c.binM2.p, c.cp[K_MID2]);
+    CKL("k_sweep_bins");
+    return;
   }
-  if (kev) CK(cudaEventRecord(kev[3], c.s));
+  if (!few) {
+    launch(k_sweep_group<WT, MODE, 8, GT>, grid_for(n_hint * 8, TPB, 6), TPB, 0, c.s, A, c.binT.p, c.cp[K_TINY]);
+    CKL("k_sweep_group<8>");
+    if (kev) CK(cudaEventRecord(kev[1], c.s));
+    launch(k_sweep_group<WT, MODE, 32, GT>, grid_for(n_hint * 32, TPB, 6), TPB, 0, c.s, A, c.binS.p, c.cp[K_SMALL]);
+    CKL("k_sweep_group<32>");
+    if (kev) CK(cudaEventRecord(kev[2], c.s));
+    const size_t sm = (size_t)tab_slot<GT> * (HB / 2);
+    launch(k_sweep_block<WT, MODE, TPB / 2, HB / 2, GT>, grid_for(n_hint, 1, 16), TPB / 2, sm, c.s, A, c.binM.p,
+           c.cp[K_MID]);
+    CKL("k_sweep_block(mid1)");
+    if (kev) CK(cudaEventRecord(kev[3], c.s));
   }
   {
     const size_t sm = (size_t)tab_slot<GT> * HB;
@@ -1588,6 +1662,7 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   // Few nodes are all swept by one block each, whatever their degree: a launch
   // per degree bin costs more than it saves (see SWEEP_FEW).
   const bool few = n_hint <= SWEEP_FEW && !c.kstats;
+  const bool fused = !few && n_hint <= SWEEP_FUSE && !c.kstats;
   // The split is only launched ahead behind such short sweeps: they mostly end
   // the level's moves, and where moves are accepted its two launches are lost
   // (one edge on 10k vertices 508 -> 486 us a batch; with it behind every sweep,
@@ -1608,8 +1683,8 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   // and the host's wait below overlaps them.  n_hint bounds every bin.
   cudaEvent_t* kev = c.kstats ? kstats_events(c) : nullptr;
   if (kev) CK(cudaEventRecord(kev[0], c.s));
-  if (sweep_gain_fits_i64(c)) sweep_bins<WT, MODE, int64_t>(c, A, n_hint, few, kev);
-  else sweep_bins<WT, MODE, i128>(c, A, n_hint, few, kev);
+  if (sweep_gain_fits_i64(c)) sweep_bins<WT, MODE, int64_t>(c, A, n_hint, few, fused, kev);
+  else sweep_bins<WT, MODE, i128>(c, A, n_hint, few, fused, kev);
   if (kev) CK(cudaEventRecord(kev[4], c.s));
   if (c.prm.cluster_max_deg > c.bin_deg[3]) {
     const size_t sm = (sizeof(int64_t) + sizeof(int32_t)) * CL_SLOTS;

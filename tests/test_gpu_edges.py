@@ -28,10 +28,10 @@ BIN_EDGES = (1, 7, 8, 9, 23, 24, 25, 31, 32, 33, 95, 96, 97, 127, 128, 129, 511,
              4100)
 
 
-def _bin_edge_graph(directed, weight, seed):
+def _bin_edge_graph(directed, weight, seed, n=6000):
     """Small cliques joined at random, and one node per degree of BIN_EDGES."""
     rng = np.random.default_rng(seed)
-    n, k = 6000, 12
+    k = 12
     v = np.arange(200, n)
     src = [np.repeat(v, 5)]
     dst = [(v // k * k)[:, None].repeat(5, 1).ravel() + rng.integers(0, k, 5 * len(v))]
@@ -49,6 +49,18 @@ def _bin_edge_graph(directed, weight, seed):
         src, dst = np.minimum(src, dst), np.maximum(src, dst)
     key = np.unique(src * n + dst)
     return csr_from_arcs(n, key // n, key % n, weight(rng, len(key)), directed)
+
+
+def _ring(n, directed):
+    """Every node beside its next neighbours, some rows of a few hundred."""
+    rng = np.random.default_rng(n)
+    v = np.arange(n)
+    src = np.concatenate([np.repeat(v, 4), np.repeat(v[:8], 300)])
+    dst = np.concatenate([(v[:, None] + np.arange(1, 5)).ravel() % n, rng.integers(8, n, 2400)])
+    if not directed:
+        src, dst = np.minimum(src, dst), np.maximum(src, dst)
+    key = np.unique(src * n + dst)
+    return csr_from_arcs(n, key // n, key % n, np.ones(len(key), np.int64), directed)
 
 
 def _unit(rng, k):
@@ -86,6 +98,22 @@ def test_sweep_bins(ldl, directed, weight):
         d.apply(b)
         msgs = compare_states(o, d, f"batch {t}")
         assert not msgs, "\n".join(msgs[:8])
+
+
+# sweeps of few nodes (one block each), of up to 131072 (one launch for all
+# bins) and of more (a launch per bin)
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("n", [1024, 1025, 131072, 131073])
+def test_sweep_sizes(ldl, directed, n):
+    g = _bin_edge_graph(directed, _unit, 7, n) if n > 4400 else _ring(n, directed)
+    o, d = Oracle(g), ldl.LDL.from_graph(g)
+    msgs = compare_states(o, d, "create")
+    assert not msgs, "\n".join(msgs[:8])
+    b = random_batch(EdgeStream.from_graph(g, 3), 60, 40, 20, 2, 5)
+    assert o.apply(b) == 0
+    d.apply(b)
+    msgs = compare_states(o, d, "batch")
+    assert not msgs, "\n".join(msgs[:8])
 
 
 def _dense_batch(g, size, seed):
