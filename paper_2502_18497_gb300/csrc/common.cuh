@@ -44,6 +44,8 @@ __device__ __forceinline__ void pdl_enter() {
 // between two short kernels was about 2 us: one edge on 10k vertices took 511
 // us a batch (70 launches), now 400; a batch of 10^4 on the R-MAT of 2^20
 // (267 launches) 4.79 ms, now 4.31.
+// Does not throw (the C entry points that must not are among its callers): an
+// error stays the thread's last one for the cudaGetLastError behind each launch.
 template <class... P, class... A>
 inline void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchConfig_t cfg{};
@@ -56,7 +58,7 @@ inline void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t s
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  CK(cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...));
+  (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
 // ---------------------------------------------------------------- device memory
