@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 from oracle import Oracle
-from synth import EdgeStream, csr_from_arcs, random_batch
+from synth import EdgeStream, csr_from_arcs, random_batch, rmat_directed, rmat_stream
 from tests.parity import compare_states
 
 pytestmark = pytest.mark.gpu
@@ -162,3 +162,20 @@ def test_batch_sizes(ldl, directed, size):
         d.apply(x)
         msgs = compare_states(o, d, f"batch {t}")
         assert not msgs, "\n".join(msgs[:8])
+
+
+# changed vertices up to 4096 come through the mapped page, more by copies
+@pytest.mark.parametrize("size,few", [(40, True), (60_000, False)])
+def test_changed_labels(ldl, size, few):
+    g = rmat_directed(scale=14, arcs=1 << 18, seed=5)
+    o, d = Oracle(g), ldl.LDL.from_graph(g)
+    before = np.array(o.labels())
+    for b in rmat_stream(g, batches=1, size=size, seed=size):
+        assert o.apply(b) == 0
+        d.apply(b)
+    want = np.flatnonzero(np.array(o.labels()) != before)
+    assert 0 < len(want) and (len(want) <= 4096) == few
+    for ids, lab in (d.changed(), d.changed_noalloc(), d.changed()):
+        order = np.argsort(ids)
+        assert np.array_equal(ids[order], want)
+        assert np.array_equal(lab[order], np.array(o.labels())[want])
