@@ -254,23 +254,6 @@ __device__ inline Best warp_best(Best x) {
   return x;
 }
 
-// The same argmax over each segment of G lanes (every lane of the warp takes
-// part; the result lands in every lane of the segment).
-template <int G>
-__device__ inline Best group_best(Best x) {
-  for (int d = G / 2; d > 0; d >>= 1) {
-    Best o;
-    o.g = shfl_down_i128_w(x.g, d, G);
-    o.c = __shfl_down_sync(0xffffffffu, x.c, d, G);
-    o.have = __shfl_down_sync(0xffffffffu, x.have, d, G);
-    if (best_better(o, x)) x = o;
-  }
-  x.g = shfl_i128_w(x.g, 0, G);
-  x.c = __shfl_sync(0xffffffffu, x.c, 0, G);
-  x.have = __shfl_sync(0xffffffffu, x.have, 0, G);
-  return x;
-}
-
 __device__ inline uint32_t hash32(uint32_t x) {
   x ^= x >> 16;
   x *= 0x7feb352dU;

@@ -130,7 +130,7 @@ struct ldl_ctx {
   DBuf<int64_t> hown;    // per hub: weight towards its own community
   // records
   DBuf<u64> rk, rv, tk, tv, rk2, rv2;
-  DBuf<int64_t> rsum, rsum2;
+  DBuf<int64_t> rsum;
   DBuf<u64> crk, crv, trk, trv;
   DBuf<u64> flk;      // a pending list's summed records (keys) ...
   DBuf<int64_t> flv;  // ... and their weight changes

@@ -319,7 +319,7 @@ void free_all(ldl_ctx& c) {
   if (c.s) cudaStreamSynchronize(c.s);
   for (auto& L : c.lv) L.release();
   DBuf<int64_t>* b64[] = {&c.Kout, &c.Kin, &c.e, &c.cghi, &c.snapKo, &c.snapKi, &c.snapE, &c.binLoff, &c.binLsz,
-                          &c.gvals, &c.rsum, &c.rsum2, 
+                          &c.gvals, &c.rsum,
                           &c.chunk_pre, &c.hub_epre, &c.pb_hi};
   for (auto* b : b64) b->release();
   DBuf<int32_t>* b32[] = {&c.stS, &c.stU, &c.stMv, &c.stB, &c.stM0, &c.stD, &c.stC, &c.stR, &c.stX, &c.stT,
@@ -506,7 +506,6 @@ static void release_build_scratch(ldl_ctx& c) {
   DBuf<u64>* bu[] = {&c.rk, &c.rv, &c.tk, &c.tv, &c.rk2, &c.rv2, &c.crk, &c.crv, &c.trk, &c.trv};
   for (auto* b : bu) b->release();
   c.rsum.release();
-  c.rsum2.release();
   c.gkeys.release();
   c.gvals.release();
   c.glist.release();

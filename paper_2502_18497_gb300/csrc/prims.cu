@@ -359,8 +359,9 @@ __global__ void __launch_bounds__(RS_THREADS, 4) k_rs_scatter(const u64* keys, c
 // goes through shared memory in digit order to its global places.  A grid
 // barrier after each.  Bound by the barriers and the passes' latency: 82 us for
 // six passes over some 10^5 pairs (2M-vertex power-law graph), 113 with four
-// small blocks per SM, a second load and a scan block per digit.  A transposing sort ping-pongs between the place
-// behind its input and (tk, tv) such that the last pass ends there.
+// small blocks per SM, a second load and a scan block per digit.  A transposing
+// sort ping-pongs between the place behind its input and (tk, tv) such that the
+// last pass ends there.
 constexpr int CO_THREADS = 512;
 constexpr int CO_ITEMS = 16;
 constexpr int CO_TILE = CO_THREADS * CO_ITEMS;

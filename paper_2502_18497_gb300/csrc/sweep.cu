@@ -454,8 +454,8 @@ __device__ inline void sweep_groups(const SweepArgs<WT>& A, const int32_t* list,
       for (int d = G / 2; d > 0; d >>= 1) wa += __shfl_xor_sync(0xffffffffu, wa, d, G);
     }
     if (act)
-      eval_slots<MODE, GT>(T, (uint32_t)H, (uint32_t)gl, (uint32_t)G, MODE == 0 ? a : v, a, (int64_t)wa, cur.ko, cur.ki, A.directed,
-                           A.Tout, A.Tin, A.m, A.gn, A.gd, mult, b, pairs);
+      eval_slots<MODE, GT>(T, (uint32_t)H, (uint32_t)gl, (uint32_t)G, MODE == 0 ? a : v, a, (int64_t)wa, cur.ko,
+                           cur.ki, A.directed, A.Tout, A.Tin, A.m, A.gn, A.gd, mult, b, pairs);
     // most nodes stay where they are: no argmax without a positive gain
     if (__any_sync(0xffffffffu, b.have)) {
       b = seg_best<GT, G>(b);
@@ -480,8 +480,6 @@ __global__ void __launch_bounds__(TPB, wide_sums<GT> ? 4 : 6) k_sweep_group(Swee
   sweep_groups<WT, MODE, G, GT>(A, list, *nlist, smem, blockIdx.x);
 }
 
-// one block per node; the hash lives in dynamic shared memory (mid degrees)
-// or in a global-memory slice (hubs, table != nullptr)
 // Entries of a node's rows staged in registers: entry k of the node is its
 // out-row entry k (k < lo) or its in-row entry k - lo; thread tid holds the
 // entries tid + j * NT.  First the neighbour ids and weights ...
@@ -611,8 +609,8 @@ __device__ inline void sweep_blocks(const SweepArgs<WT>& A, const int32_t* list,
     const int64_t ko = cur.ko, ki = cur.ki;
     BestG<GT> b{0, 0, 0};
     int64_t pairs = 0;
-    eval_slots<MODE, GT>(T, H, (uint32_t)tid, (uint32_t)NT, MODE == 0 ? a : v, a, wa, ko, ki, A.directed, A.Tout, A.Tin, A.m, A.gn, A.gd,
-                         mult, b, pairs);
+    eval_slots<MODE, GT>(T, H, (uint32_t)tid, (uint32_t)NT, MODE == 0 ? a : v, a, wa, ko, ki, A.directed,
+                         A.Tout, A.Tin, A.m, A.gn, A.gd, mult, b, pairs);
     if (has_next) stage_keys<WT, MODE, NT>(A, nxt.v, nxt.a, nxt.lo + nxt.li, tid, ek);  // label gathers overlap the argmax
     if (__any_sync(0xffffffffu, b.have)) b = seg_best<GT, 32>(b);
     if (lane == 0) wb[wid] = b;
@@ -711,7 +709,8 @@ __global__ void k_bin(Adj<WT> out, Adj<WT> in, int directed, const int32_t* list
 #pragma unroll
     for (int j = 0; j < BI; ++j) {
       d[j] = v[j] >= 0 ? (int64_t)out.len[v[j]] + (directed ? in.len[v[j]] : 0) : 0;
-      bin[j] = v[j] < 0 ? -1 : d[j] <= t0_ ? 0 : d[j] <= t1 ? 1 : d[j] <= t2 ? 2 : d[j] <= t3 ? 3 : d[j] <= cluster_max ? 4 : 5;
+      bin[j] = v[j] < 0 ? -1 : d[j] <= t0_ ? 0 : d[j] <= t1 ? 1 : d[j] <= t2 ? 2 : d[j] <= t3 ? 3
+               : d[j] <= cluster_max ? 4 : 5;
     }
     __syncthreads();
 #pragma unroll
@@ -1675,7 +1674,8 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
                                                      c.cp[K_MID2], c.binC.p, c.cp[K_CLU], c.binL.p, c.cp[K_LARGE],
                                                      c.binLsz.p, c.sums, few ? -1 : c.bin_deg[0],
                                                      few ? -1 : c.bin_deg[1], few ? -1 : c.bin_deg[2],
-                                                     few ? MID_DEG : c.bin_deg[3], std::min(c.prm.cluster_max_deg, CLUSTER_DEG),
+                                                     few ? MID_DEG : c.bin_deg[3],
+                                                     std::min(c.prm.cluster_max_deg, CLUSTER_DEG),
                                                      early ? tail_begin(c, rb, 8) : Tail{});
   CKL("k_bin");
   // Every bin but the hubs is swept by a grid-stride kernel that reads its
