@@ -164,7 +164,7 @@ struct ldl_ctx {
   // (scan.cuh), and the number of the last read
   volatile u64* h_pub = nullptr;
   u64* d_pub = nullptr;
-  uint32_t pub_seq = 0;
+  uint32_t pub_seq = 0, chg_seq = 0;
   std::string err;
   bool broken = false;  // a failed rollback left the state unknown
 

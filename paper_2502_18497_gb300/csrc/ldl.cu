@@ -81,7 +81,10 @@ DeviceScope::~DeviceScope() {
 }
 
 namespace {
-constexpr int PAGE_WORDS = 8192;  // payload words per read
+constexpr int PAGE_WORDS = 512;  // payload words per read
+// Behind them the words of ldl_copy_changed, with a sequence of their own: a
+// caller may ask for the labels while a server's worker reads on the context.
+constexpr int CHG_WORDS = 8192;
 
 // hands values of earlier kernels to the host (one block)
 __global__ void k_publish(Tail t) { pdl_enter(); put_tail(t); }
@@ -147,17 +150,16 @@ __global__ void __launch_bounds__(256) k_snapshot(SnapList l, unsigned char* dst
 // Waits for n payload words of the read under way.  Every so often it asks the
 // stream: an error ends the wait with that error; an idle stream whose write is
 // still not seen falls back to a full synchronisation before failing.
-static void wait_words(ldl_ctx& c, int n) {
-  const uint32_t seq = c.pub_seq;
+static void wait_words(ldl_ctx& c, const volatile u64* page, uint32_t seq, int n) {
   uint64_t spins = 0;
   for (int w = 0; w < n; ++w)
-    while ((uint32_t)(c.h_pub[w] >> 32) != seq) {
+    while ((uint32_t)(page[w] >> 32) != seq) {
       if ((++spins & 4095) != 0) continue;
       const cudaError_t e = cudaStreamQuery(c.s);
       if (e == cudaErrorNotReady) continue;
       CK(e);
       CK(cudaStreamSynchronize(c.s));
-      if ((uint32_t)(c.h_pub[w] >> 32) != seq) ldl_throw(LDL_E_CUDA, "internal: a published value never reached the host");
+      if ((uint32_t)(page[w] >> 32) != seq) ldl_throw(LDL_E_CUDA, "internal: a published value never reached the host");
     }
   std::atomic_thread_fence(std::memory_order_acquire);
 }
@@ -195,13 +197,13 @@ void* fresh(ldl_ctx& c, int words, void* home) {
   return home;
 }
 
-// The sequence number of the next read through the page.
-static uint32_t next_read(ldl_ctx& c) {
-  if (++c.pub_seq == 0) {  // all numbers used: no word of the page may match a new one
-    for (int w = 0; w < PAGE_WORDS; ++w) c.h_pub[w] = 0;
-    c.pub_seq = 1;  // 0 marks a tail without a read
+// The sequence number of the next read through a page of n words.
+static uint32_t next_read(uint32_t& seq, volatile u64* page, int n) {
+  if (++seq == 0) {  // all numbers used: no word of the page may match a new one
+    for (int w = 0; w < n; ++w) page[w] = 0;
+    seq = 1;  // 0 marks a tail without a read
   }
-  return c.pub_seq;
+  return seq;
 }
 
 Tail tail_begin(ldl_ctx& c, const HostRead* r, int n) {
@@ -220,14 +222,14 @@ Tail tail_begin(ldl_ctx& c, const HostRead* r, int n) {
   t.ticket = c.cp[K_TICKET];
   ++c.syncs;
   t.page = c.d_pub;
-  t.seq = next_read(c);
+  t.seq = next_read(c.pub_seq, c.h_pub, PAGE_WORDS);
   return t;
 }
 
 void tail_wait(ldl_ctx& c, const HostRead* r, int n) {
   int words = 0;
   for (int i = 0; i < n; ++i) words += r[i].bytes / 4;
-  wait_words(c, words);
+  wait_words(c, c.h_pub, c.pub_seq, words);
   int at = 0;
   for (int i = 0; i < n; ++i)
     for (int w = 0; w < r[i].bytes / 4; ++w) {
@@ -832,8 +834,8 @@ ldl_status ctx_new(const ldl_params& p, int64_t n, ldl_ctx** out) {
     c->s = (cudaStream_t)p.cuda_stream;
     {
       void* hp = nullptr;
-      CK(cudaHostAlloc(&hp, sizeof(u64) * PAGE_WORDS, cudaHostAllocMapped));
-      memset(hp, 0, sizeof(u64) * PAGE_WORDS);
+      CK(cudaHostAlloc(&hp, sizeof(u64) * (PAGE_WORDS + CHG_WORDS), cudaHostAllocMapped));
+      memset(hp, 0, sizeof(u64) * (PAGE_WORDS + CHG_WORDS));
       c->h_pub = (volatile u64*)hp;
       void* dp = nullptr;
       CK(cudaHostGetDevicePointer(&dp, hp, 0));
@@ -1261,15 +1263,17 @@ ldl_status ldl_copy_changed(const ldl_ctx* cc, int32_t* ids, int32_t* labels) {
   if (!ids) return LDL_E_INVALID;
   try {
     DeviceScope ds(c.dev);
-    if (2 * k <= PAGE_WORDS) {
+    if (2 * k <= CHG_WORDS) {
       const int32_t n = (int32_t)k;
-      const uint32_t seq = next_read(c);
-      launch(k_put_labels, grid_for(n, 256), 256, 0, c.s, c.lChg.p, n, labels ? c.lv[0].lab.p : nullptr, c.d_pub, seq);
+      volatile u64* const page = c.h_pub + PAGE_WORDS;
+      const uint32_t seq = next_read(c.chg_seq, page, CHG_WORDS);
+      launch(k_put_labels, grid_for(n, 256), 256, 0, c.s, c.lChg.p, n, labels ? c.lv[0].lab.p : nullptr,
+             c.d_pub + PAGE_WORDS, seq);
       CKL("k_put_labels");
-      wait_words(c, labels ? 2 * n : n);
-      for (int32_t i = 0; i < n; ++i) ids[i] = (int32_t)(uint32_t)c.h_pub[i];
+      wait_words(c, page, seq, labels ? 2 * n : n);
+      for (int32_t i = 0; i < n; ++i) ids[i] = (int32_t)(uint32_t)page[i];
       if (labels)
-        for (int32_t i = 0; i < n; ++i) labels[i] = (int32_t)(uint32_t)c.h_pub[n + i];
+        for (int32_t i = 0; i < n; ++i) labels[i] = (int32_t)(uint32_t)page[n + i];
       return LDL_OK;
     }
     CK(cudaMemcpyAsync(ids, c.lChg.p, sizeof(int32_t) * (size_t)k, cudaMemcpyDeviceToHost, c.s));
