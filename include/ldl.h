@@ -376,8 +376,11 @@ int64_t ldl_launch_count(void);
  * lengths, label and strengths; per evaluated (node, target) pair the
  * target's totals.  Collection adds no host synchronisation: events and
  * device counters are resolved by ldl_get_kernel_stats, which waits for the
- * context's stream.  Both return LDL_E_INVALID on a null pointer and
- * LDL_E_CUDA on a CUDA error.
+ * context's stream.  Since the groups are timed one by one, every sweep has a
+ * launch per group while statistics are collected; without them short lists
+ * share one (see ldl_params.bin_deg), so such a batch takes fewer launches.
+ * Entries and bytes are counted with statistics off too.  Both return
+ * LDL_E_INVALID on a null pointer and LDL_E_CUDA on a CUDA error.
  */
 ldl_status ldl_set_kernel_stats(ldl_ctx* ctx, int32_t on);
 ldl_status ldl_get_kernel_stats(const ldl_ctx* ctx, double* out);

@@ -400,7 +400,7 @@ struct SlackCSR {
 // accumulation kernel, 6 the rest of the hub path (table set-up, evaluation,
 // final reduction).  A sweep records KS_EVENTS events; interval j (event j to
 // j + 1) is charged to group ks_interval_group(j), or to none (-1: the host's
-// wait for the bin counts).
+// wait for the bin counts and what is launched in front of it).
 constexpr int KS_GROUPS = 7;
 constexpr int KS_EVENTS = 10;
 __host__ __device__ constexpr int ks_interval_group(int j) { return j < 5 ? j : j == 5 ? -1 : j == 7 ? 5 : 6; }

@@ -47,7 +47,9 @@ struct LevelState {
 // Device counters (indices into ldl_ctx::cp).
 enum {
   K_U = 0, K_S, K_USTAR, K_MV, K_M0, K_D, K_C, K_R, K_R2, K_X, K_T, K_CH, K_CAND, K_B,
-  K_UNDEC, K_SMALL, K_MID, K_LARGE, K_REC, K_CREC, K_ERR, K_TMP, K_TMP2, K_CHG, K_MID2, K_TINY, K_CLU,
+  K_UNDEC,
+  K_LARGE, K_TINY, K_SMALL, K_MID, K_MID2, K_CLU,  // a sweep's bins, read together (hub rows first)
+  K_REC, K_CREC, K_ERR, K_TMP, K_TMP2, K_CHG,
   K_G,
   K_HUBG,      // hubs of the current hub group
   K_A0 = 32,   // K_A0 + r: |A^r|
@@ -60,6 +62,7 @@ enum {
   K_COUNT = 64
 };
 constexpr int ARENA_WORDS = 8192;
+constexpr int N_BINS = K_CLU - K_LARGE + 1;
 
 // Exact changes of a mini-batch: the Eq. 1 numerator, sum_C K_out K_in, sum_C e_C.
 struct CommitAcc {
@@ -213,6 +216,8 @@ inline int64_t* Kin_of(ldl_ctx& c) { return c.directed ? c.Kin.p : c.Kout.p; }
 void host_read(ldl_ctx& c, const HostRead* r, int n);
 int32_t rd_cnt(ldl_ctx& c, int idx);
 void zero_cnt(ldl_ctx& c, int idx);
+// Counters first .. first + n - 1, next to one another afterwards.
+void zero_cnts(ldl_ctx& c, int first, int n);
 // `words` zeroed words, 16-byte aligned: from the arena, else `home` cleared.
 void* fresh(ldl_ctx& c, int words, void* home);
 // A read that a kernel's last block performs (scan.cuh): begin before the

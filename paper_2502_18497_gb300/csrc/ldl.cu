@@ -178,14 +178,15 @@ int32_t rd_cnt(ldl_ctx& c, int idx) {
   return v;
 }
 
-void zero_cnt(ldl_ctx& c, int idx) {
-  if (c.arena_top < ARENA_WORDS) {
-    c.cp[idx] = c.arena + c.arena_top++;
-    return;
-  }
-  c.cp[idx] = c.dcnt + idx;
-  CK(cudaMemsetAsync(c.cp[idx], 0, sizeof(int32_t), c.s));
+void zero_cnts(ldl_ctx& c, int first, int n) {
+  const bool fits = c.arena_top + n <= ARENA_WORDS;
+  int32_t* const at = fits ? c.arena + c.arena_top : c.dcnt + first;
+  for (int k = 0; k < n; ++k) c.cp[first + k] = at + k;
+  if (fits) c.arena_top += n;
+  else CK(cudaMemsetAsync(at, 0, sizeof(int32_t) * (size_t)n, c.s));
 }
+
+void zero_cnt(ldl_ctx& c, int idx) { zero_cnts(c, idx, 1); }
 
 void* fresh(ldl_ctx& c, int words, void* home) {
   const int at = (c.arena_top + 3) & ~3;

@@ -1616,7 +1616,8 @@ template <class WT, int MODE>
 static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_t* list, int idx_n,
                         int64_t n_hint, SplitRun* spec) {
   if (MODE == 0) stage_begin(c);  // refinement is timed as a whole
-  for (int k : {K_CAND, K_TINY, K_SMALL, K_MID, K_MID2, K_CLU, K_LARGE}) zero_cnt(c, k);
+  zero_cnt(c, K_CAND);
+  zero_cnts(c, K_LARGE, N_BINS);
   c.sums = (int64_t*)fresh(c, 2, c.d_sc->sums);
   LevelState& L = c.lv[r];
   SweepArgs<WT> A;
@@ -1646,12 +1647,12 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   A.scanned = &c.d_sc->scanned;
   A.stats = c.d_sc;
   // the bins' sizes, the hub tables' size and the list's length in one read
-  int32_t ct = 0, cs = 0, cm = 0, cm2 = 0, cc = 0, ch = 0, nlist = 0;
+  int32_t bins[N_BINS] = {0}, nlist = 0;
+  const int32_t& ch = bins[0];
   int64_t tab = 0;
-  const HostRead rb[8] = {{c.cp[K_TINY], &ct, sizeof(int32_t)},  {c.cp[K_SMALL], &cs, sizeof(int32_t)},
-                          {c.cp[K_MID], &cm, sizeof(int32_t)},   {c.cp[K_MID2], &cm2, sizeof(int32_t)},
-                          {c.cp[K_CLU], &cc, sizeof(int32_t)},   {c.cp[K_LARGE], &ch, sizeof(int32_t)},
-                          {c.cp[idx_n], &nlist, sizeof(int32_t)}, {c.sums, &tab, sizeof(int64_t)}};
+  const HostRead rb[3] = {{c.cp[K_LARGE], bins, sizeof(bins)},
+                          {c.cp[idx_n], &nlist, sizeof(int32_t)},
+                          {c.sums, &tab, sizeof(int64_t)}};
   // Hub rows need their tables' size on the host before they are swept.  Where
   // the last sweep of this level and mode had none, the filter is launched
   // straight behind the sweeps and one read returns its outcome and the hub
@@ -1659,16 +1660,18 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   // which leaves its scratch as it found it, runs again on all candidates.
   uint8_t& expect = c.hubs_seen[r][MODE];
   // Few nodes are all swept by one block each, whatever their degree: a launch
-  // per degree bin costs more than it saves (see SWEEP_FEW).
-  const bool few = n_hint <= SWEEP_FEW && !c.kstats;
-  const bool fused = !few && n_hint <= SWEEP_FUSE && !c.kstats;
+  // per degree bin costs more than it saves (see SWEEP_FEW).  Statistics are
+  // kept per bin, so they take a launch per bin, but no other order of waits.
+  const bool is_short = n_hint <= SWEEP_FEW;
+  const bool few = is_short && !c.kstats;
+  const bool fused = !is_short && n_hint <= SWEEP_FUSE && !c.kstats;
   // The split is only launched ahead behind such short sweeps: they mostly end
   // the level's moves, and where moves are accepted its two launches are lost
   // (one edge on 10k vertices 508 -> 486 us a batch; with it behind every sweep,
   // batches of 10^3 and more on the R-MAT graphs lost up to 1%).
   if (spec) spec->done = false;
-  if (!few) spec = nullptr;
-  const bool early = expect || c.kstats;
+  if (!is_short) spec = nullptr;
+  const bool early = expect;
   launch(k_bin<WT>, grid_for(n_hint, TPB), TPB, 0, c.s, out, in, c.directed, list, c.cp[idx_n], c.binT.p, c.cp[K_TINY],
                                                      c.binS.p, c.cp[K_SMALL], c.binM.p, c.cp[K_MID], c.binM2.p,
                                                      c.cp[K_MID2], c.binC.p, c.cp[K_CLU], c.binL.p, c.cp[K_LARGE],
@@ -1676,7 +1679,7 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
                                                      few ? -1 : c.bin_deg[1], few ? -1 : c.bin_deg[2],
                                                      few ? MID_DEG : c.bin_deg[3],
                                                      std::min(c.prm.cluster_max_deg, CLUSTER_DEG),
-                                                     early ? tail_begin(c, rb, 8) : Tail{});
+                                                     early ? tail_begin(c, rb, 3) : Tail{});
   CKL("k_bin");
   // Every bin but the hubs is swept by a grid-stride kernel that reads its
   // bin's count on the device, so these launch before the counts come back
@@ -1695,12 +1698,9 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   }
   if (kev) CK(cudaEventRecord(kev[5], c.s));
   DecoupleOut dd{};
-  if (early) tail_wait(c, rb, 8);
-  else {
-    const HostRead ro[3] = {rb[5], rb[6], rb[7]};
-    dd = decouple(c, ro, 3, spec, r, true);
-  }
-  if (kev) CK(cudaEventRecord(kev[6], c.s));  // the wait above is charged to no kernel
+  if (early) tail_wait(c, rb, 3);
+  else dd = decouple(c, rb, 3, spec, r, true);
+  if (kev) CK(cudaEventRecord(kev[6], c.s));  // the wait above (and the filter) is charged to no kernel
   if (ch > 0) {
     // Hub tables hold 2..4 slots per entry.  When all hubs' tables together
     // exceed the slot budget (static builds of the largest graphs), the hubs
@@ -1778,11 +1778,7 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
     // times and bytes are resolved when the statistics are read, so that
     // collecting them adds no host synchronisation to the sweep
     CK(cudaEventRecord(kev[9], c.s));
-    c.ks_launch[0] += ct > 0;
-    c.ks_launch[1] += cs > 0;
-    c.ks_launch[2] += cm > 0;
-    c.ks_launch[3] += cm2 > 0;
-    c.ks_launch[4] += cc > 0;
+    for (int k = 0; k < 5; ++k) c.ks_launch[k] += bins[1 + k] > 0;
     c.ks_launch[5] += ch > 0;
     c.ks_launch[6] += ch > 0 ? 2 : 0;  // evaluation, final reduction with the clearing
   }
