@@ -76,10 +76,11 @@ typedef struct {
   int32_t gamma_num, gamma_den;
   int32_t N, L, M, M_static;
   int32_t alpha_inv, beta_inv;
-  /* Sweep scheduling (no effect on results): rows of 2049 .. cluster_max_deg
-   * entries (at most 32768) are swept by one 8-block cluster with a
-   * distributed shared-memory hash instead of the whole-GPU hub path;
-   * 0 (the default) keeps every row above 2048 entries on the hub path. */
+  /* Sweep scheduling (no effect on results): rows of bin_deg[3] + 1 (2049 by
+   * default) .. cluster_max_deg entries (at most 32768) are swept by one
+   * 8-block cluster with a distributed shared-memory hash instead of the
+   * whole-GPU hub path; 0 (the default) keeps every row above bin_deg[3]
+   * entries on the hub path. */
   int32_t cluster_max_deg;
   /* 1: collect the sweep kernel statistics (ldl_get_kernel_stats) from the
    * start, so that they cover the static build inside ldl_create; 0 (the
@@ -89,6 +90,13 @@ typedef struct {
    * adjacency entries (out + in) goes to 8-lane groups if d <= bin_deg[0],
    * one warp if d <= bin_deg[1], a 128-thread block if d <= bin_deg[2], a
    * 256-thread block if d <= bin_deg[3], else to the cluster / hub paths.
+   * How the first four are launched depends on the number of nodes that a
+   * sweep can have at most (known before it starts: in a level's first round
+   * the frontier and its row entries, later the number of vertices).  Up to
+   * 1024, one kernel gives every node of at most bin_deg[3] entries a
+   * 256-thread block, and the first three bounds do not apply; up to 131072,
+   * one kernel sweeps all four bins; beyond, and always while
+   * statistics are collected (kernel_stats), each bin has its own.
    * 0 keeps an entry's default (24, 96, 1024, 2048); the bounds must not
    * decrease and must not exceed (32, 128, 1024, 2048), the largest degrees
    * whose hash tables stay at most half full (LDL_E_INVALID otherwise). */

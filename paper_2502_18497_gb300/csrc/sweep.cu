@@ -31,7 +31,8 @@ static_assert(BIN_MAX[0] == HG8 / 2 && BIN_MAX[1] == HG32 / 2 && BIN_MAX[2] == 2
               "bin bounds and table sizes");
 // Nodes up to which a sweep uses one kernel for all degrees: one edge on 10k
 // vertices took 621 us a batch with a launch per bin, 531 with one; with 4096
-// here, batches of 100 to 1000 measure the same as with 1024 (within 1%).
+// here, batches of 100 to 1000 measure the same as with 1024 (within 1%).  The
+// last bound still says which rows go to clusters or the hub path.
 constexpr int SWEEP_FEW = 1024;
 // Nodes up to which a sweep runs all four bins in one launch (k_sweep_bins), so
 // that short bins fill one another's idle blocks instead of waiting for one
@@ -1677,7 +1678,7 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
                                                      c.cp[K_MID2], c.binC.p, c.cp[K_CLU], c.binL.p, c.cp[K_LARGE],
                                                      c.binLsz.p, c.sums, few ? -1 : c.bin_deg[0],
                                                      few ? -1 : c.bin_deg[1], few ? -1 : c.bin_deg[2],
-                                                     few ? MID_DEG : c.bin_deg[3],
+                                                     c.bin_deg[3],
                                                      std::min(c.prm.cluster_max_deg, CLUSTER_DEG),
                                                      early ? tail_begin(c, rb, 3) : Tail{});
   CKL("k_bin");

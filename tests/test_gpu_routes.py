@@ -4,7 +4,9 @@ sweeps a list, what runs ahead of the host and what statistics change.
 import numpy as np
 import pytest
 
-from synth import planted_partition, planted_stream, rmat_directed, rmat_stream
+from oracle import Oracle
+from synth import csr_from_arcs, planted_partition, planted_stream, rmat_directed, rmat_stream
+from tests.parity import compare_states
 
 pytestmark = pytest.mark.gpu
 
@@ -38,3 +40,34 @@ def test_statistics_add_no_host_wait(ldl, graph):
     ks = stats.kernel_stats()
     assert sum(k["launches"] for k in ks.values()) > 0
     assert (ks["sweep_hub_acc"]["launches"] > 0) == (graph == "rmat")
+
+
+def _long_row(n, deg, seed):
+    """A ring of 5-neighbour nodes and one node with `deg` entries."""
+    rng = np.random.default_rng(seed)
+    v = np.arange(1, n)
+    src = np.concatenate([np.repeat(v, 4), np.zeros(deg // 2, np.int64), 1 + rng.permutation(n - 1)[: deg - deg // 2]])
+    dst = np.concatenate([(1 + (v[:, None] + np.arange(4)) % (n - 1)).ravel(), 1 + rng.permutation(n - 1)[: deg // 2],
+                          np.zeros(deg - deg // 2, np.int64)])
+    keep = src != dst
+    key = np.unique(src[keep] * n + dst[keep])
+    return csr_from_arcs(n, key // n, key % n, np.ones(len(key), np.int64), True)
+
+
+# the caller's last bound holds in a sweep of few nodes too: a row above it goes
+# to a cluster where those are on, else to the hub path
+@pytest.mark.parametrize("cluster_max_deg,path", [(32768, "sweep_cluster"), (0, "sweep_hub_acc")])
+def test_last_bin_bound_holds_in_short_sweeps(ldl, cluster_max_deg, path):
+    g = _long_row(1000, 1500, 3)
+    o = Oracle(g)
+    d = ldl.LDL.from_graph(g, cluster_max_deg=cluster_max_deg, bin_deg=(24, 96, 1024, 1024))
+    for t, b in enumerate(([[0, 5, 0, 3], [7, 0, 0, 3]], [[0, 5, 1, 0], [9, 11, 0, 2]])):
+        b = np.array(b, np.int32)
+        d.set_kernel_stats(False)  # clears the counts, which go on without statistics
+        assert o.apply(b) == 0
+        d.apply(b)
+        msgs = compare_states(o, d, f"batch {t}")
+        assert not msgs, "\n".join(msgs[:8])
+        entries = {k: x["entries"] for k, x in d.kernel_stats().items()}
+        if t == 0:  # touches the long row
+            assert entries[path] >= 1500
