@@ -345,7 +345,8 @@ ldl_status ldl_stage_times(const ldl_ctx* ctx, double* times);
 ldl_status ldl_set_timing(ldl_ctx* ctx, int32_t on);
 
 /* Copies the last batch's changed vertices (ids) and their new labels to host
- * arrays of length n_changed (labels may be NULL). */
+ * arrays of length n_changed (labels may be NULL).  Several threads may call it
+ * at once on one context, while no other call on that context runs. */
 ldl_status ldl_copy_changed(const ldl_ctx* ctx, int32_t* ids, int32_t* labels);
 
 /*

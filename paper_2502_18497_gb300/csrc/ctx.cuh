@@ -1,6 +1,7 @@
 // The library context: device-resident hierarchy, community statistics and
 // the scratch of one LD-Leiden instance.
 #pragma once
+#include <mutex>
 #include <vector>
 
 #include "common.cuh"
@@ -168,6 +169,14 @@ struct ldl_ctx {
   volatile u64* h_pub = nullptr;
   u64* d_pub = nullptr;
   uint32_t pub_seq = 0, chg_seq = 0;
+  // one ldl_copy_changed at a time uses its words of the page; the lock stays
+  // where it is when contexts change places (ldl_grow)
+  struct Lock {
+    std::mutex m;
+    Lock() = default;
+    Lock(Lock&&) noexcept {}
+    Lock& operator=(Lock&&) noexcept { return *this; }
+  } chg_lock;
   std::string err;
   bool broken = false;  // a failed rollback left the state unknown
 

@@ -82,8 +82,8 @@ DeviceScope::~DeviceScope() {
 
 namespace {
 constexpr int PAGE_WORDS = 512;  // payload words per read
-// Behind them the words of ldl_copy_changed, with a sequence of their own: a
-// caller may ask for the labels while a server's worker reads on the context.
+// Behind them the words of ldl_copy_changed, with a sequence and a lock of
+// their own: between batches several threads may ask a context for them.
 constexpr int CHG_WORDS = 8192;
 
 // hands values of earlier kernels to the host (one block)
@@ -1266,6 +1266,7 @@ ldl_status ldl_copy_changed(const ldl_ctx* cc, int32_t* ids, int32_t* labels) {
     DeviceScope ds(c.dev);
     if (2 * k <= CHG_WORDS) {
       const int32_t n = (int32_t)k;
+      const std::lock_guard<std::mutex> one(c.chg_lock.m);
       volatile u64* const page = c.h_pub + PAGE_WORDS;
       const uint32_t seq = next_read(c.chg_seq, page, CHG_WORDS);
       launch(k_put_labels, grid_for(n, 256), 256, 0, c.s, c.lChg.p, n, labels ? c.lv[0].lab.p : nullptr,

@@ -1,6 +1,8 @@
 """GPU parity of the launch routes a batch can take (GB300 only): which kernel
 sweeps a list, what runs ahead of the host and what statistics change.
 """
+from concurrent.futures import ThreadPoolExecutor
+
 import numpy as np
 import pytest
 
@@ -71,3 +73,18 @@ def test_last_bin_bound_holds_in_short_sweeps(ldl, cluster_max_deg, path):
         entries = {k: x["entries"] for k, x in d.kernel_stats().items()}
         if t == 0:  # touches the long row
             assert entries[path] >= 1500
+
+
+# threads that read one batch's changed labels at the same time (4096 vertices
+# and fewer come through one mapped page)
+def test_changed_labels_read_by_several_threads(ldl):
+    g = rmat_directed(scale=14, arcs=1 << 18, seed=5)
+    d = ldl.LDL.from_graph(g)
+    for b in rmat_stream(g, batches=1, size=40, seed=40):
+        d.apply(b)
+    ids, lab = d.changed()
+    assert 0 < len(ids) <= 4096
+    with ThreadPoolExecutor(8) as pool:
+        got = list(pool.map(lambda _: d.changed(), range(400)))
+    for i, x in got:
+        assert np.array_equal(i, ids) and np.array_equal(x, lab)
