@@ -340,7 +340,8 @@ ldl_status ldl_get_communities(const ldl_ctx* ctx, int64_t* kout, int64_t* kin, 
 /* Device time in milliseconds spent in each stage since timing was last
  * enabled: [ingest, repair, expand, bestmove, decouple, commit, refine,
  * aggregate, pushdown]; `times` has room for 16.  ldl_set_timing(ctx, 1)
- * enables the events (one synchronisation per stage) and resets the sums. */
+ * enables the events (one synchronisation per stage, and no stage's kernels
+ * launched ahead of it) and resets the sums. */
 ldl_status ldl_stage_times(const ldl_ctx* ctx, double* times);
 ldl_status ldl_set_timing(ldl_ctx* ctx, int32_t on);
 

@@ -240,6 +240,7 @@ void stage_begin(ldl_ctx& c);
 void stage_end(ldl_ctx& c, int stage);
 enum { ST_INGEST = 0, ST_REPAIR, ST_EXPAND, ST_BEST, ST_DECOUPLE, ST_COMMIT, ST_REFINE, ST_AGG, ST_PUSH,
        SU_AGG_EMIT, SU_AGG_SORT, SU_AGG_APPLY, SU_AGG_UP, SU_AGG_EXIST, SU_REF_DISSOLVE, SU_REF_LOOP };
-// nested sub-stage timers (their own events)
+// nested sub-stage timers (their own events; SU_AGG_UP has no launch of its
+// own any more: strengths go up the chain with the records, in SU_AGG_EMIT)
 void sub_begin(ldl_ctx& c);
 void sub_end(ldl_ctx& c, int stage);

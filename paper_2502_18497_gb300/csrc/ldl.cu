@@ -676,7 +676,8 @@ static void apply_batch(ldl_ctx& c, const ldl_update* upd, int64_t count, int on
       }
       // A short pending list of the level is planned before
       // |U| is known: one wait for both (the plan does nothing if U is empty).
-      const bool eager = c.lv[r].pend_ub > 0 && c.lv[r].pend_ub <= FLUSH_EAGER;
+      // Not while stages are timed: the flush belongs to its own.
+      const bool eager = !c.timing && c.lv[r].pend_ub > 0 && c.lv[r].pend_ub <= FLUSH_EAGER;
       int64_t tot[6];
       if (eager) {
         frontier(c, r, epU, Tail{});

@@ -1670,9 +1670,10 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   // the level's moves, and where moves are accepted its two launches are lost
   // (one edge on 10k vertices 508 -> 486 us a batch; with it behind every sweep,
   // batches of 10^3 and more on the R-MAT graphs lost up to 1%).
+  // While stages are timed, filter and split wait for the stage that is theirs.
   if (spec) spec->done = false;
-  if (!is_short) spec = nullptr;
-  const bool early = expect;
+  if (!is_short || c.timing) spec = nullptr;
+  const bool early = expect || c.timing;
   launch(k_bin<WT>, grid_for(n_hint, TPB), TPB, 0, c.s, out, in, c.directed, list, c.cp[idx_n], c.binT.p, c.cp[K_TINY],
                                                      c.binS.p, c.cp[K_SMALL], c.binM.p, c.cp[K_MID], c.binM2.p,
                                                      c.cp[K_MID2], c.binC.p, c.cp[K_CLU], c.binL.p, c.cp[K_LARGE],

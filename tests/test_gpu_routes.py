@@ -88,3 +88,19 @@ def test_changed_labels_read_by_several_threads(ldl):
         got = list(pool.map(lambda _: d.changed(), range(400)))
     for i, x in got:
         assert np.array_equal(i, ids) and np.array_equal(x, lab)
+
+
+# every round's filter is charged to its own stage, and nothing but the order of
+# launches changes while stages are timed
+def test_stage_times_charge_the_filter(ldl):
+    g = planted_partition(n=3000, block=50, seed=3)
+    plain, timed = ldl.LDL.from_graph(g), ldl.LDL.from_graph(g)
+    timed.set_timing(True)
+    rounds = 0
+    for b in planted_stream(g, batches=4, size=40, seed=3, block=50):
+        plain.apply(b)
+        rounds += timed.apply(b).decouple_rounds
+        assert np.array_equal(plain.labels(), timed.labels())
+    assert rounds > 0
+    times = timed.stage_times()
+    assert times["decouple"] > 0 and times["aggregate"] >= times["agg.emit"] > 0
