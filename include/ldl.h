@@ -434,6 +434,12 @@ ldl_status ldl_debug_sort_pairs(ldl_ctx* ctx, int64_t count, uint64_t* keys, uin
  * graphs take that path.  Process-wide. */
 void ldl_debug_hub_table_slots(int64_t slots);
 
+/* Test hook: the words of the counter arena that a batch or a static build may
+ * use (default and most 8192; words < 0 restores it).  Beyond them counters
+ * live at fixed places that a memset clears; a small value makes ordinary
+ * batches take that path.  Process-wide; set it between calls. */
+void ldl_debug_arena_words(int64_t words);
+
 /* Test hook for the bounded waits: runs a two-tile device scan in which the
  * first tile never publishes its sum, so the second tile's look-back wait
  * runs out (after about 2^20 polls).  Returns LDL_E_TIMEOUT when the wait gave

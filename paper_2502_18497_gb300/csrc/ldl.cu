@@ -178,8 +178,11 @@ int32_t rd_cnt(ldl_ctx& c, int idx) {
   return v;
 }
 
+// arena words in use (a test hook lowers it)
+static std::atomic<int32_t> g_arena_words{ARENA_WORDS};
+
 void zero_cnts(ldl_ctx& c, int first, int n) {
-  const bool fits = c.arena_top + n <= ARENA_WORDS;
+  const bool fits = c.arena_top + n <= g_arena_words.load(std::memory_order_relaxed);
   int32_t* const at = fits ? c.arena + c.arena_top : c.dcnt + first;
   for (int k = 0; k < n; ++k) c.cp[first + k] = at + k;
   if (fits) c.arena_top += n;
@@ -190,7 +193,7 @@ void zero_cnt(ldl_ctx& c, int idx) { zero_cnts(c, idx, 1); }
 
 void* fresh(ldl_ctx& c, int words, void* home) {
   const int at = (c.arena_top + 3) & ~3;
-  if (at + words <= ARENA_WORDS) {
+  if (at + words <= g_arena_words.load(std::memory_order_relaxed)) {
     c.arena_top = at + words;
     return c.arena + at;
   }
@@ -1152,6 +1155,10 @@ ldl_status ldl_set_timing(ldl_ctx* c, int32_t on) {
 }
 
 void ldl_debug_fail_alloc_after(int64_t k) { g_fail_after.store(k > 0 ? k : 0); }
+
+void ldl_debug_arena_words(int64_t words) {
+  g_arena_words.store(words < 0 ? ARENA_WORDS : (int32_t)std::min<int64_t>(words, ARENA_WORDS));
+}
 
 void ldl_debug_alloc_counts(int64_t* all, int64_t* in_batch) {
   if (all) *all = g_allocs.load();

@@ -104,3 +104,31 @@ def test_stage_times_charge_the_filter(ldl):
     assert rounds > 0
     times = timed.stage_times()
     assert times["decouple"] > 0 and times["aggregate"] >= times["agg.emit"] > 0
+
+
+# counters beyond the arena live at their home words: from the start, and from
+# some way into a batch; static build and batches with hub rows and more than
+# 8192 candidates in a sweep, and with rolled-back mini-batches
+@pytest.mark.parametrize("words", [0, 64, 500])
+@pytest.mark.parametrize("what", ["hubs", "rollbacks"])
+def test_counters_beyond_the_arena(ldl, words, what):
+    if what == "hubs":
+        g, size = rmat_directed(scale=14, arcs=1 << 18, seed=12), 1000
+        assert Oracle(g, L=0, M_static=1).counters()["candidates"] > 8192
+    else:
+        g, size = rmat_directed(scale=12, arcs=1 << 15, seed=0), 300
+    o = Oracle(g)
+    ldl.load().ldl_debug_arena_words(words)
+    try:
+        d = ldl.LDL.from_graph(g)
+        msgs = compare_states(o, d, "create")
+        assert not msgs, "\n".join(msgs[:8])
+        before = o.counters()["rollbacks"]
+        for t, b in enumerate(rmat_stream(g, batches=3, size=size, seed=12 if what == "hubs" else 0)):
+            assert o.apply(b) == 0
+            d.apply(b)
+            msgs = compare_states(o, d, f"batch {t}")
+            assert not msgs, "\n".join(msgs[:8])
+    finally:
+        ldl.load().ldl_debug_arena_words(-1)
+    assert what == "hubs" or o.counters()["rollbacks"] > before > 0
