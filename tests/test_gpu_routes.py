@@ -132,3 +132,67 @@ def test_counters_beyond_the_arena(ldl, words, what):
     finally:
         ldl.load().ldl_debug_arena_words(-1)
     assert what == "hubs" or o.counters()["rollbacks"] > before > 0
+
+
+# the routes a user's batches take (statistics off) with clusters and non-default
+# bins: rows above the last bound in lists of a few nodes and of thousands
+@pytest.mark.parametrize("cluster_max_deg,bin_deg", [(32768, None), (0, (16, 64, 256, 1024)),
+                                                     (4096, (8, 8, 32, 100))])
+@pytest.mark.parametrize("size", [3, 1000])
+def test_bins_and_clusters_without_statistics(ldl, cluster_max_deg, bin_deg, size):
+    g = rmat_directed(scale=14, arcs=1 << 18, seed=12)
+    o = Oracle(g)
+    d = ldl.LDL.from_graph(g, cluster_max_deg=cluster_max_deg, bin_deg=bin_deg)
+    for t, b in enumerate(rmat_stream(g, batches=6, size=size, seed=12)):
+        assert o.apply(b) == 0
+        d.apply(b)
+        msgs = compare_states(o, d, f"batch {t}")
+        assert not msgs, "\n".join(msgs[:8])
+
+
+def _star_and_rings(directed, leaves=2500, rings=1500):
+    """Node 0 with `leaves` neighbours, each of them in a pair, and rings of ten
+    nodes far from it."""
+    v = np.arange(1, leaves + 1)
+    w = leaves + 1 + np.arange(rings)
+    ring = w - (w - leaves - 1) % 10
+    src = np.concatenate([np.zeros(leaves, np.int64), v[::2], w])
+    dst = np.concatenate([v, v[1::2], ring + (w - ring + 1) % 10])
+    wt = np.concatenate([np.ones(leaves, np.int64), np.full(leaves // 2, 3), np.full(rings, 2)])
+    if not directed:
+        src, dst = np.minimum(src, dst), np.maximum(src, dst)
+    order = np.argsort(src * 10_000 + dst)
+    return csr_from_arcs(leaves + rings + 1, src[order], dst[order], wt[order], directed)
+
+
+# a short sweep meets a hub row where the sweep before it had none: the filter
+# and the split that were launched ahead give way to the hub path (or, with
+# clusters on, stand), in batches that move nodes and in batches that do not
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("cluster_max_deg", [0, 32768])
+def test_hub_row_appears_in_a_short_sweep(ldl, directed, cluster_max_deg):
+    g = _star_and_rings(directed)
+    o, d = Oracle(g), ldl.LDL.from_graph(g, cluster_max_deg=cluster_max_deg)
+    path = "sweep_cluster" if cluster_max_deg else "sweep_hub_acc"
+    far = 2600
+    batches = [
+        ([[far, far + 25, 0, 1]], False),
+        ([[1, 4, 0, 1]], True),  # two leaves of different pairs
+        ([[far, far + 25, 1, 0]], False),
+        ([[1, 2, 1, 0], [1, 4, 2, 9], [2, 3, 0, 9]], True),
+        ([[far + 40, far + 77, 0, 50], [far + 41, far + 78, 0, 50]], False),
+        ([[5, 6, 1, 0], [5, far + 3, 0, 4]], True),
+        ([[far + 3, far + 200, 0, 30]], None),
+        ([[0, 9, 2, 20]], True),  # the hub itself
+    ]
+    moves = []
+    for t, (b, hub) in enumerate(batches):
+        b = np.array(b, np.int32)
+        d.set_kernel_stats(False)  # clears the counts, which go on without statistics
+        assert o.apply(b) == 0
+        moves.append(d.apply(b).moves)
+        msgs = compare_states(o, d, f"batch {t}")
+        assert not msgs, "\n".join(msgs[:8])
+        if hub is not None:
+            assert (d.kernel_stats()[path]["entries"] > 0) == hub, f"batch {t}"
+    assert min(moves) == 0 < max(moves)
