@@ -94,7 +94,7 @@ typedef struct {
    * sweep can have at most (known before it starts: in a level's first round
    * the frontier and its row entries, later the number of vertices).  Up to
    * 1024, one kernel gives every node of at most bin_deg[3] entries a
-   * 256-thread block, and the first three bounds do not apply; up to 131072,
+   * 256-thread block, and the first three bounds do not apply; up to 262144,
    * one kernel sweeps all four bins; beyond, and always while
    * statistics are collected (kernel_stats), each bin has its own.
    * 0 keeps an entry's default (24, 96, 1024, 2048); the bounds must not

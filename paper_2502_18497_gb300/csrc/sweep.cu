@@ -29,20 +29,30 @@ std::atomic<int64_t> g_hub_table_slots{HUB_TABLE_SLOTS};
 static_assert(BIN_MAX[0] == HG8 / 2 && BIN_MAX[1] == HG32 / 2 && BIN_MAX[2] == 2048 / 2 &&
                   BIN_MAX[3] == HB / 2 && BIN_MAX[3] == MID_DEG,
               "bin bounds and table sizes");
-// Nodes up to which a sweep uses one kernel for all degrees: one edge on 10k
-// vertices took 621 us a batch with a launch per bin, 531 with one; with 4096
-// here, batches of 100 to 1000 measure the same as with 1024 (within 1%).  The
-// last bound still says which rows go to clusters or the hub path.
+// Bound of the list up to which a sweep uses one kernel for all degrees (the
+// bound the host has when it launches: in a level's first round the frontier and
+// its row entries, later the number of vertices).  One edge on 10k vertices took
+// 621 us a batch with a launch per bin, 531 with one; with 4096 here, batches of
+// 100 to 1000 measure the same as with 1024 (within 1%).  The last bin bound
+// still says which rows go to clusters or the hub path.
 constexpr int SWEEP_FEW = 1024;
-// Nodes up to which a sweep runs all four bins in one launch (k_sweep_bins), so
-// that short bins fill one another's idle blocks instead of waiting for one
-// another.  Against a launch per bin: a batch of 100 on 10k vertices 673 -> 626
-// us, 500 on 131k 1040 -> 994, 10^3 on the R-MAT of 131k 1782 -> 1730.  Above,
-// the groups' own kernel pays with its 6 blocks an SM to 4: with every sweep in
-// one launch a batch of 10^4 on the R-MAT of 2^20 took 4490-4600 us where this
-// bound takes 4310-4350, and one of 10^5 on the 2M-vertex power-law graph
-// 4740-4900 where it takes 4410-4650.
-constexpr int64_t SWEEP_FUSE = 131072;
+// The same bound up to which a sweep runs all four bins in one launch
+// (k_sweep_bins), so that short bins fill one another's idle blocks instead of
+// waiting for one another; with long bins the groups' own kernel pays with its 6
+// blocks an SM to 4.  As later rounds are bounded by the vertex count, the line
+// mostly tells graphs apart.  One launch for every sweep against a launch per
+// bin, in batches of 10^2, 10^3 and 10^4:
+//   vertices    R-MAT, 16 arcs a vertex    power law, 32 neighbours
+//   150k        0.990 .. 0.993             0.944 .. 0.958
+//   250k        0.989 .. 0.996             0.946 .. 0.972
+//   400k        1.004 .. 1.020             0.956 .. 0.975
+//   600k        1.036 .. 1.042             0.953 .. 0.986
+//   900k        1.025 .. 1.036             0.976 .. 1.002
+// (times as a share of the launch per bin's, 0.9 to 5.2 ms a batch, two runs of
+// one side within 0.5% but for one pair of 2.4%); at 200k and 262k vertices, 20
+// and 10^3 updates, planted graphs 0.957 .. 0.986, R-MATs of 8 and 32 neighbours
+// 0.970 .. 0.998.  Below the line no graph loses.
+constexpr int64_t SWEEP_FUSE = 262144;
 // Hub entries per block of the accumulation (four chunks for its eight warps).
 // The grid follows the tables' size, which is 2..4 slots an entry; with eight
 // blocks per hub a few rows of 10^5 entries were walked by 64 warps each, one

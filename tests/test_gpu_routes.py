@@ -7,8 +7,10 @@ import numpy as np
 import pytest
 
 from oracle import Oracle
-from synth import csr_from_arcs, planted_partition, planted_stream, rmat_directed, rmat_stream
+from synth import (EdgeStream, csr_from_arcs, planted_partition, planted_stream, random_batch, rmat_directed,
+                   rmat_stream)
 from tests.parity import compare_states
+from tests.test_gpu_edges import _bin_edge_graph, _unit
 
 pytestmark = pytest.mark.gpu
 
@@ -73,6 +75,21 @@ def test_last_bin_bound_holds_in_short_sweeps(ldl, cluster_max_deg, path):
         entries = {k: x["entries"] for k, x in d.kernel_stats().items()}
         if t == 0:  # touches the long row
             assert entries[path] >= 1500
+
+
+# one launch for all bins up to 262144 nodes, a launch per bin above
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("n", [262144, 262145])
+def test_one_launch_or_a_launch_per_bin(ldl, directed, n):
+    g = _bin_edge_graph(directed, _unit, 7, n)
+    o, d = Oracle(g), ldl.LDL.from_graph(g)
+    msgs = compare_states(o, d, "create")
+    assert not msgs, "\n".join(msgs[:8])
+    b = random_batch(EdgeStream.from_graph(g, 3), 60, 40, 20, 2, 5)
+    assert o.apply(b) == 0
+    d.apply(b)
+    msgs = compare_states(o, d, "batch")
+    assert not msgs, "\n".join(msgs[:8])
 
 
 # threads that read one batch's changed labels at the same time (4096 vertices
