@@ -247,13 +247,6 @@ struct Chain {
   int32_t* np[8];         // pending records of level q
 };
 
-// Weight records (keys, vals) of level q0 carried up the hierarchy: with
-// `self` a record joins level q0's pending list; mapped through pi_q0,
-// pi_q0+1, ... it joins the pending list of every level above up to `top`,
-// until an endpoint has no parent (W_{q+1}(pi(i), pi(j)) takes the weight of
-// every level-q arc (i, j)).  With `add_k` the strengths of those levels take
-// the weight as well.  Records are not reduced here: the pending list of a
-// level is sorted, summed and applied when the level is next read.
 // Warp-aggregated append of one record per lane that wants one (every lane
 // of the warp calls it together): one atomic per warp.
 __device__ inline void warp_append_rec(bool want, u64 key, int64_t v, u64* pk, u64* pv, int32_t* count) {
@@ -271,6 +264,13 @@ __device__ inline void warp_append_rec(bool want, u64 key, int64_t v, u64* pk, u
   }
 }
 
+// Weight records (keys, vals) of level q0 carried up the hierarchy: with
+// `self` a record joins level q0's pending list; mapped through pi_q0,
+// pi_q0+1, ... it joins the pending list of every level above up to `top`,
+// until an endpoint has no parent (W_{q+1}(pi(i), pi(j)) takes the weight of
+// every level-q arc (i, j)).  With `add_k` the strengths of those levels take
+// the weight as well.  Records are not reduced here: the pending list of a
+// level is sorted, summed and applied when the level is next read.
 __global__ void k_chain_records(const u64* keys, const int64_t* vals, int64_t n, const int32_t* n_dev, int bits, int q0, int top, int self,
                                 int add_k, int directed, Chain ch) {
   pdl_enter();
@@ -982,7 +982,6 @@ __global__ void k_alive_list(const uint8_t* alive, int64_t n, int32_t* l, int32_
   }
 }
 
-
 __global__ void k_esum(const int64_t* e, const int64_t* Kout, const int64_t* Kin, int64_t n, int64_t* E, I128* P) {
   pdl_enter();
   int64_t se = 0;
@@ -1436,7 +1435,7 @@ int32_t split(ldl_ctx& c, int r, SplitRun& sr) {
 }
 
 // deg: out-row and in-row entries of the changed nodes (k_changed); returns
-// the bound on the records (their count is at dcnt[K_REC])
+// the bound on the records (their count is at cp[K_REC])
 template <class WT>
 static int64_t emit_records(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, int32_t nC, int32_t epC, bool build,
                             const int64_t (&deg)[2]) {
@@ -1481,7 +1480,7 @@ void aggregate(ldl_ctx& c, int r, int32_t epD, int32_t epC, int32_t epA_next, bo
     CKL("k_changed");
     tail_wait(c, rr, 2);
   }
-  int64_t nr = 0;  // bound on the level r+1 records (their number is at dcnt[K_NR])
+  int64_t nr = 0;  // bound on the level r+1 records (their number is at cp[K_NR])
   if (nC > 0) {
     int64_t nrec = r == 0 ? emit_records<int32_t>(c, r, adj_out0(c), adj_in0(c), nC, epC, build, deg)
                           : emit_records<int64_t>(c, r, adj_out(c, r), adj_in(c, r), nC, epC, build, deg);

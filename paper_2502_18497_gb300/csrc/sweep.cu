@@ -491,11 +491,6 @@ __global__ void __launch_bounds__(TPB, wide_sums<GT> ? 4 : 6) k_sweep_group(Swee
   sweep_groups<WT, MODE, G, GT>(A, list, *nlist, smem, blockIdx.x);
 }
 
-// Entries of a node's rows staged in registers: entry k of the node is its
-// out-row entry k (k < lo) or its in-row entry k - lo; thread tid holds the
-// entries tid + j * NT.  First the neighbour ids and weights ...
-// Steps in which a warp has no entry are skipped by the whole warp: most rows
-// of a bin are far shorter than its longest.
 // Barrier of a block of NT threads, or of half `bar` of a block of 2 * NT.
 template <int NT>
 __device__ inline void sub_sync(int bar) {
@@ -503,6 +498,11 @@ __device__ inline void sub_sync(int bar) {
   else asm volatile("bar.sync %0, %1;" ::"r"(bar + 1), "r"(NT) : "memory");
 }
 
+// Entries of a node's rows staged in registers: entry k of the node is its
+// out-row entry k (k < lo) or its in-row entry k - lo; thread tid holds the
+// entries tid + j * NT.  First the neighbour ids and weights ...
+// Steps in which a warp has no entry are skipped by the whole warp: most rows
+// of a bin are far shorter than its longest.
 template <class WT, int NT, bool DIR, int ACC, class SW>
 __device__ inline void stage_rows(const SweepArgs<WT>& A, const NodeMeta& m, int tid, int32_t (&u)[ACC], SW (&w)[ACC]) {
   const int32_t l = DIR ? m.lo + m.li : m.lo, w0 = tid & ~31;
@@ -550,8 +550,8 @@ __device__ inline void stage_keys(const SweepArgs<WT>& A, int32_t v, int32_t a, 
 // nodes: the row entries and labels of the next node are loaded into
 // registers while the current node's table is evaluated, and the node after
 // that has its offsets, lengths and strengths loaded one node further ahead,
-// so a node's fill only inserts into shared memory.  Entries beyond the
-// staged HMAX/2 (not produced by the default bins) are inserted directly.
+// so a node's fill only inserts into shared memory.  The bins' bounds keep every
+// row within the HMAX / 2 staged entries.
 // With the evaluation emptying the table, two barriers a node instead of
 // four: 263 -> 215 us for the rows of 97..1024 entries of a 10^5 batch on the
 // 2M-vertex power-law graph, 249 -> 214 us for 10^4 on the R-MAT of 2^20.
@@ -593,16 +593,6 @@ __device__ inline void sweep_blocks(const SweepArgs<WT>& A, const int32_t* list,
       if ((tid & ~31) + j * NT >= d) continue;  // the whole warp
       if (MODE == 0 && ek[j] == a) own += ew[j];
       else if (ek[j] >= 0) T.add(H - 1, ek[j], ew[j]);
-    }
-    if (d > ACC * NT) {  // entries beyond the staged ones
-      for (int64_t k = ACC * NT + tid; k < d; k += NT) {
-        const int64_t at = (k < cur.lo ? cur.oo : cur.oi - cur.lo) + k;
-        const int64_t wx = (int64_t)A.out.w[at];
-        int32_t kx[1] = {A.out.col[at]};
-        stage_keys<WT, MODE, 0>(A, v, a, INT32_MAX, tid, kx);
-        if (MODE == 0 && kx[0] == a) own += (StageW<GT>)wx;
-        else if (kx[0] >= 0) T.add(H - 1, kx[0], wx);
-      }
     }
     if (MODE == 0) {
       if constexpr (WIDE) own = warp_sum_i64(own);
@@ -1569,7 +1559,6 @@ void union_into(ldl_ctx& c, const int32_t* list, int idx_n, int32_t* stamp, int3
   CKL("k_union");
 }
 
-// the next KS_EVENTS statistics events of the context, created on first use
 // No exact gain of a sweep, nor any intermediate product of it, reaches 2^62
 // when (2 gamma_den + 4 gamma_num) m^2 < 2^62: |w(v,.)| <= m, strengths and
 // totals are at most m, so gd*m*|dw| <= 2 gd m^2 and gn*|dd| <= 4 gn m^2.
@@ -1612,6 +1601,7 @@ static void sweep_bins(ldl_ctx& c, const SweepArgs<WT>& A, int64_t n_hint, bool 
   }
 }
 
+// the next KS_EVENTS statistics events of the context, created on first use
 static cudaEvent_t* kstats_events(ldl_ctx& c) {
   while (c.kev.size() < c.kev_used + KS_EVENTS) {
     cudaEvent_t e;
