@@ -303,7 +303,8 @@ bool read_image(Image& im, const char* path, std::string& why) {
   im.lv.assign((size_t)im.T + 1, LevelImage());
   for (LevelImage& I : im.lv) {
     r.vec(I.lab, n); r.vec(I.par, n); r.vec(I.cnt, n); r.vec(I.kout, n); r.vec(I.kin, n); r.vec(I.alive, n);
-    r.vec(I.rp, 2 * n + 1); r.vec(I.col, big); r.vec(I.w, big); r.vec(I.crp, n + 1); r.vec(I.ccol, n);
+    // (emptied nodes stay in the children lists, so those may hold more than n ids)
+    r.vec(I.rp, 2 * n + 1); r.vec(I.col, big); r.vec(I.w, big); r.vec(I.crp, n + 1); r.vec(I.ccol, big);
   }
   fclose(f);
   if (!r.ok) {
