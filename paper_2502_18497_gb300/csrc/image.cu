@@ -226,15 +226,26 @@ struct Writer {
 
 struct Reader {
   FILE* f;
+  int64_t left = INT64_MAX;  // bytes to come (unknown where the file cannot be positioned)
   bool ok = true;
-  void raw(void* p, size_t b) { ok = ok && (b == 0 || fread(p, 1, b, f) == b); }
+  explicit Reader(FILE* file) : f(file) {
+    if (fseek(f, 0, SEEK_END) != 0) return;
+    const long size = ftell(f);
+    if (size >= 0) left = size;
+    ok = fseek(f, 0, SEEK_SET) == 0;
+  }
+  void raw(void* p, size_t b) {
+    ok = ok && (int64_t)b <= left && (b == 0 || fread(p, 1, b, f) == b);
+    if (ok) left -= (int64_t)b;
+  }
   template <class T>
   void val(T& v) { raw(&v, sizeof(T)); }
   template <class T>
   void vec(std::vector<T>& v, int64_t limit) {
     int64_t k = -1;
     val(k);
-    if (!ok || k < 0 || k > limit) {
+    // (a count beyond the file would be allocated before the read fails)
+    if (!ok || k < 0 || k > limit || k > left / (int64_t)sizeof(T)) {
       ok = false;
       return;
     }
@@ -274,7 +285,7 @@ bool read_image(Image& im, const char* path, std::string& why) {
     why = "cannot open the file";
     return false;
   }
-  Reader r{f};
+  Reader r(f);
   char magic[8];
   r.raw(magic, sizeof magic);
   if (!r.ok || memcmp(magic, MAGIC, sizeof magic) != 0) {
