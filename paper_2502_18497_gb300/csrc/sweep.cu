@@ -1660,7 +1660,7 @@ static SweepOut sweep_t(ldl_ctx& c, int r, Adj<WT> out, Adj<WT> in, const int32_
   // count; should there be hubs after all, they are swept and the filter,
   // which leaves its scratch as it found it, runs again on all candidates.
   uint8_t& expect = c.hubs_seen[r][MODE];
-  // Few nodes are all swept by one block each, whatever their degree: a launch
+  // Few nodes are swept by one block each, up to the last bin bound: a launch
   // per degree bin costs more than it saves (see SWEEP_FEW).  Statistics are
   // kept per bin, so they take a launch per bin, but no other order of waits.
   const bool is_short = n_hint <= SWEEP_FEW;
