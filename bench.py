@@ -46,10 +46,10 @@ WORKLOAD = ("directed R-MAT (0.57,0.19,0.19,0.05), 2^20 vertices, 2^24 arcs, wei
 # DRAM traffic of the dominant sweep kernel from one ncu capture (dram bytes
 # read + written, summed over its launches in one timed step of the default
 # workload, divided by the launches that had nodes to sweep: the bins are
-# launched unconditionally and an empty launch moves ~23 KB), valid only for
+# launched unconditionally and an empty launch moves ~35 KB), valid only for
 # the sweep source it was taken with (sha256 of csrc/sweep.cu).
-NCU_TRAFFIC = {"sha256": "8818a9a99634cdc5b9b9f596981ec682ba71cc56abc199442c4b2f8969263ca9",
-               "bytes_per_launch": 45175268, "kernel": "sweep_block128"}
+NCU_TRAFFIC = {"sha256": "982760979872ea71583c4e019b2f848076e14d37d424db7f106d5316680734a0",
+               "bytes_per_launch": 45268196, "kernel": "sweep_block128"}
 
 
 def _set_rmat_scale(scale: int):
